@@ -38,6 +38,11 @@ cudaError_t launch_phase_tc(int mode, const Plan &p, void *ws, const double *alp
 cudaError_t launch_w_from_phi(const Plan &p, void *ws, const double *alpha, const double *beta, cudaStream_t st);
 cudaError_t launch_grad_tc(const Plan &p, void *ws, cudaStream_t st, iqp_status *why);
 int64_t grad_tc_rows(const Plan &p);
+bool x3_available();
+cudaError_t launch_x3_theta(const Plan &p, void *ws, const float *theta, cudaStream_t st);
+cudaError_t launch_phase_x3(int mode, const Plan &p, void *ws, const double *alpha, const double *beta,
+                            cudaStream_t st, iqp_status *why);
+cudaError_t launch_grad_x3(const Plan &p, void *ws, cudaStream_t st, iqp_status *why);
 // per-translation-unit self-check words (builds with -DIQP_CHECKS; 0 otherwise)
 uint32_t check_word_parity();
 uint32_t check_word_simt();
@@ -171,8 +176,29 @@ Plan make_plan(int op, int64_t n, int64_t m, int64_t l, int64_t s, int64_t N, in
     // them runs one sample tile per tile), and the scratch of their balanced
     // last round (a workspace that ends before it runs that round as single
     // tiles).
-    p.off_skp = p.off_gsum = p.off_skx = 0;
+    p.off_skp = p.off_gsum = p.off_skx = p.off_opt = 0;
+    p.x3 = false;
+    // FP32: the regions of its tensor-core form (a workspace that ends before
+    // their end runs the SIMT kernels).
+    if (prec == IQP_FP32 && !bitflip && !indep) {
+        p.off_opt = off;
+        p.off_xc = take(3 * p.mpad * 2);
+        p.off_xmax = take(128 * 4);
+        p.off_xpart = take(l * cdiv(s, (int64_t)kPartColsTc) * 16);
+        p.off_xrow = take(grad ? l * 4 : 0);
+        p.off_xw = take(grad ? 3 * l * p.ldw * 2 : 0);
+        p.off_skp = take((int64_t)kMaxSplitCtas * kSplitSlotFloats * 4 + (int64_t)kMaxSplitCtas * 4);
+        // running sums: only where the gates take more than one accumulation chunk
+        p.off_xsum = take(m > 65536 ? (int64_t)kMaxSplitCtas * kSplitSlotFloats * 4 : 0);
+        // Below 2^23 terms (and, where a gradient follows, at most 1024
+        // samples) the SIMT kernels' few tiles take no longer than the tensor
+        // form's launches do: at n = 8, m = 36, l = 64, s = 1024 a step is 0.52 ms of
+        // host time either way, 25 us more of it with the tensor maps. Past that
+        // the SIMT gradient's serial loop (4.6 us per 32 samples) decides.
+        p.x3 = x3_available() && ((double)l * (double)s * (double)m >= 8388608.0 || (grad && s > 1024));
+    }
     if (prec == IQP_SPLIT_BF16 && !bitflip && !indep) {
+        p.off_opt = off;
         p.off_skp = take((int64_t)kMaxSplitCtas * kSplitSlotFloats * 4 + (int64_t)kMaxSplitCtas * 4);
         p.off_gsum = take((int64_t)kMaxSplitCtas * kDtSumFloats * 4);
         p.off_skx = take((int64_t)kSplitSlots * kSplitSlotFloats * 4 + (int64_t)kMaxSplitCtas * 4);
@@ -183,7 +209,7 @@ Plan make_plan(int op, int64_t n, int64_t m, int64_t l, int64_t s, int64_t N, in
 
 // Bytes of the workspace below which `p` cannot run (the optional regions at
 // its end left out).
-size_t plan_min_bytes(const Plan &p) { return p.off_skp != 0 ? p.off_skp : p.total; }
+size_t plan_min_bytes(const Plan &p) { return p.off_opt != 0 ? p.off_opt : p.total; }
 
 // The smallest workspace `op` runs with (iqp_workspace_bytes less the
 // optional split-tile scratch at its end); 0 for invalid arguments (the
@@ -304,6 +330,7 @@ iqp_status check_ws(Plan &p, void *ws, size_t ws_bytes) {
     if (ws == nullptr || !aligned(ws, 256)) return IQP_ERR_WORKSPACE;
     if (ws_bytes < p.total) {
         if (ws_bytes < plan_min_bytes(p)) return IQP_ERR_WORKSPACE;
+        p.x3 = false;  // FP32: the SIMT kernels
         // The optional regions at the end, in order: each is used only where
         // the workspace reaches its end.
         p.off_skx = 0;  // the two-tile last round runs as single tiles
@@ -352,6 +379,8 @@ iqp_status prepare(const Plan &p, void *ws, const uint64_t *G, int64_t ldg, cons
         if (p.prec == IQP_SPLIT_BF16) {
             __nv_bfloat16 *hi = at<__nv_bfloat16>(ws, p.off_c);
             IQP_TRY(launch_theta_prep(theta, p.m, p.mpad, nullptr, hi, hi + p.mpad, st));
+        } else if (p.x3) {
+            IQP_TRY(launch_x3_theta(p, ws, theta, st));
         } else {
             IQP_TRY(launch_theta_prep(theta, p.m, p.mpad, at<float>(ws, p.off_c), nullptr, nullptr, st));
         }
@@ -396,6 +425,13 @@ iqp_status forward_stats(const Plan &p, void *ws, double *expval, double *std_er
                                     at<uint64_t>(ws, p.indep ? p.off_zt : p.off_pzt), p.ldzt, at<float>(ws, p.off_c),
                                     p.l, p.s, p.m, part, p.nparts, p.indep ? &ind : nullptr,
                                     p.phi_out ? p.phi : nullptr, p.ldphi, st));
+    } else if (p.x3) {
+        iqp_status why = IQP_OK;
+        if (launch_phase_x3(0, p, ws, nullptr, nullptr, st, &why) != cudaSuccess)
+            return why != IQP_OK ? why : IQP_ERR_CUDA;
+        IQP_TRY(launch_finalize(at<double2>(ws, p.off_xpart), cdiv(p.s, (int64_t)kPartColsTc), kPartColsTc, p.l, p.s,
+                                expval, std_err, S1, S2, st));
+        return IQP_OK;
     } else {
         IQP_TRY(launch_phase_simt(0, at<uint64_t>(ws, p.off_pa), at<uint64_t>(ws, p.off_pz), p.ldp,
                                   at<float>(ws, p.off_c), p.l, p.s, p.m, part, p.nparts, nullptr, nullptr, nullptr, 0,
@@ -435,6 +471,13 @@ iqp_status backward(const Plan &p, void *ws, const double *alpha, const double *
             return why != IQP_OK ? why : IQP_ERR_CUDA;
         }
         if (launch_grad_tc(p, ws, st, &why) != cudaSuccess) return why != IQP_OK ? why : IQP_ERR_CUDA;
+    } else if (p.x3) {
+        iqp_status why = IQP_OK;
+        if (launch_phase_x3(1, p, ws, alpha, beta, st, &why) != cudaSuccess ||
+            launch_grad_x3(p, ws, st, &why) != cudaSuccess)
+            return why != IQP_OK ? why : IQP_ERR_CUDA;
+        IQP_TRY(launch_grad_reduce(gpart, 2 * cdiv(p.l, kATile), p.m, grad, st));
+        return IQP_OK;
     } else {
         float *W = at<float>(ws, p.off_w);
         IQP_TRY(launch_phase_simt(1, at<uint64_t>(ws, p.off_pa), at<uint64_t>(ws, p.off_pz), p.ldp,
@@ -686,6 +729,15 @@ iqp_status iqp_expval_value_and_grad(int64_t n, const uint64_t *G, int64_t m, in
                                          at<float>(ws, p.off_c), p.l, p.s, p.m, p.nparts, part, alpha, beta,
                                          reinterpret_cast<double *>(gfx + p.m), gfx, grad, st));
         IQP_TRY(launch_finalize(part, p.nparts, p.pw, p.l, p.s, expval, std_err, nullptr, nullptr, st));
+        return IQP_OK;
+    }
+    if (p.x3) {  // one pass: the statistics and W
+        iqp_status why = IQP_OK;
+        if (launch_phase_x3(2, p, ws, alpha, beta, st, &why) != cudaSuccess) return why != IQP_OK ? why : IQP_ERR_CUDA;
+        IQP_TRY(launch_finalize(at<double2>(ws, p.off_xpart), cdiv(p.s, (int64_t)kPartColsTc), kPartColsTc, p.l, p.s,
+                                expval, std_err, nullptr, nullptr, st));
+        if (launch_grad_x3(p, ws, st, &why) != cudaSuccess) return why != IQP_OK ? why : IQP_ERR_CUDA;
+        IQP_TRY(launch_grad_reduce(at<double>(ws, p.off_gpart), 2 * cdiv(p.l, kATile), p.m, grad, st));
         return IQP_OK;
     }
     if (prec != IQP_SPLIT_BF16) {

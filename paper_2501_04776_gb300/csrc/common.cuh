@@ -52,6 +52,12 @@ struct Plan {
     size_t off_skp;  // split BF16: partial accumulators and counters of split phase tiles (0 if none)
     size_t off_gsum; // split BF16: per-CTA running sums of the two-sample-tile phase kernels (0 if none)
     size_t off_skx;  // split BF16: pieces and counters of the two-tile phase's balanced last round (0 if none)
+    // FP32 form on the tensor cores (optional region at the end of the FP32 plan; x3 = it is there and in use):
+    // the three planes of 2 theta, block maxima of |2 theta|, (S, M2) partials of 64 samples, row maxima of |W|, the
+    // three planes of W, running sums (off_skp: the split tiles' scratch)
+    size_t off_xc, off_xmax, off_xpart, off_xrow, off_xw, off_xsum;
+    bool x3;
+    size_t off_opt;  // where the optional regions begin (0: none)
     size_t off_phi;  // MMD gradient (split BF16, row-sparse): room for Phi, l x ldw fp32 (0 if none)
     // Kept Phi (l x ldphi fp32, ldphi a multiple of 64 >= s; the layout is the
     // precision's own): phi_out = the statistics pass writes it, phi_in = the
@@ -480,6 +486,21 @@ __device__ __forceinline__ void umma_stage4_ss(uint32_t d, uint64_t ahi, uint64_
         ::"r"(d), "l"(ahi), "l"(alo), "l"(b), "r"(idesc), "r"(acc)
         : "memory");
 }
+// Four K steps of one product (A, B in shared memory).
+__device__ __forceinline__ void umma_stage4_pair_ss1(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 aa, bb;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 q, %4, %4;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t"
+        "add.s64 aa, %1, 2;\n\tadd.s64 bb, %2, 2;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], aa, bb, %3, q;\n\t"
+        "add.s64 aa, %1, 4;\n\tadd.s64 bb, %2, 4;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], aa, bb, %3, q;\n\t"
+        "add.s64 aa, %1, 6;\n\tadd.s64 bb, %2, 6;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], aa, bb, %3, q;\n}\n"
+        ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        : "memory");
+}
 // Four K steps, A hi / A lo in TMEM (64 columns; K step k: hi at ta + 16 k,
 // lo at ta + 16 k + 8), B in shared memory.
 __device__ __forceinline__ void umma_stage4_pair_ts(uint32_t d, uint32_t ta, uint64_t b, uint32_t idesc, uint32_t acc) {
@@ -532,6 +553,44 @@ __device__ __forceinline__ void umma_stage8_pair_ts_b(uint32_t d, uint32_t ta, u
         "tcgen05.mma.cta_group::2.kind::f16 [%0], [t], h, %4, q;\n\t"
         "tcgen05.mma.cta_group::2.kind::f16 [%0], [t], l, %4, q;\n}\n"
         ::"r"(d), "r"(ta), "l"(bhi), "l"(blo), "r"(idesc), "r"(acc)
+        : "memory");
+}
+
+// Eight K steps of the three-plane products (two 128-byte K atoms of B), A in
+// TMEM at ta + 8 k: planes 0 and 1 side by side as one product into d (b01:
+// 128 rows per CTA, atoms 16384 bytes apart, instruction descriptor id01),
+// plane 2 into d2 (b2: 64 rows per CTA, atoms 8192 bytes apart, id2; always
+// accumulated). Two MMAs per K step instead of three of half the width: the
+// issuing thread spends about 90 clocks per MMA whatever its width.
+__device__ __forceinline__ void umma_stage8_pair_ts_x3(uint32_t d, uint32_t d2, uint32_t ta, uint64_t b01, uint64_t b2,
+                                                       uint32_t id01, uint32_t id2, uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b32 t;\n\t.reg .b64 h, l;\n\t"
+        "setp.ne.b32 p, %7, 0;\n\tsetp.eq.b32 q, %7, %7;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], [%2], %3, %5, p;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%1], [%2], %4, %6, q;\n\t"
+        "add.u32 t, %2, 8;\n\tadd.s64 h, %3, 2;\n\tadd.s64 l, %4, 2;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], [t], h, %5, q;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%1], [t], l, %6, q;\n\t"
+        "add.u32 t, %2, 16;\n\tadd.s64 h, %3, 4;\n\tadd.s64 l, %4, 4;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], [t], h, %5, q;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%1], [t], l, %6, q;\n\t"
+        "add.u32 t, %2, 24;\n\tadd.s64 h, %3, 6;\n\tadd.s64 l, %4, 6;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], [t], h, %5, q;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%1], [t], l, %6, q;\n\t"
+        "add.u32 t, %2, 32;\n\tadd.s64 h, %3, 1024;\n\tadd.s64 l, %4, 512;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], [t], h, %5, q;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%1], [t], l, %6, q;\n\t"
+        "add.u32 t, %2, 40;\n\tadd.s64 h, %3, 1026;\n\tadd.s64 l, %4, 514;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], [t], h, %5, q;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%1], [t], l, %6, q;\n\t"
+        "add.u32 t, %2, 48;\n\tadd.s64 h, %3, 1028;\n\tadd.s64 l, %4, 516;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], [t], h, %5, q;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%1], [t], l, %6, q;\n\t"
+        "add.u32 t, %2, 56;\n\tadd.s64 h, %3, 1030;\n\tadd.s64 l, %4, 518;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], [t], h, %5, q;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%1], [t], l, %6, q;\n}\n"
+        ::"r"(d), "r"(d2), "r"(ta), "l"(b01), "l"(b2), "r"(id01), "r"(id2), "r"(acc)
         : "memory");
 }
 

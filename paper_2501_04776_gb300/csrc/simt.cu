@@ -1,4 +1,5 @@
-// Plain FP32 form on the SIMT cores, plus the small kernels every form
+// Plain FP32 form on the SIMT cores (small problems, workspaces without the
+// tensor form's regions; otherwise tc.cu runs it on the tensor cores), plus the small kernels every form
 // shares: theta preparation, the per-observable statistics finalisation, the
 // fixed-order gradient reduction and the MMD combine.
 //

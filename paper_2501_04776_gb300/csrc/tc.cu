@@ -113,20 +113,24 @@ constexpr int kWPrefetch = 8;  // gradient: W tiles prefetched into L2 this many
 // DT (two sample tiles per tile): an operand stage holds A_hi, A_lo and the
 // B operands of both sample tiles, the two accumulators fill TMEM, and the
 // running sums live in global memory.
-template <int CG, bool ATMA, bool ATM = false, bool DT = false>
+// X3 (FP32 form, three planes of A): an operand stage holds the three A
+// planes and B; the two accumulators fill TMEM like DT's.
+template <int CG, bool ATMA, bool ATM = false, bool DT = false, bool X3 = false>
 struct Cfg {
     static constexpr int TNB = TN / CG;      // B rows this CTA holds (per sample tile)
-    static constexpr int NOP = DT ? 3 : (CG == 2 || ATM) ? 4 : (ATMA ? 3 : 2);  // operand stages
+    static constexpr int NOP = DT || X3 ? 3 : (CG == 2 || ATM) ? 4 : (ATMA ? 3 : 2);  // operand stages
     // Operand stage: A_hi (128 x 128 B), A_lo, B (TNB x 128 B) [DT: then the
     // second sample tile's B]; ATM: B only.
-    static constexpr uint32_t OP_A_HI = 0, OP_A_LO = 16384, OP_B = ATM ? 0 : 32768;
+    static constexpr uint32_t OP_A_HI = 0, OP_A_LO = 16384, OP_A_3 = 32768;
+    static constexpr uint32_t OP_B = ATM ? 0 : X3 ? 49152 : 32768;
     static constexpr uint32_t OP_B1 = OP_B + TNB * 128;
-    static constexpr uint32_t OP_BYTES = ATM ? TNB * 128 : 32768 + (DT ? 2 : 1) * TNB * 128;
+    static constexpr uint32_t OP_BYTES = OP_B + (DT ? 2 : 1) * TNB * 128;
     // Bits stage: A bits (128 rows x 32 B), B bits (TNB rows x 32 B) [DT: then
     // the second sample tile's], c_hi, c_lo.
     static constexpr uint32_t BT_A = 0, BT_B = 4096, BT_B1 = BT_B + TNB * 32;
     static constexpr uint32_t BT_CHI = BT_B + (DT ? 2 : 1) * TNB * 32, BT_CLO = BT_CHI + 512;
-    static constexpr uint32_t BT_BYTES = BT_CLO + 512;
+    static constexpr uint32_t BT_C3 = BT_CLO + 512;  // X3: the third plane of 2 theta
+    static constexpr uint32_t BT_BYTES = X3 ? BT_C3 + 1024 : BT_CLO + 512;
     static constexpr uint32_t SM_OP = 0;
     static constexpr uint32_t SM_BITS = SM_OP + NOP * OP_BYTES;
     static constexpr uint32_t SM_BAR = SM_BITS + NBITS * BT_BYTES;
@@ -186,6 +190,10 @@ struct TcArgs {
     uint32_t *status;
     uint64_t limit_ns;
     int serp;              // phase, whole tiles: every other round of tiles walks the gates backwards
+    // X3: the third plane of 2 theta, W as FP32 (l x ldw) and the largest |W| of each row (float bits)
+    const __nv_bfloat16 *c3;
+    float *wf;
+    uint32_t *wmax;
     // Two-sample-tile phase kernels: per CTA, the running sums of both
     // accumulators (2 x TM x TN FP32 as float4 groups of 4 columns, row-minor).
     float4 *gsum;
@@ -326,6 +334,28 @@ __device__ __forceinline__ void expand_a(const uint8_t *bitsA, const uint8_t *ch
     }
 }
 
+// The X3 form of expand_a: the three planes of 2 theta (512 bytes apart from
+// `c` on) masked into three A planes 16384 bytes apart from opA on.
+__device__ __forceinline__ void expand_a3(const uint8_t *bitsA, const uint8_t *cp, uint8_t *opA, int q, int gt) {
+    const uint32_t c = gt & 7;
+    uint4 v[3];
+#pragma unroll
+    for (int p = 0; p < 3; ++p) v[p] = *reinterpret_cast<const uint4 *>(cp + 512u * p + (uint32_t)q * 128u + c * 16u);
+    const uint32_t sub = (uint32_t)q * 8u + (c >> 2) * 4u;
+    const uint32_t sh = (c & 3u) * 8u;
+#pragma unroll
+    for (int k = 0; k < TM / kRowsPerPass; ++k) {
+        const uint32_t row = (uint32_t)(gt >> 3) + (uint32_t)kRowsPerPass * k;
+        const uint32_t w = *reinterpret_cast<const uint32_t *>(bitsA + row * 32u + sub);
+        const uint4 mk = expand_mask((w >> sh) & 0xFFu);
+        uint8_t *dst = opA + swz128(row, c);
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+            *reinterpret_cast<uint4 *>(dst + 16384 * p) =
+                make_uint4(v[p].x & mk.x, v[p].y & mk.y, v[p].z & mk.z, v[p].w & mk.w);
+    }
+}
+
 // Sum over the 32 lanes of v[lane][k]: afterwards lane L returns the sum of column L.
 __device__ __forceinline__ float reduce_scatter32(float (&v)[32], int lane) {
 #pragma unroll
@@ -378,6 +408,24 @@ __device__ __forceinline__ void load_sum32(uint32_t t, bool chunked, uint32_t (&
         tmem_ld32(t + kSumCol, acc);
 #pragma unroll
         for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) + __uint_as_float(acc[e]));
+    }
+}
+
+// X3: 32 columns of the tile at TMEM address `t`, the exact accumulator of
+// plane 0 plus the accumulator of planes 1 and 2 (kSumCol further on) plus,
+// where the tile was accumulated in more than one chunk, the running sum `ss`
+// (as in load_sum32).
+__device__ __forceinline__ void load_sum32_x3(uint32_t t, const float4 *ss, uint32_t (&r)[32]) {
+    load_sum32(t, true, r);
+    if (ss != nullptr) {
+#pragma unroll
+        for (int e4 = 0; e4 < 8; ++e4) {
+            const float4 v = ss[e4 * TM];
+            r[4 * e4] = __float_as_uint(__uint_as_float(r[4 * e4]) + v.x);
+            r[4 * e4 + 1] = __float_as_uint(__uint_as_float(r[4 * e4 + 1]) + v.y);
+            r[4 * e4 + 2] = __float_as_uint(__uint_as_float(r[4 * e4 + 2]) + v.z);
+            r[4 * e4 + 3] = __float_as_uint(__uint_as_float(r[4 * e4 + 3]) + v.w);
+        }
     }
 }
 
@@ -449,6 +497,126 @@ __global__ void __launch_bounds__(256) k_w_from_phi(const float *__restrict__ ph
     }
 }
 
+// ---- FP32 form: three BF16 planes of an FP32 value
+// A value x is taken apart on the grid of its operand (2 theta as a whole, or
+// one row of W): plane 0 is x rounded to a multiple of 2^E, an integer of at
+// most 256 in magnitude, so exact in BF16; planes 1 and 2 are the BF16 head
+// and tail of the rest (|rest| <= 2^(E-1)). 2^(E+8) is the power of two above
+// the operand's largest magnitude: the three planes keep x to 2^-26 of that
+// maximum or better, and sums of plane 0 against +-1 stay integers below
+// 2^24 of the grid, which the tensor core's FP32 accumulator holds exactly.
+// So the first plane's products need no accumulation chunks (up to 65536
+// terms), and the truncation of the other two, in an accumulator of their own,
+// is 2^-8 smaller than the sum: against FP64 the results are closer than the
+// SIMT kernels' sequential FP32 sums (one- and two-body circuit, n = 300, 1000
+// observables, 10^4 samples: gradient 2.4e-7 relative against 3.2e-6).
+// Three products per contraction, bound like the split form by producing the
+// masked planes: that circuit's autograd step takes 4.4 ms, against 59.5 ms on
+// the FP32 FMA pipe (0.54 of its peak).
+struct X3Grid {
+    float step, inv;  // 2^E and 2^-E
+};
+__device__ __forceinline__ X3Grid x3_grid(float mx) {
+    int e = (int)((__float_as_uint(mx) >> 23) & 255u) - 126;  // mx < 2^e
+    e = e < -100 ? -100 : (e > 120 ? 120 : e);
+    X3Grid g;
+    g.step = __uint_as_float((uint32_t)(e - 8 + 127) << 23);
+    g.inv = __uint_as_float((uint32_t)(8 - e + 127) << 23);
+    return g;
+}
+__device__ __forceinline__ void x3_planes(float x, const X3Grid &g, float (&p)[3]) {
+    p[0] = rintf(x * g.inv) * g.step;  // scaling by powers of two and the difference below are exact
+    const float rest = x - p[0];
+    p[1] = __bfloat162float(__float2bfloat16_rn(rest));
+    p[2] = rest - p[1];
+}
+
+// 2 theta reduced to [-pi, pi] (the phase enters only as cos and sin, and
+// every term is +-c_j, so multiples of 2 pi drop out); the reduction bounds
+// the grid's maximum.
+__device__ __forceinline__ float x3_angle(float theta) {
+    const float c = 2.0f * theta;
+    if (!(fabsf(c) > 3.1415927f)) return c;
+    const double d = (double)c;
+    return (float)(d - 6.283185307179586476925 * rint(d * 0.15915494309189533577));
+}
+
+constexpr int kX3Blocks = 128;   // blocks of the maximum's own pass, one maximum each
+constexpr int kX3Own = 8192;     // up to this many gates every block of the planes' pass takes the maximum itself
+
+// The largest finite |2 theta_j| over j = first, first + step, ... for this thread, reduced over the block.
+__device__ __forceinline__ float x3_block_max(const float *__restrict__ theta, int64_t m, int64_t first, int64_t step) {
+    __shared__ float red[8];
+    float v = 0.f;
+    for (int64_t j = first; j < m; j += step) {
+        const float c = fabsf(x3_angle(theta[j]));
+        if (c <= 4.f) v = fmaxf(v, c);
+    }
+#pragma unroll
+    for (int w = 16; w >= 1; w >>= 1) v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, w));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = red[0];
+    for (int w = 1; w < 8; ++w) v = fmaxf(v, red[w]);
+    return v;
+}
+
+__global__ void __launch_bounds__(256) k_x3_cmax(const float *__restrict__ theta, int64_t m, float *__restrict__ bmax) {
+    const float v = x3_block_max(theta, m, blockIdx.x * (int64_t)256 + threadIdx.x, (int64_t)gridDim.x * 256);
+    if (threadIdx.x == 0) bmax[blockIdx.x] = v;
+}
+
+// The planes of 2 theta (mpad BF16 each, zero beyond m), on the grid of the
+// block maxima (nb of them; nb = 0: each block takes the maximum itself, which
+// saves a launch where the gates are few). Row maxima wmax (l words, or
+// none) start at zero for the phase that follows.
+__global__ void __launch_bounds__(256) k_x3_theta(const float *__restrict__ theta, int64_t m, int64_t mpad,
+                                                  const float *__restrict__ bmax, int nb,
+                                                  __nv_bfloat16 *__restrict__ planes, uint32_t *__restrict__ wmax,
+                                                  int64_t l) {
+    float mx = 0.f;
+    if (nb == 0) mx = x3_block_max(theta, m, threadIdx.x, 256);
+    for (int b = 0; b < nb; ++b) mx = fmaxf(mx, bmax[b]);
+    const X3Grid g = x3_grid(mx);
+    for (int64_t j = blockIdx.x * (int64_t)256 + threadIdx.x; j < mpad; j += (int64_t)gridDim.x * 256) {
+        float p[3] = {0.f, 0.f, 0.f};
+        if (j < m) x3_planes(x3_angle(theta[j]), g, p);
+        if (!IQP_IN(j, mpad, 61)) continue;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) planes[k * mpad + j] = __float2bfloat16_rn(p[k]);
+    }
+    if (wmax != nullptr)
+        for (int64_t a = blockIdx.x * (int64_t)256 + threadIdx.x; a < l; a += (int64_t)gridDim.x * 256) wmax[a] = 0u;
+}
+
+// The planes of W (l x ldw BF16 each) from W as FP32 and its row maxima, eight
+// samples per thread; columns >= s are left as they are (the gradient's tensor
+// maps end at s).
+__global__ void __launch_bounds__(256) k_x3_wsplit(const float *__restrict__ W, int64_t ldw, int64_t l, int64_t s,
+                                                   const uint32_t *__restrict__ wmax, __nv_bfloat16 *__restrict__ planes) {
+    const int64_t per_row = cdiv(s, 8), total = l * per_row;
+    for (int64_t t = blockIdx.x * (int64_t)256 + threadIdx.x; t < total; t += (int64_t)gridDim.x * 256) {
+        const int64_t a = t / per_row, i0 = (t - a * per_row) * 8;  // ldw is a multiple of 64: whole words
+        if (!IQP_IN(a * ldw + i0 + 7, l * ldw, 62)) continue;
+        const X3Grid g = x3_grid(__uint_as_float(wmax[a]));
+        const float4 u = *reinterpret_cast<const float4 *>(W + a * ldw + i0);
+        const float4 v = *reinterpret_cast<const float4 *>(W + a * ldw + i0 + 4);
+        const float x[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+        uint32_t o[3][4];
+#pragma unroll
+        for (int e = 0; e < 8; e += 2) {
+            float p[3], q[3];
+            x3_planes(x[e], g, p);
+            x3_planes(x[e + 1], g, q);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) o[k][e / 2] = pack_bf16x2(p[k], q[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            *reinterpret_cast<uint4 *>(planes + (k * l + a) * ldw + i0) = make_uint4(o[k][0], o[k][1], o[k][2], o[k][3]);
+    }
+}
+
 // ------------------------------------------------------------------ kernel
 // W hi/lo (BF16 pairs) of 32 consecutive samples i0.. of observable row.
 __device__ __forceinline__ void store_w32(const TcArgs &args, int64_t row, int64_t i0, const uint32_t (&ph)[16],
@@ -472,6 +640,30 @@ __device__ __forceinline__ void store_w32(const TcArgs &args, int64_t row, int64
             sl[e] = (uint16_t)(pl[e / 2] >> ((e & 1) * 16));
         }
     }
+}
+
+// X3: 32 consecutive W values (FP32) of observable row from sample i0 on into
+// args.wf; returns the largest finite |W| among the samples below s.
+__device__ __forceinline__ float store_wf32(const TcArgs &args, int64_t row, int64_t i0, const uint32_t (&r)[32]) {
+    float mx = 0.f;
+    if (!IQP_IN(row * args.ldw + i0, args.l * args.ldw, 43) ||
+        !IQP_IN(row * args.ldw + (i0 + 32 <= args.s ? i0 + 31 : args.s - 1), args.l * args.ldw, 44))
+        return mx;
+    float *d = args.wf + row * args.ldw + i0;
+#pragma unroll
+    for (int e = 0; e < 32; ++e) {
+        const float v = fabsf(__uint_as_float(r[e]));
+        if (i0 + e < args.s && v <= 3.4e38f) mx = fmaxf(mx, v);
+    }
+    if (i0 + 32 <= args.s) {
+#pragma unroll
+        for (int e = 0; e < 32; e += 4)
+            *reinterpret_cast<float4 *>(d + e) = make_float4(__uint_as_float(r[e]), __uint_as_float(r[e + 1]),
+                                                             __uint_as_float(r[e + 2]), __uint_as_float(r[e + 3]));
+    } else {
+        for (int e = 0; e < 32 && i0 + e < args.s; ++e) d[e] = __uint_as_float(r[e]);
+    }
+    return mx;
 }
 
 // Accumulator values of 32 consecutive columns col0.. of `row`, stored into
@@ -508,11 +700,15 @@ __device__ __forceinline__ void store_out32(const TcArgs &args, int64_t row, int
 // on the stage loop). split_store: this warp's 32 rows x 64 columns of the
 // accumulator (+ running sum) into its part's slot. split_sum: the sum of
 // the tile's nsplit parts, in part order, into the accumulator columns.
+template <bool X3>
 __device__ __noinline__ void split_store(float *dst, uint32_t tbase, bool chunked, const float4 *ss0) {
     uint32_t r[32];
 #pragma unroll 1
     for (int c = 0; c < kGroupLoads; ++c) {
-        load_sum32(tbase + c * 32, chunked, r, ss0 != nullptr ? ss0 + c * 8 * TM : nullptr);
+        if (X3)
+            load_sum32_x3(tbase + c * 32, chunked ? ss0 + c * 8 * TM : nullptr, r);
+        else
+            load_sum32(tbase + c * 32, chunked, r, ss0 != nullptr ? ss0 + c * 8 * TM : nullptr);
 #pragma unroll
         for (int e = 0; e < 32; e += 4)
             *reinterpret_cast<float4 *>(dst + c * 32 + e) = make_float4(
@@ -549,7 +745,8 @@ __device__ __noinline__ void split_sum(const float *src0, int64_t part_stride, i
 // producer warps expand it from P_A bits and the hi/lo split of 2 theta.
 // CG = 1: one CTA per tile of 128 rows; CG = 2: a CTA pair per tile of 256 rows.
 // TA (phase modes of CTA pairs): 0 = A in shared memory; 1 = A in TMEM; 3 =
-// two sample tiles (2 x 256 samples) per tile against each A stage.
+// two sample tiles (2 x 256 samples) per tile against each A stage; 4 = the
+// FP32 form (X3): 2 theta as three BF16 planes (the kernel's note below).
 template <bool GRAD, int MODE, int CG, bool AT, bool SPL, int TA>
 __global__ void __launch_bounds__(kThreads, 1)
     k_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA2,
@@ -560,7 +757,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     // Two sample tiles per tile (phase modes, CTA pairs, whole tiles): A in
     // shared memory, two accumulators, running sums in global memory
     constexpr bool DT = TA == 3 && !GRAD && !AT && CG == 2;
-    using C = Cfg<CG, ATMA, ATM, DT>;
+    // FP32 form: three planes of 2 theta, the first on an integer grid, so its
+    // products (into accumulator columns 0..255) sum exactly; the other two
+    // share columns 256..511
+    constexpr bool X3 = TA == 4 && !GRAD && !AT && CG == 2;
+    using C = Cfg<CG, ATMA, ATM, DT, X3>;
     constexpr int NOP = C::NOP;
     // Serpentine gate order (phase kernels, whole tiles): the CTA groups' odd
     // rounds of tiles walk their bits stages from the last to the first, so a
@@ -666,13 +867,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                         bulk_load(bits + C::BT_CHI, args.chi + (cin ? kb * KB : 0), 512, &bar->bits_full[bs]);
                         bulk_load(bits + C::BT_CLO, args.clo + (cin ? kb * KB : 0), 512, &bar->bits_full[bs]);
                     } else {
-                        mbar_arrive_expect_tx(&bar->bits_full[bs], TM * 32 + C::TNB * 32 + 1024);
+                        mbar_arrive_expect_tx(&bar->bits_full[bs], TM * 32 + C::TNB * 32 + (X3 ? 1536 : 1024));
                         tma_load_2d(bits + C::BT_A, &tmA, &bar->bits_full[bs], x, a0);
                         tma_load_2d(bits + C::BT_B, &tmB, &bar->bits_full[bs], x, b0);
                         // the split of 2 theta is mpad long (bits stages never pass it)
                         const bool cin = IQP_IN((int64_t)kb * KB + KB - 1, args.mpad, 54);
                         bulk_load(bits + C::BT_CHI, args.chi + (cin ? kb * KB : 0), 512, &bar->bits_full[bs]);
                         bulk_load(bits + C::BT_CLO, args.clo + (cin ? kb * KB : 0), 512, &bar->bits_full[bs]);
+                        if (X3) bulk_load(bits + C::BT_C3, args.c3 + (cin ? kb * KB : 0), 512, &bar->bits_full[bs]);
                     }
                     bmask |= 1u << bs;
                     bpar = (bpar & ~(1u << bs)) | (((itb / NBITS) & 1u) << bs);
@@ -750,6 +952,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                     else if constexpr (DT) {
                         umma_stage4_pair_ss(tmem, d_hi0 + so, d_lo0 + so, d_b0 + so, C::IDESC, acc);
                         umma_stage4_pair_ss(tmem + (uint32_t)TN, d_hi0 + so, d_lo0 + so, d_b1 + so, C::IDESC, acc);
+                    } else if constexpr (X3) {
+                        umma_stage4_pair_ss1(tmem, d_hi0 + so, d_b0 + so, C::IDESC, acc);
+                        umma_stage4_pair_ss(tmem + (uint32_t)TN, d_lo0 + so,
+                                            d_lo0 + so + ((C::OP_A_3 - C::OP_A_LO) >> 4), d_b0 + so, C::IDESC, acc);
                     } else if constexpr (CG == 2)
                         umma_stage4_pair_ss(tmem, d_hi0 + so, d_lo0 + so, d_b0 + so, C::IDESC, acc);
                     else
@@ -799,7 +1005,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         // DT: this CTA's running sums (both accumulators) in global memory
         // (the host launches at most kMaxSplitCtas CTAs of this form)
         [[maybe_unused]] float4 *gsum_cta =
-            DT && IQP_IN(blockIdx.x, kMaxSplitCtas, 59) ? args.gsum + (int64_t)blockIdx.x * (kDtSumFloats / 4) : nullptr;
+            (DT || X3) && IQP_IN(blockIdx.x, kMaxSplitCtas, 59)
+                ? args.gsum + (int64_t)blockIdx.x * ((DT ? kDtSumFloats : kSplitSlotFloats) / 4)
+                : nullptr;
         // ATM: this thread's A parity bits of the current bits stage, 16 per
         // operand stage (see expand_a_tmem), packed two stages per word
         uint32_t abits01 = 0, abits23 = 0;
@@ -875,7 +1083,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
                 expand_b<C::TNB>(bits + C::BT_B, op + C::OP_B, q, gt);
                 if constexpr (DT) expand_b<C::TNB>(bits + C::BT_B1, op + C::OP_B1, q, gt);
-                if (!ATMA && !ATM)
+                if constexpr (X3)
+                    expand_a3(bits + C::BT_A, bits + C::BT_CHI, op + C::OP_A_HI, q, gt);
+                else if (!ATMA && !ATM)
                     expand_a(bits + C::BT_A, bits + C::BT_CHI, bits + C::BT_CLO, op + C::OP_A_HI, op + C::OP_A_LO, q,
                              gt);
                 if (ATM) {
@@ -907,8 +1117,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                         uint32_t r[32], acc[32];
                         const int hb = DT && c >= kGroupLoads ? 1 : 0;  // DT: accumulator of the second sample tile
                         const int cc = c - hb * kGroupLoads;
-                        tmem_ld32(tb + (uint32_t)(hb * TN + cc * 32), r);
-                        if (ATM || DT) {
+                        if (X3)
+                            load_sum32(tb + (uint32_t)(cc * 32), true, r);
+                        else
+                            tmem_ld32(tb + (uint32_t)(hb * TN + cc * 32), r);
+                        if (ATM || DT || X3) {
                             // running sum in shared memory (ATM) or global memory
                             // (DT), this thread's row only
                             float4 *sp = ATM ? sum4 + ((group * kGroupCols + cc * 32) >> 2) * TM + rl
@@ -968,6 +1181,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int64_t row = arow0 + quarter * 32 + lane;  // observable a
             const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(group * kGroupCols);
             bool chunked = nchunk > 0;
+            [[maybe_unused]] bool merged = false;  // X3: columns 0..255 hold the whole sum (a split tile's last part)
 
             if (!GRAD && MODE != 3 && SPL) {
                 // A part of a split tile: store this part's accumulator(s);
@@ -984,10 +1198,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 for (int h = 0; h < NH; ++h) {
                     const int64_t so = (((slot * CG + half) * NH + h) * TM + rl) * TN + group * kGroupCols;
                     const float4 *ss0 = ATM  ? sum4 + ((group * kGroupCols) >> 2) * TM + rl
-                                        : DT ? gsum_cta + ((h * TN + group * kGroupCols) >> 2) * TM + rl
-                                             : nullptr;
+                                        : DT || X3 ? gsum_cta + ((h * TN + group * kGroupCols) >> 2) * TM + rl
+                                                   : nullptr;
                     if (IQP_IN(so + kGroupCols - 1, kSkp, 47))
-                        split_store(args.skp + so, tbase + (uint32_t)(h * TN), chunked, ss0);
+                        split_store<X3>(args.skp + so, tbase + (uint32_t)(h * TN), chunked, ss0);
                 }
                 __threadfence();
                 __syncwarp();
@@ -1025,6 +1239,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         split_sum(args.skp + s0, pstride, (int)np, tbase + (uint32_t)(h * TN));
                 }
                 chunked = false;  // the sum of the parts is in the accumulator columns
+                merged = true;
             }
             // Phi (or Q) for 32 columns: last chunk's accumulator + running sum.
             // DT: the two sample tiles' accumulators in turn.
@@ -1036,8 +1251,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                 // else TMEM
                 auto ssum = [&](int c) -> const float4 * {
                     return ATM  ? sum4 + ((group * kGroupCols + c * 32) >> 2) * TM + rl
-                           : DT ? gsum_cta + ((hb * TN + group * kGroupCols + c * 32) >> 2) * TM + rl
-                                : nullptr;
+                           : DT || X3 ? gsum_cta + ((hb * TN + group * kGroupCols + c * 32) >> 2) * TM + rl
+                                      : nullptr;
+                };
+                auto ldsum = [&](int c, uint32_t (&r)[32]) {
+                    if (X3 && !merged)
+                        load_sum32_x3(tb_h + c * 32, chunked ? ssum(c) : nullptr, r);
+                    else
+                        load_sum32(tb_h + c * 32, chunked, r, ssum(c));
                 };
                 if (!GRAD && MODE == 0) {
                     const int64_t c0 = tn_h * TN + group * kGroupCols;  // first sample of this group
@@ -1047,7 +1268,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     uint32_t r[32];
 #pragma unroll 1
                     for (int c = 0; c < kGroupLoads; ++c) {
-                        load_sum32(tb_h + c * 32, chunked, r, ssum(c));
+                        ldsum(c, r);
 #pragma unroll
                         for (int e = 0; e < 32; ++e)
                             if (c * 32 + e < nvalid) S += cosf(__uint_as_float(r[e]));
@@ -1055,7 +1276,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const float mean = nvalid > 0 ? S / (float)nvalid : 0.f;
 #pragma unroll 1
                     for (int c = 0; c < kGroupLoads; ++c) {
-                        load_sum32(tb_h + c * 32, chunked, r, ssum(c));
+                        ldsum(c, r);
 #pragma unroll
                         for (int e = 0; e < 32; ++e)
                             if (c * 32 + e < nvalid) {
@@ -1068,7 +1289,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (args.out != nullptr) {  // uniform: every lane takes the TMEM loads
 #pragma unroll 1
                         for (int c = 0; c * 32 < nvalid; ++c) {
-                            load_sum32(tb_h + c * 32, chunked, r, ssum(c));
+                            ldsum(c, r);
                             if (row < args.l) store_out32(args, row, c0 + c * 32, r);
                         }
                     }
@@ -1083,11 +1304,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const bool rv = row < args.l;
                     const float al = rv && IQP_IN(row, args.l, 55) ? (float)args.alpha[row] : 0.f;
                     const float be = (rv && args.beta) ? (float)args.beta[row] : 0.f;
+                    [[maybe_unused]] float wmax = 0.f;
                     float S = 0.f, M2 = 0.f;
                     uint32_t r[32];
 #pragma unroll 1
                     for (int c = 0; c < kGroupLoads; ++c) {
-                        load_sum32(tb_h + c * 32, chunked, r, ssum(c));
+                        ldsum(c, r);
 #pragma unroll
                         for (int e = 0; e < 32; ++e)
                             if (c * 32 + e < nvalid) S += cosf(__uint_as_float(r[e]));
@@ -1095,7 +1317,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const float mean = nvalid > 0 ? S / (float)nvalid : 0.f;
 #pragma unroll 1
                     for (int c = 0; c < kGroupLoads; ++c) {
-                        load_sum32(tb_h + c * 32, chunked, r, ssum(c));
+                        ldsum(c, r);
                         const int64_t i0 = c0 + c * 32;
                         uint32_t ph[16], pl[16];
 #pragma unroll
@@ -1107,13 +1329,23 @@ __global__ void __launch_bounds__(kThreads, 1)
                             if (c * 32 + e < nvalid) M2 = fmaf(d0, d0, M2);
                             if (c * 32 + e + 1 < nvalid) M2 = fmaf(d1, d1, M2);
                             const float w0 = s0 * (al + be * k0), w1 = s1 * (al + be * k1);
+                            if (X3) {  // W stays FP32
+                                r[e] = __float_as_uint(w0);
+                                r[e + 1] = __float_as_uint(w1);
+                                continue;
+                            }
                             const float h0 = __bfloat162float(__float2bfloat16_rn(w0));
                             const float h1 = __bfloat162float(__float2bfloat16_rn(w1));
                             ph[e / 2] = pack_bf16x2(h0, h1);
                             pl[e / 2] = pack_bf16x2(w0 - h0, w1 - h1);
                         }
-                        if (rv && i0 < args.s) store_w32(args, row, i0, ph, pl);
+                        if (X3) {
+                            if (rv && i0 < args.s) wmax = fmaxf(wmax, store_wf32(args, row, i0, r));
+                        } else if (rv && i0 < args.s) {
+                            store_w32(args, row, i0, ph, pl);
+                        }
                     }
+                    if (X3 && wmax > 0.f && IQP_IN(row, args.l, 60)) atomicMax(args.wmax + row, __float_as_uint(wmax));
                     if (rv && nvalid > 0 && IQP_IN(row * args.nparts + c0 / kGroupCols, args.l * args.nparts, 51))
                         args.part[row * args.nparts + (c0 / kGroupCols)] = make_double2((double)S, (double)M2);
                 } else if (!GRAD && MODE == 3) {
@@ -1121,7 +1353,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     uint32_t r[32];
 #pragma unroll 1
                     for (int c = 0; c < kGroupLoads; ++c) {
-                        load_sum32(tb_h + c * 32, chunked, r, ssum(c));
+                        ldsum(c, r);
                         if (row < args.l && c0 + c * 32 < args.s) store_out32(args, row, c0 + c * 32, r);
                     }
                 } else if (!GRAD) {
@@ -1129,10 +1361,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const bool rv = row < args.l;
                     const float al = rv && IQP_IN(row, args.l, 55) ? (float)args.alpha[row] : 0.f;
                     const float be = (rv && args.beta) ? (float)args.beta[row] : 0.f;
+                    [[maybe_unused]] float wmax = 0.f;
                     uint32_t r[32];
 #pragma unroll 1
                     for (int c = 0; c < kGroupLoads; ++c) {
-                        load_sum32(tb_h + c * 32, chunked, r, ssum(c));
+                        ldsum(c, r);
                         const int64_t i0 = c0 + c * 32;
                         uint32_t ph[16], pl[16];
 #pragma unroll
@@ -1141,20 +1374,30 @@ __global__ void __launch_bounds__(kThreads, 1)
                             sincosf(__uint_as_float(r[e]), &s0, &k0);
                             sincosf(__uint_as_float(r[e + 1]), &s1, &k1);
                             const float w0 = s0 * (al + be * k0), w1 = s1 * (al + be * k1);
+                            if (X3) {  // W stays FP32
+                                r[e] = __float_as_uint(w0);
+                                r[e + 1] = __float_as_uint(w1);
+                                continue;
+                            }
                             const float h0 = __bfloat162float(__float2bfloat16_rn(w0));
                             const float h1 = __bfloat162float(__float2bfloat16_rn(w1));
                             ph[e / 2] = pack_bf16x2(h0, h1);
                             pl[e / 2] = pack_bf16x2(w0 - h0, w1 - h1);
                         }
-                        if (rv && i0 < args.s) store_w32(args, row, i0, ph, pl);
+                        if (X3) {
+                            if (rv && i0 < args.s) wmax = fmaxf(wmax, store_wf32(args, row, i0, r));
+                        } else if (rv && i0 < args.s) {
+                            store_w32(args, row, i0, ph, pl);
+                        }
                     }
+                    if (X3 && wmax > 0.f && IQP_IN(row, args.l, 60)) atomicMax(args.wmax + row, __float_as_uint(wmax));
                 } else {
                     // Gradient epilogue: mask by 2 P_A[a][j], reduce over observables.
                     const bool rv = row < args.l;
                     uint32_t r[32];
 #pragma unroll 1
                     for (int c = 0; c < kGroupLoads; ++c) {
-                        load_sum32(tb_h + c * 32, chunked, r, ssum(c));
+                        ldsum(c, r);
                         const int64_t j0 = tn_h * TN + group * kGroupCols + c * 32;
                         const uint32_t mask = (rv && j0 < args.m &&
                                                IQP_IN(row * args.ldp32 + (j0 >> 5), args.l * args.ldp32, 52))
@@ -1244,24 +1487,35 @@ constexpr int kGThreads = (GE0 + GEPI) * 32;
 // error of the tensor core's truncating FP32 accumulation.
 constexpr uint32_t kGAcol = GN;      // first A column
 
+// X3 (the FP32 form): tiles of 256 gates x 128 observables, W as three BF16
+// planes, the first on an integer grid of its row. Per K step one N = 256
+// product takes planes 0 (this CTA pair's first 128 rows of B: the even CTA's)
+// and 1 (the odd CTA's) side by side into accumulator columns 0..127 and
+// 128..255, and one N = 128 product adds plane 2 (64 rows per CTA) to columns
+// 128..255. Plane 0's sums are exact; its rounding happens once, when the
+// epilogue adds the two halves.
+template <bool X3>
 struct GCfg {
+    static constexpr int NS = X3 ? 4 : GNS;               // operand stages in flight
+    static constexpr int OBS = X3 ? 128 : GN;             // observables per tile
     static constexpr uint32_t ATOM = GNB * 128;           // one 128-byte K atom of a W tile
+    static constexpr uint32_t ATOM2 = X3 ? 64 * 128 : GNB * 128;
     static constexpr uint32_t OP_HI = 0, OP_LO = 2 * ATOM;
-    static constexpr uint32_t OP_BYTES = 4 * ATOM;        // W_hi + W_lo, two atoms each
-    static constexpr uint32_t SM_BITS = GNS * OP_BYTES;
+    static constexpr uint32_t OP_BYTES = 2 * ATOM + 2 * ATOM2;  // W_hi + W_lo (X3: plane 0 or 1, and plane 2)
+    static constexpr uint32_t SM_BITS = NS * OP_BYTES;
     static constexpr uint32_t BT_BYTES = TM * 32;         // P_Z^T: 128 gates x 256 samples
     static constexpr uint32_t SM_BAR = SM_BITS + NBITS * BT_BYTES;
     static constexpr uint32_t SM_END = SM_BAR + 256;
     static constexpr uint32_t SMEM = SM_END + 1024;
-    static constexpr uint32_t IDESC = idesc_bf16(2 * TM, GN);
+    static constexpr uint32_t IDESC = idesc_bf16(2 * TM, GN), IDESC2 = idesc_bf16(2 * TM, GN / 2);
     static_assert(OP_BYTES % 1024 == 0 && BT_BYTES % 1024 == 0, "stage alignment");
     static_assert(ATOM == 16384, "umma_stage8_pair_ts_b steps 16384 bytes between K atoms");
-    static_assert(kGAcol + GNS * GACOLS <= kTmemCols, "TMEM columns");
+    static_assert(kGAcol + NS * GACOLS <= kTmemCols, "TMEM columns");
     static_assert(SMEM <= 232448, "shared memory");
 };
 
 struct GBars {
-    uint64_t bits_full[NBITS], bits_empty[NBITS], a_full[GNS], a_peer[GNS], w_full[GNS], empty[GNS], acc_full,
+    uint64_t bits_full[NBITS], bits_empty[NBITS], a_full[4], a_peer[4], w_full[4], empty[4], acc_full,
         acc_empty, drain;
     uint32_t tmem_slot;
     int abort_flag;
@@ -1280,10 +1534,13 @@ struct GradArgs {
     uint64_t limit_ns;
 };
 
+template <bool X3>
 __global__ void __launch_bounds__(kGThreads, 1)
     k_grad_pair(const __grid_constant__ CUtensorMap tmWhi, const __grid_constant__ CUtensorMap tmWlo,
-                const __grid_constant__ CUtensorMap tmZt, const GradArgs args) {
-    using C = GCfg;
+                const __grid_constant__ CUtensorMap tmW3, const __grid_constant__ CUtensorMap tmZt,
+                const GradArgs args) {
+    using C = GCfg<X3>;
+    constexpr int GNS = C::NS, GN = C::OBS, GNB = GN / 2;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = aligned_smem(smem_raw);
     GBars *bar = reinterpret_cast<GBars *>(smem + C::SM_BAR);
@@ -1331,18 +1588,20 @@ __global__ void __launch_bounds__(kGThreads, 1)
         if (lane == 0) {
             prefetch_tmap(&tmWhi);
             prefetch_tmap(&tmWlo);
+            if (X3) prefetch_tmap(&tmW3);
             const uint32_t w_full_leader = mapa_shared(smem_u32(&bar->w_full[0]), 0u);
             uint32_t os = 0, ph = 0, omask = 0, opar = 0;  // stage ring position and its phase parity
             bool ok = true;
             for (int64_t t = group0; t < ntiles && ok; t += ngroups) {
                 int64_t to, tg;
                 tile_coords(t, args.tiles_o, args.tiles_g, args.group_o, to, tg);
-                const int a0 = (int)(to * GN) + (int)crank * GNB;  // this CTA's first W row
+                // this CTA's first W row (X3: of plane 0 or 1, then of plane 2 GNB crank further on)
+                const int a0 = (int)(to * GN) + (X3 ? 0 : (int)crank * GNB);
                 int a0n = -1;                                      // the next tile's (for L2 prefetch)
                 if (t + ngroups < ntiles) {
                     int64_t ton, tgn;
                     tile_coords(t + ngroups, args.tiles_o, args.tiles_g, args.group_o, ton, tgn);
-                    a0n = (int)(ton * GN) + (int)crank * GNB;
+                    a0n = (int)(ton * GN) + (X3 ? 0 : (int)crank * GNB);
                 }
                 for (int ks = 0; ks < nks; ++ks) {
                     if (!mbar_wait(&bar->empty[os], ph ^ 1u, abort_flag, status, lim)) {
@@ -1354,12 +1613,15 @@ __global__ void __launch_bounds__(kGThreads, 1)
 #pragma unroll
                     for (int at = 0; at < 2; ++at) {
                         const int x = ks * GKS + at * 64;
+                        const int a2 = X3 ? a0 + (int)crank * GNB : a0;
                         if (leader) {
                             tma_load_2d(op + C::OP_HI + at * C::ATOM, &tmWhi, &bar->w_full[os], x, a0);
-                            tma_load_2d(op + C::OP_LO + at * C::ATOM, &tmWlo, &bar->w_full[os], x, a0);
+                            tma_load_2d(op + C::OP_LO + at * C::ATOM2, X3 ? &tmW3 : &tmWlo, &bar->w_full[os], x, a2);
                         } else {
-                            tma_load_2d_pair(op + C::OP_HI + at * C::ATOM, &tmWhi, w_full_leader + os * 8u, x, a0);
-                            tma_load_2d_pair(op + C::OP_LO + at * C::ATOM, &tmWlo, w_full_leader + os * 8u, x, a0);
+                            tma_load_2d_pair(op + C::OP_HI + at * C::ATOM, X3 ? &tmWlo : &tmWhi, w_full_leader + os * 8u,
+                                             x, a0);
+                            tma_load_2d_pair(op + C::OP_LO + at * C::ATOM2, X3 ? &tmW3 : &tmWlo, w_full_leader + os * 8u,
+                                             x, a2);
                         }
                     }
                     // warm L2 with the tiles 512 samples beyond this load (the next tile's near the end)
@@ -1369,10 +1631,12 @@ __global__ void __launch_bounds__(kGThreads, 1)
                         ap = a0n;
                     }
                     if (ap >= 0) {
-                        tma_prefetch_2d(&tmWhi, xp, ap);
-                        tma_prefetch_2d(&tmWhi, xp + 64, ap);
-                        tma_prefetch_2d(&tmWlo, xp, ap);
-                        tma_prefetch_2d(&tmWlo, xp + 64, ap);
+                        const CUtensorMap *m1 = X3 && !leader ? &tmWlo : &tmWhi, *m2 = X3 ? &tmW3 : &tmWlo;
+                        const int ap2 = X3 ? ap + (int)crank * GNB : ap;
+                        tma_prefetch_2d(m1, xp, ap);
+                        tma_prefetch_2d(m1, xp + 64, ap);
+                        tma_prefetch_2d(m2, xp, ap2);
+                        tma_prefetch_2d(m2, xp + 64, ap2);
                     }
                     omask |= 1u << os;
                     opar = (opar & ~(1u << os)) | (ph << os);
@@ -1438,8 +1702,12 @@ __global__ void __launch_bounds__(kGThreads, 1)
                     }
                     tc_fence_after();
                     const uint64_t dhi = d_w0 + (uint64_t)(os * (C::OP_BYTES >> 4));
-                    umma_stage8_pair_ts_b(tmem, tmem + kGAcol + os * GACOLS, dhi, dhi + (C::OP_LO >> 4), C::IDESC,
-                                          kc == 0 ? 0u : 1u);
+                    if constexpr (X3)
+                        umma_stage8_pair_ts_x3(tmem, tmem + GN, tmem + kGAcol + os * GACOLS, dhi, dhi + (C::OP_LO >> 4),
+                                               C::IDESC, C::IDESC2, kc == 0 ? 0u : 1u);
+                    else
+                        umma_stage8_pair_ts_b(tmem, tmem + kGAcol + os * GACOLS, dhi, dhi + (C::OP_LO >> 4), C::IDESC,
+                                              kc == 0 ? 0u : 1u);
                     umma_commit_pair(&bar->empty[os]);
                     if (++kc == chunk || ks == nks - 1) {
                         umma_commit_pair(&bar->acc_full);
@@ -1585,9 +1853,20 @@ __global__ void __launch_bounds__(kGThreads, 1)
                 for (int w = 0; w < NW; ++w) {
                     uint32_t r[32];
                     tmem_ld32(tb + w * 32, r);
+                    if (X3) {  // planes 1 and 2
+                        uint32_t r2[32];
+                        tmem_ld32(tb + GN + w * 32, r2);
+#pragma unroll
+                        for (int x = 0; x < 32; ++x)
+                            r[x] = __float_as_uint(__uint_as_float(r[x]) + __uint_as_float(r2[x]));
+                    }
 #pragma unroll
                     for (int x = 0; x < 32; ++x)
                         if ((mk[w] >> x) & 1u) part += __uint_as_float(r[x]);
+                    if (X3 && w + 1 < NW) {
+                        gsum += 2.0 * (double)part;
+                        part = 0.f;
+                    }
                 }
                 tc_fence_before();
                 __syncwarp();
@@ -1662,7 +1941,8 @@ bool make_map(CUtensorMap *map, const void *base, CUtensorMapDataType dt, int64_
 template <bool GRAD, int MODE, int CG, bool AT = GRAD, bool SPL = false, int TA = 0>
 cudaError_t launch_k(const CUtensorMap &a, const CUtensorMap &a2, const CUtensorMap &b, const TcArgs &args,
                      cudaStream_t st) {
-    using C = Cfg<CG, GRAD || AT, TA == 1 && !GRAD && !AT && CG == 2, TA == 3 && !GRAD && !AT && CG == 2>;
+    constexpr bool kPhasePair = !GRAD && !AT && CG == 2;
+    using C = Cfg<CG, GRAD || AT, TA == 1 && kPhasePair, TA == 3 && kPhasePair, TA == 4 && kPhasePair>;
     constexpr int CL = CG;
     static bool attr_set = false;
     if (!attr_set) {
@@ -1674,7 +1954,8 @@ cudaError_t launch_k(const CUtensorMap &a, const CUtensorMap &a2, const CUtensor
     int sms = num_sms();
     if (sms < CL) sms = CL;
     const int64_t groups = args.nunits < sms / CL ? args.nunits : sms / CL;
-    LaunchScope ls(GRAD          ? IQP_KERNEL_GRAD_TC
+    LaunchScope ls(GRAD        ? IQP_KERNEL_GRAD_TC
+                   : TA == 4   ? (MODE == 1 ? IQP_KERNEL_RECOMPUTE_FP32 : IQP_KERNEL_PHASE_FP32)
                    : MODE == 1 ? IQP_KERNEL_RECOMPUTE_TC
                    : MODE == 3 ? IQP_KERNEL_LOWORDER_GEMM
                                : IQP_KERNEL_PHASE_TC,
@@ -1816,6 +2097,20 @@ int cta_group() {
     return cg;
 }
 
+// FP32 form on the tensor cores (IQP_FP32_TC; default 1; 0 = the SIMT kernels).
+bool fp32_tc() {
+    static int v = -1;
+    if (v < 0) {
+        const char *e = std::getenv("IQP_FP32_TC");
+        v = (e != nullptr && e[0] == '0') ? 0 : 1;
+    }
+    return v == 1;
+}
+
+// Gates (samples in the gradient) per accumulation chunk of the FP32 form:
+// plane 0's integers of at most 256 stay below 2^24 over 65536 terms.
+constexpr int64_t kX3Chunk = 65536;
+
 // Every tile whole (no split parts).
 void whole_tiles(TcArgs &a, int64_t ntiles) {
     a.nunits = a.whole = ntiles;
@@ -1843,6 +2138,14 @@ cudaError_t launch_phase_dt_k(int mode, const CUtensorMap &ma, const CUtensorMap
 }
 
 template <bool SPL>
+cudaError_t launch_phase_x3_k(int mode, const CUtensorMap &ma, const CUtensorMap &mb, const TcArgs &a,
+                              cudaStream_t st) {
+    if (mode == 0) return launch_k<false, 0, 2, false, SPL, 4>(ma, ma, mb, a, st);
+    if (mode == 1) return launch_k<false, 1, 2, false, SPL, 4>(ma, ma, mb, a, st);
+    return launch_k<false, 2, 2, false, SPL, 4>(ma, ma, mb, a, st);
+}
+
+template <bool SPL>
 cudaError_t launch_phase_k(int mode, int cg, const CUtensorMap &ma, const CUtensorMap &mb, const TcArgs &a,
                            cudaStream_t st) {
     if (cg == 2 && phase_tmem()) {
@@ -1860,6 +2163,54 @@ cudaError_t launch_phase_k(int mode, int cg, const CUtensorMap &ma, const CUtens
     return launch_k<false, 2, 1, false, SPL>(ma, ma, mb, a, st);
 }
 }  // namespace
+
+namespace {
+// The T single tiles of a phase: a last round of tiles that would leave CTA
+// groups idle is split along the gates across them. The whole tiles run first
+// (full rounds), then a second launch runs the remaining tiles' parts, each a
+// range of whole bits stages, and the last part of a tile to finish sums the
+// parts (in part order) and runs the epilogue. skp: the split tiles' scratch
+// (null: every tile whole).
+cudaError_t launch_single_tiles(int mode, int cg, bool x3, const CUtensorMap &ma, const CUtensorMap &mb, TcArgs a,
+                                int64_t T, float *skp, cudaStream_t st) {
+    whole_tiles(a, T);
+    int64_t R = 0, ns = 1;
+    if (split_tail() && skp != nullptr) {
+        int sms = num_sms();
+        if (sms > kMaxSplitCtas) sms = kMaxSplitCtas;
+        const int64_t P = sms / cg;  // CTA groups
+        R = T >= P ? T % P : T;
+        ns = (P >= 2 && R > 0) ? P / R : 1;
+        const int64_t nkb = cdiv(a.nks, KB / KS);
+        if (ns > nkb) ns = nkb;
+        if (ns < 2) R = 0;
+    }
+    auto run = [&](bool split, const TcArgs &w) {
+        if (x3) return split ? launch_phase_x3_k<true>(mode, ma, mb, w, st) : launch_phase_x3_k<false>(mode, ma, mb, w, st);
+        return split ? launch_phase_k<true>(mode, cg, ma, mb, w, st) : launch_phase_k<false>(mode, cg, ma, mb, w, st);
+    };
+    if (R == 0) return run(false, a);
+    if (T - R > 0) {
+        TcArgs w = a;
+        whole_tiles(w, T - R);
+        const cudaError_t e = run(false, w);
+        if (e != cudaSuccess) return e;
+    }
+    a.whole = T - R;
+    a.nsplit = (int)ns;
+    a.nunits = R * ns;
+    a.skp = skp;
+    a.skc = reinterpret_cast<int *>(a.skp + (int64_t)kMaxSplitCtas * kSplitSlotFloats);
+    a.skcap = (int64_t)kMaxSplitCtas * kSplitSlotFloats;
+    const cudaError_t e = cudaMemsetAsync(a.skc, 0, (size_t)(R * cg) * sizeof(int), st);
+    if (e != cudaSuccess) return e;
+    return run(true, a);
+}
+}  // namespace
+
+// Whether the FP32 form runs on the tensor cores here (its planes also need
+// the plan's optional regions).
+bool x3_available() { return fp32_tc() && num_sms() >= 2 && num_sms() <= kMaxSplitCtas && iqp_tensor_path_available(); }
 
 cudaError_t launch_phase_tc(int mode, const Plan &p, void *ws, const double *alpha, const double *beta,
                             cudaStream_t st, iqp_status *why) {
@@ -1955,51 +2306,81 @@ cudaError_t launch_phase_tc(int mode, const Plan &p, void *ws, const double *alp
             T = 2 * (T2 - full);
         }
     }
-    // A last round of tiles that would leave CTA groups idle is split along
-    // the gates across them: the whole tiles run first (full rounds), then a
-    // second launch runs the remaining tiles' parts, each a range of whole
-    // bits stages, and the last part of a tile to finish sums the parts (in
-    // part order) and runs the epilogue.
-    whole_tiles(a, T);
-    int64_t R = 0, ns = 1;
-    if (split_tail() && p.off_skp != 0) {
-        int sms = num_sms();
-        if (sms > kMaxSplitCtas) sms = kMaxSplitCtas;
-        const int64_t P = sms / cg;  // CTA groups
-        R = T >= P ? T % P : T;
-        ns = (P >= 2 && R > 0) ? P / R : 1;
-        const int64_t nkb = cdiv(a.nks, KB / KS);
-        if (ns > nkb) ns = nkb;
-        if (ns < 2) R = 0;
-    }
-    if (R == 0) return launch_phase_k<false>(mode, cg, ma, mb, a, st);
-    if (T - R > 0) {
-        TcArgs w = a;
-        whole_tiles(w, T - R);
-        const cudaError_t e = launch_phase_k<false>(mode, cg, ma, mb, w, st);
-        if (e != cudaSuccess) return e;
-    }
-    a.whole = T - R;
-    a.nsplit = (int)ns;
-    a.nunits = R * ns;
-    a.skp = at<float>(ws, p.off_skp);
-    a.skc = reinterpret_cast<int *>(a.skp + (int64_t)kMaxSplitCtas * kSplitSlotFloats);
-    a.skcap = (int64_t)kMaxSplitCtas * kSplitSlotFloats;
-    const cudaError_t e = cudaMemsetAsync(a.skc, 0, (size_t)(R * cg) * sizeof(int), st);
-    if (e != cudaSuccess) return e;
-    return launch_phase_k<true>(mode, cg, ma, mb, a, st);
+    return launch_single_tiles(mode, cg, false, ma, mb, a, T, p.off_skp != 0 ? at<float>(ws, p.off_skp) : nullptr, st);
 }
 
+// The FP32 form's phase (p.x3): the same contraction with 2 theta as three
+// planes (k_tc, TA = 4). mode 0: statistics; 1: W (FP32) and its row maxima;
+// 2: both.
+cudaError_t launch_phase_x3(int mode, const Plan &p, void *ws, const double *alpha, const double *beta,
+                            cudaStream_t st, iqp_status *why) {
+    CUtensorMap ma, mb;
+    if (!make_map(&ma, at<uint64_t>(ws, p.off_pa), CU_TENSOR_MAP_DATA_TYPE_UINT64, p.ldp, p.l, p.ldp * 8, 4, TM,
+                  CU_TENSOR_MAP_SWIZZLE_NONE) ||
+        !make_map(&mb, at<uint64_t>(ws, p.off_pz), CU_TENSOR_MAP_DATA_TYPE_UINT64, p.ldp, p.s, p.ldp * 8, 4,
+                  (uint32_t)(TN / 2), CU_TENSOR_MAP_SWIZZLE_NONE)) {
+        *why = IQP_ERR_UNSUPPORTED;
+        return cudaErrorNotSupported;
+    }
+    TcArgs a{};  // every field zero unless set below
+    a.l = p.l;
+    a.s = p.s;
+    a.m = p.m;
+    a.nks = cdiv(p.m, KS);
+    a.chunk = kX3Chunk / KS;
+    a.tiles_m = cdiv(p.l, 2 * TM);
+    a.tiles_n = cdiv(p.s, TN);
+    a.group_m = tile_group();
+    a.chi = at<__nv_bfloat16>(ws, p.off_xc);
+    a.clo = a.chi + p.mpad;
+    a.c3 = a.clo + p.mpad;
+    a.mpad = p.mpad;
+    a.part = at<double2>(ws, p.off_xpart);
+    a.nparts = cdiv(p.s, (int64_t)kPartColsTc);
+    a.alpha = alpha;
+    a.beta = beta;
+    a.ldw = p.ldw;
+    if (mode != 0) {
+        a.wf = at<float>(ws, p.off_w);
+        a.wmax = at<uint32_t>(ws, p.off_xrow);  // zeroed by k_x3_theta
+    }
+    a.status = at<uint32_t>(ws, p.off_status);
+    a.limit_ns = default_spin_limit_ns();
+    a.serp = phase_serp() ? 1 : 0;
+    a.gsum = at<float4>(ws, p.off_xsum);
+    return launch_single_tiles(mode, 2, true, ma, mb, a, a.tiles_m * a.tiles_n, at<float>(ws, p.off_skp), st);
+}
+
+cudaError_t launch_x3_theta(const Plan &p, void *ws, const float *theta, cudaStream_t st) {
+    float *bmax = at<float>(ws, p.off_xmax);
+    int64_t nb = p.m <= kX3Own ? 0 : cdiv(p.m, 1024);
+    if (nb > kX3Blocks) nb = kX3Blocks;
+    if (nb > 0) {
+        LaunchScope ls(IQP_KERNEL_THETA_SPLIT, st);
+        k_x3_cmax<<<(unsigned)nb, 256, 0, st>>>(theta, p.m, bmax);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    int64_t blocks = cdiv(p.mpad, 256);
+    if (blocks > 4096) blocks = 4096;
+    LaunchScope ls(IQP_KERNEL_THETA_SPLIT, st);
+    k_x3_theta<<<(unsigned)blocks, 256, 0, st>>>(theta, p.m, p.mpad, bmax, (int)nb, at<__nv_bfloat16>(ws, p.off_xc),
+                                                 p.off_xw != p.off_xrow ? at<uint32_t>(ws, p.off_xrow) : nullptr, p.l);
+    return cudaGetLastError();
+}
 
 namespace {
+template <bool X3>
 cudaError_t launch_grad_pair(const Plan &p, void *ws, cudaStream_t st, iqp_status *why) {
-    using C = GCfg;
-    CUtensorMap mhi, mlo, mz;
-    const __nv_bfloat16 *whi = at<__nv_bfloat16>(ws, p.off_w);
+    using C = GCfg<X3>;
+    CUtensorMap mhi, mlo, m3, mz;
+    const __nv_bfloat16 *whi = at<__nv_bfloat16>(ws, X3 ? p.off_xw : p.off_w);
     const __nv_bfloat16 *wlo = whi + p.l * p.ldw;
     if (!make_map(&mhi, whi, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, p.s, p.l, p.ldw * 2, KS, GNB,
                   CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map(&mlo, wlo, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, p.s, p.l, p.ldw * 2, KS, GNB,
+                  CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_map(&m3, X3 ? wlo + p.l * p.ldw : wlo, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, p.s, p.l, p.ldw * 2, KS, 64,
                   CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map(&mz, at<uint64_t>(ws, p.off_pzt), CU_TENSOR_MAP_DATA_TYPE_UINT64, p.ldzt, p.m, p.ldzt * 8, 4, TM,
                   CU_TENSOR_MAP_SWIZZLE_NONE)) {
@@ -2011,11 +2392,11 @@ cudaError_t launch_grad_pair(const Plan &p, void *ws, cudaStream_t st, iqp_statu
     a.s = p.s;
     a.m = p.m;
     a.nks = cdiv(p.s, GKS);
-    const int64_t cmax = grad_chunk_samples() / GKS;
+    const int64_t cmax = (X3 ? kX3Chunk : grad_chunk_samples()) / GKS;
     a.chunk = cdiv(a.nks, cdiv(a.nks, cmax));  // fewest chunks, balanced
     a.tiles_g = cdiv(p.m, 2 * TM);
-    a.tiles_o = cdiv(p.l, GN);
-    a.group_o = grad_group();
+    a.tiles_o = cdiv(p.l, (int64_t)C::OBS);
+    a.group_o = grad_group() * (GN / C::OBS);
     a.pat32 = at<uint32_t>(ws, p.off_pat);
     a.ldlt32 = 2 * p.ldlt;
     a.gpart = at<double>(ws, p.off_gpart);
@@ -2024,7 +2405,7 @@ cudaError_t launch_grad_pair(const Plan &p, void *ws, cudaStream_t st, iqp_statu
     static bool attr_set = false;
     if (!attr_set) {
         const cudaError_t e =
-            cudaFuncSetAttribute(k_grad_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+            cudaFuncSetAttribute(k_grad_pair<X3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
@@ -2032,7 +2413,7 @@ cudaError_t launch_grad_pair(const Plan &p, void *ws, cudaStream_t st, iqp_statu
     if (sms < 2) sms = 2;
     const int64_t ntiles = a.tiles_g * a.tiles_o;
     const int64_t groups = ntiles < sms / 2 ? ntiles : sms / 2;
-    LaunchScope ls(IQP_KERNEL_GRAD_TC, st);
+    LaunchScope ls(X3 ? IQP_KERNEL_GRAD_FP32 : IQP_KERNEL_GRAD_TC, st);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(groups * 2), 1, 1);
     cfg.blockDim = dim3(kGThreads, 1, 1);
@@ -2045,7 +2426,7 @@ cudaError_t launch_grad_pair(const Plan &p, void *ws, cudaStream_t st, iqp_statu
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_grad_pair, mhi, mlo, mz, a);
+    return cudaLaunchKernelEx(&cfg, k_grad_pair<X3>, mhi, mlo, m3, mz, a);
 }
 }  // namespace
 
@@ -2054,8 +2435,25 @@ cudaError_t launch_grad_pair(const Plan &p, void *ws, cudaStream_t st, iqp_statu
 // for the single-CTA kernel (IQP_GRAD_PAIR=0 or IQP_CTA_PAIRS=0).
 int64_t grad_tc_rows(const Plan &p) { return cta_group() == 2 && grad_pair() ? 2 * cdiv(p.l, GN) : cdiv(p.l, TM); }
 
+// The FP32 form's gradient contraction (p.x3): W taken apart into its planes,
+// then k_grad_pair<true>; 2 ceil(l / 128) rows of partials.
+cudaError_t launch_grad_x3(const Plan &p, void *ws, cudaStream_t st, iqp_status *why) {
+    const int64_t total = p.l * cdiv(p.s, (int64_t)8);
+    int64_t grid = cdiv(total, 256);
+    const int64_t cap = (int64_t)num_sms() * 8;
+    if (grid > cap) grid = cap;
+    {
+        LaunchScope ls(IQP_KERNEL_RECOMPUTE_FP32, st);
+        k_x3_wsplit<<<(unsigned)grid, 256, 0, st>>>(at<float>(ws, p.off_w), p.ldw, p.l, p.s,
+                                                    at<uint32_t>(ws, p.off_xrow), at<__nv_bfloat16>(ws, p.off_xw));
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return launch_grad_pair<true>(p, ws, st, why);
+}
+
 cudaError_t launch_grad_tc(const Plan &p, void *ws, cudaStream_t st, iqp_status *why) {
-    if (cta_group() == 2 && grad_pair()) return launch_grad_pair(p, ws, st, why);
+    if (cta_group() == 2 && grad_pair()) return launch_grad_pair<false>(p, ws, st, why);
     const int cg = 1;
     CUtensorMap mhi, mlo, mb;
     const __nv_bfloat16 *whi = at<__nv_bfloat16>(ws, p.off_w);
