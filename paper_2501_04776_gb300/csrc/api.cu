@@ -19,7 +19,13 @@ cudaError_t launch_parity_gather(int64_t n, const uint64_t *R, int64_t rows, int
                                  int64_t m, int64_t ldg, uint64_t *P, int64_t ldp, uint64_t *PT, int64_t ldpt,
                                  uint64_t *RT, cudaStream_t st, const int4 *sup = nullptr);
 cudaError_t launch_parity_sum(int64_t n, const uint64_t *A, int64_t l, int64_t lda, const uint64_t *X, int64_t N,
-                              int64_t ldx, int64_t *T, cudaStream_t st);
+                              int64_t ldx, int64_t *T, cudaStream_t st, const int *heavy = nullptr);
+cudaError_t launch_parity_sum_rows(int64_t n, const uint64_t *A, int64_t l, int64_t lda, const uint64_t *X, int64_t N,
+                                   int64_t ldx, uint64_t *XT, int64_t ldxt, int *heavy, uint32_t *counter, int64_t *T,
+                                   cudaStream_t st);
+cudaError_t launch_mmd_terms(const double2 *part, int64_t nparts, int64_t pw, const int64_t *T, int64_t l, int64_t s,
+                             int64_t N, int unbiased, bool sqrt_loss, double *terms, double *alpha, double *beta,
+                             double *loss, double *scale, uint32_t *counter, cudaStream_t st);
 cudaError_t launch_theta_prep(const float *theta, int64_t m, int64_t mpad, float *c32, __nv_bfloat16 *hi,
                               __nv_bfloat16 *lo, cudaStream_t st);
 cudaError_t launch_phase_simt(int mode, const uint64_t *PA, const uint64_t *PZ, int64_t ldp, const float *c,
@@ -58,7 +64,8 @@ cudaError_t launch_sparse_stats(const uint64_t *PA, int64_t ldp, const uint64_t 
 cudaError_t launch_sparse_grad(const uint64_t *PA, int64_t ldp, const uint64_t *PZT, int64_t ldzt, const float *c,
                                int64_t l, int64_t s, int64_t m, int64_t nparts, const double *alpha,
                                const double *beta, double *scale, unsigned long long *gfx, double *grad,
-                               const SparseIndep *indep, const float *phi, int64_t ldphi, cudaStream_t st);
+                               const SparseIndep *indep, const float *phi, int64_t ldphi, bool scale_set,
+                               cudaStream_t st);
 cudaError_t launch_sparse_value_grad(const uint64_t *PA, int64_t ldp, const uint64_t *PZT, int64_t ldzt,
                                      const float *c, int64_t l, int64_t s, int64_t m, int64_t nparts, double2 *part,
                                      const double *alpha, const double *beta, double *scale, unsigned long long *gfx,
@@ -89,7 +96,7 @@ cudaError_t launch_lo_grad(const uint64_t *A, int64_t lda, int64_t n, int64_t l,
                            const float *M, int64_t lds, const float *C, int64_t ldc, int64_t s, int64_t m,
                            const int4 *sup, const double *alpha, const double *beta, uint64_t *AT, int64_t ldlt,
                            float *W, float *V, double *H, double *gsp, unsigned long long *Kfx, double *grad,
-                           __nv_bfloat16 *split, const float *phi, int64_t ldphi, uint32_t *status,
+                           __nv_bfloat16 *split, const float *phi, int64_t ldphi, bool scale_set, uint32_t *status,
                            cudaStream_t st);
 cudaError_t launch_bitflip_gates(const float *theta, int64_t m, int64_t mpad, double *c, double *t, cudaStream_t st);
 cudaError_t launch_bitflip_rows(const uint64_t *PA, int64_t ldp, int64_t l, const double *c, double *expval,
@@ -202,6 +209,16 @@ Plan make_plan(int op, int64_t n, int64_t m, int64_t l, int64_t s, int64_t N, in
         p.off_skp = take((int64_t)kMaxSplitCtas * kSplitSlotFloats * 4 + (int64_t)kMaxSplitCtas * 4);
         p.off_gsum = take((int64_t)kMaxSplitCtas * kDtSumFloats * 4);
         p.off_skx = take((int64_t)kSplitSlots * kSplitSlotFloats * 4 + (int64_t)kMaxSplitCtas * 4);
+    }
+    // MMD: scratch of the data parities by row gather (a workspace that ends
+    // before its end folds them densely).
+    p.off_xt = p.off_heavy = 0;
+    p.ldxt = round_up(cdiv(N, 64), 4);
+    p.scale_set = false;
+    if (mmd) {
+        if (p.off_opt == 0) p.off_opt = off;
+        p.off_xt = take(n * p.ldxt * 8);
+        p.off_heavy = take(256 + cdiv(l, 32) * 4);  // the counter, then the marks
     }
     p.total = off;
     return p;
@@ -331,9 +348,12 @@ iqp_status check_ws(Plan &p, void *ws, size_t ws_bytes) {
     if (ws_bytes < p.total) {
         if (ws_bytes < plan_min_bytes(p)) return IQP_ERR_WORKSPACE;
         p.x3 = false;  // FP32: the SIMT kernels
+        p.off_xt = 0;  // data parities folded densely
         // The optional regions at the end, in order: each is used only where
         // the workspace reaches its end.
-        p.off_skx = 0;  // the two-tile last round runs as single tiles
+        if (p.off_skx != 0 && ws_bytes < p.off_skx + (size_t)round_up((int64_t)kSplitSlots * kSplitSlotFloats * 4 +
+                                                                       (int64_t)kMaxSplitCtas * 4, 256))
+            p.off_skx = 0;  // the two-tile last round runs as single tiles
         if (p.off_gsum != 0 && ws_bytes < p.off_gsum + (size_t)kMaxSplitCtas * kDtSumFloats * 4)
             p.off_gsum = 0;  // one sample tile per tile
         if (p.off_skp != 0 && ws_bytes < p.off_skp + (size_t)round_up((int64_t)kMaxSplitCtas * kSplitSlotFloats * 4 +
@@ -407,12 +427,16 @@ iqp_status prepare(const Plan &p, void *ws, const uint64_t *G, int64_t ldg, cons
     return IQP_OK;
 }
 
-// Phase contraction with the statistics epilogue -> (expval, std_err, S1, S2).
-iqp_status forward_stats(const Plan &p, void *ws, double *expval, double *std_err, double *S1, double *S2,
-                         cudaStream_t st) {
-    double2 *part = at<double2>(ws, p.off_part);
+// Phase contraction with the statistics epilogue: (sum cos, M2) partials of
+// `pw` samples, `nparts` per observable.
+iqp_status forward_partials(const Plan &p, void *ws, cudaStream_t st, const double2 **parts, int64_t *nparts,
+                            int64_t *pw) {
+    double2 *part = at<double2>(ws, p.x3 ? p.off_xpart : p.off_part);
+    *parts = part;
+    *nparts = p.x3 ? cdiv(p.s, (int64_t)kPartColsTc) : p.nparts;
+    *pw = p.x3 ? kPartColsTc : p.pw;
+    iqp_status why = IQP_OK;
     if (p.prec == IQP_SPLIT_BF16) {
-        iqp_status why = IQP_OK;
         if (launch_phase_tc(0, p, ws, nullptr, nullptr, st, &why) != cudaSuccess)
             return why != IQP_OK ? why : IQP_ERR_CUDA;
     } else if (p.prec == IQP_LOWORDER_FP32) {
@@ -426,18 +450,24 @@ iqp_status forward_stats(const Plan &p, void *ws, double *expval, double *std_er
                                     p.l, p.s, p.m, part, p.nparts, p.indep ? &ind : nullptr,
                                     p.phi_out ? p.phi : nullptr, p.ldphi, st));
     } else if (p.x3) {
-        iqp_status why = IQP_OK;
         if (launch_phase_x3(0, p, ws, nullptr, nullptr, st, &why) != cudaSuccess)
             return why != IQP_OK ? why : IQP_ERR_CUDA;
-        IQP_TRY(launch_finalize(at<double2>(ws, p.off_xpart), cdiv(p.s, (int64_t)kPartColsTc), kPartColsTc, p.l, p.s,
-                                expval, std_err, S1, S2, st));
-        return IQP_OK;
     } else {
         IQP_TRY(launch_phase_simt(0, at<uint64_t>(ws, p.off_pa), at<uint64_t>(ws, p.off_pz), p.ldp,
                                   at<float>(ws, p.off_c), p.l, p.s, p.m, part, p.nparts, nullptr, nullptr, nullptr, 0,
                                   st));
     }
-    IQP_TRY(launch_finalize(part, p.nparts, p.pw, p.l, p.s, expval, std_err, S1, S2, st));
+    return IQP_OK;
+}
+
+// The same merged per observable -> (expval, std_err, S1, S2).
+iqp_status forward_stats(const Plan &p, void *ws, double *expval, double *std_err, double *S1, double *S2,
+                         cudaStream_t st) {
+    const double2 *part;
+    int64_t nparts, pw;
+    const iqp_status rc = forward_partials(p, ws, st, &part, &nparts, &pw);
+    if (rc != IQP_OK) return rc;
+    IQP_TRY(launch_finalize(part, nparts, pw, p.l, p.s, expval, std_err, S1, S2, st));
     return IQP_OK;
 }
 
@@ -451,7 +481,7 @@ iqp_status backward(const Plan &p, void *ws, const double *alpha, const double *
                                at<uint64_t>(ws, p.off_rt), p.ldlt, at<float>(ws, p.off_w), at<float>(ws, p.off_lo_v),
                                at<double>(ws, p.off_lo_h), at<double>(ws, p.off_lo_gs),
                                at<unsigned long long>(ws, p.off_gpart), grad, at<__nv_bfloat16>(ws, p.off_lo_a),
-                               p.phi_in ? p.phi : nullptr, p.ldphi, at<uint32_t>(ws, p.off_status), st));
+                               p.phi_in ? p.phi : nullptr, p.ldphi, p.scale_set, at<uint32_t>(ws, p.off_status), st));
         return IQP_OK;
     }
     if (p.prec == IQP_SPARSE_FP32) {
@@ -460,7 +490,7 @@ iqp_status backward(const Plan &p, void *ws, const double *alpha, const double *
         IQP_TRY(launch_sparse_grad(at<uint64_t>(ws, p.off_pa), p.ldp,
                                    at<uint64_t>(ws, p.indep ? p.off_zt : p.off_pzt), p.ldzt, at<float>(ws, p.off_c),
                                    p.l, p.s, p.m, p.nparts, alpha, beta, reinterpret_cast<double *>(gfx + p.m), gfx,
-                                   grad, p.indep ? &ind : nullptr, p.phi_in ? p.phi : nullptr, p.ldphi, st));
+                                   grad, p.indep ? &ind : nullptr, p.phi_in ? p.phi : nullptr, p.ldphi, p.scale_set, st));
         return IQP_OK;
     }
     if (p.prec == IQP_SPLIT_BF16) {
@@ -520,12 +550,27 @@ iqp_status mmd_core(int op, int64_t n, const uint64_t *G, int64_t m, int64_t ldg
         p.ldphi = p.ldw;
         p.phi_out = p.phi_in = true;
     }
-    if ((rc = forward_stats(p, ws, nullptr, nullptr, S1, S2, st)) != IQP_OK) return rc;
     int64_t *T = at<int64_t>(ws, p.off_T);
-    IQP_TRY(launch_parity_sum(n, A, l, lda, X, N, ldx, T, st));
     double *alpha = at<double>(ws, p.off_ab), *beta = alpha + l;
-    IQP_TRY(launch_mmd_combine(T, S1, S2, l, s, N, unbiased, (flags & IQP_MMD_SQRT) != 0,
-                               at<double>(ws, p.off_terms), alpha, beta, loss, st));
+    const bool sq = (flags & IQP_MMD_SQRT) != 0;
+    if (p.off_xt != 0) {
+        const double2 *part;
+        int64_t nparts, pw;
+        if ((rc = forward_partials(p, ws, st, &part, &nparts, &pw)) != IQP_OK) return rc;
+        uint32_t *counter = at<uint32_t>(ws, p.off_heavy);
+        IQP_TRY(launch_parity_sum_rows(n, A, l, lda, X, N, ldx, at<uint64_t>(ws, p.off_xt), p.ldxt,
+                                       reinterpret_cast<int *>(counter) + 64, counter, T, st));
+        double *scale = nullptr;  // where the gradient's fixed-point accumulators keep it
+        if (g && p.prec == IQP_LOWORDER_FP32) scale = at<double>(ws, p.off_gpart) + n * n;
+        if (g && p.prec == IQP_SPARSE_FP32) scale = at<double>(ws, p.off_gpart) + m;
+        IQP_TRY(launch_mmd_terms(part, nparts, pw, T, l, s, N, unbiased, sq, at<double>(ws, p.off_terms), alpha, beta, loss,
+                                 scale, counter, st));
+        p.scale_set = scale != nullptr;
+    } else {
+        if ((rc = forward_stats(p, ws, nullptr, nullptr, S1, S2, st)) != IQP_OK) return rc;
+        IQP_TRY(launch_parity_sum(n, A, l, lda, X, N, ldx, T, st));
+        IQP_TRY(launch_mmd_combine(T, S1, S2, l, s, N, unbiased, sq, at<double>(ws, p.off_terms), alpha, beta, loss, st));
+    }
     if (g) return backward(p, ws, alpha, beta, grad, st);
     return IQP_OK;
 }

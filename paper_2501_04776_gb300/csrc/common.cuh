@@ -58,6 +58,11 @@ struct Plan {
     size_t off_xc, off_xmax, off_xpart, off_xrow, off_xw, off_xsum;
     bool x3;
     size_t off_opt;  // where the optional regions begin (0: none)
+    // MMD (optional, at the end): the data transposed (n x ldxt words), marks of the heavy observable blocks, the counter
+    // of the pass over the terms
+    size_t off_xt, off_heavy;
+    int64_t ldxt;
+    bool scale_set;  // the gradient's fixed-point scale is in place already (set with the MMD terms)
     size_t off_phi;  // MMD gradient (split BF16, row-sparse): room for Phi, l x ldw fp32 (0 if none)
     // Kept Phi (l x ldphi fp32, ldphi a multiple of 64 >= s; the layout is the
     // precision's own): phi_out = the statistics pass writes it, phi_in = the
@@ -102,6 +107,16 @@ iqp_status expval_arg_check(int64_t n, const uint64_t *G, int64_t m, int64_t ldg
 cudaError_t launch_tc_dense(const __nv_bfloat16 *a_hi, const __nv_bfloat16 *a_lo, int64_t rows, int64_t kpad,
                             int64_t k, const uint64_t *b_bits, int64_t nb, int64_t ldb, void *out, int64_t ldo,
                             bool out_f64, uint32_t *status, cudaStream_t st);
+
+// Fixed-point scale of a gradient accumulator: 2^k with B 2^k < 2^61 for a
+// bound B of every partial sum; k clamped so that 2^(k+1) is a normal FP32 number.
+__device__ __forceinline__ double fixed_scale(double B) {
+    // B in [2^e, 2^(e+1)); scale = 2^(60-e) gives B scale < 2^61.
+    int e = (B > 0.0 && B < 1e300) ? ilogb(B) : 0;
+    if (e < -58) e = -58;
+    if (e > 180) e = 180;
+    return ldexp(1.0, 60 - e);
+}
 
 // ---------------------------------------------------------------- status
 

@@ -1076,7 +1076,7 @@ cudaError_t launch_lo_grad(const uint64_t *A, int64_t lda, int64_t n, int64_t l,
                            const float *M, int64_t lds, const float *C, int64_t ldc, int64_t s, int64_t m,
                            const int4 *sup, const double *alpha, const double *beta, uint64_t *AT, int64_t ldlt,
                            float *W, float *V, double *H, double *gsp, unsigned long long *Kfx, double *grad,
-                           __nv_bfloat16 *split, const float *phi, int64_t ldphi, uint32_t *status,
+                           __nv_bfloat16 *split, const float *phi, int64_t ldphi, bool scale_set, uint32_t *status,
                            cudaStream_t st) {
     const int64_t nblk = cdiv(s, kBlk);
     double *scale = reinterpret_cast<double *>(Kfx + n * n);
@@ -1086,7 +1086,7 @@ cudaError_t launch_lo_grad(const uint64_t *A, int64_t lda, int64_t n, int64_t l,
     cudaError_t e = launch_bit_transpose_batched(A, 1, l, n, lda, AT, ldlt, st);
     if (e != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(Kfx, 0, (size_t)n * n * sizeof(unsigned long long), st)) != cudaSuccess) return e;
-    if ((e = launch_fixed_scale(alpha, beta, l, s, scale, st)) != cudaSuccess) return e;
+    if (!scale_set && (e = launch_fixed_scale(alpha, beta, l, s, scale, st)) != cudaSuccess) return e;
     if (phi != nullptr) {  // Phi kept by the statistics pass (possibly in W itself)
         LaunchScope ls(IQP_KERNEL_LOWORDER, st);
         k_lo_w<<<grid_1d(l * (lds / 4)), 256, 0, st>>>(phi, ldphi, W, lds, l, s, alpha, beta);

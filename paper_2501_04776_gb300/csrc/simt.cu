@@ -271,6 +271,24 @@ __device__ __forceinline__ double warp_sum_f64(double v) {
     return v;
 }
 
+// S = sum cos and M2 = sum (cos - S/s)^2 of one observable's partials, on every lane of the warp.
+__device__ __forceinline__ void merge_partials(const double2 *__restrict__ p, int64_t nparts, int64_t pw, int64_t s,
+                                               int lane, double &S, double &mean, double &M2) {
+    S = 0.0;
+    for (int64_t k = lane; k < nparts; k += 32) S += p[k].x;
+    S = warp_sum_f64(S);
+    mean = S / (double)s;
+    const double inv_pw = 1.0 / (double)pw;
+    M2 = 0.0;
+    for (int64_t k = lane; k < nparts; k += 32) {
+        const int64_t nk = (s - k * pw) < pw ? (s - k * pw) : pw;
+        const double2 v = p[k];
+        const double d = (nk == pw ? v.x * inv_pw : v.x / (double)nk) - mean;
+        M2 += v.y + (double)nk * d * d;
+    }
+    M2 = warp_sum_f64(M2);
+}
+
 __global__ void __launch_bounds__(256) k_finalize(const double2 *__restrict__ part, int64_t nparts, int64_t pw,
                                                   int64_t l, int64_t s, double *__restrict__ expval,
                                                   double *__restrict__ std_err, double *__restrict__ S1,
@@ -279,20 +297,8 @@ __global__ void __launch_bounds__(256) k_finalize(const double2 *__restrict__ pa
     const int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (a >= l) return;  // whole warps
     if (!IQP_IN(a * nparts + nparts - 1, l * nparts, 30)) return;
-    const double2 *p = part + a * nparts;
-    double S = 0.0;
-    for (int64_t k = lane; k < nparts; k += 32) S += p[k].x;
-    S = warp_sum_f64(S);
-    const double mean = S / (double)s;
-    const double inv_pw = 1.0 / (double)pw;
-    double M2 = 0.0;
-    for (int64_t k = lane; k < nparts; k += 32) {
-        const int64_t nk = (s - k * pw) < pw ? (s - k * pw) : pw;
-        const double2 v = p[k];
-        const double d = (nk == pw ? v.x * inv_pw : v.x / (double)nk) - mean;
-        M2 += v.y + (double)nk * d * d;
-    }
-    M2 = warp_sum_f64(M2);
+    double S, mean, M2;
+    merge_partials(part + a * nparts, nparts, pw, s, lane, S, mean, M2);
     if (lane != 0) return;
     if (expval) expval[a] = mean;
     if (std_err) std_err[a] = sqrt(M2 / (double)s) / sqrt((double)s);
@@ -358,6 +364,81 @@ __global__ void __launch_bounds__(1024) k_mmd_combine(const long long *__restric
         if (beta) beta[a] *= f;
     }
     if (threadIdx.x == 0) *loss = r;
+}
+
+// The same from the statistics' partials, one warp per observable over the
+// whole grid (the kernel above runs its FP64 divisions, a few hundred thousand
+// operations, on one SM: 53 us for 2000 observables; with k_finalize and the
+// gradient's scale 71 us, this 19). The last block to finish adds the terms up in a fixed order and,
+// with `scale`, sets the fixed-point scale of the gradient's accumulators.
+struct MmdConst {
+    double inv_s, inv_N, inv_l, inv_ss1, inv_NN1;  // 1 / (s (s - 1)), 1 / (N (N - 1))
+};
+__global__ void __launch_bounds__(256) k_mmd_terms(const double2 *__restrict__ part, int64_t nparts, int64_t pw,
+                                                   const long long *__restrict__ T, int64_t l, int64_t s, int64_t N,
+                                                   int unbiased, int sqrt_loss, MmdConst k, double *__restrict__ terms,
+                                                   double *__restrict__ alpha, double *__restrict__ beta,
+                                                   double *__restrict__ loss, double *__restrict__ scale,
+                                                   uint32_t *__restrict__ counter) {
+    const int lane = threadIdx.x & 31;
+    const int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (a < l && IQP_IN(a * nparts + nparts - 1, l * nparts, 30)) {  // whole warps
+        double S, mean, M2;
+        merge_partials(part + a * nparts, nparts, pw, s, lane, S, mean, M2);
+        if (lane == 0) {
+            const double t = (double)T[a], dN = (double)N;
+            const double p = t * k.inv_N, S2 = M2 + S * mean;
+            double term, al, be = 0.0;
+            if (unbiased) {
+                term = (t * t - dN) * k.inv_NN1 - 2.0 * p * mean + (S * S - S2) * k.inv_ss1;
+                al = (2.0 * p * k.inv_s - 2.0 * S * k.inv_ss1) * k.inv_l;
+                be = 2.0 * k.inv_ss1 * k.inv_l;
+            } else {
+                term = (p - mean) * (p - mean);
+                al = 2.0 * (p - mean) * k.inv_s * k.inv_l;
+            }
+            terms[a] = term;
+            alpha[a] = al;
+            beta[a] = be;
+        }
+    }
+    __shared__ bool last;
+    __shared__ double red[2][256];
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double sum = 0.0, mag = 0.0;
+    for (int64_t b = threadIdx.x; b < l; b += 256) {
+        sum += __ldcg(terms + b);
+        mag += fabs(__ldcg(alpha + b)) + fabs(__ldcg(beta + b));
+    }
+    red[0][threadIdx.x] = sum;
+    red[1][threadIdx.x] = mag;
+    __syncthreads();
+    for (int w = 128; w >= 1; w >>= 1) {
+        if ((int)threadIdx.x < w) {
+            red[0][threadIdx.x] += red[0][threadIdx.x + w];
+            red[1][threadIdx.x] += red[1][threadIdx.x + w];
+        }
+        __syncthreads();
+    }
+    const double L = red[0][0] * k.inv_l;
+    double f = 1.0, out = L;
+    if (sqrt_loss) {
+        out = L > 0.0 ? sqrt(L) : 0.0;
+        f = L > 0.0 ? 0.5 / out : 0.0;
+        for (int64_t b = threadIdx.x; b < l; b += 256) {
+            alpha[b] = __ldcg(alpha + b) * f;
+            beta[b] = __ldcg(beta + b) * f;
+        }
+    }
+    if (threadIdx.x == 0) {
+        *loss = out;
+        if (scale != nullptr) *scale = fixed_scale(2.0 * (double)s * red[1][0] * f);
+    }
 }
 
 // alpha_a = -w_a / s for a linear loss given weights (device helper).
@@ -436,6 +517,20 @@ cudaError_t launch_mmd_combine(const int64_t *T, const double *S1, const double 
     LaunchScope ls(IQP_KERNEL_MMD_COMBINE, st);
     k_mmd_combine<<<1, 1024, 0, st>>>(reinterpret_cast<const long long *>(T), S1, S2, l, s, N, unbiased,
                                       sqrt_loss ? 1 : 0, terms, alpha, beta, loss);
+    return cudaGetLastError();
+}
+
+// T, terms, alpha, beta: l each; scale: null or the gradient's fixed-point
+// scale; counter: zero (launch_parity_sum_rows leaves it so).
+cudaError_t launch_mmd_terms(const double2 *part, int64_t nparts, int64_t pw, const int64_t *T, int64_t l, int64_t s,
+                             int64_t N, int unbiased, bool sqrt_loss, double *terms, double *alpha, double *beta,
+                             double *loss, double *scale, uint32_t *counter, cudaStream_t st) {
+    const double ds = (double)s, dN = (double)N;
+    const MmdConst k{1.0 / ds, 1.0 / dN, 1.0 / (double)l, 1.0 / (ds * (ds - 1.0)), 1.0 / (dN * (dN - 1.0))};
+    LaunchScope ls(IQP_KERNEL_MMD_COMBINE, st);
+    k_mmd_terms<<<(unsigned)cdiv(l, 8), 256, 0, st>>>(part, nparts, pw, reinterpret_cast<const long long *>(T), l, s, N,
+                                                      unbiased, sqrt_loss ? 1 : 0, k, terms, alpha, beta, loss, scale,
+                                                      counter);
     return cudaGetLastError();
 }
 

@@ -492,13 +492,7 @@ __global__ void __launch_bounds__(256) k_sparse_scale(const double *__restrict__
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        // B in [2^e, 2^(e+1)); scale = 2^(60-e) gives B scale < 2^61. e is
-        // clamped to [-58, 180] so that 2 scale is a normal FP32 number.
-        const double B = 2.0 * (double)s * red[0];
-        int e = (B > 0.0 && B < 1e300) ? ilogb(B) : 0;
-        if (e < -58) e = -58;
-        if (e > 180) e = 180;
-        *scale = ldexp(1.0, 60 - e);
+        *scale = fixed_scale(2.0 * (double)s * red[0]);
     }
 }
 
@@ -589,10 +583,10 @@ cudaError_t launch_sparse_stats(const uint64_t *PA, int64_t ldp, const uint64_t 
 cudaError_t launch_sparse_grad(const uint64_t *PA, int64_t ldp, const uint64_t *PZT, int64_t ldzt, const float *c,
                                int64_t l, int64_t s, int64_t m, int64_t nparts, const double *alpha,
                                const double *beta, double *scale, unsigned long long *gfx, double *grad,
-                               const SparseIndep *indep, const float *phi, int64_t ldphi, cudaStream_t st) {
+                               const SparseIndep *indep, const float *phi, int64_t ldphi, bool scale_set, cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(gfx, 0, (size_t)m * sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
-    {
+    if (!scale_set) {
         LaunchScope ls(IQP_KERNEL_GRAD_SPARSE, st);
         k_sparse_scale<<<1, 256, 0, st>>>(alpha, beta, l, s, scale);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
