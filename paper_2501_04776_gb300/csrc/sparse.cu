@@ -28,9 +28,10 @@
 // lanes' sums of 32 gates are combined by one reduce-scatter.
 //
 // Measured, MMD loss and gradient of the n = 1000 one- and two-body circuit
-// (500500 gates, 2000 observables, 5000 samples): 18.9 -> 8.6 ms; independent
-// batches (n = 200, 5000 gates, 256 x 2000 samples), forward and backward: 1.43
-// -> 0.52 ms. What is left is mostly the latency of the P_Z^T loads.
+// (500500 gates, 2000 observables, 5000 samples): 18.9 -> 5.9 ms (8.6 with the
+// parity words loaded into registers and the list made again for every range);
+// independent batches (n = 200, 5000 gates, 256 x 2000 samples), forward and
+// backward: 1.43 -> 0.51 ms.
 //
 // Statistics: (sum cos, sum (cos - mean)^2) partials of 1024 samples (FP32
 // within a warp, FP64 across warps), merged by the shared finaliser.
@@ -102,10 +103,31 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 // Dynamic shared memory: the list (gate, bits of c), then the partial phases
 // (16 x 1024 floats) or the sign tables (4 x 256 x 32 floats) in the same
 // place, then W (1024 floats), then the dense words of a listing step, then
-// the reductions' words.
+// the reductions' words, then (gradient, shared batches) the rings of its
+// P_Z^T words. The phase's rings lie in the tables' place.
 constexpr int kSmList = 0, kSmTab = kList * 8, kWordBytes = kThreads * kScan * 4;
 constexpr int kPartBytes = kWarps * kRange * 4, kTabBytes = 4 * 256 * 32 * 4;
-constexpr int smem_bytes(bool grad) { return kSmTab + (grad ? kTabBytes : kPartBytes) + kRange * 4 + kWordBytes + 256; }
+// P_Z^T words in flight: per warp kRing stages of kPhaseStage (kGradStage) gates
+// x 128 bytes, brought in by 16-byte asynchronous copies (four gates per warp
+// instruction), two stages ahead of their use: 82 KB per SM in the phase. With
+// the next five words in registers, 10 to 20 KB per SM, the phase waited on
+// them for most of its time.
+constexpr int kRing = 3, kPhaseStage = 20, kGradStage = 8;
+constexpr int kPhaseRing = kRing * kPhaseStage * 32, kGradRing = kRing * kGradStage * 32;  // words per warp
+static_assert(kWarps * kPhaseRing * 4 <= kTabBytes && kPartBytes <= kTabBytes, "the tables' place");
+// bytes of the tables' place, and in all (independent batches stage nothing)
+__host__ __device__ constexpr int tab_bytes(bool grad, bool indep) { return grad || !indep ? kTabBytes : kPartBytes; }
+constexpr int smem_bytes(bool grad, bool indep) {
+    return kSmTab + tab_bytes(grad, indep) + kRange * 4 + kWordBytes + 256 + (grad && !indep ? kWarps * kGradRing * 4 : 0);
+}
+static_assert(smem_bytes(true, false) <= 232448 && 2 * (smem_bytes(false, true) + 1024) <= 233472, "shared memory");
+
+__device__ __forceinline__ void copy16_async(uint32_t *dst, const uint32_t *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// Every group but the newest kRing - 2 of this thread has landed.
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(kRing - 2) : "memory"); }
 
 // Exclusive prefix sum of v over the CTA; *total receives the sum. Every thread calls it.
 __device__ __forceinline__ int block_excl(int v, int *red, int *total) {
@@ -286,6 +308,15 @@ __device__ __forceinline__ float reduce_scatter(float (&v)[32], int lane) {
     return v[0];
 }
 
+// x sc (a power of two, |x sc| < 2^61) rounded to an integer without FP64 (slow
+// on this GPU): split exactly into hi 2^31 + lo.
+__device__ __forceinline__ long long to_fixed(float x, float sc) {
+    const float xs = sc * x;
+    const float hi = truncf(xs * 0x1.0p-31f);
+    const float lo = fmaf(-hi, 0x1.0p31f, xs);
+    return ((long long)__float2int_rz(hi) << 31) + (long long)__float2int_rn(lo);
+}
+
 // Adds 2 scale sum_i W_i s_ij of this warp's share of the listed gates into
 // their accumulators: batches of 32 gates, every 16th batch. sc = 2 scale, a
 // power of two in [2^-119, 2^119].
@@ -310,14 +341,102 @@ __device__ __forceinline__ void grad_list(const int2 *list, int n, const ZSource
         }
         const float d = reduce_scatter(v, lane);
         if (e0 + lane < n) {
-            // Fixed-point value without FP64 (slow on this GPU): x = sc d,
-            // |x| < 2^61, split exactly into hi 2^31 + lo.
             const int64_t j = (int64_t)(uint32_t)list[e0 + lane].x;
-            const float x = sc * d;
-            const float hi = truncf(x * 0x1.0p-31f);
-            const float lo = fmaf(-hi, 0x1.0p31f, x);
-            const long long q = ((long long)__float2int_rz(hi) << 31) + (long long)__float2int_rn(lo);
+            const long long q = to_fixed(d, sc);
             if (IQP_IN(j, zs.m, 72)) atomicAdd(gfx + j, (unsigned long long)q);
+        }
+    }
+}
+
+// The words of gates e0 .. e0 + STAGE - 1 (below `end`) of the list into `dst`
+// (STAGE x 32 words): 16-byte piece c of a gate's 128 bytes where c < nch.
+template <int STAGE>
+__device__ __forceinline__ void fetch_stage(uint32_t *dst, const int2 *list, int e0, int end, const uint32_t *pzt,
+                                            int64_t ldzt, int nch, [[maybe_unused]] int64_t m, int lane) {
+#pragma unroll
+    for (int i = 0; i < STAGE / 4; ++i) {
+        const int g = 4 * i + (lane >> 3), c = lane & 7;
+        if (e0 + g < end && c < nch) {
+            const int64_t j = (int64_t)(uint32_t)list[e0 + g].x;
+            if (IQP_IN(j, m, 70)) copy16_async(dst + g * 32 + 4 * c, pzt + j * ldzt + 4 * c);
+        }
+    }
+    copy_commit();
+}
+
+// phase_list for shared batches: this warp's share of the list is a run of
+// gates, its words staged in `ring`. pzt: P_Z^T at this range's words.
+__device__ __forceinline__ void phase_list_staged(float (&acc)[32], const int2 *list, int n, const uint32_t *pzt,
+                                                  int64_t ldzt, int nch, int64_t m, uint32_t *ring, int warp, int lane) {
+    const int per = 5 * ((n + 5 * kWarps - 1) / (5 * kWarps));
+    const int b0 = warp * per, end = b0 + per < n ? b0 + per : n;
+#pragma unroll
+    for (int k = 0; k < kRing - 1; ++k)
+        fetch_stage<kPhaseStage>(ring + k * kPhaseStage * 32, list, b0 + k * kPhaseStage, end, pzt, ldzt, nch, m, lane);
+    int st = 0;
+    for (int e0 = b0; e0 < end; e0 += kPhaseStage) {
+        copy_wait();
+        __syncwarp();
+        const uint32_t *zw = ring + st * kPhaseStage * 32 + lane;
+#pragma unroll 1
+        for (int h = 0; h < kPhaseStage && e0 + h < end; h += 5) {
+            uint32_t z[5], R[8];
+            float t = 0.f;
+#pragma unroll
+            for (int g = 0; g < 5; ++g) {
+                z[g] = zw[(h + g) * 32];
+                const float cv = e0 + h + g < end ? __int_as_float(list[e0 + h + g].y) : 0.f;  // a short batch: c = 0
+                t += ((lane >> g) & 1) ? -cv : cv;
+            }
+            indices5(z, R);
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) acc[8 * k + q] += __shfl_sync(kFull, t, (int)(R[q] >> (8 * k)));
+        }
+        __syncwarp();  // every lane has read the stage that comes free
+        const int nx = st == 0 ? kRing - 1 : st - 1;
+        fetch_stage<kPhaseStage>(ring + nx * kPhaseStage * 32, list, e0 + (kRing - 1) * kPhaseStage, end, pzt, ldzt, nch, m,
+                                 lane);
+        st = st + 1 == kRing ? 0 : st + 1;
+    }
+}
+
+// grad_list for shared batches, staged likewise.
+__device__ __forceinline__ void grad_list_staged(const int2 *list, int n, const uint32_t *pzt, int64_t ldzt, int nch,
+                                                 int64_t m, uint32_t *ring, const float *tab,
+                                                 unsigned long long *__restrict__ gfx, float sc, int warp, int lane) {
+    const float *tl = tab + lane;
+    const int per = 8 * ((n + 8 * kWarps - 1) / (8 * kWarps));
+    const int b0 = warp * per, end = b0 + per < n ? b0 + per : n;
+#pragma unroll
+    for (int k = 0; k < kRing - 1; ++k)
+        fetch_stage<kGradStage>(ring + k * kGradStage * 32, list, b0 + k * kGradStage, end, pzt, ldzt, nch, m, lane);
+    int st = 0;
+    for (int e0 = b0; e0 < end; e0 += 32) {
+        float v[32];
+#pragma unroll
+        for (int h = 0; h < 32; h += kGradStage) {
+            copy_wait();
+            __syncwarp();
+            const uint32_t *zw = ring + st * kGradStage * 32 + lane;
+#pragma unroll
+            for (int g = 0; g < kGradStage; ++g) {
+                const uint32_t z = e0 + h + g < end ? zw[g * 32] : 0u;
+                const float a0 = tl[(z & 0xFFu) * 32], a1 = tl[8192 + ((z >> 8) & 0xFFu) * 32];
+                const float a2 = tl[16384 + ((z >> 16) & 0xFFu) * 32], a3 = tl[24576 + (z >> 24) * 32];
+                v[h + g] = (a0 + a1) + (a2 + a3);
+            }
+            __syncwarp();
+            const int nx = st == 0 ? kRing - 1 : st - 1;
+            fetch_stage<kGradStage>(ring + nx * kGradStage * 32, list, e0 + h + (kRing - 1) * kGradStage, end, pzt, ldzt, nch,
+                                    m, lane);
+            st = st + 1 == kRing ? 0 : st + 1;
+        }
+        const float d = reduce_scatter(v, lane);
+        if (e0 + lane < end) {
+            const int64_t j = (int64_t)(uint32_t)list[e0 + lane].x;
+            if (IQP_IN(j, m, 72)) atomicAdd(gfx + j, (unsigned long long)to_fixed(d, sc));
         }
     }
 }
@@ -346,30 +465,38 @@ __device__ __forceinline__ double block_sum(float v, float *red) {
 // phi: element e = 32-sample position k, lane q of a range's nl valid lanes at
 // range start + k nl + q.
 template <int MODE, bool INDEP>
-__global__ void __launch_bounds__(kThreads, MODE == 0 ? 2 : 1)
+__global__ void __launch_bounds__(kThreads, MODE == 0 && INDEP ? 2 : 1)
     k_sparse(const uint64_t *__restrict__ PA, int64_t ldp, const uint64_t *__restrict__ PZT, int64_t ldzt,
              int64_t m, const float *__restrict__ c, int64_t s, int64_t nparts, double2 *__restrict__ part,
              const double *__restrict__ alpha, const double *__restrict__ beta, const double *__restrict__ scale,
              unsigned long long *__restrict__ gfx, const int4 *__restrict__ sup, const uint64_t *__restrict__ G,
-             int64_t ldg, int64_t n, float *__restrict__ phi, int64_t ldphi, int64_t r0) {
+             int64_t ldg, int64_t n, float *__restrict__ phi, int64_t ldphi, int64_t r0,
+             int64_t rpc) {
     extern __shared__ __align__(16) uint8_t sm[];
     int2 *list = reinterpret_cast<int2 *>(sm + kSmList);
     float *tab = reinterpret_cast<float *>(sm + kSmTab);
-    float *wsm = reinterpret_cast<float *>(sm + kSmTab + (MODE == 0 ? kPartBytes : kTabBytes));
+    float *wsm = reinterpret_cast<float *>(sm + kSmTab + tab_bytes(MODE != 0, INDEP));
     uint32_t *dense = reinterpret_cast<uint32_t *>(wsm + kRange);
     int *red = reinterpret_cast<int *>(dense + kThreads * kScan);
+    [[maybe_unused]] uint32_t *ring = reinterpret_cast<uint32_t *>(red + 64);  // the gradient's
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t a = blockIdx.x, r = r0 + blockIdx.y;
+    const int64_t a = blockIdx.x;
     const int64_t vwords = cdiv(s, 32);
+    const uint64_t *parow = PA + a * ldp;
+    [[maybe_unused]] const int64_t l = gridDim.x;
+    int held = -1;  // gates in the list when it holds all of J_a: listed once for all of the CTA's ranges
+    const int64_t rbeg = r0 + blockIdx.y * rpc, rend = rbeg + rpc < nparts ? rbeg + rpc : nparts;
+    for (int64_t r = rbeg; r < rend; ++r) {
+    if (r > rbeg) __syncthreads();  // the previous range is done with shared memory
     const int nl = (int)(vwords - r * 32 < 32 ? vwords - r * 32 : 32);  // lanes with samples
     const int64_t word = r * 32 + (lane < nl ? lane : nl - 1);          // in-bounds load, result masked
-    const uint64_t *parow = PA + a * ldp;
     const ZSource zs{reinterpret_cast<const uint32_t *>(INDEP ? PZT + a * n * ldzt : PZT), 2 * ldzt, word, sup, G, ldg, n, m};
-    [[maybe_unused]] const int64_t l = gridDim.x;
+    // shared batches: this range's words of P_Z^T row 0, and its 16-byte pieces inside a row (2 ldzt is a multiple of 8)
+    const uint32_t *pzt = reinterpret_cast<const uint32_t *>(PZT) + r * 32;
+    const int nch = (int)(2 * ldzt - r * 32 < 32 ? (2 * ldzt - r * 32) / 4 : 8);
 
     // Phi of elements tid and tid + 512 (element e: sample 32 (e % 32) + e / 32 of the range)
     float ph[2];
-    int held = -1;  // gates in the list when it holds all of J_a
     const bool kept = MODE == 1 && !INDEP && phi != nullptr;
     float *prow = phi == nullptr ? nullptr : phi + a * ldphi + r * kRange;
     if (kept) {
@@ -383,22 +510,28 @@ __global__ void __launch_bounds__(kThreads, MODE == 0 ? 2 : 1)
         float acc[32];
 #pragma unroll
         for (int k = 0; k < 32; ++k) acc[k] = 0.f;
-        RowCursor cur{0, 0};
-        bool first = true;
-        while (true) {
-            const int cnt = list_gates(parow, ldp, m, c, list, dense, red, cur);
-            if (cnt == 0) {
-                if (first) held = 0;
-                break;
+        auto phase = [&](int cnt) {
+            if constexpr (INDEP)
+                phase_list<true>(acc, list, cnt, zs, warp, lane);
+            else
+                phase_list_staged(acc, list, cnt, pzt, 2 * ldzt, nch, m, reinterpret_cast<uint32_t *>(tab) + warp * kPhaseRing,
+                                  warp, lane);
+        };
+        if (held >= 0) {
+            phase(held);
+        } else {
+            RowCursor cur{0, 0};
+            for (bool first = true;; first = false) {
+                const int cnt = list_gates(parow, ldp, m, c, list, dense, red, cur);
+                phase(cnt);
+                if (cur.w0 >= ldp) {
+                    if (first) held = cnt;
+                    break;
+                }
+                __syncthreads();  // the list is read before it is filled again
             }
-            phase_list<INDEP>(acc, list, cnt, zs, warp, lane);
-            if (cur.w0 >= ldp) {
-                if (first) held = cnt;
-                break;
-            }
-            first = false;
-            __syncthreads();  // the list is read before it is filled again
         }
+        __syncthreads();  // the partial phases lie where other warps' rings were
 #pragma unroll
         for (int k = 0; k < 32; ++k) tab[warp * kRange + k * 32 + lane] = acc[k];
         __syncthreads();
@@ -461,20 +594,29 @@ __global__ void __launch_bounds__(kThreads, MODE == 0 ? 2 : 1)
             for (int e = 0; e < 16; ++e) t[e * 32] = hi + (p01[e & 3] + p23[e >> 2]);
         }
         const float sc = (float)(2.0 * *scale);
-        if (held < 0) {
+        auto grad = [&](int cnt) {
+            if constexpr (INDEP)
+                grad_list<true>(list, cnt, zs, tab, gfx, sc, warp, lane);
+            else
+                grad_list_staged(list, cnt, pzt, 2 * ldzt, nch, m, ring + warp * kGradRing, tab, gfx, sc, warp, lane);
+        };
+        if (held >= 0) {
+            __syncthreads();
+            grad(held);
+        } else {
             RowCursor cur{0, 0};
-            while (true) {
+            for (bool first = true;; first = false) {
                 const int cnt = list_gates(parow, ldp, m, c, list, dense, red, cur);  // its barriers also publish the tables
-                if (cnt == 0) break;
-                grad_list<INDEP>(list, cnt, zs, tab, gfx, sc, warp, lane);
-                if (cur.w0 >= ldp) break;
+                grad(cnt);
+                if (cur.w0 >= ldp) {
+                    if (first) held = cnt;
+                    break;
+                }
                 __syncthreads();
             }
-        } else {
-            __syncthreads();
-            grad_list<INDEP>(list, held, zs, tab, gfx, sc, warp, lane);
         }
     }
+    }  // ranges
 }
 
 // scale = 2^k with B 2^k < 2^61, B = sum_a 2 s (|alpha_a| + |beta_a|)
@@ -509,7 +651,7 @@ cudaError_t launch_k(int64_t l, int64_t nparts, int kernel, const uint64_t *PA, 
                      int64_t ldzt, int64_t m, const float *c, int64_t s, double2 *part, const double *alpha,
                      const double *beta, const double *scale, unsigned long long *gfx, const SparseIndep *ind, float *phi,
                      int64_t ldphi, cudaStream_t st) {
-    constexpr int smem = smem_bytes(MODE != 0);
+    constexpr int smem = smem_bytes(MODE != 0, INDEP);
     static bool attr_set = false;
     if (!attr_set) {
         const cudaError_t e =
@@ -518,13 +660,18 @@ cudaError_t launch_k(int64_t l, int64_t nparts, int kernel, const uint64_t *PA, 
         attr_set = true;
     }
     // Observables on grid x (the CTAs running at once share a range's P_Z^T
-    // segments in L2), ranges on y, at most 65535 per launch.
-    for (int64_t r0 = 0; r0 < nparts; r0 += 65535) {
-        const int64_t nr = nparts - r0 < 65535 ? nparts - r0 : 65535;
+    // segments in L2), ranges on y: a CTA takes as many of them as leave four
+    // CTAs per SM, so that J_a is listed once for them all (5% of the time where
+    // P_A's density is 0.008), at most 65535 blocks per launch.
+    int64_t rpc = l * nparts / (4 * (int64_t)num_sms() + 1);
+    rpc = rpc < 1 ? 1 : (rpc > nparts ? nparts : rpc);
+    rpc = cdiv(nparts, cdiv(nparts, rpc));  // equal shares
+    for (int64_t r0 = 0; r0 < nparts; r0 += 65535 * rpc) {
+        const int64_t nr = cdiv(nparts - r0, rpc) < 65535 ? cdiv(nparts - r0, rpc) : 65535;
         LaunchScope ls(kernel, st);
         k_sparse<MODE, INDEP><<<dim3((unsigned)l, (unsigned)nr), kThreads, smem, st>>>(
             PA, ldp, PZT, ldzt, m, c, s, nparts, part, alpha, beta, scale, gfx, ind ? ind->sup : nullptr,
-            ind ? ind->G : nullptr, ind ? ind->ldg : 0, ind ? ind->n : 0, phi, ldphi, r0);
+            ind ? ind->G : nullptr, ind ? ind->ldg : 0, ind ? ind->n : 0, phi, ldphi, r0, rpc);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
