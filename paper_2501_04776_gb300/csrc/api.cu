@@ -72,7 +72,8 @@ cudaError_t launch_sparse_value_grad(const uint64_t *PA, int64_t ldp, const uint
                                      double *grad, cudaStream_t st);
 cudaError_t launch_bit_transpose_batched(const uint64_t *in, int64_t batch, int64_t in_rows, int64_t in_cols,
                                          int64_t ld_in, uint64_t *out, int64_t ld_out, cudaStream_t st);
-cudaError_t launch_support_list(const uint64_t *G, int64_t m, int64_t ldg, int64_t n, int4 *sup, cudaStream_t st);
+cudaError_t launch_support_list(const uint64_t *G, int64_t m, int64_t ldg, int64_t n, int4 *sup, cudaStream_t st,
+                                const float *theta = nullptr, unsigned *cmax = nullptr);
 cudaError_t launch_expand_params(const float *theta_p, int64_t np, const int64_t *start, int64_t m, float *theta_gen,
                                  cudaStream_t st);
 cudaError_t launch_reduce_params(const double *grad_gen, int64_t m, const int64_t *start, int64_t np,
@@ -85,19 +86,11 @@ cudaError_t launch_bernoulli_bits(uint64_t seed, uint64_t stream, int64_t rows, 
                                   uint64_t *out, cudaStream_t st);
 int64_t lo_part_samples();
 int64_t lo_split_elems(int64_t n, int64_t lds);
-cudaError_t launch_lo_prepare(int64_t n, const uint64_t *G, int64_t m, int64_t ldg, const uint64_t *Z, int64_t s,
-                              int64_t ldz, const float *c, int4 *sup, uint64_t *ZT, int64_t ldzt, float *C,
-                              int64_t ldc, float *M, int64_t lds, __nv_bfloat16 *split, unsigned long long *fx,
-                              uint32_t *status, cudaStream_t st);
-cudaError_t launch_lo_stats(const uint64_t *A, int64_t lda, int64_t n, int64_t l, const uint64_t *ZT, int64_t ldzt,
-                            const float *M, int64_t lds, const float *C, int64_t ldc, int64_t s, double2 *part,
-                            int64_t nparts, float *phi, int64_t ldphi, uint32_t *status, cudaStream_t st);
-cudaError_t launch_lo_grad(const uint64_t *A, int64_t lda, int64_t n, int64_t l, const uint64_t *ZT, int64_t ldzt,
-                           const float *M, int64_t lds, const float *C, int64_t ldc, int64_t s, int64_t m,
-                           const int4 *sup, const double *alpha, const double *beta, uint64_t *AT, int64_t ldlt,
-                           float *W, float *V, double *H, double *gsp, unsigned long long *Kfx, double *grad,
-                           __nv_bfloat16 *split, const float *phi, int64_t ldphi, bool scale_set, uint32_t *status,
-                           cudaStream_t st);
+cudaError_t launch_lo_prepare(const LoArgs &a, cudaStream_t st);
+cudaError_t launch_lo_stats(const LoArgs &a, double2 *part, float *phi, int64_t ldphi, cudaStream_t st);
+cudaError_t launch_lo_grad(const LoArgs &a, double2 *part, const double *alpha, const double *beta, uint64_t *AT,
+                           int64_t ldlt, float *W, float *V, double *gsp, double *grad, float *phi, int64_t ldphi,
+                           bool scale_set, cudaStream_t st);
 cudaError_t launch_bitflip_gates(const float *theta, int64_t m, int64_t mpad, double *c, double *t, cudaStream_t st);
 cudaError_t launch_bitflip_rows(const uint64_t *PA, int64_t ldp, int64_t l, const double *c, double *expval,
                                 cudaStream_t st);
@@ -209,6 +202,17 @@ Plan make_plan(int op, int64_t n, int64_t m, int64_t l, int64_t s, int64_t N, in
         p.off_skp = take((int64_t)kMaxSplitCtas * kSplitSlotFloats * 4 + (int64_t)kMaxSplitCtas * 4);
         p.off_gsum = take((int64_t)kMaxSplitCtas * kDtSumFloats * 4);
         p.off_skx = take((int64_t)kSplitSlots * kSplitSlotFloats * 4 + (int64_t)kMaxSplitCtas * 4);
+    }
+    // Low-order: the lists and the K pieces of H (a workspace that ends before
+    // their end takes the one-CTA form for every observable, and H in one piece).
+    p.off_lo_zp = p.off_lo_q = p.off_lo_p = p.off_lo_cnt = p.off_lo_hp = 0;
+    if (lo) {
+        p.off_opt = off;
+        p.off_lo_zp = take(n * cdiv(s, (int64_t)1024) * 32 * 4);
+        p.off_lo_q = take(l * kLoQ * 4);
+        p.off_lo_p = take(l * kLoP * 8);
+        p.off_lo_cnt = take(2 * l * 4);
+        p.off_lo_hp = take(grad ? n * p.ldc * 4 * lo_hparts(n, s) : 0);
     }
     // MMD: scratch of the data parities by row gather (a workspace that ends
     // before its end folds them densely).
@@ -349,6 +353,7 @@ iqp_status check_ws(Plan &p, void *ws, size_t ws_bytes) {
         if (ws_bytes < plan_min_bytes(p)) return IQP_ERR_WORKSPACE;
         p.x3 = false;  // FP32: the SIMT kernels
         p.off_xt = 0;  // data parities folded densely
+        p.off_lo_zp = p.off_lo_hp = 0;  // low-order: no lists, H in one piece
         // The optional regions at the end, in order: each is used only where
         // the workspace reaches its end.
         if (p.off_skx != 0 && ws_bytes < p.off_skx + (size_t)round_up((int64_t)kSplitSlots * kSplitSlotFloats * 4 +
@@ -374,6 +379,37 @@ T *at(void *ws, size_t off) {
         if (e_ != cudaSuccess) return IQP_ERR_CUDA;     \
     } while (0)
 
+LoArgs lo_args(const Plan &p, void *ws) {
+    LoArgs a{};
+    a.n = p.n;
+    a.m = p.m;
+    a.l = p.l;
+    a.s = p.s;
+    a.A = p.A;
+    a.lda = p.lda;
+    a.sup = at<int4>(ws, p.off_sup);
+    a.ZT = at<uint64_t>(ws, p.off_pzt);
+    a.ldzt = p.ldzt;
+    a.X = at<float>(ws, p.off_lo_m);
+    a.lds = p.ldw;
+    a.C = at<float>(ws, p.off_lo_c);
+    a.ldc = p.ldc;
+    a.d = a.C + p.n * p.ldc;
+    a.E = reinterpret_cast<unsigned long long *>(a.d + p.ldc);
+    a.fx = at<unsigned long long>(ws, p.off_gpart);
+    a.split = at<__nv_bfloat16>(ws, p.off_lo_a);
+    if (p.off_lo_zp != 0) {
+        a.ZP = at<uint32_t>(ws, p.off_lo_zp);
+        a.Lq = at<int>(ws, p.off_lo_q);
+        a.Lp = at<uint2>(ws, p.off_lo_p);
+        a.cnt = at<int>(ws, p.off_lo_cnt);
+    }
+    a.H = at<float>(ws, p.off_lo_hp != 0 ? p.off_lo_hp : p.off_lo_h);
+    a.hparts = p.off_lo_hp != 0 ? lo_hparts(p.n, p.s) : 1;
+    a.status = at<uint32_t>(ws, p.off_status);
+    return a;
+}
+
 // Parities of A and Z by support gather (P_A, P_A^T, P_Z, P_Z^T) + theta split.
 // Independent batches: P_A, every batch of Z transposed, and the gate
 // supports (the sample parities are formed inside the row-sparse kernels).
@@ -382,11 +418,13 @@ iqp_status prepare(const Plan &p, void *ws, const uint64_t *G, int64_t ldg, cons
     uint64_t *rt = at<uint64_t>(ws, p.off_rt);
     if (p.prec == IQP_LOWORDER_FP32 && !p.indep) {
         // no parity matrices: C, d, the samples transposed and M = C S
-        IQP_TRY(launch_theta_prep(theta, p.m, p.mpad, at<float>(ws, p.off_c), nullptr, nullptr, st));
-        IQP_TRY(launch_lo_prepare(p.n, G, p.m, ldg, Z, p.s, ldz, at<float>(ws, p.off_c), at<int4>(ws, p.off_sup),
-                                  at<uint64_t>(ws, p.off_pzt), p.ldzt, at<float>(ws, p.off_lo_c), p.ldc,
-                                  at<float>(ws, p.off_lo_m), p.ldw, at<__nv_bfloat16>(ws, p.off_lo_a),
-                                  at<unsigned long long>(ws, p.off_gpart), at<uint32_t>(ws, p.off_status), st));
+        LoArgs lo = lo_args(p, ws);
+        lo.G = G;
+        lo.ldg = ldg;
+        lo.Z = Z;
+        lo.ldz = ldz;
+        lo.theta = theta;
+        IQP_TRY(launch_lo_prepare(lo, st));
         return IQP_OK;
     }
     const int4 *sup = at<int4>(ws, p.off_sup);
@@ -440,9 +478,7 @@ iqp_status forward_partials(const Plan &p, void *ws, cudaStream_t st, const doub
         if (launch_phase_tc(0, p, ws, nullptr, nullptr, st, &why) != cudaSuccess)
             return why != IQP_OK ? why : IQP_ERR_CUDA;
     } else if (p.prec == IQP_LOWORDER_FP32) {
-        IQP_TRY(launch_lo_stats(p.A, p.lda, p.n, p.l, at<uint64_t>(ws, p.off_pzt), p.ldzt, at<float>(ws, p.off_lo_m),
-                                p.ldw, at<float>(ws, p.off_lo_c), p.ldc, p.s, part, p.nparts,
-                                p.phi_out ? p.phi : nullptr, p.ldphi, at<uint32_t>(ws, p.off_status), st));
+        IQP_TRY(launch_lo_stats(lo_args(p, ws), part, p.phi_out ? p.phi : nullptr, p.ldphi, st));
     } else if (p.prec == IQP_SPARSE_FP32) {
         const SparseIndep ind{at<int4>(ws, p.off_sup), p.G, p.ldg, p.n};
         IQP_TRY(launch_sparse_stats(at<uint64_t>(ws, p.off_pa), p.ldp,
@@ -476,12 +512,9 @@ iqp_status backward(const Plan &p, void *ws, const double *alpha, const double *
                     cudaStream_t st) {
     double *gpart = at<double>(ws, p.off_gpart);
     if (p.prec == IQP_LOWORDER_FP32) {
-        IQP_TRY(launch_lo_grad(p.A, p.lda, p.n, p.l, at<uint64_t>(ws, p.off_pzt), p.ldzt, at<float>(ws, p.off_lo_m),
-                               p.ldw, at<float>(ws, p.off_lo_c), p.ldc, p.s, p.m, at<int4>(ws, p.off_sup), alpha, beta,
-                               at<uint64_t>(ws, p.off_rt), p.ldlt, at<float>(ws, p.off_w), at<float>(ws, p.off_lo_v),
-                               at<double>(ws, p.off_lo_h), at<double>(ws, p.off_lo_gs),
-                               at<unsigned long long>(ws, p.off_gpart), grad, at<__nv_bfloat16>(ws, p.off_lo_a),
-                               p.phi_in ? p.phi : nullptr, p.ldphi, p.scale_set, at<uint32_t>(ws, p.off_status), st));
+        IQP_TRY(launch_lo_grad(lo_args(p, ws), nullptr, alpha, beta, at<uint64_t>(ws, p.off_rt), p.ldlt,
+                               at<float>(ws, p.off_w), at<float>(ws, p.off_lo_v), at<double>(ws, p.off_lo_gs), grad,
+                               p.phi_in ? p.phi : nullptr, p.ldphi, p.scale_set, st));
         return IQP_OK;
     }
     if (p.prec == IQP_SPARSE_FP32) {
@@ -786,10 +819,13 @@ iqp_status iqp_expval_value_and_grad(int64_t n, const uint64_t *G, int64_t m, in
         return IQP_OK;
     }
     if (prec != IQP_SPLIT_BF16) {
-        if (prec == IQP_LOWORDER_FP32) {  // W from the kept Phi (in the W buffer), no second phase pass
-            p.phi = at<float>(ws, p.off_w);
-            p.ldphi = p.ldw;
-            p.phi_out = p.phi_in = true;
+        if (prec == IQP_LOWORDER_FP32) {  // one pass over Phi: the statistics, W and the pair corrections
+            double2 *part = at<double2>(ws, p.off_part);
+            IQP_TRY(launch_lo_grad(lo_args(p, ws), part, alpha, beta, at<uint64_t>(ws, p.off_rt), p.ldlt,
+                                   at<float>(ws, p.off_w), at<float>(ws, p.off_lo_v), at<double>(ws, p.off_lo_gs), grad,
+                                   nullptr, 0, false, st));
+            IQP_TRY(launch_finalize(part, p.nparts, p.pw, p.l, p.s, expval, std_err, nullptr, nullptr, st));
+            return IQP_OK;
         }
         if ((rc = forward_stats(p, ws, expval, std_err, nullptr, nullptr, st)) != IQP_OK) return rc;
         return backward(p, ws, alpha, beta, grad, st);

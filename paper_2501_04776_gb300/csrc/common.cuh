@@ -62,6 +62,8 @@ struct Plan {
     // of the pass over the terms
     size_t off_xt, off_heavy;
     int64_t ldxt;
+    // low-order lists (optional): lane-ordered sample bits, the observables' qubits, pairs and counts
+    size_t off_lo_zp, off_lo_q, off_lo_p, off_lo_cnt, off_lo_hp;
     bool scale_set;  // the gradient's fixed-point scale is in place already (set with the MMD terms)
     size_t off_phi;  // MMD gradient (split BF16, row-sparse): room for Phi, l x ldw fp32 (0 if none)
     // Kept Phi (l x ldphi fp32, ldphi a multiple of 64 >= s; the layout is the
@@ -77,6 +79,40 @@ struct Plan {
     const uint64_t *A;  // observables (read by the low-order kernels)
     int64_t lda;
 };
+
+// The low-order form's buffers and inputs (loworder.cu).
+struct LoArgs {
+    int64_t n, m, l, s;
+    const uint64_t *G, *A, *Z;
+    int64_t ldg, lda, ldz;
+    const float *theta;
+    int4 *sup;                 // m: the gates' supports
+    uint64_t *ZT;              // n x ldzt words: the samples transposed
+    int64_t ldzt;
+    float *X;                  // n x lds: s_q (d_q + (C S)_q)
+    int64_t lds;
+    float *C, *d;              // C (n x ldc; only where the contractions run as sums), d (n)
+    int64_t ldc;
+    unsigned long long *E;     // pair-existence bits
+    unsigned long long *fx;    // n x n fixed-point sums (C, then the gradient's K), n more (d, then the scale), cmax, counter
+    __nv_bfloat16 *split;      // split-BF16 operand of the contractions
+    uint32_t *ZP;              // n x 32 ceil(s / 1024): the sample bits in lane order (null: no lists, the one-CTA form)
+    int *Lq;                   // l x kLoQ: the observables' qubits
+    uint2 *Lp;                 // l x kLoP: their pairs with a generator (q | r << 16, bits of -2 C_qr)
+    int *cnt;                  // l: qubits | pairs << 16, or -1 for an observable too heavy for the lists; then those
+    float *H;                  // hparts x n x ldc
+    int hparts;
+    uint32_t *status;
+};
+constexpr int kLoQ = 64, kLoP = 256;  // qubits and pairs listed per observable
+// K pieces of the gradient's pair contraction (tiles of 256 x 256, 76 CTA
+// pairs): as many as fill the chip with at least eight 64-sample stages each.
+__host__ __device__ inline int lo_hparts(int64_t n, int64_t s) {
+    const int64_t t = cdiv(n, 256) * cdiv(n, 256), nks = cdiv(s, 64);
+    int64_t p = t < 76 ? 76 / t : 1;
+    if (p > nks / 8) p = nks / 8;
+    return (int)(p < 1 ? 1 : p);
+}
 
 // Independent-batch arguments of the row-sparse kernels.
 struct SparseIndep {
@@ -102,11 +138,15 @@ iqp_status expval_arg_check(int64_t n, const uint64_t *G, int64_t m, int64_t ldg
 // for r < rows, c < nb. a_hi / a_lo: rows x kpad BF16 (row-major, kpad a
 // multiple of 64, zero for k >= K); b_bits: nb rows of ldb words (even,
 // >= 4, bits >= K zero or multiplied by zero); out: row-major, ldo elements
-// per row (a multiple of 4), FP32 or FP64. cudaErrorNotSupported when a
+// per row (a multiple of 4). cudaErrorNotSupported when a
 // shape or layout rule does not hold (nothing is launched then).
+// kparts > 1: the K range in kparts pieces (whole 256-wide bits stages), piece
+// p's sums into out + p rows ldo; d != nullptr: out[r][c] = (d[r] + that sum)
+// with the sign bit c of row r of zt (rows of ldzt words) applied.
 cudaError_t launch_tc_dense(const __nv_bfloat16 *a_hi, const __nv_bfloat16 *a_lo, int64_t rows, int64_t kpad,
-                            int64_t k, const uint64_t *b_bits, int64_t nb, int64_t ldb, void *out, int64_t ldo,
-                            bool out_f64, uint32_t *status, cudaStream_t st);
+                            int64_t k, const uint64_t *b_bits, int64_t nb, int64_t ldb, float *out, int64_t ldo,
+                            int kparts, const float *d, const uint64_t *zt, int64_t ldzt, uint32_t *status,
+                            cudaStream_t st);
 
 // Fixed-point scale of a gradient accumulator: 2^k with B 2^k < 2^61 for a
 // bound B of every partial sum; k clamped so that 2^(k+1) is a normal FP32 number.
@@ -116,6 +156,46 @@ __device__ __forceinline__ double fixed_scale(double B) {
     if (e < -58) e = -58;
     if (e > 180) e = 180;
     return ldexp(1.0, 60 - e);
+}
+
+// x sc (a power of two, |x sc| < 2^61) rounded to an integer without FP64 (slow
+// on this GPU): split exactly into hi 2^31 + lo.
+__device__ __forceinline__ long long to_fixed(float x, float sc) {
+    const float xs = sc * x;
+    const float hi = truncf(xs * 0x1.0p-31f);
+    const float lo = fmaf(-hi, 0x1.0p31f, xs);
+    return ((long long)__float2int_rz(hi) << 31) + (long long)__float2int_rn(lo);
+}
+
+// Five words (bit i of word g = sample i's sign under gate g) to a 5-bit index
+// per sample: byte b of R[q] holds, in its low five bits, the index of sample
+// 8 b + q (the bits above them are zero).
+__device__ __forceinline__ void indices5(const uint32_t (&w)[5], uint32_t (&R)[8]) {
+    constexpr uint32_t m1 = 0x55555555u, m2 = 0x33333333u, m4 = 0x0F0F0F0Fu, mh = 0x10101010u;
+    const uint32_t x0 = (w[0] & m1) | ((w[1] << 1) & ~m1), x1 = ((w[0] >> 1) & m1) | (w[1] & ~m1);
+    const uint32_t y0 = (w[2] & m1) | ((w[3] << 1) & ~m1), y1 = ((w[2] >> 1) & m1) | (w[3] & ~m1);
+    const uint32_t u[4] = {(x0 & m2) | ((y0 << 2) & ~m2), (x1 & m2) | ((y1 << 2) & ~m2),
+                           ((x0 >> 2) & m2) | (y0 & ~m2), ((x1 >> 2) & m2) | (y1 & ~m2)};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        R[q] = (u[q] & m4) | ((w[4] << (4 - q)) & mh);
+        R[q + 4] = ((u[q] >> 4) & m4) | ((w[4] >> q) & mh);
+    }
+}
+
+// Sum over the 32 lanes of v[lane][k]: afterwards lane L returns the sum of column L.
+__device__ __forceinline__ float reduce_scatter(float (&v)[32], int lane) {
+#pragma unroll
+    for (int w = 16; w >= 1; w >>= 1) {
+        const bool upper = (lane & w) != 0;
+#pragma unroll
+        for (int k = 0; k < w; ++k) {
+            const float send = upper ? v[k] : v[k + w];
+            const float keep = upper ? v[k + w] : v[k];
+            v[k] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, w);
+        }
+    }
+    return v[0];
 }
 
 // ---------------------------------------------------------------- status

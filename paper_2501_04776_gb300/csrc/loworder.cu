@@ -8,6 +8,7 @@
 // so the phase of eq. expvalsample regroups exactly into
 //   Phi[a,i] = sum_{q in Q_a} s_q(i) (d_q + M[q,i]) - 2 sum_{q<r in Q_a} C_qr s_q(i) s_r(i),
 //   M = C S,  S[r][i] = s_r(i)        (an n x n x s contraction over the pairs with a generator),
+// held as X[q,i] = s_q(i) (d_q + M[q,i]), formed in the contraction's epilogue,
 // and with W[a,i] = sin Phi (alpha_a + beta_a cos Phi), V[q,i] = sum_{a : q in Q_a} W[a,i]:
 //   grad(gate e_q)       = 2 sum_i s_q(i) V[q,i],
 //   grad(gate e_q + e_r) = 2 (H[q,r] + H[r,q]) - 4 K[q,r],
@@ -33,7 +34,8 @@ namespace {
 
 constexpr int kQMax = 1024;  // observable weight limit (support list in shared memory)
 constexpr int kPairMax = 512;  // pairs of Q_a held in shared memory per round
-constexpr int kBlk = 256;    // samples per CTA in the per-observable kernels
+constexpr int kBlk = 256;    // samples per partial, and per block of the heavy observables' kernels
+constexpr int kLane = 1024;  // samples per warp in the listed observables' kernels (32 per lane)
 constexpr int kQ4 = 256;     // supports up to this size take four sample blocks per pass in k_lo_phase
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
@@ -68,28 +70,11 @@ __device__ __forceinline__ int lo_fx_exp(unsigned cmax_bits, int64_t m) {
     return k < -60 ? -60 : (k > 100 ? 100 : k);
 }
 
-__global__ void k_lo_cmax(const int4 *__restrict__ sup, const float *__restrict__ c, int64_t m,
-                          unsigned *__restrict__ cmax) {
-    unsigned v = 0u;
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
-        const int w = sup[j].w;
-        if (w == 1 || w == 2) {
-            const unsigned b = __float_as_uint(fabsf(c[j]));  // non-negative floats order like their bits
-            v = b > v ? b : v;
-        }
-    }
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) {
-        const unsigned o = __shfl_xor_sync(kFull, v, off);
-        v = o > v ? o : v;
-    }
-    if ((threadIdx.x & 31) == 0 && v != 0u) atomicMax(cmax, v);
-}
-
-// Cfx (n x n) and dfx (n): fixed-point sums of c_j; E bits.
-__global__ void k_lo_build(const int4 *__restrict__ sup, const float *__restrict__ c, int64_t m, int64_t n,
+// Cfx (n x n, upper triangle) and dfx (n): fixed-point sums of c_j = 2 theta_j;
+// E bits (upper triangle, both with `full`).
+__global__ void k_lo_build(const int4 *__restrict__ sup, const float *__restrict__ theta, int64_t m, int64_t n,
                            unsigned long long *__restrict__ Cfx, unsigned long long *__restrict__ dfx,
-                           const unsigned *__restrict__ cmax, unsigned long long *__restrict__ E, int64_t lde,
+                           const unsigned *__restrict__ cmax, unsigned long long *__restrict__ E, int64_t lde, int full,
                            uint32_t *__restrict__ status) {
     [[maybe_unused]] uint32_t *status_dbg = status;
     const int k = lo_fx_exp(*cmax, m);
@@ -97,14 +82,13 @@ __global__ void k_lo_build(const int4 *__restrict__ sup, const float *__restrict
         const int4 sp = sup[j];
         if (!LO_OK(sp.w <= 0 || (sp.x >= 0 && sp.x < n && (sp.w < 2 || (sp.y > sp.x && sp.y < n))), 8)) continue;
         if (sp.w == 1 || sp.w == 2) {
-            const unsigned long long v = (unsigned long long)llrint(ldexp((double)c[j], k));
+            const unsigned long long v = (unsigned long long)llrint(ldexp((double)(2.0f * theta[j]), k));
             if (sp.w == 1) {
                 atomicAdd(dfx + sp.x, v);
             } else {
                 atomicAdd(Cfx + (int64_t)sp.x * n + sp.y, v);
-                atomicAdd(Cfx + (int64_t)sp.y * n + sp.x, v);
                 atomicOr(E + (int64_t)sp.x * lde + (sp.y >> 6), 1ull << (sp.y & 63));
-                atomicOr(E + (int64_t)sp.y * lde + (sp.x >> 6), 1ull << (sp.x & 63));
+                if (full) atomicOr(E + (int64_t)sp.y * lde + (sp.x >> 6), 1ull << (sp.x & 63));
             }
         } else if (sp.w > 2) {
             record_status(status, IQP_ERR_ARG);
@@ -112,21 +96,144 @@ __global__ void k_lo_build(const int4 *__restrict__ sup, const float *__restrict
     }
 }
 
-// C (n x ldc, zero in columns >= n) and d (n) from their fixed-point sums,
-// each rounded to FP32 once.
-__global__ void k_lo_fx_float(const unsigned long long *__restrict__ Cfx, const unsigned long long *__restrict__ dfx,
-                              const unsigned *__restrict__ cmax, int64_t m, int64_t n, float *__restrict__ C,
-                              int64_t ldc, float *__restrict__ d) {
+// C from the upper triangle of its fixed-point sums, each rounded to FP32
+// once, as the split-BF16 operand (n x kc, zero in columns >= n) and, where the
+// contractions run as sums, as FP32 (n x ldc); d (n) likewise. One block per
+// pair of 64 x 64 tiles (bi <= bj), which reads the upper tile once and writes
+// it and its transpose.
+__global__ void __launch_bounds__(256) k_lo_convert(const unsigned long long *__restrict__ Cfx,
+                                                    const unsigned long long *__restrict__ dfx,
+                                                    const unsigned *__restrict__ cmax, int64_t m, int64_t n, int nb,
+                                                    __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo,
+                                                    int64_t kc, float *__restrict__ C, int64_t ldc,
+                                                    float *__restrict__ d) {
+    __shared__ float tile[64][65];
     const float inv = ldexpf(1.0f, -lo_fx_exp(*cmax, m));
-    const int64_t total = n * ldc;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total + n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        if (i < total) {
-            const int64_t q = i / ldc, r = i - q * ldc;
-            C[i] = r < n ? __ll2float_rn((long long)Cfx[q * n + r]) * inv : 0.f;
-        } else {
-            d[i - total] = __ll2float_rn((long long)dfx[i - total]) * inv;
+    int bi = 0, left = blockIdx.x;  // block number -> (bi, bj), row by row
+    while (left >= nb - bi) {
+        left -= nb - bi;
+        ++bi;
+    }
+    const int bj = bi + left;
+    const int64_t q0 = 64 * (int64_t)bi, r0 = 64 * (int64_t)bj;
+    for (int e = threadIdx.x; e < 64 * 64; e += 256) {
+        const int64_t q = q0 + (e >> 6), r = r0 + (e & 63);
+        tile[e >> 6][e & 63] = q < r && r < n ? __ll2float_rn((long long)Cfx[q * n + r]) * inv : 0.f;
+    }
+    if (bi == bj && threadIdx.x < 64 && q0 + threadIdx.x < n)
+        d[q0 + threadIdx.x] = __ll2float_rn((long long)dfx[q0 + threadIdx.x]) * inv;
+    __syncthreads();
+    // side 0: rows q0.. (columns r0..); side 1: rows r0.. (columns q0..), the transpose
+    for (int side = 0; side < (bi == bj ? 1 : 2); ++side) {
+        const int64_t row0 = side ? r0 : q0, col0 = side ? q0 : r0;
+        for (int e = threadIdx.x; e < 64 * 8; e += 256) {
+            const int a = e >> 3, b = (e & 7) * 8;
+            if (row0 + a >= n) continue;
+            uint32_t ph[4], pl[4];
+            float x[8];
+#pragma unroll
+            for (int t = 0; t < 8; ++t)
+                x[t] = side ? tile[b + t][a] : (bi == bj && b + t < a ? tile[b + t][a] : tile[a][b + t]);
+#pragma unroll
+            for (int t = 0; t < 8; t += 2) {
+                const __nv_bfloat16 h0 = __float2bfloat16_rn(x[t]), h1 = __float2bfloat16_rn(x[t + 1]);
+                const __nv_bfloat16 l0 = __float2bfloat16_rn(x[t] - __bfloat162float(h0));
+                const __nv_bfloat16 l1 = __float2bfloat16_rn(x[t + 1] - __bfloat162float(h1));
+                ph[t / 2] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
+                pl[t / 2] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+            }
+            const int64_t at = (row0 + a) * kc + col0 + b;
+            *reinterpret_cast<uint4 *>(hi + at) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
+            *reinterpret_cast<uint4 *>(lo + at) = make_uint4(pl[0], pl[1], pl[2], pl[3]);
+            if (C != nullptr)
+                for (int t = 0; t < 8; ++t)
+                    if (col0 + b + t < ldc) C[(row0 + a) * ldc + col0 + b + t] = x[t];
         }
+    }
+}
+
+// The sample bits in lane order: word (q, 32 b + L) of ZP holds lane L's 32
+// samples of the 1024-sample block b, bit 4 k + j being sample
+// 1024 b + 128 k + 4 L + j (so that a lane's floats are eight coalesced 16-byte
+// words). One warp per (q, b).
+__global__ void __launch_bounds__(256) k_lo_zpack(const uint32_t *__restrict__ ZT, int64_t ldzt32, int64_t n, int64_t nb,
+                                                  uint32_t *__restrict__ ZP) {
+    const int lane = threadIdx.x & 31;
+    const int64_t total = n * nb;
+    for (int64_t i = (blockIdx.x * (int64_t)256 + threadIdx.x) >> 5; i < total; i += (int64_t)gridDim.x * 8) {
+        const int64_t q = i / nb, b = i - q * nb;
+        const uint32_t w = 32 * b + lane < ldzt32 ? ZT[q * ldzt32 + 32 * b + lane] : 0u;
+        uint32_t o = 0u;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            o |= ((__shfl_sync(kFull, w, 4 * k + (lane >> 3)) >> (4 * (lane & 7))) & 0xFu) << (4 * k);
+        ZP[(q * nb + b) * 32 + lane] = o;
+    }
+}
+
+// Every observable's qubits (in increasing order) and, with C, the pairs among
+// them that carry a generator, one warp per observable. One of more than kLoQ
+// qubits or kLoP pairs is left to the heavy observables' kernels: cnt = -1, and
+// its number in `heavy` (counted in *nheavy).
+__global__ void __launch_bounds__(256) k_lo_lists(const uint64_t *__restrict__ A, int64_t lda, int64_t l, int64_t n,
+                                                  const unsigned long long *__restrict__ E, int64_t lde,
+                                                  const unsigned long long *__restrict__ Cfx,
+                                                  const unsigned *__restrict__ cmax, int64_t m, int *__restrict__ Lq,
+                                                  uint2 *__restrict__ Lp, int *__restrict__ cnt, int *__restrict__ heavy,
+                                                  unsigned *__restrict__ nheavy, uint32_t *__restrict__ status) {
+    [[maybe_unused]] uint32_t *status_dbg = status;
+    __shared__ int sq[8][kLoQ];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t a = (int64_t)blockIdx.x * 8 + warp;
+    if (a >= l) return;
+    const float inv = ldexpf(1.0f, -lo_fx_exp(*cmax, m));
+    const int64_t nw = (n + 63) >> 6;
+    int nq = 0;
+    for (int64_t wb = 0; wb < nw; wb += 32) {
+        uint64_t w = wb + lane < nw ? A[a * lda + wb + lane] : 0ull;
+        if (wb + lane == nw - 1 && (n & 63)) w &= (1ull << (n & 63)) - 1ull;  // never a qubit >= n
+        const int c = __popcll(w);
+        int incl = c;
+#pragma unroll
+        for (int s = 1; s < 32; s <<= 1) {
+            const int u = __shfl_up_sync(kFull, incl, s);
+            if (lane >= s) incl += u;
+        }
+        int p = nq + incl - c;
+        while (w) {
+            if (p < kLoQ) sq[warp][p] = (int)(64 * (wb + lane)) + __ffsll((long long)w) - 1;
+            w &= w - 1ull;
+            ++p;
+        }
+        nq += __shfl_sync(kFull, incl, 31);
+    }
+    __syncwarp();
+    int np = 0;
+    if (nq <= kLoQ) {
+        for (int t = lane; t < nq; t += 32) Lq[a * kLoQ + t] = sq[warp][t];
+        for (int t = 0; t + 1 < nq; ++t) {
+            const int q = sq[warp][t];
+            for (int u0 = t + 1; u0 < nq; u0 += 32) {
+                const int u = u0 + lane;
+                const int r = u < nq ? sq[warp][u] : 0;
+                const bool ok = u < nq && LO_OK(q >= 0 && q < r && r < n, 10) &&
+                                ((E[(int64_t)q * lde + (r >> 6)] >> (r & 63)) & 1ull) != 0ull;
+                const uint32_t bal = __ballot_sync(kFull, ok);
+                const int pos = np + __popc(bal & ((1u << lane) - 1u));
+                if (ok && pos < kLoP) {
+                    const float c = __ll2float_rn((long long)Cfx[(int64_t)q * n + r]) * inv;
+                    Lp[a * kLoP + pos] = make_uint2((uint32_t)q | ((uint32_t)r << 16), __float_as_uint(-2.0f * c));
+                }
+                np += __popc(bal);
+            }
+        }
+    }
+    if (lane != 0) return;
+    const bool listed = nq <= kLoQ && np <= kLoP;
+    cnt[a] = listed ? nq | (np << 16) : -1;
+    if (!listed) {
+        const unsigned h = atomicAdd(nheavy, 1u);
+        if (h < l) heavy[h] = (int)a;
     }
 }
 
@@ -158,12 +265,12 @@ __device__ __forceinline__ void for_each_bit(const unsigned long long *__restric
     }
 }
 
-// M[q][i] = sum_{r in E_q} C_qr s_r(i) (M = C S restricted to the pairs with
-// a generator, which is all of C's nonzeros). Grid (n, ranges) x 32 threads.
+// X[q][i] = s_q(i) (d_q + sum_{r in E_q} C_qr s_r(i)) (C S restricted to the
+// pairs with a generator, which is all of C's nonzeros). Grid (n, ranges) x 32 threads.
 __global__ void __launch_bounds__(32) k_lo_cs(const unsigned long long *__restrict__ E, int64_t lde,
                                               const float *__restrict__ C, int64_t ldc,
-                                              const uint64_t *__restrict__ ZT, int64_t ldzt, int64_t s,
-                                              float *__restrict__ M, int64_t lds) {
+                                              const float *__restrict__ d, const uint64_t *__restrict__ ZT,
+                                              int64_t ldzt, int64_t s, float *__restrict__ M, int64_t lds) {
     const int lane = threadIdx.x;
     const int64_t q = blockIdx.x, r0 = blockIdx.y;
     const int64_t vwords = cdiv(s, 64);
@@ -210,6 +317,10 @@ __global__ void __launch_bounds__(32) k_lo_cs(const unsigned long long *__restri
         if (t >= kCsBatch - nb) add(__ldg(ZT + rb[t] * ldzt + word), __float_as_uint(__ldg(crow + rb[t])));
     if (wraw < vwords) {
         float *mrow = M + q * lds + wraw * 64;  // lds is a multiple of 64
+        const uint64_t zq = __ldg(ZT + q * ldzt + word);
+        const float dq = d[q];
+#pragma unroll
+        for (int k = 0; k < 64; ++k) acc[k] = ((zq >> k) & 1ull) ? -(dq + acc[k]) : dq + acc[k];
 #pragma unroll
         for (int k = 0; k < 64; k += 4) *reinterpret_cast<float4 *>(mrow + k) = make_float4(acc[k], acc[k + 1], acc[k + 2], acc[k + 3]);
     }
@@ -218,8 +329,7 @@ __global__ void __launch_bounds__(32) k_lo_cs(const unsigned long long *__restri
 // H[q][r] = sum_i s_q(i) V[q][i] s_r(i) for r in E_q. Warp (q, k) takes
 // every kHSplit-th set bit of E_q starting at the k-th (listed in shared
 // memory, kRMax at a time) and walks the sample ranges in order, so each
-// H[q][r] is accumulated by one warp alone (fixed order, FP32 per range,
-// FP64 across ranges).
+// H[q][r] is accumulated by one warp alone (fixed order).
 constexpr int kHSplit = 8;
 constexpr int kRMax = 1024;
 constexpr int kHPre = 4;
@@ -227,14 +337,14 @@ constexpr int kHPre = 4;
 __global__ void __launch_bounds__(32) k_lo_h(const unsigned long long *__restrict__ E, int64_t lde,
                                              const uint64_t *__restrict__ ZT, int64_t ldzt,
                                              const float *__restrict__ V, int64_t lds, int64_t s,
-                                             double *__restrict__ Hd, int64_t ldh) {
+                                             float *__restrict__ Hf, int64_t ldh) {
     __shared__ int rl[kRMax];
     const int lane = threadIdx.x;
     const int64_t q = blockIdx.x;
     const int split = blockIdx.y;
     const int64_t vwords = cdiv(s, 64);
     const int64_t nranges = cdiv(vwords, 32);
-    double *hrow = Hd + q * ldh;
+    float *hrow = Hf + q * ldh;
     const unsigned long long *erow = E + q * lde;
     int seen = 0;        // set bits of E_q visited so far
     int64_t w0 = 0;      // next E word to scan
@@ -307,7 +417,7 @@ __global__ void __launch_bounds__(32) k_lo_h(const unsigned long long *__restric
                 float dsum = ((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]));
 #pragma unroll
                 for (int off = 16; off >= 1; off >>= 1) dsum += __shfl_xor_sync(kFull, dsum, off);
-                if (lane == 0) hrow[r] = r0 == 0 ? (double)dsum : hrow[r] + (double)dsum;
+                if (lane == 0) hrow[r] = r0 == 0 ? dsum : hrow[r] + dsum;
                 }
             }
         }
@@ -315,38 +425,10 @@ __global__ void __launch_bounds__(32) k_lo_h(const unsigned long long *__restric
     }
 }
 
-// ------------------------------------- the contractions on the tensor cores
 // With the tensor cores both contractions are dense GEMMs with one +-1
 // operand from bits, M = C S (K = the n qubits r) and H = (s o V) S^T
 // (K = the s samples), like the phase contraction; the FP32 operand goes in
-// as a hi + lo BF16 split. k_lo_split writes that split: element (q, k) of
-// a rows x cols FP32 matrix, multiplied by s_q(k) = (-1)^(bit k of zt row q)
-// when zt is given, into rows x kpad BF16 matrices (zero for k >= cols).
-// One thread per 8 consecutive elements.
-__global__ void k_lo_split(const float *__restrict__ in, int64_t ld_in, int64_t rows, int64_t cols,
-                           const uint64_t *__restrict__ zt, int64_t ldzt, int64_t kpad, __nv_bfloat16 *__restrict__ hi,
-                           __nv_bfloat16 *__restrict__ lo) {
-    const int64_t per_row = kpad / 8, total = rows * per_row;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t q = e / per_row, k0 = (e - q * per_row) * 8;
-        const uint32_t sb = zt ? (uint32_t)(zt[q * ldzt + (k0 >> 6)] >> (k0 & 63)) & 0xFFu : 0u;
-        uint32_t ph[4], pl[4];
-#pragma unroll
-        for (int t = 0; t < 8; t += 2) {
-            float x0 = k0 + t < cols ? in[q * ld_in + k0 + t] : 0.f;
-            float x1 = k0 + t + 1 < cols ? in[q * ld_in + k0 + t + 1] : 0.f;
-            if ((sb >> t) & 1u) x0 = -x0;
-            if ((sb >> (t + 1)) & 1u) x1 = -x1;
-            const __nv_bfloat16 h0 = __float2bfloat16_rn(x0), h1 = __float2bfloat16_rn(x1);
-            const __nv_bfloat16 l0 = __float2bfloat16_rn(x0 - __bfloat162float(h0));
-            const __nv_bfloat16 l1 = __float2bfloat16_rn(x1 - __bfloat162float(h1));
-            ph[t / 2] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-            pl[t / 2] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
-        }
-        *reinterpret_cast<uint4 *>(hi + q * kpad + k0) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
-        *reinterpret_cast<uint4 *>(lo + q * kpad + k0) = make_uint4(pl[0], pl[1], pl[2], pl[3]);
-    }
-}
+// as a hi + lo BF16 split, written by k_lo_convert and k_lo_v.
 
 // Exclusive prefix sum of v over the CTA (every thread calls it); *total
 // receives the sum.
@@ -437,9 +519,8 @@ __device__ void lo_load_bits(LoShared &sh, int nq, int64_t n, const uint64_t *__
 // entries or the candidates run out. Returns the list length; every thread
 // calls it and gets the same value.
 __device__ int lo_fill_pairs(LoShared &sh, int nq, int64_t *c0, const unsigned long long *__restrict__ E,
-                             int64_t lde, const float *__restrict__ C, int64_t ldc, int64_t n,
+                             int64_t lde, const unsigned long long *__restrict__ Cfx, float inv, int64_t n,
                              [[maybe_unused]] uint32_t *__restrict__ status_dbg) {
-    (void)n;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t ncand = (int64_t)nq * nq;
     int np = 0;
@@ -468,7 +549,8 @@ __device__ int lo_fill_pairs(LoShared &sh, int nq, int64_t *c0, const unsigned l
         const int pos = off + __popc(bal & ((1u << lane) - 1u));
         if (ok && LO_OK(pos >= 0 && pos < kPairMax, 5)) {
             sh.pr[pos] = t | (u << 16);
-            sh.pc[pos] = C[(int64_t)sh.Q[t] * ldc + sh.Q[u]];
+            if (Cfx != nullptr)
+                sh.pc[pos] = __ll2float_rn((long long)Cfx[(int64_t)sh.Q[t] * n + sh.Q[u]]) * inv;
         }
         np += tot;
         *c0 += kBlk;
@@ -523,12 +605,14 @@ __device__ void lo_load_bits4(LoShared &sh, int nq, int64_t n, const uint64_t *_
     __syncthreads();
 }
 
+// The observables too heavy for the lists (or all of them, without lists):
+// work item (h, g) is observable heavy[h] (h itself without `heavy`).
 // MODE 0: (sum cos, sum (cos - mean)^2) per (observable, 256 samples) into
 // part, and Phi itself into phi (row stride ldphi >= lds, columns < lds) when
 // phi is not null (a gradient pass follows). MODE 1: W[a][i] = sin Phi
-// (alpha_a + beta_a cos Phi), zero for i >= s.
+// (alpha_a + beta_a cos Phi), zero for i >= s. MODE 2: the partials and W.
 // The pair term visits only the pairs of Q_a that carry a generator (C_qr is
-// zero on the others). CTA (a, g) takes sample blocks kPGroup g ..
+// zero on the others). Item (a, g) takes sample blocks kPGroup g ..
 // kPGroup g + kPGroup - 1. For |Q_a| <= kQ4 a thread owns four consecutive
 // samples of a 1024-sample pass (four blocks; block b is warps 2b, 2b + 1),
 // so every support qubit costs one 16-byte load of M and every pair one
@@ -537,39 +621,44 @@ __device__ void lo_load_bits4(LoShared &sh, int nq, int64_t n, const uint64_t *_
 template <int MODE>
 __global__ void __launch_bounds__(kBlk) k_lo_phase(const uint64_t *__restrict__ A, int64_t lda, int64_t n,
                                                    const uint64_t *__restrict__ ZT, int64_t ldzt,
-                                                   const float *__restrict__ M, int64_t lds,
-                                                   const float *__restrict__ C, int64_t ldc,
-                                                   const float *__restrict__ d, const unsigned long long *__restrict__ E,
-                                                   int64_t lde, int64_t s, int64_t nparts, double2 *__restrict__ part,
+                                                   const float *__restrict__ X, int64_t lds,
+                                                   const unsigned long long *__restrict__ Cfx,
+                                                   const unsigned *__restrict__ cmax, int64_t m,
+                                                   const unsigned long long *__restrict__ E, int64_t lde, int64_t l,
+                                                   const int *__restrict__ heavy, const unsigned *__restrict__ nheavy,
+                                                   int64_t s, int64_t nparts, double2 *__restrict__ part,
                                                    const double *__restrict__ alpha, const double *__restrict__ beta,
                                                    float *__restrict__ W, float *__restrict__ phi, int64_t ldphi,
                                                    uint32_t *__restrict__ status) {
     [[maybe_unused]] uint32_t *status_dbg = status;
     __shared__ LoShared sh;
-    __shared__ const float *mrow[kQ4];  // M + Q[t] lds (four-block form)
-    __shared__ float dq[kQ4];           // d[Q[t]] (four-block form)
-    const int64_t a = blockIdx.x;
+    __shared__ const float *mrow[kQ4];  // X + Q[t] lds (four-block form)
+    const int64_t ngroups = cdiv(nparts, (int64_t)kPGroup);
+    const int64_t nobs = heavy ? (int64_t)*nheavy : l;
+    const float inv = ldexpf(1.0f, -lo_fx_exp(*cmax, m));
+    for (int64_t it = blockIdx.x; it < nobs * ngroups; it += gridDim.x) {
+    __syncthreads();  // the previous item's readers of sh are done
+    const int64_t h = it % nobs, a = heavy ? heavy[h] : h;
     const int nq = support_of_row(A + a * lda, n, sh.Q, sh.scan, status);
     const int tid = threadIdx.x, w = tid >> 5, bit = tid & 31;
     const int64_t ncand = (int64_t)nq * nq;
     int64_t c0 = 0;
-    int np = lo_fill_pairs(sh, nq, &c0, E, lde, C, ldc, n, status);
+    int np = lo_fill_pairs(sh, nq, &c0, E, lde, Cfx, inv, n, status);
     const bool complete = c0 >= ncand;  // the whole list fits: reuse it for every block
-    const float al = MODE == 1 ? (float)alpha[a] : 0.f;
-    const float be = (MODE == 1 && beta) ? (float)beta[a] : 0.f;
-    const int64_t bstart = blockIdx.y * (int64_t)kPGroup;
+    const float al = MODE != 0 ? (float)alpha[a] : 0.f;
+    const float be = (MODE != 0 && beta) ? (float)beta[a] : 0.f;
+    const int64_t bstart = it / nobs * (int64_t)kPGroup;
     const int64_t b1 = bstart + kPGroup < nparts ? bstart + kPGroup : nparts;
     if (nq <= kQ4) {
         for (int t = tid; t < nq; t += kBlk) {
             const int q = sh.Q[t];
             const bool ok = LO_OK(q >= 0 && q < n, 7);
-            mrow[t] = M + (ok ? (int64_t)q * lds : 0);
-            dq[t] = ok ? d[q] : 0.f;
+            mrow[t] = X + (ok ? (int64_t)q * lds : 0);
         }
         const int word = tid >> 3;              // bits4 word of this thread's samples
         const int sh4 = 28 - 4 * (tid & 7);     // moves their four bits to bits 28 .. 31
         for (int64_t blk0 = bstart; blk0 < b1; blk0 += 4) {
-            lo_load_bits4(sh, nq, n, ZT, ldzt, blk0, status);  // also orders the mrow/dq stores
+            lo_load_bits4(sh, nq, n, ZT, ldzt, blk0, status);  // also orders the mrow stores
             const int64_t i0 = blk0 * kBlk + 4 * (int64_t)tid;
             const int64_t blk = blk0 + (tid >> 6);  // this thread's block
             const int64_t i0c = i0 < lds ? i0 : lds - 4;  // lds is a multiple of 64
@@ -577,17 +666,15 @@ __global__ void __launch_bounds__(kBlk) k_lo_phase(const uint64_t *__restrict__ 
             for (int t = 0; t < nq; ++t) {
                 if (!LO_OK(i0c >= 0 && i0c + 3 < lds, 8)) break;
                 const float4 mv = *reinterpret_cast<const float4 *>(mrow[t] + i0c);
-                const float dv = dq[t];
-                const uint32_t y = sh.bits4[t][word] << sh4;
-                p0 = p0 + flip_if(dv + mv.x, y << 3);
-                p1 = p1 + flip_if(dv + mv.y, y << 2);
-                p2 = p2 + flip_if(dv + mv.z, y << 1);
-                p3 = p3 + flip_if(dv + mv.w, y);
+                p0 += mv.x;
+                p1 += mv.y;
+                p2 += mv.z;
+                p3 += mv.w;
             }
             float q0 = 0.f, q1 = 0.f, q2 = 0.f, q3 = 0.f;
             if (!complete && blk0 != bstart) {
                 c0 = 0;  // the list is rebuilt round by round for every pass
-                np = lo_fill_pairs(sh, nq, &c0, E, lde, C, ldc, n, status);
+                np = lo_fill_pairs(sh, nq, &c0, E, lde, Cfx, inv, n, status);
             }
             while (true) {
                 for (int p = 0; p < np; ++p) {
@@ -602,13 +689,13 @@ __global__ void __launch_bounds__(kBlk) k_lo_phase(const uint64_t *__restrict__ 
                 }
                 if (complete || c0 >= ncand) break;
                 __syncthreads();
-                np = lo_fill_pairs(sh, nq, &c0, E, lde, C, ldc, n, status);
+                np = lo_fill_pairs(sh, nq, &c0, E, lde, Cfx, inv, n, status);
             }
             const float ph[4] = {p0 - 2.f * q0, p1 - 2.f * q1, p2 - 2.f * q2, p3 - 2.f * q3};
             bool valid[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) valid[k] = i0 + k < s && blk < b1;
-            if (MODE == 0) {
+            if (MODE != 1) {
                 float cv[4], S1 = 0.f;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
@@ -637,9 +724,10 @@ __global__ void __launch_bounds__(kBlk) k_lo_phase(const uint64_t *__restrict__ 
                 __syncthreads();
                 if ((tid & 63) == 0 && blk < b1)
                     part[a * nparts + blk] = make_double2((double)S, (double)(sh.redf[w] + sh.redf[w + 1]));
-                if (phi != nullptr && i0 < lds && blk < b1)
+                if (MODE == 0 && phi != nullptr && i0 < lds && blk < b1)
                     *reinterpret_cast<float4 *>(phi + a * ldphi + i0) = make_float4(ph[0], ph[1], ph[2], ph[3]);
-            } else if (i0 < lds && blk < b1) {
+            }
+            if (MODE != 0 && i0 < lds && blk < b1) {
                 float o[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
@@ -650,7 +738,7 @@ __global__ void __launch_bounds__(kBlk) k_lo_phase(const uint64_t *__restrict__ 
                 *reinterpret_cast<float4 *>(W + a * lds + i0) = make_float4(o[0], o[1], o[2], o[3]);
             }
         }
-        return;
+        continue;
     }
     for (int64_t blk = bstart; blk < b1; ++blk) {
         lo_load_bits(sh, nq, n, ZT, ldzt, blk, status);
@@ -661,13 +749,12 @@ __global__ void __launch_bounds__(kBlk) k_lo_phase(const uint64_t *__restrict__ 
         for (int t = 0; t < nq; ++t) {
             const int q = sh.Q[t];
             if (!LO_OK(q >= 0 && q < n && ic >= 0 && ic < lds, 7)) continue;
-            const float v = d[q] + M[(int64_t)q * lds + ic];
-            ph += ((sh.bits[t][w] >> bit) & 1u) ? -v : v;
+            ph += X[(int64_t)q * lds + ic];
         }
         float pairs = 0.f;
         if (!complete && blk != bstart) {
             c0 = 0;  // the list is rebuilt round by round for every block
-            np = lo_fill_pairs(sh, nq, &c0, E, lde, C, ldc, n, status);
+            np = lo_fill_pairs(sh, nq, &c0, E, lde, Cfx, inv, n, status);
         }
         while (true) {
             for (int p = 0; p < np; ++p) {
@@ -679,10 +766,10 @@ __global__ void __launch_bounds__(kBlk) k_lo_phase(const uint64_t *__restrict__ 
             }
             if (complete || c0 >= ncand) break;
             __syncthreads();
-            np = lo_fill_pairs(sh, nq, &c0, E, lde, C, ldc, n, status);
+            np = lo_fill_pairs(sh, nq, &c0, E, lde, Cfx, inv, n, status);
         }
         ph -= 2.f * pairs;
-        if (MODE == 0) {
+        if (MODE != 1) {
             const float cv = valid ? cosf(ph) : 0.f;
             const float S = block_sum_f(cv, sh.redf);
             const int64_t nb = s - blk * kBlk < kBlk ? s - blk * kBlk : kBlk;
@@ -690,24 +777,211 @@ __global__ void __launch_bounds__(kBlk) k_lo_phase(const uint64_t *__restrict__ 
             const float dv = cv - mean;
             const float M2 = block_sum_f(valid ? dv * dv : 0.f, sh.redf);
             if (tid == 0) part[a * nparts + blk] = make_double2((double)S, (double)M2);
-            if (phi != nullptr && i < lds) phi[a * ldphi + i] = ph;
-        } else {
+            if (MODE == 0 && phi != nullptr && i < lds) phi[a * ldphi + i] = ph;
+        }
+        if (MODE != 0) {
             float sn, cn;
             sincosf(ph, &sn, &cn);
             if (i < lds) W[a * lds + i] = valid ? sn * (al + be * cn) : 0.f;
         }
     }
+    }  // items
+}
+
+// ---------------------------------------------------- the listed observables
+// One warp per (observable, 1024 samples), 32 samples per lane, no barriers: the
+// observable's qubits and pairs come from its lists (k_lo_lists).
+//   Phi: X is added up row by row (eight coalesced 16-byte loads per lane and
+// qubit, no sign or addend left to apply); the pair term goes five pairs at a
+// time, their 32 sign combinations one per lane, indexed by the lane's transposed
+// sample bits (indices5), one shuffle and one add per sample.
+//   K: W's signed sums over all 16 sign patterns of every four samples of a lane
+// are tabulated (16 KB per warp); a pair then costs eight table loads per lane,
+// and the lanes' sums of 32 pairs are combined by one reduce-scatter.
+// The loads of X from L2 bound the phase where the observables are wide: n =
+// 5000, 4096 observables of 50 qubits, 16384 samples 1762 us in the one-CTA form
+// (18 instructions per qubit and four samples), the pair term 1278 us.
+// MODE 0: statistics partials, and Phi into phi when it is not null; 1: W and K
+// from Phi formed here; 2: partials, W and K; 3: W and K from Phi read from phi
+// (which may be W itself: each lane reads its samples before it writes them).
+// Heavy observables (cnt < 0) take part in MODE 3 only, for W.
+constexpr int kLoWarps = 4;
+constexpr int kLoTab = 8 * 16 * 32;  // floats of a warp's tables
+template <int MODE>
+__global__ void __launch_bounds__(32 * kLoWarps) k_lo_obs(
+    const int *__restrict__ cnt, const int *__restrict__ Lq, const uint2 *__restrict__ Lp, const uint32_t *__restrict__ ZP,
+    int64_t nb, const float *__restrict__ X, int64_t lds, int64_t n, int64_t l, int64_t s, int64_t nparts,
+    double2 *__restrict__ part, const double *__restrict__ alpha, const double *__restrict__ beta, float *W, float *phi,
+    int64_t ldphi, const double *__restrict__ scale, unsigned long long *__restrict__ Kfx, uint32_t *__restrict__ status) {
+    [[maybe_unused]] uint32_t *status_dbg = status;
+    extern __shared__ float lo_tab[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t a = (int64_t)blockIdx.x * kLoWarps + warp, blk = blockIdx.y;
+    if (a >= l) return;
+    const int c = cnt[a];
+    if (c < 0 && MODE != 3) return;
+    const int nq = c & 0xFFFF, np = c < 0 ? 0 : c >> 16;
+    const int64_t i0 = blk * kLane + 4 * lane;  // the lane's samples: i0 + 128 k .. + 3
+    const uint32_t *zp = ZP + blk * 32 + lane;
+    const uint2 *pairs = Lp + a * kLoP;
+    float acc[32];
+    if (MODE == 3) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const float4 v = i0 + 128 * k < lds ? *reinterpret_cast<const float4 *>(phi + a * ldphi + i0 + 128 * k)
+                                                : make_float4(0.f, 0.f, 0.f, 0.f);
+            acc[4 * k] = v.x;
+            acc[4 * k + 1] = v.y;
+            acc[4 * k + 2] = v.z;
+            acc[4 * k + 3] = v.w;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 32; ++k) acc[k] = 0.f;
+        const int *Q = Lq + a * kLoQ;
+#pragma unroll 2
+        for (int t = 0; t < nq; ++t) {
+            const int q = __ldg(Q + t);
+            if (!LO_OK(q >= 0 && q < n, 11)) continue;
+            const float *xr = X + (int64_t)q * lds + i0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                if (i0 + 128 * k >= lds) continue;
+                const float4 v = __ldg(reinterpret_cast<const float4 *>(xr + 128 * k));
+                acc[4 * k] += v.x;
+                acc[4 * k + 1] += v.y;
+                acc[4 * k + 2] += v.z;
+                acc[4 * k + 3] += v.w;
+            }
+        }
+        for (int p0 = 0; p0 < np; p0 += 5) {
+            uint32_t z[5], R[8];
+            float t = 0.f;
+#pragma unroll
+            for (int g = 0; g < 5; ++g) {
+                z[g] = 0u;
+                if (p0 + g < np) {
+                    const uint2 e = __ldg(pairs + p0 + g);
+                    const int64_t q = e.x & 0xFFFFu, r = e.x >> 16;
+                    if (!LO_OK(q < r && r < n, 12)) continue;
+                    z[g] = __ldg(zp + q * nb * 32) ^ __ldg(zp + r * nb * 32);
+                    const float cv = __uint_as_float(e.y);
+                    t += ((lane >> g) & 1) ? -cv : cv;
+                }
+            }
+            indices5(z, R);
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) acc[8 * k + q] += __shfl_sync(kFull, t, (int)(R[q] >> (8 * k)));
+        }
+        if (MODE == 0 && phi != nullptr) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (i0 + 128 * k < lds)
+                    *reinterpret_cast<float4 *>(phi + a * ldphi + i0 + 128 * k) =
+                        make_float4(acc[4 * k], acc[4 * k + 1], acc[4 * k + 2], acc[4 * k + 3]);
+        }
+    }
+    const int64_t left = s - i0;  // sample k of the lane is valid when 128 (k / 4) + k % 4 < left
+    const float al = MODE != 0 ? (float)alpha[a] : 0.f;
+    const float be = (MODE != 0 && beta) ? (float)beta[a] : 0.f;
+    if (MODE == 0 || MODE == 2) {
+        float cv[32], S[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) S[b] = 0.f;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+            const bool valid = 128 * (k / 4) + k % 4 < left;
+            if (MODE == 2) {
+                float sn, cn;
+                sincosf(acc[k], &sn, &cn);
+                cv[k] = valid ? cn : 0.f;
+                acc[k] = valid ? sn * (al + be * cn) : 0.f;  // W
+            } else {
+                cv[k] = valid ? cosf(acc[k]) : 0.f;
+            }
+            S[k / 8] += cv[k];
+        }
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {  // the 256-sample blocks of the range
+            const int64_t pb = blk * 4 + b;
+#pragma unroll
+            for (int off = 16; off >= 1; off >>= 1) S[b] += __shfl_xor_sync(kFull, S[b], off);
+            const int64_t nbv = s - pb * kBlk < kBlk ? s - pb * kBlk : kBlk;
+            const float mean = nbv > 0 ? S[b] / (float)nbv : 0.f;
+            float M2 = 0.f;
+#pragma unroll
+            for (int k = 8 * b; k < 8 * b + 8; ++k) {
+                const float dv = cv[k] - mean;
+                M2 += 128 * (k / 4) + k % 4 < left ? dv * dv : 0.f;
+            }
+#pragma unroll
+            for (int off = 16; off >= 1; off >>= 1) M2 += __shfl_xor_sync(kFull, M2, off);
+            if (lane == 0 && pb < nparts) part[a * nparts + pb] = make_double2((double)S[b], (double)M2);
+        }
+    }
+    if (MODE != 0) {
+        if (MODE != 2) {
+#pragma unroll
+            for (int k = 0; k < 32; ++k) {
+                float sn, cn;
+                sincosf(acc[k], &sn, &cn);
+                acc[k] = 128 * (k / 4) + k % 4 < left ? sn * (al + be * cn) : 0.f;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (i0 + 128 * k < lds)
+                *reinterpret_cast<float4 *>(W + a * lds + i0 + 128 * k) =
+                    make_float4(acc[4 * k], acc[4 * k + 1], acc[4 * k + 2], acc[4 * k + 3]);
+        if (np == 0) return;  // uniform in the warp
+        float *tab = lo_tab + warp * kLoTab + lane;
+#pragma unroll
+        for (int g = 0; g < 8; ++g) {
+            const float w0 = acc[4 * g], w1 = acc[4 * g + 1], w2 = acc[4 * g + 2], w3 = acc[4 * g + 3];
+            const float p01[4] = {w0 + w1, w1 - w0, w0 - w1, -w0 - w1};
+            const float p23[4] = {w2 + w3, w3 - w2, w2 - w3, -w2 - w3};
+#pragma unroll
+            for (int e = 0; e < 16; ++e) tab[(g * 16 + e) * 32] = p01[e & 3] + p23[e >> 2];
+        }
+        const float sc = (float)*scale;
+        for (int p0 = 0; p0 < np; p0 += 32) {
+            float v[32];
+#pragma unroll
+            for (int g = 0; g < 32; ++g) {
+                v[g] = 0.f;
+                if (p0 + g < np) {  // uniform
+                    const uint32_t e = __ldg(&pairs[p0 + g].x);
+                    const uint32_t z = __ldg(zp + (int64_t)(e & 0xFFFFu) * nb * 32) ^ __ldg(zp + (int64_t)(e >> 16) * nb * 32);
+                    float u[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        u[k] = tab[(2 * k * 16 + ((z >> (8 * k)) & 15u)) * 32] +
+                               tab[((2 * k + 1) * 16 + ((z >> (8 * k + 4)) & 15u)) * 32];
+                    v[g] = (u[0] + u[1]) + (u[2] + u[3]);
+                }
+            }
+            const float d = reduce_scatter(v, lane);
+            if (p0 + lane < np) {
+                const uint32_t e = pairs[p0 + lane].x;
+                atomicAdd(Kfx + (int64_t)(e & 0xFFFFu) * n + (e >> 16), (unsigned long long)to_fixed(d, sc));
+            }
+        }
+    }
 }
 
 // V[q][i] = sum over the observables a containing q of W[a][i] (in a order),
-// zero for i >= s; gsp[q * nblk + blk] = sum_i s_q(i) V[q][i] over the
+// zero for i >= s: s_q V as the hi + lo BF16 operand of H (row stride lds), or V
+// itself where H is summed without the tensor cores; gsp[q * nblk + blk] = sum_i s_q(i) V[q][i] over the
 // CTA's 256 samples (FP64). A thread owns four consecutive samples of each
 // 1024-sample pass (block b of the pass is warps 2b, 2b + 1), so every
 // observable costs one 16-byte load of W per thread and pass.
 __global__ void __launch_bounds__(kBlk) k_lo_v(const uint64_t *__restrict__ AT, int64_t ldlt,
                                                const uint64_t *__restrict__ ZT, int64_t ldzt,
                                                const float *__restrict__ W, int64_t lds, int64_t s, int64_t nblk,
-                                               float *__restrict__ V, double *__restrict__ gsp) {
+                                               float *__restrict__ V, __nv_bfloat16 *__restrict__ hi,
+                                               __nv_bfloat16 *__restrict__ lo, double *__restrict__ gsp) {
     __shared__ float red[kBlk / 32];
     __shared__ int obs[kObsMax];
     __shared__ int wsum[kBlk / 32];
@@ -777,12 +1051,23 @@ __global__ void __launch_bounds__(kBlk) k_lo_v(const uint64_t *__restrict__ AT, 
         const bool in = blk < b1 && i0 < lds;
         const float vv[4] = {in && i0 < s ? v[g].x : 0.f, in && i0 + 1 < s ? v[g].y : 0.f,
                              in && i0 + 2 < s ? v[g].z : 0.f, in && i0 + 3 < s ? v[g].w : 0.f};
-        if (in) *reinterpret_cast<float4 *>(V + q * lds + i0) = make_float4(vv[0], vv[1], vv[2], vv[3]);
+        if (in && V != nullptr) *reinterpret_cast<float4 *>(V + q * lds + i0) = make_float4(vv[0], vv[1], vv[2], vv[3]);
         // lds <= 64 ldzt, so the word of i0 is inside row q of ZT when i0 < lds.
         const uint32_t nib = in ? (uint32_t)(ZT[q * ldzt + (i0 >> 6)] >> (i0 & 63)) : 0u;
         float u = 0.f;
+        uint32_t ph[4], pl[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) u += ((nib >> k) & 1u) ? -vv[k] : vv[k];
+        for (int k = 0; k < 4; ++k) {
+            const float x = ((nib >> k) & 1u) ? -vv[k] : vv[k];
+            u += x;
+            const __nv_bfloat16 b = __float2bfloat16_rn(x);
+            ph[k] = __bfloat16_as_ushort(b);
+            pl[k] = __bfloat16_as_ushort(__float2bfloat16_rn(x - __bfloat162float(b)));
+        }
+        if (in && hi != nullptr) {
+            *reinterpret_cast<uint2 *>(hi + q * lds + i0) = make_uint2(ph[0] | (ph[1] << 16), ph[2] | (ph[3] << 16));
+            *reinterpret_cast<uint2 *>(lo + q * lds + i0) = make_uint2(pl[0] | (pl[1] << 16), pl[2] | (pl[3] << 16));
+        }
 #pragma unroll
         for (int off = 16; off >= 1; off >>= 1) u += __shfl_xor_sync(kFull, u, off);
         __syncthreads();
@@ -818,13 +1103,6 @@ __global__ void __launch_bounds__(256) k_lo_w(const float *phi, int64_t ldphi, f
     }
 }
 
-__device__ __forceinline__ long long to_fixed(float x, float sc) {
-    const float xs = sc * x;  // |xs| < 2^60, exact power-of-two scaling
-    const float hi = truncf(xs * 0x1.0p-31f);
-    const float lo = fmaf(-hi, 0x1.0p31f, xs);
-    return ((long long)__float2int_rz(hi) << 31) + (long long)__float2int_rn(lo);
-}
-
 // K[q][r] += sum over the samples of W[a][i] s_q(i) s_r(i) for the pairs
 // q < r of Q_a that carry a generator (the only K entries the gradient
 // reads). The pair list is taken kPairPass pairs at a time; warp w owns
@@ -833,12 +1111,12 @@ __device__ __forceinline__ long long to_fixed(float x, float sc) {
 // then one shuffle reduction and one fixed-point atomic per (pair, CTA).
 // For supports of at most kQ4 qubits the sample bits and W of four blocks
 // are staged per pair of barriers (one block at a time otherwise).
-// CTA (a, g) takes blocks kPGroup g ...
+// Work item (a, g) takes blocks kPGroup g ...; heavy observables as in k_lo_phase.
 constexpr int kPairPass = 128;
 __global__ void __launch_bounds__(kBlk) k_lo_pairs(const uint64_t *__restrict__ A, int64_t lda, int64_t n,
                                                    const uint64_t *__restrict__ ZT, int64_t ldzt,
-                                                   const float *__restrict__ C, int64_t ldc,
-                                                   const unsigned long long *__restrict__ E, int64_t lde,
+                                                   const unsigned long long *__restrict__ E, int64_t lde, int64_t l,
+                                                   const int *__restrict__ heavy, const unsigned *__restrict__ nheavy,
                                                    const float *__restrict__ W, int64_t lds, int64_t s,
                                                    int64_t nblk, const double *__restrict__ scale,
                                                    unsigned long long *__restrict__ Kfx,
@@ -847,17 +1125,21 @@ __global__ void __launch_bounds__(kBlk) k_lo_pairs(const uint64_t *__restrict__ 
     __shared__ LoShared sh;
     __shared__ __align__(16) float wb[4 * kBlk];
     constexpr int kPerWarp = kPairPass / (kBlk / 32);
-    const int64_t a = blockIdx.x;
+    const int64_t ngroups = cdiv(nblk, (int64_t)kPGroup);
+    const int64_t nobs = heavy ? (int64_t)*nheavy : l;
+    for (int64_t it = blockIdx.x; it < nobs * ngroups; it += gridDim.x) {
+    __syncthreads();  // the previous item's readers of sh are done
+    const int64_t h = it % nobs, a = heavy ? heavy[h] : h;
     const int nq = support_of_row(A + a * lda, n, sh.Q, sh.scan, status);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int sa = 31 - lane;  // moves this lane's sample bit to bit 31
     const float sc = (float)*scale;
     const int64_t ncand = (int64_t)nq * nq;
-    const int64_t b0 = blockIdx.y * (int64_t)kPGroup;
+    const int64_t b0 = it / nobs * (int64_t)kPGroup;
     const int64_t b1 = b0 + kPGroup < nblk ? b0 + kPGroup : nblk;
     int64_t c0 = 0;
     while (c0 < ncand) {
-        const int np = lo_fill_pairs(sh, nq, &c0, E, lde, C, ldc, n, status);
+        const int np = lo_fill_pairs(sh, nq, &c0, E, lde, nullptr, 0.f, n, status);
         for (int p0 = 0; p0 < np; p0 += kPairPass) {
             float acc[kPerWarp];
 #pragma unroll
@@ -940,11 +1222,12 @@ __global__ void __launch_bounds__(kBlk) k_lo_pairs(const uint64_t *__restrict__ 
         }
         __syncthreads();  // the list is read before the next round rebuilds it
     }
+    }  // items
 }
 
 // grad_j from the parts above (see the header).
 __global__ void k_lo_grad_out(const int4 *__restrict__ sup, int64_t m, int64_t n, const double *__restrict__ gsp,
-                              int64_t nblk, const double *__restrict__ H, int64_t ldh,
+                              int64_t nblk, const float *__restrict__ H, int64_t ldh, int hparts,
                               const unsigned long long *__restrict__ Kfx, const double *__restrict__ scale,
                               double *__restrict__ grad) {
     const double inv = 1.0 / *scale;
@@ -957,7 +1240,9 @@ __global__ void k_lo_grad_out(const int4 *__restrict__ sup, int64_t m, int64_t n
             g = 2.0 * t;
         } else if (sp.w == 2) {
             const int64_t q = sp.x, r = sp.y;
-            const double h = H[q * ldh + r] + H[r * ldh + q];
+            double h = 0.0;
+            for (int p = 0; p < hparts; ++p)
+                h += (double)H[((int64_t)p * n + q) * ldh + r] + (double)H[((int64_t)p * n + r) * ldh + q];
             const double k = (double)(long long)Kfx[q * n + r] * inv;
             g = 2.0 * h - 4.0 * k;
         }
@@ -974,7 +1259,8 @@ int grid_1d(int64_t work) {
 
 }  // namespace
 
-cudaError_t launch_support_list(const uint64_t *G, int64_t m, int64_t ldg, int64_t n, int4 *sup, cudaStream_t st);
+cudaError_t launch_support_list(const uint64_t *G, int64_t m, int64_t ldg, int64_t n, int4 *sup, cudaStream_t st,
+                                const float *theta, unsigned *cmax);
 cudaError_t launch_bit_transpose_batched(const uint64_t *in, int64_t batch, int64_t in_rows, int64_t in_cols,
                                          int64_t ld_in, uint64_t *out, int64_t ld_out, cudaStream_t st);
 cudaError_t launch_fixed_scale(const double *alpha, const double *beta, int64_t l, int64_t s, double *scale,
@@ -1000,133 +1286,159 @@ int64_t lo_split_elems(int64_t n, int64_t lds) {
     return 2 * n * (kc > lds ? kc : lds);
 }
 
-namespace {
-cudaError_t launch_split(const float *in, int64_t ld_in, int64_t rows, int64_t cols, const uint64_t *zt,
-                         int64_t ldzt, int64_t kpad, __nv_bfloat16 *hi, __nv_bfloat16 *lo, cudaStream_t st) {
-    LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-    k_lo_split<<<grid_1d(rows * (kpad / 8)), 256, 0, st>>>(in, ld_in, rows, cols, zt, ldzt, kpad, hi, lo);
-    return cudaGetLastError();
-}
-}  // namespace
-
-// C, d and M = C S. C: n x ldc fp32 (+ d: ldc fp32 after it), M: n x lds,
-// ZT: n x ldzt words (the samples transposed), sup: m int4.
 int64_t lo_lde(int64_t n) { return cdiv(n, 64); }
 
-// C, d, E and M = C S. C: n x ldc fp32 (+ d: ldc fp32 after it), E: n x
-// lo_lde(n) words right after d, M: n x lds, ZT: n x ldzt words (the samples
-// transposed), sup: m int4.
-cudaError_t launch_lo_prepare(int64_t n, const uint64_t *G, int64_t m, int64_t ldg, const uint64_t *Z, int64_t s,
-                              int64_t ldz, const float *c, int4 *sup, uint64_t *ZT, int64_t ldzt, float *C,
-                              int64_t ldc, float *M, int64_t lds, __nv_bfloat16 *split, unsigned long long *fx,
-                              uint32_t *status, cudaStream_t st) {
-    cudaError_t e = launch_support_list(G, m, ldg, n, sup, st);
-    if (e != cudaSuccess) return e;
-    if ((e = launch_bit_transpose_batched(Z, 1, s, n, ldz, ZT, ldzt, st)) != cudaSuccess) return e;
-    float *d = C + n * ldc;
-    unsigned long long *E = reinterpret_cast<unsigned long long *>(d + ldc);
-    const int64_t lde = lo_lde(n);
-    // fx: Cfx (n x n), dfx (n), then the largest |c_j| (float bits).
-    unsigned long long *Cfx = fx, *dfx = fx + n * n;
-    unsigned *cmax = reinterpret_cast<unsigned *>(dfx + n);
-    if ((e = cudaMemsetAsync(E, 0, (size_t)n * lde * 8, st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(fx, 0, (size_t)(n * n + n) * 8 + 16, st)) != cudaSuccess) return e;
-    {
-        LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-        k_lo_cmax<<<grid_1d(m), 256, 0, st>>>(sup, c, m, cmax);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        k_lo_build<<<grid_1d(m), 256, 0, st>>>(sup, c, m, n, Cfx, dfx, cmax, E, lde, status);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        k_lo_fx_float<<<grid_1d(n * ldc + n), 256, 0, st>>>(Cfx, dfx, cmax, m, n, C, ldc, d);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    // M = C S: rows q, columns the samples (Z's rows), K the qubits r.
-    const int64_t kc = round_up(n, 64);
-    bool done = false;
-    if (lo_tensor() && split != nullptr && ldz >= 4 && ldz % 2 == 0 && (reinterpret_cast<uintptr_t>(Z) & 15) == 0) {
-        __nv_bfloat16 *hi = split, *lo = split + n * kc;
-        if ((e = launch_split(C, ldc, n, n, nullptr, 0, kc, hi, lo, st)) != cudaSuccess) return e;
-        e = launch_tc_dense(hi, lo, n, kc, n, Z, s, ldz, M, lds, false, status, st);
-        if (e != cudaSuccess && e != cudaErrorNotSupported) return e;
-        done = e == cudaSuccess;
-    }
-    if (!done) {
-        LaunchScope ls(IQP_KERNEL_LOWORDER_GEMM, st);
-        k_lo_cs<<<dim3((unsigned)n, (unsigned)cdiv(s, 2048)), 32, 0, st>>>(E, lde, C, ldc, ZT, ldzt, s, M, lds);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+namespace {
+
+unsigned *lo_cmax(const LoArgs &a) { return reinterpret_cast<unsigned *>(a.fx + a.n * a.n + a.n); }
+unsigned *lo_nheavy(const LoArgs &a) { return lo_cmax(a) + 1; }
+double *lo_scale(const LoArgs &a) { return reinterpret_cast<double *>(a.fx + a.n * a.n); }
+const int *lo_heavy(const LoArgs &a) { return a.ZP != nullptr ? a.cnt + a.l : nullptr; }
+
+// Blocks of the heavy observables' kernels: two per SM take what there is
+// (usually nothing); without lists one per work item.
+unsigned lo_heavy_blocks(const LoArgs &a, int64_t nblk) {
+    int64_t b = a.l * cdiv(nblk, (int64_t)kPGroup);
+    if (a.ZP != nullptr && b > 2 * num_sms()) b = 2 * num_sms();
+    if (b > 0x7FFFFFFF) b = 0x7FFFFFFF;
+    return (unsigned)(b < 1 ? 1 : b);
 }
 
-cudaError_t launch_lo_stats(const uint64_t *A, int64_t lda, int64_t n, int64_t l, const uint64_t *ZT, int64_t ldzt,
-                            const float *M, int64_t lds, const float *C, int64_t ldc, int64_t s, double2 *part,
-                            int64_t nparts, float *phi, int64_t ldphi, uint32_t *status, cudaStream_t st) {
+template <int MODE>
+cudaError_t launch_obs(const LoArgs &a, double2 *part, const double *alpha, const double *beta, float *W, float *phi,
+                       int64_t ldphi, cudaStream_t st) {
+    constexpr int smem = MODE == 0 ? 0 : kLoWarps * kLoTab * 4;
+    static bool attr_set = false;
+    if (!attr_set) {
+        const cudaError_t e = cudaFuncSetAttribute(k_lo_obs<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        attr_set = true;
+    }
+    const int64_t nb = cdiv(a.s, (int64_t)kLane);
     LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-    const float *d = C + n * ldc;
-    const unsigned long long *E = reinterpret_cast<const unsigned long long *>(d + ldc);
-    k_lo_phase<0><<<dim3((unsigned)l, (unsigned)cdiv(nparts, kPGroup)), kBlk, 0, st>>>(A, lda, n, ZT, ldzt, M, lds, C, ldc, d, E,
-                                                                       lo_lde(n), s, nparts, part, nullptr, nullptr,
-                                                                       nullptr, phi, ldphi, status);
+    k_lo_obs<MODE><<<dim3((unsigned)cdiv(a.l, (int64_t)kLoWarps), (unsigned)nb), 32 * kLoWarps, smem, st>>>(
+        a.cnt, a.Lq, a.Lp, a.ZP, nb, a.X, a.lds, a.n, a.l, a.s, cdiv(a.s, (int64_t)kBlk), part, alpha, beta, W, phi, ldphi,
+        lo_scale(a), a.fx, a.status);
     return cudaGetLastError();
 }
 
-// AT: n x ldlt words (A transposed), W: l x lds, V: n x lds, H: n x ldc,
-// gsp: n x nblk doubles, Kfx: n x n int64 followed by the scale (double).
-cudaError_t launch_lo_grad(const uint64_t *A, int64_t lda, int64_t n, int64_t l, const uint64_t *ZT, int64_t ldzt,
-                           const float *M, int64_t lds, const float *C, int64_t ldc, int64_t s, int64_t m,
-                           const int4 *sup, const double *alpha, const double *beta, uint64_t *AT, int64_t ldlt,
-                           float *W, float *V, double *H, double *gsp, unsigned long long *Kfx, double *grad,
-                           __nv_bfloat16 *split, const float *phi, int64_t ldphi, bool scale_set, uint32_t *status,
-                           cudaStream_t st) {
-    const int64_t nblk = cdiv(s, kBlk);
-    double *scale = reinterpret_cast<double *>(Kfx + n * n);
-    const float *d = C + n * ldc;
-    const unsigned long long *E = reinterpret_cast<const unsigned long long *>(d + ldc);
-    const int64_t lde = lo_lde(n);
-    cudaError_t e = launch_bit_transpose_batched(A, 1, l, n, lda, AT, ldlt, st);
-    if (e != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(Kfx, 0, (size_t)n * n * sizeof(unsigned long long), st)) != cudaSuccess) return e;
-    if (!scale_set && (e = launch_fixed_scale(alpha, beta, l, s, scale, st)) != cudaSuccess) return e;
-    if (phi != nullptr) {  // Phi kept by the statistics pass (possibly in W itself)
-        LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-        k_lo_w<<<grid_1d(l * (lds / 4)), 256, 0, st>>>(phi, ldphi, W, lds, l, s, alpha, beta);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    } else {
-        LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-        k_lo_phase<1><<<dim3((unsigned)l, (unsigned)cdiv(nblk, kPGroup)), kBlk, 0, st>>>(A, lda, n, ZT, ldzt, M, lds, C, ldc, d,
-                                                                         E, lde, s, nblk, nullptr, alpha, beta, W, nullptr, 0,
-                                                                         status);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
+template <int MODE>
+cudaError_t launch_phase(const LoArgs &a, double2 *part, const double *alpha, const double *beta, float *W, float *phi,
+                         int64_t ldphi, cudaStream_t st) {
+    const int64_t nblk = cdiv(a.s, (int64_t)kBlk);
+    LaunchScope ls(IQP_KERNEL_LOWORDER, st);
+    k_lo_phase<MODE><<<lo_heavy_blocks(a, nblk), kBlk, 0, st>>>(
+        a.A, a.lda, a.n, a.ZT, a.ldzt, a.X, a.lds, a.fx, lo_cmax(a), a.m, a.E, lo_lde(a.n), a.l, lo_heavy(a), lo_nheavy(a),
+        a.s, nblk, part, alpha, beta, W, phi, ldphi, a.status);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+// Supports, C, d, E, the samples transposed, X, and the observables' lists.
+cudaError_t launch_lo_prepare(const LoArgs &a, cudaStream_t st) {
+    const int64_t n = a.n, m = a.m, lde = lo_lde(n), kc = round_up(n, 64);
+    const bool tc = lo_tensor() && a.split != nullptr && a.ldz >= 4 && a.ldz % 2 == 0 &&
+                    (reinterpret_cast<uintptr_t>(a.Z) & 15) == 0;
+    cudaError_t e;
+    // fx: Cfx (n x n), dfx (n), then the largest |c_j| (float bits) and the count of heavy observables.
+    if ((e = cudaMemsetAsync(a.E, 0, (size_t)n * lde * 8, st)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(a.fx, 0, (size_t)(n * n + n) * 8 + 16, st)) != cudaSuccess) return e;
+    if ((e = launch_support_list(a.G, m, a.ldg, n, a.sup, st, a.theta, lo_cmax(a))) != cudaSuccess) return e;
+    if ((e = launch_bit_transpose_batched(a.Z, 1, a.s, n, a.ldz, a.ZT, a.ldzt, st)) != cudaSuccess) return e;
+    __nv_bfloat16 *hi = a.split, *lo = a.split + n * kc;
     {
         LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-        k_lo_v<<<dim3((unsigned)n, (unsigned)cdiv(nblk, kGroup)), kBlk, 0, st>>>(AT, ldlt, ZT, ldzt, W, lds, s, nblk,
-                                                                                  V, gsp);
+        k_lo_build<<<grid_1d(m), 256, 0, st>>>(a.sup, a.theta, m, n, a.fx, a.fx + n * n, lo_cmax(a), a.E, lde, tc ? 0 : 1,
+                                              a.status);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        const int nb = (int)(kc / 64);
+        k_lo_convert<<<(unsigned)((int64_t)nb * (nb + 1) / 2), 256, 0, st>>>(a.fx, a.fx + n * n, lo_cmax(a), m, n, nb, hi,
+                                                                             lo, kc, tc ? nullptr : a.C, a.ldc, a.d);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    if (a.ZP != nullptr) {
+        LaunchScope ls(IQP_KERNEL_LOWORDER, st);
+        const int64_t nb = cdiv(a.s, (int64_t)kLane);
+        k_lo_zpack<<<grid_1d(32 * n * nb), 256, 0, st>>>(reinterpret_cast<const uint32_t *>(a.ZT), 2 * a.ldzt, n, nb, a.ZP);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        k_lo_lists<<<(unsigned)cdiv(a.l, (int64_t)8), 256, 0, st>>>(a.A, a.lda, a.l, n, a.E, lde, a.fx, lo_cmax(a), m, a.Lq,
+                                                                    a.Lp, a.cnt, a.cnt + a.l, lo_nheavy(a), a.status);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    // X = s o (d + C S): rows q, columns the samples (Z's rows), K the qubits r.
+    if (tc) {
+        e = launch_tc_dense(hi, lo, n, kc, n, a.Z, a.s, a.ldz, a.X, a.lds, 1, a.d, a.ZT, a.ldzt, a.status, st);
+        if (e != cudaErrorNotSupported) return e;
+    }
+    LaunchScope ls(IQP_KERNEL_LOWORDER_GEMM, st);
+    k_lo_cs<<<dim3((unsigned)n, (unsigned)cdiv(a.s, 2048)), 32, 0, st>>>(a.E, lde, a.C, a.ldc, a.d, a.ZT, a.ldzt, a.s, a.X,
+                                                                         a.lds);
+    return cudaGetLastError();
+}
+
+// Statistics partials and, if phi is not null, Phi.
+cudaError_t launch_lo_stats(const LoArgs &a, double2 *part, float *phi, int64_t ldphi, cudaStream_t st) {
+    const cudaError_t e = launch_phase<0>(a, part, nullptr, nullptr, nullptr, phi, ldphi, st);
+    if (e != cudaSuccess || a.ZP == nullptr) return e;
+    return launch_obs<0>(a, part, nullptr, nullptr, nullptr, phi, ldphi, st);
+}
+
+// The gradient. part: also the statistics partials (one pass over Phi); phi:
+// read from there (it may be W) instead of formed; scale_set: the fixed-point
+// scale is in place. AT: n x ldlt words (A transposed), W: l x lds, V: n x lds
+// (only without the tensor cores), gsp: n x nblk doubles.
+cudaError_t launch_lo_grad(const LoArgs &a, double2 *part, const double *alpha, const double *beta, uint64_t *AT,
+                           int64_t ldlt, float *W, float *V, double *gsp, double *grad, float *phi, int64_t ldphi,
+                           bool scale_set, cudaStream_t st) {
+    const int64_t n = a.n, s = a.s, nblk = cdiv(s, (int64_t)kBlk), lde = lo_lde(n);
+    const bool listed = a.ZP != nullptr, tc = lo_tensor() && a.split != nullptr;
+    cudaError_t e = launch_bit_transpose_batched(a.A, 1, a.l, n, a.lda, AT, ldlt, st);
+    if (e != cudaSuccess) return e;
+    // The heavy observables' phase reads C's sums, which K then takes the place of.
+    if (phi == nullptr) {
+        e = part != nullptr ? launch_phase<2>(a, part, alpha, beta, W, nullptr, 0, st)
+                            : launch_phase<1>(a, nullptr, alpha, beta, W, nullptr, 0, st);
+        if (e != cudaSuccess) return e;
+    }
+    if (!scale_set && (e = launch_fixed_scale(alpha, beta, a.l, s, lo_scale(a), st)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(a.fx, 0, (size_t)n * n * sizeof(unsigned long long), st)) != cudaSuccess) return e;
+    if (listed) {
+        e = phi != nullptr    ? launch_obs<3>(a, nullptr, alpha, beta, W, phi, ldphi, st)
+            : part != nullptr ? launch_obs<2>(a, part, alpha, beta, W, nullptr, 0, st)
+                              : launch_obs<1>(a, nullptr, alpha, beta, W, nullptr, 0, st);
+        if (e != cudaSuccess) return e;
+    } else if (phi != nullptr) {
+        LaunchScope ls(IQP_KERNEL_LOWORDER, st);
+        k_lo_w<<<grid_1d(a.l * (a.lds / 4)), 256, 0, st>>>(phi, ldphi, W, a.lds, a.l, s, alpha, beta);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    __nv_bfloat16 *hi = a.split, *lo = a.split + n * a.lds;
+    {
+        LaunchScope ls(IQP_KERNEL_LOWORDER, st);
+        k_lo_v<<<dim3((unsigned)n, (unsigned)cdiv(nblk, (int64_t)kGroup)), kBlk, 0, st>>>(
+            AT, ldlt, a.ZT, a.ldzt, W, a.lds, s, nblk, tc ? nullptr : V, tc ? hi : nullptr, lo, gsp);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     // H = (s o V) S^T: rows q, columns r (ZT's rows), K the samples.
-    bool h_done = false;
-    if (lo_tensor() && split != nullptr) {
-        __nv_bfloat16 *hi = split, *lo = split + n * lds;
-        if ((e = launch_split(V, lds, n, s, ZT, ldzt, lds, hi, lo, st)) != cudaSuccess) return e;
-        e = launch_tc_dense(hi, lo, n, lds, s, ZT, n, ldzt, H, ldc, true, status, st);
-        if (e != cudaSuccess && e != cudaErrorNotSupported) return e;
-        h_done = e == cudaSuccess;
-    }
-    if (!h_done) {
+    int hparts = 1;
+    if (tc) {
+        hparts = a.hparts;
+        e = launch_tc_dense(hi, lo, n, a.lds, s, a.ZT, n, a.ldzt, a.H, a.ldc, hparts, nullptr, nullptr, 0, a.status, st);
+    } else {
         LaunchScope ls(IQP_KERNEL_LOWORDER_GEMM, st);
-        k_lo_h<<<dim3((unsigned)n, (unsigned)kHSplit), 32, 0, st>>>(E, lde, ZT, ldzt, V, lds, s, H, ldc);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        k_lo_h<<<dim3((unsigned)n, (unsigned)kHSplit), 32, 0, st>>>(a.E, lde, a.ZT, a.ldzt, V, a.lds, s, a.H, a.ldc);
+        e = cudaGetLastError();
     }
+    if (e != cudaSuccess) return e;
     {
         LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-        k_lo_pairs<<<dim3((unsigned)l, (unsigned)cdiv(nblk, kPGroup)), kBlk, 0, st>>>(A, lda, n, ZT, ldzt, C, ldc, E,
-                                                                                     lde, W, lds, s, nblk, scale, Kfx,
-                                                                                     status);
+        k_lo_pairs<<<lo_heavy_blocks(a, nblk), kBlk, 0, st>>>(a.A, a.lda, n, a.ZT, a.ldzt, a.E, lde, a.l, lo_heavy(a),
+                                                              lo_nheavy(a), W, a.lds, s, nblk, lo_scale(a), a.fx, a.status);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-    k_lo_grad_out<<<grid_1d(m), 256, 0, st>>>(sup, m, n, gsp, nblk, H, ldc, Kfx, scale, grad);
+    k_lo_grad_out<<<grid_1d(a.m), 256, 0, st>>>(a.sup, a.m, n, gsp, nblk, a.H, a.ldc, hparts, a.fx, lo_scale(a), grad);
     return cudaGetLastError();
 }
 

@@ -10,6 +10,9 @@
 
 namespace iqp {
 
+cudaError_t launch_support_list(const uint64_t *G, int64_t m, int64_t ldg, int64_t n, int4 *sup, cudaStream_t st,
+                                const float *theta = nullptr, unsigned *cmax = nullptr);
+
 uint32_t check_word_parity() { return take_check_word(); }
 
 namespace {
@@ -659,42 +662,79 @@ cudaError_t bit_transpose(const uint64_t *in, int64_t in_rows, int64_t in_cols, 
 }
 
 // Support list of every generator: (q0, q1, q2, |supp g_j|), the first three
-// qubits of its support in increasing order. One warp per generator.
-__global__ void __launch_bounds__(256) k_support_list(const uint64_t *__restrict__ G, int64_t m, int64_t ldg,
-                                                       int64_t n, int4 *__restrict__ sup) {
-    const int lane = threadIdx.x & 31;
-    const int64_t j = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (j >= m) return;
-    const int64_t nw = (n + 63) >> 6;
-    int cnt = 0, q0 = 0, q1 = 0, q2 = 0;
-    for (int64_t wb = 0; wb < nw; wb += 32) {
-        const uint64_t word = (wb + lane < nw) ? G[j * ldg + wb + lane] : 0ull;
-        uint32_t nz = __ballot_sync(0xFFFFFFFFu, word != 0ull);
-        while (nz) {
-            const int src = __ffs(nz) - 1;
-            nz &= nz - 1u;
-            uint64_t wv = __shfl_sync(0xFFFFFFFFu, word, src);
-            while (wv) {
-                const int b = __ffsll((long long)wv) - 1;
-                wv &= wv - 1ull;
-                const int64_t q = 64 * (wb + src) + b;
-                if (q >= n) break;
-                if (cnt == 0) q0 = (int)q;
-                else if (cnt == 1) q1 = (int)q;
-                else if (cnt == 2) q2 = (int)q;
-                ++cnt;
+// qubits of its support in increasing order. A block takes R gates and reads
+// their rows as one run of 16-byte units, eight loads per thread in flight; the
+// few set bits go to the row's slots in shared memory, in any order, and one
+// thread per row sorts them (a row of more than three set bits is scanned
+// again). The rows are read once, which bounds it: 500500 rows of 128 bytes in
+// 38.7 us by one thread per row (each load behind the previous word's scan),
+// 254 us for 10^6 rows of 640 bytes by one warp per row.
+// With theta, the largest |2 theta_j| of the gates on one or two qubits goes to
+// *cmax (its float bits; zero before the launch).
+constexpr int kSuRows = 256, kSuLoads = 8;
+__global__ void __launch_bounds__(256) k_support_rows(const uint64_t *__restrict__ G, int64_t m, int64_t ldg, int64_t n,
+                                                      int nu, int R, int4 *__restrict__ sup,
+                                                      const float *__restrict__ theta, unsigned *__restrict__ cmax) {
+    __shared__ int cnt[kSuRows], qs[kSuRows][3];
+    const int64_t j0 = (int64_t)blockIdx.x * R;
+    const int rows = (int)(m - j0 < R ? m - j0 : R);
+    for (int r = threadIdx.x; r < rows; r += 256) cnt[r] = 0;
+    __syncthreads();
+    const int total = rows * nu;  // R nu <= 2048, or one row of any length
+    for (int b = 0; b < total; b += 256 * kSuLoads) {
+        ulonglong2 v[kSuLoads];
+#pragma unroll
+        for (int k = 0; k < kSuLoads; ++k) {
+            const int i = b + (int)threadIdx.x + 256 * k;
+            const int r = i / nu, u = i - r * nu;
+            v[k] = make_ulonglong2(0ull, 0ull);
+            if (i < total && IQP_IN((j0 + r) * ldg + 2 * u + 1, m * ldg, 16))
+                v[k] = *reinterpret_cast<const ulonglong2 *>(G + (j0 + r) * ldg + 2 * u);
+        }
+#pragma unroll
+        for (int k = 0; k < kSuLoads; ++k) {
+            if ((v[k].x | v[k].y) == 0ull) continue;
+            const int i = b + (int)threadIdx.x + 256 * k;
+            const int r = i / nu, u = i - r * nu;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                uint64_t w = h ? v[k].y : v[k].x;
+                while (w) {
+                    const int64_t q = 128 * (int64_t)u + 64 * h + __ffsll((long long)w) - 1;
+                    w &= w - 1ull;
+                    if (q >= n) break;  // never a qubit >= n
+                    const int at = atomicAdd(&cnt[r], 1);
+                    if (at < 3) qs[r][at] = (int)q;
+                }
             }
         }
     }
-    if (lane == 0 && IQP_IN(j, m, 12)) sup[j] = make_int4(q0, q1, q2, cnt);
-}
-
-// The same list with one thread per generator, for rows of at most 16 words
-// (n <= 1024): a warp per generator would leave most lanes idle there.
-__global__ void __launch_bounds__(256) k_support_list_short(const uint64_t *__restrict__ G, int64_t m, int64_t ldg,
-                                                             int64_t n, int4 *__restrict__ sup) {
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x)
-        if (IQP_IN(j, m, 13)) sup[j] = support_entry(G + j * ldg, n);
+    __syncthreads();
+    unsigned mx = 0u;
+    for (int r = threadIdx.x; r < rows; r += 256) {
+        const int c = cnt[r];
+        int4 e;
+        if (c <= 3) {
+            int q0 = c > 0 ? qs[r][0] : 0, q1 = c > 1 ? qs[r][1] : 0, q2 = c > 2 ? qs[r][2] : 0;
+            if (c >= 2 && q0 > q1) { const int x = q0; q0 = q1; q1 = x; }
+            if (c == 3) {
+                if (q1 > q2) { const int x = q1; q1 = q2; q2 = x; }
+                if (q0 > q1) { const int x = q0; q0 = q1; q1 = x; }
+            }
+            e = make_int4(q0, q1, q2, c);
+        } else {
+            e = support_entry(G + (j0 + r) * ldg, n);
+        }
+        if (IQP_IN(j0 + r, m, 12)) sup[j0 + r] = e;
+        if (theta != nullptr && (c == 1 || c == 2)) {
+            const unsigned b = __float_as_uint(fabsf(2.0f * theta[j0 + r]));  // non-negative floats order like their bits
+            mx = b > mx ? b : mx;
+        }
+    }
+    if (theta != nullptr) {
+        mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+        if ((threadIdx.x & 31) == 0 && mx != 0u) atomicMax(cmax, mx);
+    }
 }
 
 }  // namespace
@@ -720,15 +760,14 @@ cudaError_t launch_bit_transpose_batched(const uint64_t *in, int64_t batch, int6
     return cudaSuccess;
 }
 
-cudaError_t launch_support_list(const uint64_t *G, int64_t m, int64_t ldg, int64_t n, int4 *sup, cudaStream_t st) {
+cudaError_t launch_support_list(const uint64_t *G, int64_t m, int64_t ldg, int64_t n, int4 *sup, cudaStream_t st,
+                                const float *theta, unsigned *cmax) {
+    const int64_t nu = cdiv(n, 128);  // 16-byte units per row (ldg is even)
+    int64_t R = 256 * kSuLoads / nu;
+    R = R < 1 ? 1 : (R > kSuRows ? kSuRows : R);
+    if (cdiv(m, R) > 0x7FFFFFFFll) return cudaErrorInvalidValue;
     LaunchScope ls(IQP_KERNEL_PARITY, st);
-    if (cdiv(n, 64) <= 16) {
-        int64_t blocks = cdiv(m, 256);
-        if (blocks > 16384) blocks = 16384;
-        k_support_list_short<<<(unsigned)(blocks < 1 ? 1 : blocks), 256, 0, st>>>(G, m, ldg, n, sup);
-    } else {
-        k_support_list<<<(unsigned)cdiv(m, 8), 256, 0, st>>>(G, m, ldg, n, sup);
-    }
+    k_support_rows<<<(unsigned)cdiv(m, R), 256, 0, st>>>(G, m, ldg, n, (int)nu, (int)R, sup, theta, cmax);
     return cudaGetLastError();
 }
 

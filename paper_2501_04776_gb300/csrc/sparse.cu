@@ -236,22 +236,6 @@ __device__ __forceinline__ int list_gates(const uint64_t *__restrict__ row, int6
 }
 static_assert(kThreads * kScan <= 2048 && kThreads * kScan * 64 <= (1 << 21), "packing of `dense`");
 
-// Five words (bit i of word g = sample i's sign under gate g) to a 5-bit index
-// per sample: byte b of R[q] holds, in its low five bits, the index of sample
-// 8 b + q (the bits above them are zero).
-__device__ __forceinline__ void indices5(const uint32_t (&w)[5], uint32_t (&R)[8]) {
-    constexpr uint32_t m1 = 0x55555555u, m2 = 0x33333333u, m4 = 0x0F0F0F0Fu, mh = 0x10101010u;
-    const uint32_t x0 = (w[0] & m1) | ((w[1] << 1) & ~m1), x1 = ((w[0] >> 1) & m1) | (w[1] & ~m1);
-    const uint32_t y0 = (w[2] & m1) | ((w[3] << 1) & ~m1), y1 = ((w[2] >> 1) & m1) | (w[3] & ~m1);
-    const uint32_t u[4] = {(x0 & m2) | ((y0 << 2) & ~m2), (x1 & m2) | ((y1 << 2) & ~m2),
-                           ((x0 >> 2) & m2) | (y0 & ~m2), ((x1 >> 2) & m2) | (y1 & ~m2)};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        R[q] = (u[q] & m4) | ((w[4] << (4 - q)) & mh);
-        R[q + 4] = ((u[q] >> 4) & m4) | ((w[4] >> q) & mh);
-    }
-}
-
 // acc[k] += sum over this warp's share of the listed gates of +-c_j for
 // sample k of the lane (batches of five gates, every 16th batch; the next
 // batch's words are loaded before the current one is used). A short last
@@ -291,30 +275,6 @@ __device__ __forceinline__ void phase_list(float (&acc)[32], const int2 *list, i
         for (int g = 0; g < 5; ++g) z[g] = zn[g];
         t = tn;
     }
-}
-
-// Sum over the 32 lanes of v[lane][k]: afterwards lane L returns the sum of column L.
-__device__ __forceinline__ float reduce_scatter(float (&v)[32], int lane) {
-#pragma unroll
-    for (int w = 16; w >= 1; w >>= 1) {
-        const bool upper = (lane & w) != 0;
-#pragma unroll
-        for (int k = 0; k < w; ++k) {
-            const float send = upper ? v[k] : v[k + w];
-            const float keep = upper ? v[k + w] : v[k];
-            v[k] = keep + __shfl_xor_sync(kFull, send, w);
-        }
-    }
-    return v[0];
-}
-
-// x sc (a power of two, |x sc| < 2^61) rounded to an integer without FP64 (slow
-// on this GPU): split exactly into hi 2^31 + lo.
-__device__ __forceinline__ long long to_fixed(float x, float sc) {
-    const float xs = sc * x;
-    const float hi = truncf(xs * 0x1.0p-31f);
-    const float lo = fmaf(-hi, 0x1.0p31f, xs);
-    return ((long long)__float2int_rz(hi) << 31) + (long long)__float2int_rn(lo);
 }
 
 // Adds 2 scale sum_i W_i s_ij of this warp's share of the listed gates into

@@ -177,9 +177,14 @@ struct TcArgs {
     const uint32_t *pa32;  // P_A, for the gradient mask
     int64_t ldp32;
     double *gpart;
-    void *out;             // mode 3: the accumulator stored as is (FP32, or FP64 if out_f64)
+    float *out;            // mode 0: Phi; mode 3: the accumulator (+ dvec[row], sign bits of zt32)
     int64_t ldo;
-    int out_f64;
+    // mode 3: K pieces (1 = whole), floats between their outputs, addend and sign bits (null = neither)
+    int kparts;
+    int64_t out_part;
+    const float *dvec;
+    const uint32_t *zt32;
+    int64_t ldzt32;
     // Work units of this launch: the tiles, whole (nunits tiles); or, for a
     // split launch, nunits parts of the tiles from `whole` on, nsplit parts
     // per tile (phase modes only).
@@ -236,9 +241,19 @@ struct Bars {
 // units are the tiles, whole. SPL = true: unit u is part u % nsplit of tile
 // whole + u / nsplit; the parts cover the tile's stages in ranges of whole
 // bits stages (KB / KS operand stages), in order.
-template <bool SPL>
+// KP (the dense form): unit u is K piece u / whole of tile u % whole, v the piece.
+template <bool SPL, bool KP = false>
 __device__ __forceinline__ void unit_of(int64_t u, const TcArgs &a, int nks, int64_t &tile, int &ks0, int &ks1,
                                         int64_t &v) {
+    if (KP) {
+        tile = u % a.whole;
+        v = u / a.whole;
+        const int64_t nkb = (nks + KB / KS - 1) / (KB / KS);
+        ks0 = (KB / KS) * (int)(v * nkb / a.kparts);
+        const int e = (KB / KS) * (int)((v + 1) * nkb / a.kparts);
+        ks1 = e < nks ? e : nks;
+        return;
+    }
     if (!SPL) {
         tile = u;
         ks0 = 0;
@@ -666,33 +681,22 @@ __device__ __forceinline__ float store_wf32(const TcArgs &args, int64_t row, int
     return mx;
 }
 
-// Accumulator values of 32 consecutive columns col0.. of `row`, stored into
-// args.out (row-major, args.ldo elements per row, columns < args.s): FP32, or
-// FP64 when args.out_f64. Rows start 16-byte aligned (ldo a multiple of 4).
-__device__ __forceinline__ void store_out32(const TcArgs &args, int64_t row, int64_t col0, const uint32_t (&r)[32]) {
+// Values of 32 consecutive columns col0.. of `row`, stored into out
+// (row-major, args.ldo elements per row, columns < args.s). Rows start 16-byte
+// aligned (ldo a multiple of 4).
+__device__ __forceinline__ void store_out32(const TcArgs &args, float *out, int64_t row, int64_t col0,
+                                            const uint32_t (&r)[32]) {
     if (!IQP_IN(row * args.ldo + col0, args.l * args.ldo, 45) ||
         !IQP_IN(row * args.ldo + (col0 + 32 <= args.s ? col0 + 31 : args.s - 1), args.l * args.ldo, 46))
         return;
-    if (args.out_f64) {
-        double *d = static_cast<double *>(args.out) + row * args.ldo + col0;
-        if (col0 + 32 <= args.s) {
+    float *f = out + row * args.ldo + col0;
+    if (col0 + 32 <= args.s) {
 #pragma unroll
-            for (int e = 0; e < 32; e += 2)
-                *reinterpret_cast<double2 *>(d + e) =
-                    make_double2((double)__uint_as_float(r[e]), (double)__uint_as_float(r[e + 1]));
-        } else {
-            for (int e = 0; e < 32 && col0 + e < args.s; ++e) d[e] = (double)__uint_as_float(r[e]);
-        }
+        for (int e = 0; e < 32; e += 4)
+            *reinterpret_cast<float4 *>(f + e) = make_float4(__uint_as_float(r[e]), __uint_as_float(r[e + 1]),
+                                                             __uint_as_float(r[e + 2]), __uint_as_float(r[e + 3]));
     } else {
-        float *f = static_cast<float *>(args.out) + row * args.ldo + col0;
-        if (col0 + 32 <= args.s) {
-#pragma unroll
-            for (int e = 0; e < 32; e += 4)
-                *reinterpret_cast<float4 *>(f + e) = make_float4(__uint_as_float(r[e]), __uint_as_float(r[e + 1]),
-                                                                 __uint_as_float(r[e + 2]), __uint_as_float(r[e + 3]));
-        } else {
-            for (int e = 0; e < 32 && col0 + e < args.s; ++e) f[e] = __uint_as_float(r[e]);
-        }
+        for (int e = 0; e < 32 && col0 + e < args.s; ++e) f[e] = __uint_as_float(r[e]);
     }
 }
 
@@ -836,7 +840,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int64_t u = group0; u < nunits && ok; u += ngroups) {
                 int64_t t, uv;
                 int ks0, ks1;
-                unit_of<SPL>(u, args, nks, t, ks0, ks1, uv);
+                unit_of<SPL, MODE == 3>(u, args, nks, t, ks0, ks1, uv);
                 int64_t tm64, tc64;
                 tile_rc(t, args, tm64, tc64);
                 const int tm = (int)tm64;
@@ -925,7 +929,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int64_t u = group0; u < nunits && ok; u += ngroups) {
                 int64_t t, uv;
                 int ks0, ks1;
-                unit_of<SPL>(u, args, nks, t, ks0, ks1, uv);
+                unit_of<SPL, MODE == 3>(u, args, nks, t, ks0, ks1, uv);
                 int kc = 0;  // stage index within the current accumulation chunk
                 for (int ks = ks0; ks < ks1; ++ks, ++ito) {
                     const uint32_t os = ito % NOP;
@@ -984,7 +988,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int64_t u = group0; u < nunits && ok; u += ngroups) {
                 int64_t t, uv;
                 int ks0, ks1;
-                unit_of<SPL>(u, args, nks, t, ks0, ks1, uv);
+                unit_of<SPL, MODE == 3>(u, args, nks, t, ks0, ks1, uv);
                 for (int ks = ks0; ks < ks1; ++ks, ++ito) {
                     const uint32_t os = ito % NOP;
                     if (!mbar_wait(&bar->peer_full[os], (ito / NOP) & 1u, abort_flag, status, lim)) {
@@ -1017,7 +1021,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             int64_t tm, tc, slot;
             {
                 int64_t t;
-                unit_of<SPL>(u, args, nks, t, ks0, ks1, slot);
+                unit_of<SPL, MODE == 3>(u, args, nks, t, ks0, ks1, slot);
                 tile_rc(t, args, tm, tc);
             }
             if (ks0 >= ks1) continue;      // an empty piece of a balanced split: no work
@@ -1290,7 +1294,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll 1
                         for (int c = 0; c * 32 < nvalid; ++c) {
                             ldsum(c, r);
-                            if (row < args.l) store_out32(args, row, c0 + c * 32, r);
+                            if (row < args.l) store_out32(args, args.out, row, c0 + c * 32, r);
                         }
                     }
                     if (row < args.l && nvalid > 0 && IQP_IN(row * args.nparts + c0 / kGroupCols, args.l * args.nparts, 50))
@@ -1354,7 +1358,15 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll 1
                     for (int c = 0; c < kGroupLoads; ++c) {
                         ldsum(c, r);
-                        if (row < args.l && c0 + c * 32 < args.s) store_out32(args, row, c0 + c * 32, r);
+                        if (row >= args.l || c0 + c * 32 >= args.s) continue;
+                        if (args.dvec != nullptr) {  // uniform
+                            const float dv = args.dvec[row];
+                            const uint32_t zw = args.zt32[row * args.ldzt32 + ((c0 + c * 32) >> 5)];
+#pragma unroll
+                            for (int e = 0; e < 32; ++e)
+                                r[e] = __float_as_uint(dv + __uint_as_float(r[e])) ^ ((zw << (31 - e)) & 0x80000000u);
+                        }
+                        store_out32(args, args.out + slot * args.out_part, row, c0 + c * 32, r);
                     }
                 } else if (!GRAD) {
                     const int64_t c0 = tn_h * TN + group * kGroupCols;
@@ -2246,9 +2258,8 @@ cudaError_t launch_phase_tc(int mode, const Plan &p, void *ws, const double *alp
     a.ldp32 = 2 * p.ldp;
     a.gpart = nullptr;
     // MODE 0 keeps Phi (FP32, l x ldw) when a gradient pass follows.
-    a.out = (mode == 0 && p.phi_out) ? static_cast<void *>(p.phi) : nullptr;
+    a.out = (mode == 0 && p.phi_out) ? p.phi : nullptr;
     a.ldo = p.ldphi;
-    a.out_f64 = 0;
     a.status = at<uint32_t>(ws, p.off_status);
     a.limit_ns = default_spin_limit_ns();
     a.serp = phase_serp() ? 1 : 0;
@@ -2489,7 +2500,6 @@ cudaError_t launch_grad_tc(const Plan &p, void *ws, cudaStream_t st, iqp_status 
     a.gpart = at<double>(ws, p.off_gpart);
     a.out = nullptr;
     a.ldo = 0;
-    a.out_f64 = 0;
     whole_tiles(a, a.tiles_m * a.tiles_n);
     a.status = at<uint32_t>(ws, p.off_status);
     a.limit_ns = default_spin_limit_ns();
@@ -2511,9 +2521,19 @@ cudaError_t launch_w_from_phi(const Plan &p, void *ws, const double *alpha, cons
 }
 
 cudaError_t launch_tc_dense(const __nv_bfloat16 *a_hi, const __nv_bfloat16 *a_lo, int64_t rows, int64_t kpad,
-                            int64_t k, const uint64_t *b_bits, int64_t nb, int64_t ldb, void *out, int64_t ldo,
-                            bool out_f64, uint32_t *status, cudaStream_t st) {
-    const int cg = cta_group();
+                            int64_t k, const uint64_t *b_bits, int64_t nb, int64_t ldb, float *out, int64_t ldo,
+                            int kparts, const float *d, const uint64_t *zt, int64_t ldzt, uint32_t *status,
+                            cudaStream_t st) {
+    // CTA pairs, or single CTAs where their half-size tiles need less than
+    // three quarters of the pairs' time in rounds (a single CTA expands twice the
+    // +-1 rows per product, about 1.3 times the time of a pair's tile half):
+    // 1000 x 5000 (80 pair tiles on 76 pairs, two rounds) 41 -> 29 us.
+    int cg = cta_group();
+    if (cg == 2 && kparts == 1) {
+        const int sms = num_sms();
+        const int64_t r2 = 2 * cdiv(cdiv(rows, 2 * TM) * cdiv(nb, TN), sms / 2), r1 = cdiv(cdiv(rows, TM) * cdiv(nb, TN), sms);
+        if (r1 * 4 < r2 * 3) cg = 1;
+    }
     CUtensorMap mhi, mlo, mb;
     if (kpad % KS != 0 || k > kpad || k > 64 * ldb || ldb % 2 != 0 || ldb < 4 || ldo % 4 != 0 ||
         !make_map(&mhi, a_hi, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, kpad, rows, kpad * 2, KS, TM,
@@ -2544,8 +2564,13 @@ cudaError_t launch_tc_dense(const __nv_bfloat16 *a_hi, const __nv_bfloat16 *a_lo
     a.gpart = nullptr;
     a.out = out;
     a.ldo = ldo;
-    a.out_f64 = out_f64 ? 1 : 0;
+    a.kparts = kparts;
+    a.out_part = rows * ldo;
+    a.dvec = d;
+    a.zt32 = reinterpret_cast<const uint32_t *>(zt);
+    a.ldzt32 = 2 * ldzt;
     whole_tiles(a, a.tiles_m * a.tiles_n);
+    a.nunits *= kparts;
     a.status = status;
     a.limit_ns = default_spin_limit_ns();
     if (cg == 2) return launch_k<false, 3, 2, true>(mhi, mlo, mb, a, st);
