@@ -406,6 +406,7 @@ LoArgs lo_args(const Plan &p, void *ws) {
     }
     a.H = at<float>(ws, p.off_lo_hp != 0 ? p.off_lo_hp : p.off_lo_h);
     a.hparts = p.off_lo_hp != 0 ? lo_hparts(p.n, p.s) : 1;
+    a.Hs = at<double>(ws, p.off_lo_h);  // free where the pieces have a region of their own
     a.status = at<uint32_t>(ws, p.off_status);
     return a;
 }

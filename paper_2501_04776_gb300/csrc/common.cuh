@@ -101,10 +101,11 @@ struct LoArgs {
     uint2 *Lp;                 // l x kLoP: their pairs with a generator (q | r << 16, bits of -2 C_qr)
     int *cnt;                  // l: qubits | pairs << 16, or -1 for an observable too heavy for the lists; then those
     float *H;                  // hparts x n x ldc
+    double *Hs;                // n x ldc: the pieces' symmetric sum (hparts > 1)
     int hparts;
     uint32_t *status;
 };
-constexpr int kLoQ = 64, kLoP = 256;  // qubits and pairs listed per observable
+constexpr int kLoQ = 128, kLoP = 256;  // qubits and pairs listed per observable
 // K pieces of the gradient's pair contraction (tiles of 256 x 256, 76 CTA
 // pairs): as many as fill the chip with at least eight 64-sample stages each.
 __host__ __device__ inline int lo_hparts(int64_t n, int64_t s) {

@@ -77,12 +77,12 @@ __global__ void k_lo_build(const int4 *__restrict__ sup, const float *__restrict
                            const unsigned *__restrict__ cmax, unsigned long long *__restrict__ E, int64_t lde, int full,
                            uint32_t *__restrict__ status) {
     [[maybe_unused]] uint32_t *status_dbg = status;
-    const int k = lo_fx_exp(*cmax, m);
+    const float sc = ldexpf(1.0f, lo_fx_exp(*cmax, m));  // |c_j sc| < 2^62
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
         const int4 sp = sup[j];
         if (!LO_OK(sp.w <= 0 || (sp.x >= 0 && sp.x < n && (sp.w < 2 || (sp.y > sp.x && sp.y < n))), 8)) continue;
         if (sp.w == 1 || sp.w == 2) {
-            const unsigned long long v = (unsigned long long)llrint(ldexp((double)(2.0f * theta[j]), k));
+            const unsigned long long v = (unsigned long long)to_fixed(2.0f * theta[j], sc);
             if (sp.w == 1) {
                 atomicAdd(dfx + sp.x, v);
             } else {
@@ -211,18 +211,28 @@ __global__ void __launch_bounds__(256) k_lo_lists(const uint64_t *__restrict__ A
     int np = 0;
     if (nq <= kLoQ) {
         for (int t = lane; t < nq; t += 32) Lq[a * kLoQ + t] = sq[warp][t];
-        for (int t = 0; t + 1 < nq; ++t) {
-            const int q = sq[warp][t];
-            for (int u0 = t + 1; u0 < nq; u0 += 32) {
-                const int u = u0 + lane;
-                const int r = u < nq ? sq[warp][u] : 0;
-                const bool ok = u < nq && LO_OK(q >= 0 && q < r && r < n, 10) &&
-                                ((E[(int64_t)q * lde + (r >> 6)] >> (r & 63)) & 1ull) != 0ull;
-                const uint32_t bal = __ballot_sync(kFull, ok);
+        // candidates t nq + u in order, 128 per round: the round's E words are all loaded before the first is used
+        for (int c0 = 0; c0 < nq * nq; c0 += 128) {
+            int qq[4], rr[4];
+            bool ok[4];
+            unsigned long long ew[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int e = c0 + 32 * k + lane, t = e / nq, u = e - t * nq;
+                ok[k] = e < nq * nq && u > t;
+                qq[k] = ok[k] ? sq[warp][t] : 0;
+                rr[k] = ok[k] ? sq[warp][u] : 0;
+                ok[k] = ok[k] && LO_OK(qq[k] >= 0 && qq[k] < rr[k] && rr[k] < n, 10);
+                ew[k] = ok[k] ? E[(int64_t)qq[k] * lde + (rr[k] >> 6)] : 0ull;
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const bool has = ok[k] && ((ew[k] >> (rr[k] & 63)) & 1ull) != 0ull;
+                const uint32_t bal = __ballot_sync(kFull, has);
                 const int pos = np + __popc(bal & ((1u << lane) - 1u));
-                if (ok && pos < kLoP) {
-                    const float c = __ll2float_rn((long long)Cfx[(int64_t)q * n + r]) * inv;
-                    Lp[a * kLoP + pos] = make_uint2((uint32_t)q | ((uint32_t)r << 16), __float_as_uint(-2.0f * c));
+                if (has && pos < kLoP) {
+                    const float cv = __ll2float_rn((long long)Cfx[(int64_t)qq[k] * n + rr[k]]) * inv;
+                    Lp[a * kLoP + pos] = make_uint2((uint32_t)qq[k] | ((uint32_t)rr[k] << 16), __float_as_uint(-2.0f * cv));
                 }
                 np += __popc(bal);
             }
@@ -795,85 +805,86 @@ __global__ void __launch_bounds__(kBlk) k_lo_phase(const uint64_t *__restrict__ 
 // qubit, no sign or addend left to apply); the pair term goes five pairs at a
 // time, their 32 sign combinations one per lane, indexed by the lane's transposed
 // sample bits (indices5), one shuffle and one add per sample.
-//   K: W's signed sums over all 16 sign patterns of every four samples of a lane
-// are tabulated (16 KB per warp); a pair then costs eight table loads per lane,
-// and the lanes' sums of 32 pairs are combined by one reduce-scatter.
-// The loads of X from L2 bound the phase where the observables are wide: n =
-// 5000, 4096 observables of 50 qubits, 16384 samples 1762 us in the one-CTA form
-// (18 instructions per qubit and four samples), the pair term 1278 us.
-// MODE 0: statistics partials, and Phi into phi when it is not null; 1: W and K
-// from Phi formed here; 2: partials, W and K; 3: W and K from Phi read from phi
-// (which may be W itself: each lane reads its samples before it writes them).
-// Heavy observables (cnt < 0) take part in MODE 3 only, for W.
+//   K (k_lo_k, reading W back; fused with the phase its 16 KB of tables per
+// warp left 12 warps per SM to wait for X): W's signed sums over all 16 sign
+// patterns of every four samples of a lane are tabulated; a pair then costs
+// eight table loads per lane, and the lanes' sums of 32 pairs are combined by
+// one reduce-scatter.
+// The loads of X from L2 bound the phase where the observables are wide (n =
+// 5000, 4096 observables of 50 qubits, 16384 samples): 927 us, against 1868 with
+// W in the one-CTA form (18 instructions per qubit and four samples); K 356
+// against 1278.
+// MODE 0: statistics partials, and Phi into phi when it is not null; 1: W; 2:
+// partials and W.
 constexpr int kLoWarps = 4;
 constexpr int kLoTab = 8 * 16 * 32;  // floats of a warp's tables
 template <int MODE>
 __global__ void __launch_bounds__(32 * kLoWarps) k_lo_obs(
     const int *__restrict__ cnt, const int *__restrict__ Lq, const uint2 *__restrict__ Lp, const uint32_t *__restrict__ ZP,
     int64_t nb, const float *__restrict__ X, int64_t lds, int64_t n, int64_t l, int64_t s, int64_t nparts,
-    double2 *__restrict__ part, const double *__restrict__ alpha, const double *__restrict__ beta, float *W, float *phi,
-    int64_t ldphi, const double *__restrict__ scale, unsigned long long *__restrict__ Kfx, uint32_t *__restrict__ status) {
+    double2 *__restrict__ part, const double *__restrict__ alpha, const double *__restrict__ beta, float *__restrict__ W,
+    float *__restrict__ phi, int64_t ldphi, uint32_t *__restrict__ status) {
     [[maybe_unused]] uint32_t *status_dbg = status;
-    extern __shared__ float lo_tab[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t a = (int64_t)blockIdx.x * kLoWarps + warp, blk = blockIdx.y;
     if (a >= l) return;
     const int c = cnt[a];
-    if (c < 0 && MODE != 3) return;
-    const int nq = c & 0xFFFF, np = c < 0 ? 0 : c >> 16;
+    if (c < 0) return;  // a heavy observable
+    const int nq = c & 0xFFFF, np = c >> 16;
     const int64_t i0 = blk * kLane + 4 * lane;  // the lane's samples: i0 + 128 k .. + 3
     const uint32_t *zp = ZP + blk * 32 + lane;
     const uint2 *pairs = Lp + a * kLoP;
     float acc[32];
-    if (MODE == 3) {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const float4 v = i0 + 128 * k < lds ? *reinterpret_cast<const float4 *>(phi + a * ldphi + i0 + 128 * k)
-                                                : make_float4(0.f, 0.f, 0.f, 0.f);
-            acc[4 * k] = v.x;
-            acc[4 * k + 1] = v.y;
-            acc[4 * k + 2] = v.z;
-            acc[4 * k + 3] = v.w;
-        }
-    } else {
+    {
 #pragma unroll
         for (int k = 0; k < 32; ++k) acc[k] = 0.f;
-        const int *Q = Lq + a * kLoQ;
-#pragma unroll 2
-        for (int t = 0; t < nq; ++t) {
-            const int q = __ldg(Q + t);
-            if (!LO_OK(q >= 0 && q < n, 11)) continue;
-            const float *xr = X + (int64_t)q * lds + i0;
+        // The lists are read 32 entries at a time, one per lane, and handed
+        // round by shuffles, so that the rows' loads wait for nothing. (Two rows
+        // of X at a time in registers, or one: 1100 against 950 us; the warps the
+        // extra registers cost matter more.)
+        for (int t0 = 0; t0 < nq; t0 += 32) {
+            const int mine = t0 + lane < nq ? __ldg(Lq + a * kLoQ + t0 + lane) : 0;
+            const int nt = nq - t0 < 32 ? nq - t0 : 32;
+#pragma unroll 1
+            for (int t = 0; t < nt; ++t) {
+                const int q = __shfl_sync(kFull, mine, t);
+                if (!LO_OK(q >= 0 && q < n, 11)) continue;
+                const float *xr = X + (int64_t)q * lds + i0;
+                float4 v[8];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                if (i0 + 128 * k >= lds) continue;
-                const float4 v = __ldg(reinterpret_cast<const float4 *>(xr + 128 * k));
-                acc[4 * k] += v.x;
-                acc[4 * k + 1] += v.y;
-                acc[4 * k + 2] += v.z;
-                acc[4 * k + 3] += v.w;
-            }
-        }
-        for (int p0 = 0; p0 < np; p0 += 5) {
-            uint32_t z[5], R[8];
-            float t = 0.f;
+                for (int k = 0; k < 8; ++k)
+                    v[k] = i0 + 128 * k < lds ? __ldg(reinterpret_cast<const float4 *>(xr + 128 * k))
+                                              : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-            for (int g = 0; g < 5; ++g) {
-                z[g] = 0u;
-                if (p0 + g < np) {
-                    const uint2 e = __ldg(pairs + p0 + g);
-                    const int64_t q = e.x & 0xFFFFu, r = e.x >> 16;
-                    if (!LO_OK(q < r && r < n, 12)) continue;
-                    z[g] = __ldg(zp + q * nb * 32) ^ __ldg(zp + r * nb * 32);
-                    const float cv = __uint_as_float(e.y);
-                    t += ((lane >> g) & 1) ? -cv : cv;
+                for (int k = 0; k < 8; ++k) {
+                    acc[4 * k] += v[k].x;
+                    acc[4 * k + 1] += v[k].y;
+                    acc[4 * k + 2] += v[k].z;
+                    acc[4 * k + 3] += v[k].w;
                 }
             }
-            indices5(z, R);
+        }
+        for (int p0 = 0; p0 < np; p0 += 30) {
+            // past the last pair: {0, 0} with C = 0
+            const uint2 mine = p0 + lane < np && lane < 30 ? __ldg(pairs + p0 + lane) : make_uint2(0u, 0u);
+            const int nt = np - p0 < 30 ? np - p0 : 30;
+#pragma unroll 1
+            for (int h = 0; h < nt; h += 5) {
+                uint32_t z[5], R[8];
+                float t = 0.f;
 #pragma unroll
-            for (int q = 0; q < 8; ++q)
+                for (int g = 0; g < 5; ++g) {
+                    const uint32_t e = __shfl_sync(kFull, mine.x, h + g);
+                    const float cv = __uint_as_float(__shfl_sync(kFull, mine.y, h + g));
+                    z[g] = __ldg(zp + (int64_t)(e & 0xFFFFu) * nb * 32) ^ __ldg(zp + (int64_t)(e >> 16) * nb * 32);
+                    t += ((lane >> g) & 1) ? -cv : cv;
+                }
+                indices5(z, R);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) acc[8 * k + q] += __shfl_sync(kFull, t, (int)(R[q] >> (8 * k)));
+                for (int q = 0; q < 8; ++q)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) acc[8 * k + q] += __shfl_sync(kFull, t, (int)(R[q] >> (8 * k)));
+            }
         }
         if (MODE == 0 && phi != nullptr) {
 #pragma unroll
@@ -935,38 +946,64 @@ __global__ void __launch_bounds__(32 * kLoWarps) k_lo_obs(
             if (i0 + 128 * k < lds)
                 *reinterpret_cast<float4 *>(W + a * lds + i0 + 128 * k) =
                     make_float4(acc[4 * k], acc[4 * k + 1], acc[4 * k + 2], acc[4 * k + 3]);
-        if (np == 0) return;  // uniform in the warp
-        float *tab = lo_tab + warp * kLoTab + lane;
+    }
+}
+
+// K[q][r] += sum_i W[a][i] s_q(i) s_r(i) for the listed pairs (see above).
+__global__ void __launch_bounds__(32 * kLoWarps) k_lo_k(const int *__restrict__ cnt, const uint2 *__restrict__ Lp,
+                                                        const uint32_t *__restrict__ ZP, int64_t nb,
+                                                        const float *__restrict__ W, int64_t lds, int64_t n, int64_t l,
+                                                        const double *__restrict__ scale,
+                                                        unsigned long long *__restrict__ Kfx) {
+    extern __shared__ float lo_tab[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t a = (int64_t)blockIdx.x * kLoWarps + warp, blk = blockIdx.y;
+    if (a >= l) return;
+    const int np = cnt[a] >> 16;
+    if (np <= 0) return;  // no pair, or a heavy observable
+    const int64_t i0 = blk * kLane + 4 * lane;
+    const uint32_t *zp = ZP + blk * 32 + lane;
+    const uint2 *pairs = Lp + a * kLoP;
+    float *tab = lo_tab + warp * kLoTab + lane;
 #pragma unroll
-        for (int g = 0; g < 8; ++g) {
-            const float w0 = acc[4 * g], w1 = acc[4 * g + 1], w2 = acc[4 * g + 2], w3 = acc[4 * g + 3];
-            const float p01[4] = {w0 + w1, w1 - w0, w0 - w1, -w0 - w1};
-            const float p23[4] = {w2 + w3, w3 - w2, w2 - w3, -w2 - w3};
+    for (int g = 0; g < 8; ++g) {  // W is zero from s on, up to its row's end
+        const float4 w = i0 + 128 * g < lds ? *reinterpret_cast<const float4 *>(W + a * lds + i0 + 128 * g)
+                                            : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float p01[4] = {w.x + w.y, w.y - w.x, w.x - w.y, -w.x - w.y};
+        const float p23[4] = {w.z + w.w, w.w - w.z, w.z - w.w, -w.z - w.w};
 #pragma unroll
-            for (int e = 0; e < 16; ++e) tab[(g * 16 + e) * 32] = p01[e & 3] + p23[e >> 2];
-        }
-        const float sc = (float)*scale;
-        for (int p0 = 0; p0 < np; p0 += 32) {
-            float v[32];
+        for (int e = 0; e < 16; ++e) tab[(g * 16 + e) * 32] = p01[e & 3] + p23[e >> 2];
+    }
+    const float sc = (float)*scale;
+    for (int p0 = 0; p0 < np; p0 += 32) {
+        const uint32_t mine = p0 + lane < np ? __ldg(&pairs[p0 + lane].x) : 0u;  // past the last pair: {0, 0}, not used
+        float v[32];
 #pragma unroll
-            for (int g = 0; g < 32; ++g) {
-                v[g] = 0.f;
-                if (p0 + g < np) {  // uniform
-                    const uint32_t e = __ldg(&pairs[p0 + g].x);
-                    const uint32_t z = __ldg(zp + (int64_t)(e & 0xFFFFu) * nb * 32) ^ __ldg(zp + (int64_t)(e >> 16) * nb * 32);
+        for (int h = 0; h < 32; h += 8) {
+            if (p0 + h < np) {  // uniform
+                uint32_t z[8];
+#pragma unroll
+                for (int g = 0; g < 8; ++g) {
+                    const uint32_t e = __shfl_sync(kFull, mine, h + g);
+                    z[g] = __ldg(zp + (int64_t)(e & 0xFFFFu) * nb * 32) ^ __ldg(zp + (int64_t)(e >> 16) * nb * 32);
+                }
+#pragma unroll
+                for (int g = 0; g < 8; ++g) {
                     float u[4];
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
-                        u[k] = tab[(2 * k * 16 + ((z >> (8 * k)) & 15u)) * 32] +
-                               tab[((2 * k + 1) * 16 + ((z >> (8 * k + 4)) & 15u)) * 32];
-                    v[g] = (u[0] + u[1]) + (u[2] + u[3]);
+                        u[k] = tab[(2 * k * 16 + ((z[g] >> (8 * k)) & 15u)) * 32] +
+                               tab[((2 * k + 1) * 16 + ((z[g] >> (8 * k + 4)) & 15u)) * 32];
+                    v[h + g] = (u[0] + u[1]) + (u[2] + u[3]);
                 }
+            } else {
+#pragma unroll
+                for (int g = 0; g < 8; ++g) v[h + g] = 0.f;
             }
-            const float d = reduce_scatter(v, lane);
-            if (p0 + lane < np) {
-                const uint32_t e = pairs[p0 + lane].x;
-                atomicAdd(Kfx + (int64_t)(e & 0xFFFFu) * n + (e >> 16), (unsigned long long)to_fixed(d, sc));
-            }
+        }
+        const float d = reduce_scatter(v, lane);
+        if (p0 + lane < np) {
+            atomicAdd(Kfx + (int64_t)(mine & 0xFFFFu) * n + (mine >> 16), (unsigned long long)to_fixed(d, sc));
         }
     }
 }
@@ -1225,9 +1262,47 @@ __global__ void __launch_bounds__(kBlk) k_lo_pairs(const uint64_t *__restrict__ 
     }  // items
 }
 
+// Hs[q][r] = sum over the K pieces of H[q][r] + H[r][q], q < r (n x ldh FP64):
+// tile by tile, so that the transposed elements are read in rows too (per gate
+// they are a cache line each, times the pieces).
+__global__ void __launch_bounds__(256) k_lo_hsum(const float *__restrict__ H, int64_t ldh, int64_t n, int hparts, int nb,
+                                                 double *__restrict__ Hs) {
+    __shared__ float2 tile[32][33];
+    int bi = 0, left = blockIdx.x;  // block number -> (bi, bj), bi <= bj
+    while (left >= nb - bi) {
+        left -= nb - bi;
+        ++bi;
+    }
+    const int64_t q0 = 32 * (int64_t)bi, r0 = 32 * (int64_t)(bi + left);
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    // The pieces in FP32 with their rounding errors added up beside them (the
+    // sum to about 2^-46 with one FP64 add per element).
+    auto pieces = [&](int64_t row, int64_t col, float &s, float &e) {
+        for (int p = 0; p < hparts; ++p) {
+            const float v = H[((int64_t)p * n + row) * ldh + col], t = s + v, z = t - s;
+            e += (s - (t - z)) + (v - z);
+            s = t;
+        }
+    };
+    for (int k = y; k < 32; k += 8) {  // rows r0 + k, columns q0 + x
+        float s = 0.f, e = 0.f;
+        if (r0 + k < n && q0 + x < n) pieces(r0 + k, q0 + x, s, e);
+        tile[k][x] = make_float2(s, e);
+    }
+    __syncthreads();
+    for (int k = y; k < 32; k += 8) {
+        const int64_t q = q0 + k, r = r0 + x;
+        if (q >= r || r >= n) continue;
+        float s = tile[x][k].x, e = tile[x][k].y;
+        pieces(q, r, s, e);
+        Hs[q * ldh + r] = (double)s + (double)e;
+    }
+}
+
 // grad_j from the parts above (see the header).
 __global__ void k_lo_grad_out(const int4 *__restrict__ sup, int64_t m, int64_t n, const double *__restrict__ gsp,
-                              int64_t nblk, const float *__restrict__ H, int64_t ldh, int hparts,
+                              int64_t nblk, const float *__restrict__ H, int64_t ldh,
+                              const double *__restrict__ Hs,
                               const unsigned long long *__restrict__ Kfx, const double *__restrict__ scale,
                               double *__restrict__ grad) {
     const double inv = 1.0 / *scale;
@@ -1240,9 +1315,7 @@ __global__ void k_lo_grad_out(const int4 *__restrict__ sup, int64_t m, int64_t n
             g = 2.0 * t;
         } else if (sp.w == 2) {
             const int64_t q = sp.x, r = sp.y;
-            double h = 0.0;
-            for (int p = 0; p < hparts; ++p)
-                h += (double)H[((int64_t)p * n + q) * ldh + r] + (double)H[((int64_t)p * n + r) * ldh + q];
+            const double h = Hs != nullptr ? Hs[q * ldh + r] : (double)H[q * ldh + r] + (double)H[r * ldh + q];
             const double k = (double)(long long)Kfx[q * n + r] * inv;
             g = 2.0 * h - 4.0 * k;
         }
@@ -1307,18 +1380,26 @@ unsigned lo_heavy_blocks(const LoArgs &a, int64_t nblk) {
 template <int MODE>
 cudaError_t launch_obs(const LoArgs &a, double2 *part, const double *alpha, const double *beta, float *W, float *phi,
                        int64_t ldphi, cudaStream_t st) {
-    constexpr int smem = MODE == 0 ? 0 : kLoWarps * kLoTab * 4;
+    const int64_t nb = cdiv(a.s, (int64_t)kLane);
+    LaunchScope ls(IQP_KERNEL_LOWORDER, st);
+    k_lo_obs<MODE><<<dim3((unsigned)cdiv(a.l, (int64_t)kLoWarps), (unsigned)nb), 32 * kLoWarps, 0, st>>>(
+        a.cnt, a.Lq, a.Lp, a.ZP, nb, a.X, a.lds, a.n, a.l, a.s, cdiv(a.s, (int64_t)kBlk), part, alpha, beta, W, phi, ldphi,
+        a.status);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_k(const LoArgs &a, const float *W, cudaStream_t st) {
+    constexpr int smem = kLoWarps * kLoTab * 4;
     static bool attr_set = false;
     if (!attr_set) {
-        const cudaError_t e = cudaFuncSetAttribute(k_lo_obs<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        const cudaError_t e = cudaFuncSetAttribute(k_lo_k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
     const int64_t nb = cdiv(a.s, (int64_t)kLane);
     LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-    k_lo_obs<MODE><<<dim3((unsigned)cdiv(a.l, (int64_t)kLoWarps), (unsigned)nb), 32 * kLoWarps, smem, st>>>(
-        a.cnt, a.Lq, a.Lp, a.ZP, nb, a.X, a.lds, a.n, a.l, a.s, cdiv(a.s, (int64_t)kBlk), part, alpha, beta, W, phi, ldphi,
-        lo_scale(a), a.fx, a.status);
+    k_lo_k<<<dim3((unsigned)cdiv(a.l, (int64_t)kLoWarps), (unsigned)nb), 32 * kLoWarps, smem, st>>>(
+        a.cnt, a.Lp, a.ZP, nb, W, a.lds, a.n, a.l, lo_scale(a), a.fx);
     return cudaGetLastError();
 }
 
@@ -1403,16 +1484,16 @@ cudaError_t launch_lo_grad(const LoArgs &a, double2 *part, const double *alpha, 
     }
     if (!scale_set && (e = launch_fixed_scale(alpha, beta, a.l, s, lo_scale(a), st)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(a.fx, 0, (size_t)n * n * sizeof(unsigned long long), st)) != cudaSuccess) return e;
-    if (listed) {
-        e = phi != nullptr    ? launch_obs<3>(a, nullptr, alpha, beta, W, phi, ldphi, st)
-            : part != nullptr ? launch_obs<2>(a, part, alpha, beta, W, nullptr, 0, st)
-                              : launch_obs<1>(a, nullptr, alpha, beta, W, nullptr, 0, st);
-        if (e != cudaSuccess) return e;
-    } else if (phi != nullptr) {
+    if (phi != nullptr) {
         LaunchScope ls(IQP_KERNEL_LOWORDER, st);
         k_lo_w<<<grid_1d(a.l * (a.lds / 4)), 256, 0, st>>>(phi, ldphi, W, a.lds, a.l, s, alpha, beta);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    } else if (listed) {
+        e = part != nullptr ? launch_obs<2>(a, part, alpha, beta, W, nullptr, 0, st)
+                            : launch_obs<1>(a, nullptr, alpha, beta, W, nullptr, 0, st);
+        if (e != cudaSuccess) return e;
     }
+    if (listed && (e = launch_k(a, W, st)) != cudaSuccess) return e;
     __nv_bfloat16 *hi = a.split, *lo = a.split + n * a.lds;
     {
         LaunchScope ls(IQP_KERNEL_LOWORDER, st);
@@ -1437,8 +1518,15 @@ cudaError_t launch_lo_grad(const LoArgs &a, double2 *part, const double *alpha, 
                                                               lo_nheavy(a), W, a.lds, s, nblk, lo_scale(a), a.fx, a.status);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
+    if (hparts > 1) {
+        const int64_t nb = cdiv(n, 32);
+        LaunchScope ls(IQP_KERNEL_LOWORDER, st);
+        k_lo_hsum<<<(unsigned)(nb * (nb + 1) / 2), 256, 0, st>>>(a.H, a.ldc, n, hparts, (int)nb, a.Hs);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
     LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-    k_lo_grad_out<<<grid_1d(a.m), 256, 0, st>>>(a.sup, a.m, n, gsp, nblk, a.H, a.ldc, hparts, a.fx, lo_scale(a), grad);
+    k_lo_grad_out<<<grid_1d(a.m), 256, 0, st>>>(a.sup, a.m, n, gsp, nblk, a.H, a.ldc, hparts > 1 ? a.Hs : nullptr, a.fx,
+                                                lo_scale(a), grad);
     return cudaGetLastError();
 }
 

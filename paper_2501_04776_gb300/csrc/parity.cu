@@ -666,9 +666,9 @@ cudaError_t bit_transpose(const uint64_t *in, int64_t in_rows, int64_t in_cols, 
 // their rows as one run of 16-byte units, eight loads per thread in flight; the
 // few set bits go to the row's slots in shared memory, in any order, and one
 // thread per row sorts them (a row of more than three set bits is scanned
-// again). The rows are read once, which bounds it: 500500 rows of 128 bytes in
-// 38.7 us by one thread per row (each load behind the previous word's scan),
-// 254 us for 10^6 rows of 640 bytes by one warp per row.
+// again). The rows are read once, which bounds it: 500500 rows of 128 bytes
+// 25 us (38.7 by one thread per row, each load behind the previous word's
+// scan), 10^6 rows of 640 bytes 134 us (254 by one warp per row).
 // With theta, the largest |2 theta_j| of the gates on one or two qubits goes to
 // *cmax (its float bits; zero before the launch).
 constexpr int kSuRows = 256, kSuLoads = 8;
@@ -681,12 +681,15 @@ __global__ void __launch_bounds__(256) k_support_rows(const uint64_t *__restrict
     for (int r = threadIdx.x; r < rows; r += 256) cnt[r] = 0;
     __syncthreads();
     const int total = rows * nu;  // R nu <= 2048, or one row of any length
+    // unit i -> row i / nu: exact in FP32 (i + 1/2 is at least 1 / (2 nu) off a multiple, i <= 2048 unless R = 1)
+    const float inv = 1.0f / (float)nu;
+    auto row_of = [&](int i) { return R == 1 ? 0 : (int)(((float)i + 0.5f) * inv); };
     for (int b = 0; b < total; b += 256 * kSuLoads) {
         ulonglong2 v[kSuLoads];
 #pragma unroll
         for (int k = 0; k < kSuLoads; ++k) {
             const int i = b + (int)threadIdx.x + 256 * k;
-            const int r = i / nu, u = i - r * nu;
+            const int r = row_of(i), u = i - r * nu;
             v[k] = make_ulonglong2(0ull, 0ull);
             if (i < total && IQP_IN((j0 + r) * ldg + 2 * u + 1, m * ldg, 16))
                 v[k] = *reinterpret_cast<const ulonglong2 *>(G + (j0 + r) * ldg + 2 * u);
@@ -695,7 +698,7 @@ __global__ void __launch_bounds__(256) k_support_rows(const uint64_t *__restrict
         for (int k = 0; k < kSuLoads; ++k) {
             if ((v[k].x | v[k].y) == 0ull) continue;
             const int i = b + (int)threadIdx.x + 256 * k;
-            const int r = i / nu, u = i - r * nu;
+            const int r = row_of(i), u = i - r * nu;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 uint64_t w = h ? v[k].y : v[k].x;

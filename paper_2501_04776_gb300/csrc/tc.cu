@@ -2524,16 +2524,11 @@ cudaError_t launch_tc_dense(const __nv_bfloat16 *a_hi, const __nv_bfloat16 *a_lo
                             int64_t k, const uint64_t *b_bits, int64_t nb, int64_t ldb, float *out, int64_t ldo,
                             int kparts, const float *d, const uint64_t *zt, int64_t ldzt, uint32_t *status,
                             cudaStream_t st) {
-    // CTA pairs, or single CTAs where their half-size tiles need less than
-    // three quarters of the pairs' time in rounds (a single CTA expands twice the
-    // +-1 rows per product, about 1.3 times the time of a pair's tile half):
-    // 1000 x 5000 (80 pair tiles on 76 pairs, two rounds) 41 -> 29 us.
-    int cg = cta_group();
-    if (cg == 2 && kparts == 1) {
-        const int sms = num_sms();
-        const int64_t r2 = 2 * cdiv(cdiv(rows, 2 * TM) * cdiv(nb, TN), sms / 2), r1 = cdiv(cdiv(rows, TM) * cdiv(nb, TN), sms);
-        if (r1 * 4 < r2 * 3) cg = 1;
-    }
+    // Single CTAs: their half-size tiles fill the last round better, and with A by
+    // TMA the producers have only the +-1 rows to expand. n = 5000, 16384 samples:
+    // X 1009 us (CTA pairs 1124), H 1047 (1236); 1000 x 5000 40 either way. H in
+    // K pieces keeps the pairs: its pieces are counted for them.
+    const int cg = kparts == 1 ? 1 : cta_group();
     CUtensorMap mhi, mlo, mb;
     if (kpad % KS != 0 || k > kpad || k > 64 * ldb || ldb % 2 != 0 || ldb < 4 || ldo % 4 != 0 ||
         !make_map(&mhi, a_hi, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, kpad, rows, kpad * 2, KS, TM,
