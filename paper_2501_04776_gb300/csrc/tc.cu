@@ -27,10 +27,10 @@
 // takes sixteen MMAs, and the A expansion per flop halves. The running sums
 // of the accumulation chunks go to a per-CTA buffer in global memory (it
 // stays in L2). The double tiles of a last, partial round run as a balanced
-// split (TcArgs::sk): their bits stages, end to end, in one equal range per
-// CTA pair, each range's piece of a tile a split part; or, without room for
-// its scratch, as single tiles (TcArgs::dtmap), split along the gates as
-// below.
+// split (TcArgs::skW): their bits stages, end to end, in one equal range per
+// CTA pair, each range's piece of a tile a split part that k_split_reduce adds
+// up; or, without room for its scratch, as single tiles (TcArgs::dtmap), whose
+// last round is split the same way.
 //
 // Dense form (mode 3, A by TMA): out = (A_hi + A_lo) (1 - 2 B_bits)^T for a
 // dense split-BF16 matrix A brought in by TMA and a +-1 operand expanded from
@@ -186,12 +186,10 @@ struct TcArgs {
     const uint32_t *zt32;
     int64_t ldzt32;
     // Work units of this launch: the tiles, whole (nunits tiles); or, for a
-    // split launch, nunits parts of the tiles from `whole` on, nsplit parts
-    // per tile (phase modes only).
+    // split launch, nunits parts of the tiles from `whole` on (phase modes
+    // only; see skW).
     int64_t nunits, whole;
-    int nsplit;
     float *skp;            // split parts' partial accumulators, TM x TN FP32 per (part, CTA of the pair)
-    int *skc;              // per (split tile, CTA of the pair): parts finished so far
     uint32_t *status;
     uint64_t limit_ns;
     int serp;              // phase, whole tiles: every other round of tiles walks the gates backwards
@@ -207,13 +205,12 @@ struct TcArgs {
     // tiles_m x tiles_n2 walk.
     int dtmap;
     int64_t dbase, tiles_n2;
-    // Balanced split of a last round (sk = 1; split units only): the skW
+    // Balanced split of a last round (split units only): the skW
     // bits stages of the tiles from `whole` on, laid end to end, are cut into
     // skP equal contiguous ranges, one per CTA group; unit u is piece u / skP
     // of range u % skP (the part of the range inside one tile; empty when the
     // range has fewer pieces). The pieces of tile whole + t take the slots
     // t * skKP + j, j = 0, 1, ... in range order.
-    int sk;
     int64_t skW, skP, skKP;
     int64_t skcap;  // floats of split-part scratch at skp
 };
@@ -230,17 +227,16 @@ __device__ __forceinline__ void tile_rc(int64_t t, const TcArgs &a, int64_t &tm,
 
 struct Bars {
     uint64_t bits_full[NBITS], bits_empty[NBITS], op_full[kMaxOp], op_empty[kMaxOp], w_full[kMaxOp],
-        peer_full[kMaxOp], acc_full, drain, red_full, part_done, part_flag;
+        peer_full[kMaxOp], acc_full, drain, red_full;
     uint32_t tmem_slot;
     int abort_flag;
-    int last_flag;  // this CTA finished the last part of a split tile
 };
 
 // Work unit u -> its tile, its operand-stage range [ks0, ks1) and, for a
 // part of a split tile, its slot v (-1 for a whole tile). SPL = false: the
-// units are the tiles, whole. SPL = true: unit u is part u % nsplit of tile
-// whole + u / nsplit; the parts cover the tile's stages in ranges of whole
-// bits stages (KB / KS operand stages), in order.
+// units are the tiles, whole. SPL = true: unit u is a piece of the balanced
+// split (see skW); the parts cover a tile's stages in ranges of whole bits
+// stages (KB / KS operand stages), in order.
 // KP (the dense form): unit u is K piece u / whole of tile u % whole, v the piece.
 template <bool SPL, bool KP = false>
 __device__ __forceinline__ void unit_of(int64_t u, const TcArgs &a, int nks, int64_t &tile, int &ks0, int &ks1,
@@ -262,49 +258,31 @@ __device__ __forceinline__ void unit_of(int64_t u, const TcArgs &a, int nks, int
         return;
     }
     const int64_t nkb = (nks + KB / KS - 1) / (KB / KS);
-    if (a.sk) {
-        const int64_t g = u % a.skP, k = u / a.skP;
-        const int64_t A = g * a.skW / a.skP, B = (g + 1) * a.skW / a.skP;
-        const int64_t start = k == 0 ? A : (A / nkb + k) * nkb;
-        tile = a.whole;
-        ks0 = ks1 = 0;
-        v = -1;
-        if (start >= B) return;  // this range has no piece k
-        const int64_t t = start / nkb;
-        const int64_t end = B < (t + 1) * nkb ? B : (t + 1) * nkb;
-        tile = a.whole + t;
-        ks0 = (KB / KS) * (int)(start - t * nkb);
-        const int64_t e = (KB / KS) * (end - t * nkb);
-        ks1 = e < nks ? (int)e : nks;
-        // the range holding the tile's first bits stage: the largest g0 with g0 W / P <= t nkb
-        const int64_t g0 = ((t * nkb + 1) * a.skP - 1) / a.skW;
-        v = t * a.skKP + (g - g0);
-        return;
-    }
-    v = u;
-    tile = a.whole + v / a.nsplit;
-    const int64_t part = v % a.nsplit;
-    ks0 = (KB / KS) * (int)(part * nkb / a.nsplit);
-    const int e = (KB / KS) * (int)((part + 1) * nkb / a.nsplit);
-    ks1 = e < nks ? e : nks;
+    const int64_t g = u % a.skP, k = u / a.skP;
+    const int64_t A = g * a.skW / a.skP, B = (g + 1) * a.skW / a.skP;
+    const int64_t start = k == 0 ? A : (A / nkb + k) * nkb;
+    tile = a.whole;
+    ks0 = ks1 = 0;
+    v = -1;
+    if (start >= B) return;  // this range has no piece k
+    const int64_t tt = start / nkb;
+    const int64_t end = B < (tt + 1) * nkb ? B : (tt + 1) * nkb;
+    tile = a.whole + tt;
+    ks0 = (KB / KS) * (int)(start - tt * nkb);
+    const int64_t e = (KB / KS) * (end - tt * nkb);
+    ks1 = e < nks ? (int)e : nks;
+    // the range holding the tile's first bits stage: the largest g0 with g0 W / P <= tt nkb
+    const int64_t g0 = ((tt * nkb + 1) * a.skP - 1) / a.skW;
+    v = tt * a.skKP + (g - g0);
 }
 
-// A split unit's slot v -> its tile's index tt among the split tiles, the
-// number of parts of that tile and the slot of its first part.
-__device__ __forceinline__ void part_info(int64_t v, const TcArgs &a, int nks, int64_t &tt, int64_t &np,
-                                          int64_t &base) {
-    if (a.sk) {
-        const int64_t nkb = (nks + KB / KS - 1) / (KB / KS);
-        tt = v / a.skKP;
-        const int64_t g0 = ((tt * nkb + 1) * a.skP - 1) / a.skW;
-        const int64_t g1 = ((tt + 1) * nkb * a.skP - 1) / a.skW;
-        np = g1 - g0 + 1;
-        base = tt * a.skKP;
-        return;
-    }
-    tt = v / a.nsplit;
-    np = a.nsplit;
-    base = tt * a.nsplit;
+// Split tile tt (from `whole` on): the number of its parts and the slot of the first.
+__device__ __forceinline__ void part_info(int64_t tt, const TcArgs &a, int nks, int64_t &np, int64_t &base) {
+    const int64_t nkb = (nks + KB / KS - 1) / (KB / KS);
+    const int64_t g0 = ((tt * nkb + 1) * a.skP - 1) / a.skW;
+    const int64_t g1 = ((tt + 1) * nkb * a.skP - 1) / a.skW;
+    np = g1 - g0 + 1;
+    base = tt * a.skKP;
 }
 
 __device__ __forceinline__ uint8_t *aligned_smem(uint8_t *raw) {
@@ -700,10 +678,9 @@ __device__ __forceinline__ void store_out32(const TcArgs &args, float *out, int6
     }
 }
 
-// Split phase tiles (kept out of line, so that their registers do not weigh
-// on the stage loop). split_store: this warp's 32 rows x 64 columns of the
-// accumulator (+ running sum) into its part's slot. split_sum: the sum of
-// the tile's nsplit parts, in part order, into the accumulator columns.
+// Split phase tiles (kept out of line, so that its registers do not weigh on
+// the stage loop): this warp's 32 rows x 64 columns of the accumulator (+
+// running sum) into its part's slot.
 template <bool X3>
 __device__ __noinline__ void split_store(float *dst, uint32_t tbase, bool chunked, const float4 *ss0) {
     uint32_t r[32];
@@ -720,24 +697,89 @@ __device__ __noinline__ void split_store(float *dst, uint32_t tbase, bool chunke
     }
 }
 
-__device__ __noinline__ void split_sum(const float *src0, int64_t part_stride, int nsplit, uint32_t tbase) {
-#pragma unroll 1
-    for (int c = 0; c < kGroupLoads; ++c) {
-        uint32_t r[32];
+// The split tiles' epilogue: one warp per (row, 64 columns) of a split tile adds
+// the tile's parts up in part order (two columns per lane, 256 coalesced bytes
+// per part) and forms what the whole tiles' epilogue forms, over the whole chip.
+// With the last part's CTA doing both, a tile of 20 parts cost 0.47 ms of one SM's
+// time for 45 us of products (1000 observables x 10^4 samples, 45150 gates).
+template <int MODE, bool X3>
+__global__ void __launch_bounds__(256) k_split_reduce(const TcArgs args, int CG, int NH, int64_t tiles) {
+    const int lane = threadIdx.x & 31;
+    const int64_t w = (blockIdx.x * (int64_t)256 + threadIdx.x) >> 5;
+    const int group = (int)(w & 3), rl = (int)((w >> 2) & (TM - 1));
+    const int64_t v = w >> 9;  // (tile, half, accumulator)
+    const int h = (int)(v % NH), half = (int)((v / NH) % CG);
+    const int64_t tt = v / (NH * CG);
+    if (tt >= tiles) return;
+    int64_t tm, tc, np, base;
+    tile_rc(args.whole + tt, args, tm, tc);
+    part_info(tt, args, (int)args.nks, np, base);
+    const int64_t row = (tm * CG + half) * TM + rl;
+    const int64_t c0 = (NH == 2 ? 2 * tc + h : tc) * TN + group * kGroupCols;  // first sample of this group
+    if (row >= args.l || c0 >= args.s) return;
+    const int64_t so = (((base * CG + half) * NH + h) * TM + rl) * TN + group * kGroupCols + 2 * lane;
+    const int64_t pstride = (int64_t)CG * NH * TM * TN;
+    if (!IQP_IN(so + (np - 1) * pstride + 1, args.skcap, 49)) return;
+    float x = 0.f, y = 0.f;
+#pragma unroll 4
+    for (int64_t p = 0; p < np; ++p) {
+        const float2 u = __ldcg(reinterpret_cast<const float2 *>(args.skp + so + p * pstride));
+        x += u.x;
+        y += u.y;
+    }
+    const int64_t i = c0 + 2 * lane;
+    const bool v0 = i < args.s, v1 = i + 1 < args.s;
+    float s0 = 0.f, k0, s1 = 0.f, k1;
+    if (MODE == 0) {
+        k0 = cosf(x);
+        k1 = cosf(y);
+    } else {
+        sincosf(x, &s0, &k0);
+        sincosf(y, &s1, &k1);
+    }
+    if (MODE != 1) {
+        const int64_t nvalid = args.s - c0 < kGroupCols ? args.s - c0 : kGroupCols;
+        float S = (v0 ? k0 : 0.f) + (v1 ? k1 : 0.f);
 #pragma unroll
-        for (int e = 0; e < 32; ++e) r[e] = 0u;  // +0.0f
-        for (int pp = 0; pp < nsplit; ++pp) {
-            const float *src = src0 + pp * part_stride + c * 32;
+        for (int o = 16; o >= 1; o >>= 1) S += __shfl_xor_sync(0xFFFFFFFFu, S, o);
+        const float mean = S / (float)nvalid;
+        float M2 = (v0 ? (k0 - mean) * (k0 - mean) : 0.f) + (v1 ? (k1 - mean) * (k1 - mean) : 0.f);
 #pragma unroll
-            for (int e = 0; e < 32; e += 4) {
-                const float4 x = __ldcg(reinterpret_cast<const float4 *>(src + e));
-                r[e] = __float_as_uint(__uint_as_float(r[e]) + x.x);
-                r[e + 1] = __float_as_uint(__uint_as_float(r[e + 1]) + x.y);
-                r[e + 2] = __float_as_uint(__uint_as_float(r[e + 2]) + x.z);
-                r[e + 3] = __float_as_uint(__uint_as_float(r[e + 3]) + x.w);
+        for (int o = 16; o >= 1; o >>= 1) M2 += __shfl_xor_sync(0xFFFFFFFFu, M2, o);
+        if (lane == 0 && IQP_IN(row * args.nparts + c0 / kGroupCols, args.l * args.nparts, 50))
+            args.part[row * args.nparts + c0 / kGroupCols] = make_double2((double)S, (double)M2);
+    }
+    if (MODE == 0) {
+        if (args.out != nullptr && IQP_IN(row * args.ldo + (v1 ? i + 1 : c0), args.l * args.ldo, 45)) {
+            float *f = args.out + row * args.ldo + i;
+            if (v1) *reinterpret_cast<float2 *>(f) = make_float2(x, y);
+            else if (v0) *f = x;
+        }
+    } else {
+        const float al = (float)args.alpha[row], be = args.beta ? (float)args.beta[row] : 0.f;
+        const float w0 = s0 * (al + be * k0), w1 = s1 * (al + be * k1);
+        if (!IQP_IN(row * args.ldw + (v1 ? i + 1 : c0), args.l * args.ldw, 44)) return;
+        if (X3) {
+            float *f = args.wf + row * args.ldw + i;
+            if (v1) *reinterpret_cast<float2 *>(f) = make_float2(w0, w1);
+            else if (v0) *f = w0;
+            const float a0 = fabsf(w0), a1 = fabsf(w1);
+            float mx = v0 && a0 <= 3.4e38f ? a0 : 0.f;
+            if (v1 && a1 <= 3.4e38f) mx = fmaxf(mx, a1);
+            const uint32_t mb = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(mx));
+            if (lane == 0 && mb != 0u) atomicMax(args.wmax + row, mb);
+        } else {
+            const float h0 = __bfloat162float(__float2bfloat16_rn(w0)), h1 = __bfloat162float(__float2bfloat16_rn(w1));
+            const uint32_t ph = pack_bf16x2(h0, h1), pl = pack_bf16x2(w0 - h0, w1 - h1);
+            __nv_bfloat16 *dh = args.whi + row * args.ldw + i, *dl = args.wlo + row * args.ldw + i;
+            if (v1) {
+                *reinterpret_cast<uint32_t *>(dh) = ph;
+                *reinterpret_cast<uint32_t *>(dl) = pl;
+            } else if (v0) {
+                *reinterpret_cast<uint16_t *>(dh) = (uint16_t)ph;
+                *reinterpret_cast<uint16_t *>(dl) = (uint16_t)pl;
             }
         }
-        tmem_st32(tbase + c * 32, r);
     }
 }
 
@@ -802,9 +844,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_init(&bar->acc_full, 1);
         mbar_init(&bar->drain, 1);
         mbar_init(&bar->red_full, NGEN);
-        mbar_init(&bar->part_done, NGEN);
-        mbar_init(&bar->part_flag, 1);
-        bar->last_flag = 0;
         bar->abort_flag = 0;
         fence_barrier_init();
         fence_proxy_async_smem();
@@ -1184,66 +1223,26 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc_fence_after();
             const int64_t row = arow0 + quarter * 32 + lane;  // observable a
             const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(group * kGroupCols);
-            bool chunked = nchunk > 0;
-            [[maybe_unused]] bool merged = false;  // X3: columns 0..255 hold the whole sum (a split tile's last part)
+            const bool chunked = nchunk > 0;
 
-            if (!GRAD && MODE != 3 && SPL) {
+            if constexpr (!GRAD && MODE != 3 && SPL) {
                 // A part of a split tile: store this part's accumulator(s);
-                // the CTA that finishes the tile's last part sums every
-                // part's, in part order, back into TMEM and runs the
-                // epilogue. Slot layout: ((slot * CG + CTA) * NH + h) per
-                // TM x TN accumulator h (DT: two).
+                // k_split_reduce, launched next, adds the tile's parts up and
+                // runs the epilogue. Slot layout: ((slot * CG + CTA) * NH + h)
+                // per TM x TN accumulator h (DT: two).
                 constexpr int NH = DT ? 2 : 1;
                 const int64_t half = CG == 2 ? (int64_t)crank : 0;
-                [[maybe_unused]] const int64_t kSkp = args.skcap;  // floats of part scratch
-                int64_t tt, np, pbase;  // index among the split tiles, its parts, its first part's slot
-                part_info(slot, args, nks, tt, np, pbase);
 #pragma unroll 1
                 for (int h = 0; h < NH; ++h) {
                     const int64_t so = (((slot * CG + half) * NH + h) * TM + rl) * TN + group * kGroupCols;
                     const float4 *ss0 = ATM  ? sum4 + ((group * kGroupCols) >> 2) * TM + rl
                                         : DT || X3 ? gsum_cta + ((h * TN + group * kGroupCols) >> 2) * TM + rl
                                                    : nullptr;
-                    if (IQP_IN(so + kGroupCols - 1, kSkp, 47))
+                    if (IQP_IN(so + kGroupCols - 1, args.skcap, 47))
                         split_store<X3>(args.skp + so, tbase + (uint32_t)(h * TN), chunked, ss0);
                 }
-                __threadfence();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&bar->part_done);
-                const uint32_t nsu = tix;  // split parts this CTA finished before
-                if (warp == 2 && lane == 0) {
-                    if (mbar_wait(&bar->part_done, nsu & 1u, abort_flag, status, lim)) {
-                        int last = 0;
-                        if (IQP_IN(tt * CG + half, kMaxSplitCtas, 48)) {
-                            int *cnt = args.skc + tt * CG + half;
-                            last = atomicAdd(cnt, 1) == np - 1;
-                            if (last) {
-                                atomicExch(cnt, 0);  // ready for the next launch
-                                __threadfence();
-                            }
-                        }
-                        bar->last_flag = last;
-                    }
-                    mbar_arrive(&bar->part_flag);
-                }
-                if (!wait_warp(&bar->part_flag, nsu & 1u, abort_flag, status, lim) || *abort_flag) {
-                    ok = false;
-                    break;
-                }
-                if (*reinterpret_cast<volatile int *>(&bar->last_flag) == 0) {
-                    tc_fence_before();
-                    continue;  // another CTA finishes this tile
-                }
-                __threadfence();
-#pragma unroll 1
-                for (int h = 0; h < NH; ++h) {
-                    const int64_t s0 = (((pbase * CG + half) * NH + h) * TM + rl) * TN + group * kGroupCols;
-                    const int64_t pstride = (int64_t)CG * NH * TM * TN;
-                    if (IQP_IN(s0 + (np - 1) * pstride + kGroupCols - 1, kSkp, 49))
-                        split_sum(args.skp + s0, pstride, (int)np, tbase + (uint32_t)(h * TN));
-                }
-                chunked = false;  // the sum of the parts is in the accumulator columns
-                merged = true;
+                tc_fence_before();
+                continue;
             }
             // Phi (or Q) for 32 columns: last chunk's accumulator + running sum.
             // DT: the two sample tiles' accumulators in turn.
@@ -1259,7 +1258,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                                       : nullptr;
                 };
                 auto ldsum = [&](int c, uint32_t (&r)[32]) {
-                    if (X3 && !merged)
+                    if (X3)
                         load_sum32_x3(tb_h + c * 32, chunked ? ssum(c) : nullptr, r);
                     else
                         load_sum32(tb_h + c * 32, chunked, r, ssum(c));
@@ -2126,9 +2125,7 @@ constexpr int64_t kX3Chunk = 65536;
 // Every tile whole (no split parts).
 void whole_tiles(TcArgs &a, int64_t ntiles) {
     a.nunits = a.whole = ntiles;
-    a.nsplit = 1;
     a.skp = nullptr;
-    a.skc = nullptr;
 }
 
 template <class T>
@@ -2177,46 +2174,87 @@ cudaError_t launch_phase_k(int mode, int cg, const CUtensorMap &ma, const CUtens
 }  // namespace
 
 namespace {
-// The T single tiles of a phase: a last round of tiles that would leave CTA
-// groups idle is split along the gates across them. The whole tiles run first
-// (full rounds), then a second launch runs the remaining tiles' parts, each a
-// range of whole bits stages, and the last part of a tile to finish sums the
-// parts (in part order) and runs the epilogue. skp: the split tiles' scratch
-// (null: every tile whole).
-cudaError_t launch_single_tiles(int mode, int cg, bool x3, const CUtensorMap &ma, const CUtensorMap &mb, TcArgs a,
-                                int64_t T, float *skp, cudaStream_t st) {
-    whole_tiles(a, T);
-    int64_t R = 0, ns = 1;
-    if (split_tail() && skp != nullptr) {
-        int sms = num_sms();
-        if (sms > kMaxSplitCtas) sms = kMaxSplitCtas;
-        const int64_t P = sms / cg;  // CTA groups
-        R = T >= P ? T % P : T;
-        ns = (P >= 2 && R > 0) ? P / R : 1;
-        const int64_t nkb = cdiv(a.nks, KB / KS);
-        if (ns > nkb) ns = nkb;
-        if (ns < 2) R = 0;
+// Times the choices below weigh, in us: a bits stage of a tile (of two sample
+// tiles: DT), and what a split costs beside its products (parts of 256 or 512 KB
+// per CTA pair to store, add up and launch; about P + tiles of them whatever the
+// sizes: 17 us of adding up for 84 DT parts, as much again for the rest).
+constexpr double kStageUs = 2.6, kStageDtUs = 4.8, kSplitUs = 20.0, kSplitDtUs = 35.0;
+
+// Balanced split of `left` tiles (from tile `first` on) over P CTA groups: their
+// bits stages, end to end, in equal ranges, one per group, each range's piece of
+// a tile a part (see unit_of). skp: scratch of `slots` accumulators. Returns
+// false, and leaves the tiles whole, where that saves less than it costs: (1 -
+// left / P) of the tiles' K loop. 4 double tiles left on 76 pairs, 177 stages: 517
+// -> 83 us with the parts added up over the chip (k_split_reduce). 40 tiles of 12
+// stages: whole 72 us, split 80. Where the tiles fill half the groups at most,
+// or `always`, they are split in any case: there are few parts to add up, and
+// sums of shorter ranges lose less to the tensor core's truncation (standard
+// errors of small circuits 6e-7 relative, 1.1e-6 with whole tiles).
+bool balance(TcArgs &a, int64_t first, int64_t left, int64_t P, int cg, int nh, float *skp, int64_t slots,
+             bool always = false) {
+    const int64_t nkb = cdiv(a.nks, KB / KS), W = left * nkb;
+    const double stage = nh == 2 ? kStageDtUs : kStageUs, cost = nh == 2 ? kSplitDtUs : kSplitUs;
+    if (!split_tail() || skp == nullptr || left <= 0 || nkb < 2) return false;
+    if (!always && 2 * left > P && (double)(nkb * (P - left)) * stage <= cost * (double)P) return false;
+    if (P > W) P = W;  // at least one bits stage per range
+    for (; P >= left && P >= 1; --P) {
+        int64_t KP = 1;
+        for (int64_t t = 0; t < left; ++t) {
+            const int64_t g0 = ((t * nkb + 1) * P - 1) / W, g1 = ((t + 1) * nkb * P - 1) / W;
+            if (g1 - g0 + 1 > KP) KP = g1 - g0 + 1;
+        }
+        if (left * KP * cg * nh > slots) continue;
+        a.whole = first;
+        a.nunits = P * (cdiv(W / P + 1, nkb) + 2);
+        a.skW = W;
+        a.skP = P;
+        a.skKP = KP;
+        a.skp = skp;
+        a.skcap = slots * kSplitSlotFloats;
+        return true;
     }
+    return false;
+}
+
+cudaError_t launch_split_reduce(int mode, bool x3, const TcArgs &a, int cg, int nh, int64_t tiles, cudaStream_t st) {
+    const unsigned blocks = (unsigned)(tiles * cg * nh * TM * 4 / 8);
+    LaunchScope ls(x3 ? (mode == 1 ? IQP_KERNEL_RECOMPUTE_FP32 : IQP_KERNEL_PHASE_FP32)
+                      : (mode == 1 ? IQP_KERNEL_RECOMPUTE_TC : IQP_KERNEL_PHASE_TC),
+                   st);
+    if (x3) {
+        if (mode == 0) k_split_reduce<0, true><<<blocks, 256, 0, st>>>(a, cg, nh, tiles);
+        else if (mode == 1) k_split_reduce<1, true><<<blocks, 256, 0, st>>>(a, cg, nh, tiles);
+        else k_split_reduce<2, true><<<blocks, 256, 0, st>>>(a, cg, nh, tiles);
+    } else {
+        if (mode == 0) k_split_reduce<0, false><<<blocks, 256, 0, st>>>(a, cg, nh, tiles);
+        else if (mode == 1) k_split_reduce<1, false><<<blocks, 256, 0, st>>>(a, cg, nh, tiles);
+        else k_split_reduce<2, false><<<blocks, 256, 0, st>>>(a, cg, nh, tiles);
+    }
+    return cudaGetLastError();
+}
+
+// The T single tiles of a phase: full rounds of whole tiles, then the last
+// round's tiles as a balanced split where that pays (skp: its scratch, or null).
+cudaError_t launch_single_tiles(int mode, int cg, bool x3, const CUtensorMap &ma, const CUtensorMap &mb, TcArgs a,
+                                int64_t T, float *skp, int64_t slots, cudaStream_t st) {
+    int sms = num_sms();
+    if (sms > kMaxSplitCtas) sms = kMaxSplitCtas;
+    const int64_t P = sms / cg;  // CTA groups
     auto run = [&](bool split, const TcArgs &w) {
         if (x3) return split ? launch_phase_x3_k<true>(mode, ma, mb, w, st) : launch_phase_x3_k<false>(mode, ma, mb, w, st);
         return split ? launch_phase_k<true>(mode, cg, ma, mb, w, st) : launch_phase_k<false>(mode, cg, ma, mb, w, st);
     };
-    if (R == 0) return run(false, a);
+    const int64_t R = P >= 1 ? T % P : 0;
+    TcArgs b = a;
+    whole_tiles(a, T);
+    if (!balance(b, T - R, R, P, cg, 1, skp, slots)) return run(false, a);
     if (T - R > 0) {
-        TcArgs w = a;
-        whole_tiles(w, T - R);
-        const cudaError_t e = run(false, w);
+        whole_tiles(a, T - R);
+        const cudaError_t e = run(false, a);
         if (e != cudaSuccess) return e;
     }
-    a.whole = T - R;
-    a.nsplit = (int)ns;
-    a.nunits = R * ns;
-    a.skp = skp;
-    a.skc = reinterpret_cast<int *>(a.skp + (int64_t)kMaxSplitCtas * kSplitSlotFloats);
-    a.skcap = (int64_t)kMaxSplitCtas * kSplitSlotFloats;
-    const cudaError_t e = cudaMemsetAsync(a.skc, 0, (size_t)(R * cg) * sizeof(int), st);
-    if (e != cudaSuccess) return e;
-    return run(true, a);
+    const cudaError_t e = run(true, b);
+    return e != cudaSuccess ? e : launch_split_reduce(mode, x3, b, cg, 1, R, st);
 }
 }  // namespace
 
@@ -2273,51 +2311,42 @@ cudaError_t launch_phase_tc(int mode, const Plan &p, void *ws, const double *alp
         const int64_t P = sms / 2;  // CTA pairs
         const int64_t tiles_n2 = cdiv(p.s, 2 * TN);
         const int64_t T2 = a.tiles_m * tiles_n2;
-        if (cg == 2 && phase_dt() && p.off_gsum != 0 && num_sms() <= kMaxSplitCtas && P >= 1 && T2 >= P) {
-            const int64_t full = (T2 / P) * P;
+        if (cg == 2 && phase_dt() && p.off_gsum != 0 && num_sms() <= kMaxSplitCtas && P >= 1) {
+            const int64_t full = (T2 / P) * P, left = T2 - full;
             TcArgs d = a;
             d.tiles_n = tiles_n2;
-            whole_tiles(d, full);
             d.gsum = at<float4>(ws, p.off_gsum);
-            const cudaError_t e = launch_phase_dt_k<false>(mode, ma, mb, d, st);
-            if (e != cudaSuccess) return e;
-            if (full == T2) return cudaSuccess;
-            // The last round, balanced: its double tiles' bits stages, end to
-            // end, in P equal ranges, one per CTA pair (pieces of at most two
-            // or three tiles each; see unit_of).
-            const int64_t left = T2 - full;
-            const int64_t nkb = cdiv(a.nks, KB / KS);
-            const int64_t W = left * nkb;
-            if (split_tail() && p.off_skx != 0 && W >= P && left * 2 <= kMaxSplitCtas) {
-                int64_t KP = 1;
-                for (int64_t t = 0; t < left; ++t) {
-                    const int64_t g0 = ((t * nkb + 1) * P - 1) / W, g1 = ((t + 1) * nkb * P - 1) / W;
-                    if (g1 - g0 + 1 > KP) KP = g1 - g0 + 1;
-                }
-                if (left * KP * 2 * 2 <= kSplitSlots) {
-                    TcArgs e2 = d;
-                    e2.whole = full;
-                    e2.nsplit = 1;
-                    e2.nunits = P * (cdiv(W / P + 1, nkb) + 2);
-                    e2.sk = 1;
-                    e2.skW = W;
-                    e2.skP = P;
-                    e2.skKP = KP;
-                    e2.skp = at<float>(ws, p.off_skx);
-                    e2.skc = reinterpret_cast<int *>(e2.skp + (int64_t)kSplitSlots * kSplitSlotFloats);
-                    e2.skcap = (int64_t)kSplitSlots * kSplitSlotFloats;
-                    const cudaError_t e3 = cudaMemsetAsync(e2.skc, 0, (size_t)(left * 2) * sizeof(int), st);
-                    if (e3 != cudaSuccess) return e3;
-                    return launch_phase_dt_k<true>(mode, ma, mb, e2, st);
-                }
+            TcArgs b = d;
+            bool bal = left > 0 && p.off_skx != 0 && balance(b, full, left, P, 2, 2, at<float>(ws, p.off_skx), kSplitSlots, full > 0);
+            if (bal && full == 0) {  // less than a round: against single tiles, whole or split
+                const double k = (double)cdiv(a.nks, KB / KS) * kStageUs, w = k * (double)cdiv(T, P);
+                const double sp = k * (double)T / (double)P + kSplitUs;
+                bal = (double)left / (double)P * (double)cdiv(a.nks, KB / KS) * kStageDtUs + kSplitDtUs < (w < sp ? w : sp);
             }
-            a.dtmap = 1;
-            a.dbase = full;
-            a.tiles_n2 = tiles_n2;
-            T = 2 * (T2 - full);
+            if (full > 0 || bal) {
+                if (full > 0) {
+                    whole_tiles(d, full);
+                    const cudaError_t e = launch_phase_dt_k<false>(mode, ma, mb, d, st);
+                    if (e != cudaSuccess || left == 0) return e;
+                }
+                if (bal) {
+                    const cudaError_t e = launch_phase_dt_k<true>(mode, ma, mb, b, st);
+                    return e != cudaSuccess ? e : launch_split_reduce(mode, false, b, 2, 2, left, st);
+                }
+                a.dtmap = 1;
+                a.dbase = full;
+                a.tiles_n2 = tiles_n2;
+                T = 2 * left;
+            }
         }
     }
-    return launch_single_tiles(mode, cg, false, ma, mb, a, T, p.off_skp != 0 ? at<float>(ws, p.off_skp) : nullptr, st);
+    float *skp = p.off_skp != 0 ? at<float>(ws, p.off_skp) : nullptr;
+    int64_t slots = kMaxSplitCtas;
+    if (p.off_skx != 0) {
+        skp = at<float>(ws, p.off_skx);
+        slots = kSplitSlots;
+    }
+    return launch_single_tiles(mode, cg, false, ma, mb, a, T, skp, slots, st);
 }
 
 // The FP32 form's phase (p.x3): the same contraction with 2 theta as three
@@ -2359,7 +2388,7 @@ cudaError_t launch_phase_x3(int mode, const Plan &p, void *ws, const double *alp
     a.limit_ns = default_spin_limit_ns();
     a.serp = phase_serp() ? 1 : 0;
     a.gsum = at<float4>(ws, p.off_xsum);
-    return launch_single_tiles(mode, 2, true, ma, mb, a, a.tiles_m * a.tiles_n, at<float>(ws, p.off_skp), st);
+    return launch_single_tiles(mode, 2, true, ma, mb, a, a.tiles_m * a.tiles_n, at<float>(ws, p.off_skp), kMaxSplitCtas, st);
 }
 
 cudaError_t launch_x3_theta(const Plan &p, void *ws, const float *theta, cudaStream_t st) {
