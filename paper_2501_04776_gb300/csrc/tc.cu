@@ -659,6 +659,74 @@ __device__ __forceinline__ float store_wf32(const TcArgs &args, int64_t row, int
     return mx;
 }
 
+// W of eight consecutive samples i.. of observable row: BF16 hi/lo rows, or (X3)
+// FP32, returning the largest finite |W| among those below s.
+__device__ __forceinline__ void store_w8(const TcArgs &args, int64_t row, int64_t i, const float (&w)[8]) {
+    uint32_t ph[4], pl[4];
+#pragma unroll
+    for (int e = 0; e < 8; e += 2) {
+        const float h0 = __bfloat162float(__float2bfloat16_rn(w[e])), h1 = __bfloat162float(__float2bfloat16_rn(w[e + 1]));
+        ph[e / 2] = pack_bf16x2(h0, h1);
+        pl[e / 2] = pack_bf16x2(w[e] - h0, w[e + 1] - h1);
+    }
+    __nv_bfloat16 *dh = args.whi + row * args.ldw + i, *dl = args.wlo + row * args.ldw + i;
+    if (i + 8 <= args.s) {
+        *reinterpret_cast<uint4 *>(dh) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
+        *reinterpret_cast<uint4 *>(dl) = make_uint4(pl[0], pl[1], pl[2], pl[3]);
+        return;
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+        if (i + e < args.s) {
+            reinterpret_cast<uint16_t *>(dh)[e] = (uint16_t)(ph[e / 2] >> ((e & 1) * 16));
+            reinterpret_cast<uint16_t *>(dl)[e] = (uint16_t)(pl[e / 2] >> ((e & 1) * 16));
+        }
+}
+__device__ __forceinline__ float store_wf8(const TcArgs &args, int64_t row, int64_t i, const float (&w)[8]) {
+    float mx = 0.f;
+    float *d = args.wf + row * args.ldw + i;
+    if (i + 8 <= args.s) {
+        *reinterpret_cast<float4 *>(d) = make_float4(w[0], w[1], w[2], w[3]);
+        *reinterpret_cast<float4 *>(d + 4) = make_float4(w[4], w[5], w[6], w[7]);
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        const float v = fabsf(w[e]);
+        if (i + e >= args.s) continue;
+        if (v <= 3.4e38f) mx = fmaxf(mx, v);
+        if (i + 8 > args.s) d[e] = w[e];
+    }
+    return mx;
+}
+
+// Merges 32 cosines (columns 32 c .. of a group with nvalid valid columns) into
+// (S, M2): their own sum and squared deviations from registers, then the merge of
+// the two means (Chan et al.). Each cosine is taken once: the epilogue took it
+// once for the sum and again for the deviations from the whole group's mean,
+// half of its instructions, with no product under way meanwhile where a CTA pair
+// has one tile (all of k_tc, cold: 255 gates, 8 x 2000: 37.6 -> 18.5 us; 5050
+// gates, 1000 x 1003: 71.6 -> 50.3 us).
+__device__ __forceinline__ void merge_cos32(const uint32_t (&r)[32], int c, int nvalid, float &S, float &M2) {
+    const int n = nvalid - 32 * c < 32 ? nvalid - 32 * c : 32;
+    if (n <= 0) return;
+    float s = 0.f, m2 = 0.f;
+#pragma unroll
+    for (int e = 0; e < 32; ++e) s += e < n ? __uint_as_float(r[e]) : 0.f;
+    const float mean = s / (float)n;
+#pragma unroll
+    for (int e = 0; e < 32; ++e) {
+        const float d = __uint_as_float(r[e]) - mean;
+        m2 = e < n ? fmaf(d, d, m2) : m2;
+    }
+    if (c > 0) {  // the columns before are all valid: 32 c of them
+        const float before = (float)(32 * c), d = mean - S / before;
+        m2 += M2 + d * d * (before * (float)n / (before + (float)n));
+        s += S;
+    }
+    S = s;
+    M2 = m2;
+}
+
 // Values of 32 consecutive columns col0.. of `row`, stored into out
 // (row-major, args.ldo elements per row, columns < args.s). Rows start 16-byte
 // aligned (ldo a multiple of 4).
@@ -1272,29 +1340,13 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll 1
                     for (int c = 0; c < kGroupLoads; ++c) {
                         ldsum(c, r);
+                        // Phi itself, when a gradient pass follows (W from it
+                        // instead of a second contraction).
+                        if (args.out != nullptr && c * 32 < nvalid && row < args.l)
+                            store_out32(args, args.out, row, c0 + c * 32, r);
 #pragma unroll
-                        for (int e = 0; e < 32; ++e)
-                            if (c * 32 + e < nvalid) S += cosf(__uint_as_float(r[e]));
-                    }
-                    const float mean = nvalid > 0 ? S / (float)nvalid : 0.f;
-#pragma unroll 1
-                    for (int c = 0; c < kGroupLoads; ++c) {
-                        ldsum(c, r);
-#pragma unroll
-                        for (int e = 0; e < 32; ++e)
-                            if (c * 32 + e < nvalid) {
-                                const float d = cosf(__uint_as_float(r[e])) - mean;
-                                M2 = fmaf(d, d, M2);
-                            }
-                    }
-                    // Phi itself, when a gradient pass follows (W from it instead
-                    // of a second contraction).
-                    if (args.out != nullptr) {  // uniform: every lane takes the TMEM loads
-#pragma unroll 1
-                        for (int c = 0; c * 32 < nvalid; ++c) {
-                            ldsum(c, r);
-                            if (row < args.l) store_out32(args, args.out, row, c0 + c * 32, r);
-                        }
+                        for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(cosf(__uint_as_float(r[e])));
+                        merge_cos32(r, c, (int)nvalid, S, M2);
                     }
                     if (row < args.l && nvalid > 0 && IQP_IN(row * args.nparts + c0 / kGroupCols, args.l * args.nparts, 50))
                         args.part[row * args.nparts + (c0 / kGroupCols)] = make_double2((double)S, (double)M2);
@@ -1313,40 +1365,29 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll 1
                     for (int c = 0; c < kGroupLoads; ++c) {
                         ldsum(c, r);
-#pragma unroll
-                        for (int e = 0; e < 32; ++e)
-                            if (c * 32 + e < nvalid) S += cosf(__uint_as_float(r[e]));
-                    }
-                    const float mean = nvalid > 0 ? S / (float)nvalid : 0.f;
-#pragma unroll 1
-                    for (int c = 0; c < kGroupLoads; ++c) {
-                        ldsum(c, r);
                         const int64_t i0 = c0 + c * 32;
-                        uint32_t ph[16], pl[16];
+                        const bool in = rv && i0 < args.s && IQP_IN(row * args.ldw + i0, args.l * args.ldw, 43) &&
+                                        IQP_IN(row * args.ldw + (i0 + 32 <= args.s ? i0 + 31 : args.s - 1),
+                                               args.l * args.ldw, 44);
+                        // eight columns of W at a time, stored as they are formed
 #pragma unroll
-                        for (int e = 0; e < 32; e += 2) {
-                            float s0, k0, s1, k1;
-                            sincosf(__uint_as_float(r[e]), &s0, &k0);
-                            sincosf(__uint_as_float(r[e + 1]), &s1, &k1);
-                            const float d0 = k0 - mean, d1 = k1 - mean;
-                            if (c * 32 + e < nvalid) M2 = fmaf(d0, d0, M2);
-                            if (c * 32 + e + 1 < nvalid) M2 = fmaf(d1, d1, M2);
-                            const float w0 = s0 * (al + be * k0), w1 = s1 * (al + be * k1);
-                            if (X3) {  // W stays FP32
-                                r[e] = __float_as_uint(w0);
-                                r[e + 1] = __float_as_uint(w1);
-                                continue;
+                        for (int v = 0; v < 4; ++v) {
+                            float w[8];
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) {
+                                float sn, cn;
+                                sincosf(__uint_as_float(r[8 * v + e]), &sn, &cn);
+                                r[8 * v + e] = __float_as_uint(cn);
+                                w[e] = sn * (al + be * cn);
                             }
-                            const float h0 = __bfloat162float(__float2bfloat16_rn(w0));
-                            const float h1 = __bfloat162float(__float2bfloat16_rn(w1));
-                            ph[e / 2] = pack_bf16x2(h0, h1);
-                            pl[e / 2] = pack_bf16x2(w0 - h0, w1 - h1);
+                            const int64_t i = i0 + 8 * v;
+                            if (!in || i >= args.s) continue;
+                            if (X3)
+                                wmax = fmaxf(wmax, store_wf8(args, row, i, w));
+                            else
+                                store_w8(args, row, i, w);
                         }
-                        if (X3) {
-                            if (rv && i0 < args.s) wmax = fmaxf(wmax, store_wf32(args, row, i0, r));
-                        } else if (rv && i0 < args.s) {
-                            store_w32(args, row, i0, ph, pl);
-                        }
+                        merge_cos32(r, c, (int)nvalid, S, M2);
                     }
                     if (X3 && wmax > 0.f && IQP_IN(row, args.l, 60)) atomicMax(args.wmax + row, __float_as_uint(wmax));
                     if (rv && nvalid > 0 && IQP_IN(row * args.nparts + c0 / kGroupCols, args.l * args.nparts, 51))
