@@ -18,7 +18,8 @@
 // value per lane; each lane transposes the gates' five words into a 5-bit
 // index per sample and takes that sample's combination with one shuffle and
 // one add, about 30 instructions per gate and word against 160 per gate and
-// two words for a sign flip and an add per term.
+// two words for a sign flip and an add per term. Two batches are added to a pair
+// of samples by one packed FP32 add (3.14 -> 2.81 ms of the loss below).
 // The warps' partial phases are added in shared memory in a fixed order.
 //
 // Gradient: W of the range is tabulated, once per CTA, as the signed sums of
@@ -28,7 +29,7 @@
 // lanes' sums of 32 gates are combined by one reduce-scatter.
 //
 // Measured, MMD loss and gradient of the n = 1000 one- and two-body circuit
-// (500500 gates, 2000 observables, 5000 samples): 18.9 -> 5.9 ms (8.6 with the
+// (500500 gates, 2000 observables, 5000 samples): 18.9 -> 5.6 ms (8.6 with the
 // parity words loaded into registers and the list made again for every range);
 // independent batches (n = 200, 5000 gates, 256 x 2000 samples), forward and
 // backward: 1.43 -> 0.51 ms.
@@ -114,7 +115,7 @@ constexpr int kPartBytes = kWarps * kRange * 4, kTabBytes = 4 * 256 * 32 * 4;
 // them for most of its time.
 constexpr int kRing = 3, kPhaseStage = 20, kGradStage = 8;
 constexpr int kPhaseRing = kRing * kPhaseStage * 32, kGradRing = kRing * kGradStage * 32;  // words per warp
-static_assert(kWarps * kPhaseRing * 4 <= kTabBytes && kPartBytes <= kTabBytes, "the tables' place");
+static_assert(kPhaseStage % 10 == 0 && kWarps * kPhaseRing * 4 <= kTabBytes && kPartBytes <= kTabBytes, "the tables' place");
 // bytes of the tables' place, and in all (independent batches stage nothing)
 __host__ __device__ constexpr int tab_bytes(bool grad, bool indep) { return grad || !indep ? kTabBytes : kPartBytes; }
 constexpr int smem_bytes(bool grad, bool indep) {
@@ -324,35 +325,61 @@ __device__ __forceinline__ void fetch_stage(uint32_t *dst, const int2 *list, int
     copy_commit();
 }
 
+// Two FP32 adds in one instruction, each rounded to nearest like a scalar add.
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, float lo, float hi) {
+    uint64_t b, d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(b) : "f"(lo), "f"(hi));
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
 // phase_list for shared batches: this warp's share of the list is a run of
-// gates, its words staged in `ring`. pzt: P_Z^T at this range's words.
-__device__ __forceinline__ void phase_list_staged(float (&acc)[32], const int2 *list, int n, const uint32_t *pzt,
+// gates, its words staged in `ring`. pzt: P_Z^T at this range's words. acc: pair
+// t holds samples 2 t and 2 t + 1 of the lane. Two batches of five at a time, so
+// that one's index and shuffle latencies lie behind the other's.
+__device__ __forceinline__ void phase_list_staged(uint64_t (&acc)[16], const int2 *list, int n, const uint32_t *pzt,
                                                   int64_t ldzt, int nch, int64_t m, uint32_t *ring, int warp, int lane) {
     const int per = 5 * ((n + 5 * kWarps - 1) / (5 * kWarps));
     const int b0 = warp * per, end = b0 + per < n ? b0 + per : n;
+    uint32_t sign[5];
+#pragma unroll
+    for (int g = 0; g < 5; ++g) sign[g] = (uint32_t)((lane >> g) & 1) << 31;
 #pragma unroll
     for (int k = 0; k < kRing - 1; ++k)
         fetch_stage<kPhaseStage>(ring + k * kPhaseStage * 32, list, b0 + k * kPhaseStage, end, pzt, ldzt, nch, m, lane);
+    // a batch's five words and this lane's sign combination of its c_j; gates past the end count as c = 0
+    auto load = [&](const uint32_t *zw, const int2 *lp, int left, uint32_t (&z)[5]) {
+        float t = 0.f;
+#pragma unroll
+        for (int g = 0; g < 5; ++g) {
+            z[g] = zw[g * 32];
+            const uint32_t cb = g < left ? (uint32_t)lp[g].y : 0u;
+            t += __uint_as_float(cb ^ sign[g]);
+        }
+        return t;
+    };
     int st = 0;
     for (int e0 = b0; e0 < end; e0 += kPhaseStage) {
         copy_wait();
         __syncwarp();
         const uint32_t *zw = ring + st * kPhaseStage * 32 + lane;
 #pragma unroll 1
-        for (int h = 0; h < kPhaseStage && e0 + h < end; h += 5) {
-            uint32_t z[5], R[8];
-            float t = 0.f;
+        for (int h = 0; h < kPhaseStage && e0 + h < end; h += 10) {
+            uint32_t z0[5], z1[5], R0[8], R1[8];
+            const float t0 = load(zw + h * 32, list + e0 + h, end - e0 - h, z0);
+            const float t1 = load(zw + (h + 5) * 32, list + e0 + h + 5, end - e0 - h - 5, z1);
+            indices5(z0, R0);
+            indices5(z1, R1);
 #pragma unroll
-            for (int g = 0; g < 5; ++g) {
-                z[g] = zw[(h + g) * 32];
-                const float cv = e0 + h + g < end ? __int_as_float(list[e0 + h + g].y) : 0.f;  // a short batch: c = 0
-                t += ((lane >> g) & 1) ? -cv : cv;
-            }
-            indices5(z, R);
+            for (int q = 0; q < 8; q += 2)
 #pragma unroll
-            for (int q = 0; q < 8; ++q)
-#pragma unroll
-                for (int k = 0; k < 4; ++k) acc[8 * k + q] += __shfl_sync(kFull, t, (int)(R[q] >> (8 * k)));
+                for (int k = 0; k < 4; ++k) {
+                    const float a0 = __shfl_sync(kFull, t0, (int)(R0[q] >> (8 * k)));
+                    const float a1 = __shfl_sync(kFull, t0, (int)(R0[q + 1] >> (8 * k)));
+                    const float c0 = __shfl_sync(kFull, t1, (int)(R1[q] >> (8 * k)));
+                    const float c1 = __shfl_sync(kFull, t1, (int)(R1[q + 1] >> (8 * k)));
+                    acc[4 * k + q / 2] = add_f32x2(add_f32x2(acc[4 * k + q / 2], a0, a1), c0, c1);
+                }
         }
         __syncwarp();  // every lane has read the stage that comes free
         const int nx = st == 0 ? kRing - 1 : st - 1;
@@ -402,7 +429,8 @@ __device__ __forceinline__ void grad_list_staged(const int2 *list, int n, const 
 }
 
 // Sum of v over the CTA: shuffles in FP32 within a warp, the warps' sums in
-// FP64 in a fixed order. Every thread calls it and gets the sum.
+// FP64 in a fixed order, by warp 0 alone (16 FP64 adds by every warp took a
+// tenth of the statistics pass). Every thread calls it; warp 0 gets the sum.
 __device__ __forceinline__ double block_sum(float v, float *red) {
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) v += __shfl_xor_sync(kFull, v, off);
@@ -410,8 +438,10 @@ __device__ __forceinline__ double block_sum(float v, float *red) {
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
     double t = 0.0;
+    if (threadIdx.x < 32) {
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) t += (double)red[w];
+        for (int w = 0; w < kWarps; ++w) t += (double)red[w];
+    }
     return t;
 }
 
@@ -468,13 +498,16 @@ __global__ void __launch_bounds__(kThreads, MODE == 0 && INDEP ? 2 : 1)
         }
     } else {
         float acc[32];
+        uint64_t acc2[16];
 #pragma unroll
         for (int k = 0; k < 32; ++k) acc[k] = 0.f;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) acc2[k] = 0ull;
         auto phase = [&](int cnt) {
             if constexpr (INDEP)
                 phase_list<true>(acc, list, cnt, zs, warp, lane);
             else
-                phase_list_staged(acc, list, cnt, pzt, 2 * ldzt, nch, m, reinterpret_cast<uint32_t *>(tab) + warp * kPhaseRing,
+                phase_list_staged(acc2, list, cnt, pzt, 2 * ldzt, nch, m, reinterpret_cast<uint32_t *>(tab) + warp * kPhaseRing,
                                   warp, lane);
         };
         if (held >= 0) {
@@ -492,6 +525,13 @@ __global__ void __launch_bounds__(kThreads, MODE == 0 && INDEP ? 2 : 1)
             }
         }
         __syncthreads();  // the partial phases lie where other warps' rings were
+        if constexpr (!INDEP) {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                acc[2 * k] = __uint_as_float((uint32_t)acc2[k]);
+                acc[2 * k + 1] = __uint_as_float((uint32_t)(acc2[k] >> 32));
+            }
+        }
 #pragma unroll
         for (int k = 0; k < 32; ++k) tab[warp * kRange + k * 32 + lane] = acc[k];
         __syncthreads();
@@ -516,15 +556,18 @@ __global__ void __launch_bounds__(kThreads, MODE == 0 && INDEP ? 2 : 1)
         float cv[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) cv[h] = valid[h] ? cosf(ph[h]) : 0.f;
-        const double S = block_sum(cv[0] + cv[1], reinterpret_cast<float *>(red));
-        const float mean = (float)(S / (double)(left < kRange ? left : kRange));
+        float *redf = reinterpret_cast<float *>(red);
+        const double S = block_sum(cv[0] + cv[1], redf);
+        if (tid == 0) redf[kWarps] = (float)(S / (double)(left < kRange ? left : kRange));
+        __syncthreads();
+        const float mean = redf[kWarps];
         float m2 = 0.f;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const float d = cv[h] - mean;
             m2 += valid[h] ? d * d : 0.f;
         }
-        const double M2 = block_sum(m2, reinterpret_cast<float *>(red));
+        const double M2 = block_sum(m2, redf);
         if (tid == 0 && IQP_IN(a * nparts + r, l * nparts, 75)) part[a * nparts + r] = make_double2(S, M2);
     }
     if (MODE != 0) {
