@@ -96,6 +96,11 @@ cudaError_t launch_bitflip_rows(const uint64_t *PA, int64_t ldp, int64_t l, cons
                                 cudaStream_t st);
 cudaError_t launch_bitflip_grad(const uint64_t *PAT, int64_t ldlt, int64_t m, int64_t l, const double *w,
                                 const double *ev, double *v, const double *t, double *grad, cudaStream_t st);
+bool bitflip_ints(int64_t m, int64_t l);
+int64_t bitflip_int_words(int64_t m, int64_t l);
+cudaError_t launch_bitflip_ints(const uint64_t *PA, int64_t ldp, const uint64_t *PAT, int64_t ldlt, int64_t m, int64_t l,
+                                const float *theta, double *c, double *t, int64_t mpad, double *expval, const double *w,
+                                double *v, double *grad, double *s, cudaStream_t st);
 
 // ---------------------------------------------------------------- plan
 
@@ -213,6 +218,13 @@ Plan make_plan(int op, int64_t n, int64_t m, int64_t l, int64_t s, int64_t N, in
         p.off_lo_p = take(l * kLoP * 8);
         p.off_lo_cnt = take(2 * l * 4);
         p.off_lo_hp = take(grad ? n * p.ldc * 4 * lo_hparts(n, s) : 0);
+    }
+    // Bitflip: scratch of the integer sums (a workspace that ends before its
+    // end takes the FP64 kernels).
+    p.off_bf = 0;
+    if (bitflip && bitflip_ints(m, l)) {
+        p.off_opt = off;
+        p.off_bf = take(8 * bitflip_int_words(m, l));
     }
     // MMD: scratch of the data parities by row gather (a workspace that ends
     // before its end folds them densely).
@@ -353,6 +365,7 @@ iqp_status check_ws(Plan &p, void *ws, size_t ws_bytes) {
         if (ws_bytes < plan_min_bytes(p)) return IQP_ERR_WORKSPACE;
         p.x3 = false;  // FP32: the SIMT kernels
         p.off_xt = 0;  // data parities folded densely
+        p.off_bf = 0;
         p.off_lo_zp = p.off_lo_hp = 0;  // low-order: no lists, H in one piece
         // The optional regions at the end, in order: each is used only where
         // the workspace reaches its end.
@@ -952,11 +965,17 @@ iqp_status bitflip_core(int64_t n, const uint64_t *G, int64_t m, int64_t ldg, co
     Plan p = make_plan(IQP_OP_BITFLIP, n, m, l, 1, 0, IQP_FP32);
     if ((rc = check_ws(p, ws, ws_bytes)) != IQP_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    IQP_TRY(launch_support_list(G, m, ldg, n, at<int4>(ws, p.off_sup), st));
-    IQP_TRY(launch_parity_gather(n, A, l, lda, G, m, ldg, at<uint64_t>(ws, p.off_pa), p.ldp,
-                                 at<uint64_t>(ws, p.off_pat), p.ldlt, at<uint64_t>(ws, p.off_rt), st,
-                                 at<int4>(ws, p.off_sup)));
+    const ParitySide side{A, l, lda, at<uint64_t>(ws, p.off_pa), at<uint64_t>(ws, p.off_pat), p.ldlt,
+                          at<uint64_t>(ws, p.off_rt)};
+    IQP_TRY(launch_parity_gather_fused(n, G, m, ldg, at<int4>(ws, p.off_sup), true, p.ldp, &side, 1, st));
     double *c = at<double>(ws, p.off_c), *t = c + p.mpad;
+    if (p.off_bf != 0) {
+        double *part = at<double>(ws, p.off_part);
+        IQP_TRY(launch_bitflip_ints(at<uint64_t>(ws, p.off_pa), p.ldp, at<uint64_t>(ws, p.off_pat), p.ldlt, m, l, theta, c,
+                                    t, p.mpad, expval ? expval : part, grad ? w : nullptr, part + l, grad,
+                                    at<double>(ws, p.off_bf), st));
+        return IQP_OK;
+    }
     IQP_TRY(launch_bitflip_gates(theta, m, p.mpad, c, t, st));
     double *ev = expval ? expval : at<double>(ws, p.off_part);
     IQP_TRY(launch_bitflip_rows(at<uint64_t>(ws, p.off_pa), p.ldp, l, c, ev, st));
