@@ -447,15 +447,16 @@ iqp_status prepare(const Plan &p, void *ws, const uint64_t *G, int64_t ldg, cons
         const ParitySide sides[2] = {
             {A, p.l, lda, at<uint64_t>(ws, p.off_pa), at<uint64_t>(ws, p.off_pat), p.ldlt, rt},
             {Z, p.s, ldz, at<uint64_t>(ws, p.off_pz), at<uint64_t>(ws, p.off_pzt), p.ldzt, rt + p.n * p.ldlt}};
-        IQP_TRY(launch_parity_gather_fused(p.n, G, p.m, ldg, at<int4>(ws, p.off_sup), true, p.ldp, sides, 2, st));
+        ThetaJob tj{theta, p.m, p.mpad, nullptr, nullptr, nullptr};
         if (p.prec == IQP_SPLIT_BF16) {
-            __nv_bfloat16 *hi = at<__nv_bfloat16>(ws, p.off_c);
-            IQP_TRY(launch_theta_prep(theta, p.m, p.mpad, nullptr, hi, hi + p.mpad, st));
-        } else if (p.x3) {
-            IQP_TRY(launch_x3_theta(p, ws, theta, st));
+            tj.hi = at<__nv_bfloat16>(ws, p.off_c);
+            tj.lo = tj.hi + p.mpad;
         } else {
-            IQP_TRY(launch_theta_prep(theta, p.m, p.mpad, at<float>(ws, p.off_c), nullptr, nullptr, st));
+            tj.c32 = at<float>(ws, p.off_c);
         }
+        if (p.x3) tj.theta = nullptr;  // the planes are formed by their own kernels
+        IQP_TRY(launch_parity_gather_fused(p.n, G, p.m, ldg, at<int4>(ws, p.off_sup), true, p.ldp, sides, 2, st, tj));
+        if (p.x3) IQP_TRY(launch_x3_theta(p, ws, theta, st));
         return IQP_OK;
     }
     IQP_TRY(launch_support_list(G, p.m, ldg, p.n, at<int4>(ws, p.off_sup), st));

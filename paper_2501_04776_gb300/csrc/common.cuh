@@ -234,6 +234,21 @@ static inline uint32_t take_check_word() {
 static inline uint32_t take_check_word() { return 0u; }
 #endif
 
+// c_j = 2 theta_j (exact in FP32); hi = RN_bf16(c), lo = RN_bf16(c - hi)
+// (c - hi is exact in FP32). Zero beyond m, up to mpad.
+__device__ __forceinline__ void theta_prep_one(const float *__restrict__ theta, int64_t j, int64_t m,
+                                               [[maybe_unused]] int64_t mpad, float *__restrict__ c32,
+                                               __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo) {
+    const float c = j < m ? 2.0f * theta[j] : 0.0f;
+    if (!IQP_IN(j, mpad, 20)) return;
+    if (c32) c32[j] = c;
+    if (hi) {
+        const __nv_bfloat16 h = __float2bfloat16_rn(c);
+        hi[j] = h;
+        lo[j] = __float2bfloat16_rn(c - __bfloat162float(h));
+    }
+}
+
 // Host-side launch accounting (iqp_launch_count) and optional per-kernel
 // event timing (iqp_profile_*). Construct one right before each launch.
 struct LaunchScope {

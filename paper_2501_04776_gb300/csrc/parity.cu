@@ -346,9 +346,17 @@ struct SupportJob {
     int4 *sup;
 };
 constexpr int kSlGates = 256;  // gates per support-list block of k_parity_prep
-__global__ void __launch_bounds__(kTT) k_parity_prep(BitTransposeJob a, BitTransposeJob b, SupportJob g) {
+// The last tblocks blocks prepare theta (a launch of its own cost every call 2.4
+// us on the GPU and a few on the host).
+__global__ void __launch_bounds__(kTT) k_parity_prep(BitTransposeJob a, BitTransposeJob b, SupportJob g, ThetaJob t,
+                                                     int64_t tblocks) {
     __shared__ __align__(16) uint32_t tin[kTT][kTW + 1];  // transposed in place
     const int64_t bid = blockIdx.x;
+    if (bid >= (int64_t)gridDim.x - tblocks) {
+        for (int64_t j = (bid - ((int64_t)gridDim.x - tblocks)) * kTT + threadIdx.x; j < t.mpad; j += tblocks * kTT)
+            theta_prep_one(t.theta, j, t.m, t.mpad, t.c32, t.hi, t.lo);
+        return;
+    }
     if (bid >= a.tiles + b.tiles) {
         // 256 gates: their rows (at most 16 words) staged in tin with coalesced loads, all in flight
         // together (row r at 17 r), then one thread scans each row there
@@ -812,7 +820,7 @@ cudaError_t launch_gather_transpose(bool i32, int64_t gx, const int4 *sup, const
 
 cudaError_t launch_parity_gather_fused(int64_t n, const uint64_t *G, int64_t m, int64_t ldg, int4 *sup,
                                        bool form_sup, int64_t ldp, const ParitySide *side, int nside,
-                                       cudaStream_t st) {
+                                       cudaStream_t st, const ThetaJob &theta) {
     if (nside < 1 || nside > 2 || ldp % 2 != 0) return cudaErrorInvalidValue;
     // the support list in the preparation launch where its rows are short, else on its own first
     const bool sup_in_prep = form_sup && cdiv(n, 64) <= 16;
@@ -828,11 +836,13 @@ cudaError_t launch_parity_gather_fused(int64_t n, const uint64_t *G, int64_t m, 
         bt[k].tiles = bt[k].gx * cdiv(n, kTT);
     }
     const int64_t sl_blocks = sup_in_prep ? cdiv(m, kSlGates) : 0;
-    if (bt[0].tiles + bt[1].tiles + sl_blocks > 0x7FFFFFFFll) return cudaErrorInvalidValue;
+    int64_t tblocks = theta.theta != nullptr ? cdiv(theta.mpad, kTT) : 0;
+    if (tblocks > 1024) tblocks = 1024;
+    if (bt[0].tiles + bt[1].tiles + sl_blocks + tblocks > 0x7FFFFFFFll) return cudaErrorInvalidValue;
     {
         LaunchScope ls(IQP_KERNEL_PARITY, st);
-        k_parity_prep<<<(unsigned)(bt[0].tiles + bt[1].tiles + sl_blocks), kTT, 0, st>>>(
-            bt[0], bt[1], SupportJob{G, m, ldg, n, sup});
+        k_parity_prep<<<(unsigned)(bt[0].tiles + bt[1].tiles + sl_blocks + tblocks), kTT, 0, st>>>(
+            bt[0], bt[1], SupportJob{G, m, ldg, n, sup}, theta, tblocks);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }

@@ -20,20 +20,11 @@ constexpr int BM = 128, BN = 128, BK = 32, PADF = 4;
 
 // ------------------------------------------------------------ theta split
 
-// c_j = 2 theta_j (exact in FP32); hi = RN_bf16(c), lo = RN_bf16(c - hi)
-// (c - hi is exact in FP32). Zero beyond m, up to mpad.
+// c_j, hi_j and lo_j of theta_prep_one for every j < mpad.
 __global__ void k_theta_prep(const float *__restrict__ theta, int64_t m, int64_t mpad, float *__restrict__ c32,
                              __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo) {
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < mpad; j += (int64_t)gridDim.x * blockDim.x) {
-        const float c = j < m ? 2.0f * theta[j] : 0.0f;
-        if (!IQP_IN(j, mpad, 20)) continue;
-        if (c32) c32[j] = c;
-        if (hi) {
-            const __nv_bfloat16 h = __float2bfloat16_rn(c);
-            hi[j] = h;
-            lo[j] = __float2bfloat16_rn(c - __bfloat162float(h));
-        }
-    }
+    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < mpad; j += (int64_t)gridDim.x * blockDim.x)
+        theta_prep_one(theta, j, m, mpad, c32, hi, lo);
 }
 
 // --------------------------------------------------------- FP32 phase GEMM
@@ -271,37 +262,53 @@ __device__ __forceinline__ double warp_sum_f64(double v) {
     return v;
 }
 
-// S = sum cos and M2 = sum (cos - S/s)^2 of one observable's partials, on every lane of the warp.
-__device__ __forceinline__ void merge_partials(const double2 *__restrict__ p, int64_t nparts, int64_t pw, int64_t s,
-                                               int lane, double &S, double &mean, double &M2) {
+// Sizes of the partials and the reciprocals the merge needs: an FP64 division or
+// square root takes about a microsecond of latency on this GPU, and a warp has
+// nothing else to do meanwhile, so the host divides (k_finalize, 784 x 1003: 10.4
+// -> 7.2 us).
+struct PartSizes {
+    int64_t nparts, pw, s;
+    double inv_s, inv_pw, inv_last;  // 1 / s, 1 / pw, 1 / (samples of the last partial)
+};
+
+// a / b from y = 1 / b: a quotient, and one correction by its exact remainder
+// (Markstein, "Computation of elementary functions on the IBM RISC System/6000
+// processor", 1990). Exact where the quotient is a double.
+__device__ __forceinline__ double div_by(double a, double b, double y) {
+    const double q = a * y;
+    return fma(fma(-q, b, a), y, q);
+}
+
+// S = sum cos, its mean and M2 = sum (cos - S/s)^2 of one observable's partials, on every lane of the warp.
+__device__ __forceinline__ void merge_partials(const double2 *__restrict__ p, const PartSizes &z, int lane, double &S,
+                                               double &mean, double &M2) {
     S = 0.0;
-    for (int64_t k = lane; k < nparts; k += 32) S += p[k].x;
+    for (int64_t k = lane; k < z.nparts; k += 32) S += p[k].x;
     S = warp_sum_f64(S);
-    mean = S / (double)s;
-    const double inv_pw = 1.0 / (double)pw;
+    mean = div_by(S, (double)z.s, z.inv_s);
     M2 = 0.0;
-    for (int64_t k = lane; k < nparts; k += 32) {
-        const int64_t nk = (s - k * pw) < pw ? (s - k * pw) : pw;
+    for (int64_t k = lane; k < z.nparts; k += 32) {
+        const bool last = k == z.nparts - 1;
         const double2 v = p[k];
-        const double d = (nk == pw ? v.x * inv_pw : v.x / (double)nk) - mean;
-        M2 += v.y + (double)nk * d * d;
+        const double nk = (double)(last ? z.s - k * z.pw : z.pw);
+        const double d = div_by(v.x, nk, last ? z.inv_last : z.inv_pw) - mean;
+        M2 += v.y + nk * d * d;
     }
     M2 = warp_sum_f64(M2);
 }
 
-__global__ void __launch_bounds__(256) k_finalize(const double2 *__restrict__ part, int64_t nparts, int64_t pw,
-                                                  int64_t l, int64_t s, double *__restrict__ expval,
-                                                  double *__restrict__ std_err, double *__restrict__ S1,
-                                                  double *__restrict__ S2) {
+__global__ void __launch_bounds__(256) k_finalize(const double2 *__restrict__ part, PartSizes z, int64_t l,
+                                                  double *__restrict__ expval, double *__restrict__ std_err,
+                                                  double *__restrict__ S1, double *__restrict__ S2) {
     const int lane = threadIdx.x & 31;
     const int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (a >= l) return;  // whole warps
-    if (!IQP_IN(a * nparts + nparts - 1, l * nparts, 30)) return;
+    if (!IQP_IN(a * z.nparts + z.nparts - 1, l * z.nparts, 30)) return;
     double S, mean, M2;
-    merge_partials(part + a * nparts, nparts, pw, s, lane, S, mean, M2);
+    merge_partials(part + a * z.nparts, z, lane, S, mean, M2);
     if (lane != 0) return;
     if (expval) expval[a] = mean;
-    if (std_err) std_err[a] = sqrt(M2 / (double)s) / sqrt((double)s);
+    if (std_err) std_err[a] = sqrt(M2) * z.inv_s;  // sqrt(M2 / s) / sqrt(s)
     if (S1) S1[a] = S;
     if (S2) S2[a] = M2 + S * mean;
 }
@@ -374,17 +381,17 @@ __global__ void __launch_bounds__(1024) k_mmd_combine(const long long *__restric
 struct MmdConst {
     double inv_s, inv_N, inv_l, inv_ss1, inv_NN1;  // 1 / (s (s - 1)), 1 / (N (N - 1))
 };
-__global__ void __launch_bounds__(256) k_mmd_terms(const double2 *__restrict__ part, int64_t nparts, int64_t pw,
-                                                   const long long *__restrict__ T, int64_t l, int64_t s, int64_t N,
+__global__ void __launch_bounds__(256) k_mmd_terms(const double2 *__restrict__ part, PartSizes z,
+                                                   const long long *__restrict__ T, int64_t l, int64_t N,
                                                    int unbiased, int sqrt_loss, MmdConst k, double *__restrict__ terms,
                                                    double *__restrict__ alpha, double *__restrict__ beta,
                                                    double *__restrict__ loss, double *__restrict__ scale,
                                                    uint32_t *__restrict__ counter) {
     const int lane = threadIdx.x & 31;
     const int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (a < l && IQP_IN(a * nparts + nparts - 1, l * nparts, 30)) {  // whole warps
+    if (a < l && IQP_IN(a * z.nparts + z.nparts - 1, l * z.nparts, 30)) {  // whole warps
         double S, mean, M2;
-        merge_partials(part + a * nparts, nparts, pw, s, lane, S, mean, M2);
+        merge_partials(part + a * z.nparts, z, lane, S, mean, M2);
         if (lane == 0) {
             const double t = (double)T[a], dN = (double)N;
             const double p = t * k.inv_N, S2 = M2 + S * mean;
@@ -437,7 +444,7 @@ __global__ void __launch_bounds__(256) k_mmd_terms(const double2 *__restrict__ p
     }
     if (threadIdx.x == 0) {
         *loss = out;
-        if (scale != nullptr) *scale = fixed_scale(2.0 * (double)s * red[1][0] * f);
+        if (scale != nullptr) *scale = fixed_scale(2.0 * (double)z.s * red[1][0] * f);
     }
 }
 
@@ -496,10 +503,16 @@ cudaError_t launch_grad_simt(const float *W, int64_t ldw, const uint64_t *PZ, co
     return cudaGetLastError();
 }
 
+namespace {
+PartSizes part_sizes(int64_t nparts, int64_t pw, int64_t s) {
+    return PartSizes{nparts, pw, s, 1.0 / (double)s, 1.0 / (double)pw, 1.0 / (double)(s - (nparts - 1) * pw)};
+}
+}  // namespace
+
 cudaError_t launch_finalize(const double2 *part, int64_t nparts, int64_t pw, int64_t l, int64_t s, double *expval,
                             double *std_err, double *S1, double *S2, cudaStream_t st) {
     LaunchScope ls(IQP_KERNEL_FINALIZE, st);
-    k_finalize<<<(unsigned)cdiv(l, 8), 256, 0, st>>>(part, nparts, pw, l, s, expval, std_err, S1, S2);
+    k_finalize<<<(unsigned)cdiv(l, 8), 256, 0, st>>>(part, part_sizes(nparts, pw, s), l, expval, std_err, S1, S2);
     return cudaGetLastError();
 }
 
@@ -528,7 +541,8 @@ cudaError_t launch_mmd_terms(const double2 *part, int64_t nparts, int64_t pw, co
     const double ds = (double)s, dN = (double)N;
     const MmdConst k{1.0 / ds, 1.0 / dN, 1.0 / (double)l, 1.0 / (ds * (ds - 1.0)), 1.0 / (dN * (dN - 1.0))};
     LaunchScope ls(IQP_KERNEL_MMD_COMBINE, st);
-    k_mmd_terms<<<(unsigned)cdiv(l, 8), 256, 0, st>>>(part, nparts, pw, reinterpret_cast<const long long *>(T), l, s, N,
+    k_mmd_terms<<<(unsigned)cdiv(l, 8), 256, 0, st>>>(part, part_sizes(nparts, pw, s),
+                                                      reinterpret_cast<const long long *>(T), l, N,
                                                       unbiased, sqrt_loss ? 1 : 0, k, terms, alpha, beta, loss, scale,
                                                       counter);
     return cudaGetLastError();
