@@ -9,8 +9,6 @@ float32 for the kernels; gradients come back in theta's dtype).
 """
 from __future__ import annotations
 
-import ctypes
-
 import torch
 
 from . import _lib
@@ -30,8 +28,15 @@ def precision_code(precision) -> int:
                          f"got {precision!r}") from None
 
 
+# The current stream's raw handle without a Stream object around it.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
+    lambda index: torch.cuda.current_stream(index).cuda_stream)
+
+
 def _stream(device) -> int:
-    return torch.cuda.current_stream(device).cuda_stream
+    if not isinstance(device, torch.device) or device.index is None:
+        device = _resolve(device)
+    return _raw_stream(device.index)
 
 
 def _bits(t: torch.Tensor, name: str) -> torch.Tensor:
@@ -51,7 +56,14 @@ def _resolve(device) -> torch.device:
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+def _f64(t, device):
+    """t as a contiguous float64 tensor on `device` (t itself where it is one already)."""
+    if t is None or (t.dtype is torch.float64 and t.device == device and t.is_contiguous()):
+        return t
+    return t.detach().to(device=device, dtype=torch.float64).contiguous()
 
 
 class _Workspace:
@@ -60,9 +72,10 @@ class _Workspace:
     def __init__(self):
         self._bufs = {}
 
-    def get(self, nbytes: int, device) -> torch.Tensor:
-        device = _resolve(device)
-        key = (device.index, _stream(device))
+    def get(self, nbytes: int, device, stream: int | None = None) -> torch.Tensor:
+        if not isinstance(device, torch.device) or device.index is None:
+            device = _resolve(device)
+        key = (device.index, _stream(device) if stream is None else stream)
         buf = self._bufs.get(key)
         if buf is None or buf.numel() < nbytes:
             buf = torch.zeros(max(nbytes, 256), dtype=torch.uint8, device=device)
@@ -73,8 +86,12 @@ class _Workspace:
 _WS = _Workspace()
 
 
+def _ws_bytes(op: int, n: int, m: int, l: int, s: int, N: int, prec: int) -> int:
+    return int(_lib.load().iqp_workspace_bytes(op, n, m, l, s, N, prec))
+
+
 def workspace_bytes(op: int, n: int, m: int, l: int, s: int, N: int = 0, precision="split_bf16") -> int:
-    return int(_lib.load().iqp_workspace_bytes(op, n, m, l, s, N, precision_code(precision)))
+    return _ws_bytes(op, n, m, l, s, N, precision_code(precision))
 
 
 def parity(n: int, R: torch.Tensor, G: torch.Tensor, ldp: int | None = None) -> torch.Tensor:
@@ -86,7 +103,7 @@ def parity(n: int, R: torch.Tensor, G: torch.Tensor, ldp: int | None = None) -> 
         ldp += ldp & 1
     P = torch.empty((R.shape[0], ldp), dtype=torch.int64, device=R.device)
     check(_lib.load().iqp_parity(n, _ptr(R), R.shape[0], R.shape[1], _ptr(G), m, G.shape[1], _ptr(P), ldp,
-                                 ctypes.c_void_p(_stream(R.device))), "iqp_parity")
+                                 _stream(R.device)), "iqp_parity")
     return P
 
 
@@ -103,7 +120,7 @@ def parity_gather(n: int, R: torch.Tensor, G: torch.Tensor):
     PT = torch.empty((m, ldpt), dtype=torch.int64, device=R.device)
     scratch = torch.empty((n * ldpt + 2 * m,), dtype=torch.int64, device=R.device)  # R^T, then the support list
     check(_lib.load().iqp_parity_gather(n, _ptr(R), rows, R.shape[1], _ptr(G), m, G.shape[1], _ptr(P), ldp, _ptr(PT),
-                                        ldpt, _ptr(scratch), ctypes.c_void_p(_stream(R.device))), "iqp_parity_gather")
+                                        ldpt, _ptr(scratch), _stream(R.device)), "iqp_parity_gather")
     return P, PT
 
 
@@ -112,13 +129,15 @@ def parity_sum(n: int, A: torch.Tensor, X: torch.Tensor) -> torch.Tensor:
     _bits(A, "A"), _bits(X, "X")
     T = torch.empty(A.shape[0], dtype=torch.int64, device=A.device)
     check(_lib.load().iqp_parity_sum(n, _ptr(A), A.shape[0], A.shape[1], _ptr(X), X.shape[0], X.shape[1], _ptr(T),
-                                     ctypes.c_void_p(_stream(A.device))), "iqp_parity_sum")
+                                     _stream(A.device)), "iqp_parity_sum")
     return T
 
 
 def _theta32(theta: torch.Tensor) -> torch.Tensor:
     if not theta.is_cuda:
         raise ValueError("theta must be a CUDA tensor")
+    if theta.dtype is torch.float32 and theta.is_contiguous():
+        return theta  # only its address is used, in this call
     return theta.detach().to(torch.float32).contiguous()
 
 
@@ -130,12 +149,12 @@ def expval_raw(n, theta, G, A, Z, precision="split_bf16"):
     m, l, s = G.shape[0], A.shape[0], Z.shape[0]
     prec = precision_code(precision)
     lib = _lib.load()
-    nbytes = lib.iqp_workspace_bytes(OP_EXPVAL, n, m, l, s, 0, prec)
-    ws = _WS.get(nbytes, G.device)
+    st = _stream(G.device)
+    ws = _WS.get(_ws_bytes(OP_EXPVAL, n, m, l, s, 0, prec), G.device, st)
     ev = torch.empty(l, dtype=torch.float64, device=G.device)
     se = torch.empty(l, dtype=torch.float64, device=G.device)
     check(lib.iqp_expval(n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(Z), s, Z.shape[1], _ptr(th), prec,
-                         _ptr(ev), _ptr(se), _ptr(ws), ws.numel(), ctypes.c_void_p(_stream(G.device))), "iqp_expval")
+                         _ptr(ev), _ptr(se), _ptr(ws), ws.numel(), st), "iqp_expval")
     return ev, se
 
 
@@ -146,15 +165,15 @@ def expval_grad(n, theta, G, A, Z, alpha, beta=None, precision="split_bf16") -> 
     th = _theta32(theta)
     m, l, s = G.shape[0], A.shape[0], Z.shape[0]
     prec = precision_code(precision)
-    al = alpha.detach().to(device=G.device, dtype=torch.float64).contiguous()
-    be = None if beta is None else beta.detach().to(device=G.device, dtype=torch.float64).contiguous()
+    al = _f64(alpha, G.device)
+    be = _f64(beta, G.device)
     lib = _lib.load()
-    nbytes = lib.iqp_workspace_bytes(OP_EXPVAL_GRAD, n, m, l, s, 0, prec)
-    ws = _WS.get(nbytes, G.device)
+    st = _stream(G.device)
+    ws = _WS.get(_ws_bytes(OP_EXPVAL_GRAD, n, m, l, s, 0, prec), G.device, st)
     grad = torch.empty(m, dtype=torch.float64, device=G.device)
     check(lib.iqp_expval_grad(n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(Z), s, Z.shape[1], _ptr(th),
                               _ptr(al), _ptr(be), prec, _ptr(grad), _ptr(ws), ws.numel(),
-                              ctypes.c_void_p(_stream(G.device))), "iqp_expval_grad")
+                              st), "iqp_expval_grad")
     return grad
 
 
@@ -168,16 +187,17 @@ def expval_value_and_grad(n, theta, G, A, Z, alpha, beta=None, precision="split_
     th = _theta32(theta)
     m, l, s = G.shape[0], A.shape[0], Z.shape[0]
     prec = precision_code(precision)
-    al = alpha.detach().to(device=G.device, dtype=torch.float64).contiguous()
-    be = None if beta is None else beta.detach().to(device=G.device, dtype=torch.float64).contiguous()
+    al = _f64(alpha, G.device)
+    be = _f64(beta, G.device)
     lib = _lib.load()
-    ws = _WS.get(lib.iqp_workspace_bytes(OP_EXPVAL_GRAD, n, m, l, s, 0, prec), G.device)
+    st = _stream(G.device)
+    ws = _WS.get(_ws_bytes(OP_EXPVAL_GRAD, n, m, l, s, 0, prec), G.device, st)
     ev = torch.empty(l, dtype=torch.float64, device=G.device)
     se = torch.empty(l, dtype=torch.float64, device=G.device)
     grad = torch.empty(m, dtype=torch.float64, device=G.device)
     check(lib.iqp_expval_value_and_grad(n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(Z), s, Z.shape[1],
                                         _ptr(th), _ptr(al), _ptr(be), prec, _ptr(ev), _ptr(se), _ptr(grad), _ptr(ws),
-                                        ws.numel(), ctypes.c_void_p(_stream(G.device))), "iqp_expval_value_and_grad")
+                                        ws.numel(), st), "iqp_expval_value_and_grad")
     return ev, se, grad
 
 
@@ -200,14 +220,15 @@ def expval_keep_phi_raw(n, theta, G, A, Z, precision="split_bf16", ld=None):
     m, l, s = G.shape[0], A.shape[0], Z.shape[0]
     prec = precision_code(precision)
     lib = _lib.load()
-    ws = _WS.get(lib.iqp_workspace_bytes(OP_EXPVAL, n, m, l, s, 0, prec), G.device)
+    st = _stream(G.device)
+    ws = _WS.get(_ws_bytes(OP_EXPVAL, n, m, l, s, 0, prec), G.device, st)
     ev = torch.empty(l, dtype=torch.float64, device=G.device)
     se = torch.empty(l, dtype=torch.float64, device=G.device)
     ld = phi_ld(s) if ld is None else int(ld)
     phi = torch.empty((l, ld), dtype=torch.float32, device=G.device)
     check(lib.iqp_expval_keep_phi(n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(Z), s, Z.shape[1], _ptr(th),
                                   prec, _ptr(ev), _ptr(se), _ptr(phi), ld, _ptr(ws), ws.numel(),
-                                  ctypes.c_void_p(_stream(G.device))), "iqp_expval_keep_phi")
+                                  st), "iqp_expval_keep_phi")
     return ev, se, phi
 
 
@@ -222,14 +243,15 @@ def expval_grad_from_phi(n, theta, G, A, Z, phi, alpha, beta=None, precision="sp
     if not (phi.is_cuda and phi.dtype == torch.float32 and phi.dim() == 2 and phi.is_contiguous()
             and phi.shape[0] == l):
         raise ValueError("phi must be the contiguous l x ld float32 CUDA tensor expval_keep_phi_raw returned")
-    al = alpha.detach().to(device=G.device, dtype=torch.float64).contiguous()
-    be = None if beta is None else beta.detach().to(device=G.device, dtype=torch.float64).contiguous()
+    al = _f64(alpha, G.device)
+    be = _f64(beta, G.device)
     lib = _lib.load()
-    ws = _WS.get(lib.iqp_workspace_bytes(OP_EXPVAL_GRAD, n, m, l, s, 0, prec), G.device)
+    st = _stream(G.device)
+    ws = _WS.get(_ws_bytes(OP_EXPVAL_GRAD, n, m, l, s, 0, prec), G.device, st)
     grad = torch.empty(m, dtype=torch.float64, device=G.device)
     check(lib.iqp_expval_grad_from_phi(n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(Z), s, Z.shape[1],
                                        _ptr(th), _ptr(al), _ptr(be), prec, _ptr(phi), phi.shape[1], _ptr(grad),
-                                       _ptr(ws), ws.numel(), ctypes.c_void_p(_stream(G.device))),
+                                       _ptr(ws), ws.numel(), st),
           "iqp_expval_grad_from_phi")
     return grad
 
@@ -253,7 +275,7 @@ class _ExpvalFn(torch.autograd.Function):
         if g_ev is None:
             return (None,) * 7
         s = Z.shape[0]
-        alpha = -g_ev.to(torch.float64) / s
+        alpha = g_ev.to(torch.float64) / -s
         if phi is not None:
             grad = expval_grad_from_phi(ctx.n, theta, G, A, Z, phi, alpha, None, ctx.precision)
         else:
@@ -288,9 +310,9 @@ def mmd_loss_raw(n, theta, G, A, Z, X, precision="split_bf16", unbiased=True, wi
     else:
         op = OP_MMD_LOSS_GRAD if with_grad else OP_MMD_LOSS
     flags = (MMD_UNBIASED if unbiased else 0) | (MMD_SQRT if sqrt_loss else 0) | (MMD_INDEP if indep else 0)
-    ws = _WS.get(lib.iqp_workspace_bytes(op, n, m, l, s, N, prec), G.device)
+    st = _stream(G.device)
+    ws = _WS.get(_ws_bytes(op, n, m, l, s, N, prec), G.device, st)
     loss = torch.empty(1, dtype=torch.float64, device=G.device)
-    st = ctypes.c_void_p(_stream(G.device))
     args = (n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(Z), s, Z.shape[1], _ptr(X), N, X.shape[1],
             _ptr(th), prec, flags)
     if with_grad:
@@ -338,11 +360,12 @@ def expval_indep_raw(n, theta, G, A, Z):
         raise ValueError("Z must have l * s rows")
     s = Z.shape[0] // l
     lib = _lib.load()
-    ws = _WS.get(lib.iqp_workspace_bytes(OP_EXPVAL_INDEP, n, m, l, s, 0, SPARSE_FP32), G.device)
+    st = _stream(G.device)
+    ws = _WS.get(_ws_bytes(OP_EXPVAL_INDEP, n, m, l, s, 0, SPARSE_FP32), G.device, st)
     ev = torch.empty(l, dtype=torch.float64, device=G.device)
     se = torch.empty(l, dtype=torch.float64, device=G.device)
     check(lib.iqp_expval_indep(n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(Z), s, Z.shape[1], _ptr(th),
-                               _ptr(ev), _ptr(se), _ptr(ws), ws.numel(), ctypes.c_void_p(_stream(G.device))),
+                               _ptr(ev), _ptr(se), _ptr(ws), ws.numel(), st),
           "iqp_expval_indep")
     return ev, se
 
@@ -354,14 +377,15 @@ def expval_indep_grad(n, theta, G, A, Z, alpha, beta=None) -> torch.Tensor:
     th = _theta32(theta)
     m, l = G.shape[0], A.shape[0]
     s = Z.shape[0] // l
-    al = alpha.detach().to(device=G.device, dtype=torch.float64).contiguous()
-    be = None if beta is None else beta.detach().to(device=G.device, dtype=torch.float64).contiguous()
+    al = _f64(alpha, G.device)
+    be = _f64(beta, G.device)
     lib = _lib.load()
-    ws = _WS.get(lib.iqp_workspace_bytes(OP_EXPVAL_INDEP_GRAD, n, m, l, s, 0, SPARSE_FP32), G.device)
+    st = _stream(G.device)
+    ws = _WS.get(_ws_bytes(OP_EXPVAL_INDEP_GRAD, n, m, l, s, 0, SPARSE_FP32), G.device, st)
     grad = torch.empty(m, dtype=torch.float64, device=G.device)
     check(lib.iqp_expval_indep_grad(n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(Z), s, Z.shape[1],
                                     _ptr(th), _ptr(al), _ptr(be), _ptr(grad), _ptr(ws), ws.numel(),
-                                    ctypes.c_void_p(_stream(G.device))), "iqp_expval_indep_grad")
+                                    st), "iqp_expval_indep_grad")
     return grad
 
 
@@ -380,7 +404,7 @@ class _ExpvalIndepFn(torch.autograd.Function):
         if g_ev is None:
             return (None,) * 5
         s = Z.shape[0] // A.shape[0]
-        grad = expval_indep_grad(ctx.n, theta, G, A, Z, -g_ev.to(torch.float64) / s, None)
+        grad = expval_indep_grad(ctx.n, theta, G, A, Z, g_ev.to(torch.float64) / -s, None)
         return grad.to(theta.dtype), None, None, None, None
 
 
@@ -403,7 +427,7 @@ class _ExpandFn(torch.autograd.Function):
         th = _theta32(theta_p)
         out = torch.empty(m, dtype=torch.float32, device=th.device)
         check(_lib.load().iqp_expand_params(_ptr(th), th.shape[0], _ptr(start), _ptr(out), m,
-                                            ctypes.c_void_p(_stream(th.device))), "iqp_expand_params")
+                                            _stream(th.device)), "iqp_expand_params")
         ctx.save_for_backward(start)
         ctx.np, ctx.m, ctx.dtype = th.shape[0], m, theta_p.dtype
         return out
@@ -414,7 +438,7 @@ class _ExpandFn(torch.autograd.Function):
         gg = g.detach().to(torch.float64).contiguous()
         out = torch.empty(ctx.np, dtype=torch.float64, device=gg.device)
         check(_lib.load().iqp_reduce_params(_ptr(gg), ctx.m, _ptr(start), ctx.np, _ptr(out),
-                                            ctypes.c_void_p(_stream(gg.device))), "iqp_reduce_params")
+                                            _stream(gg.device)), "iqp_reduce_params")
         return out.to(ctx.dtype), None, None
 
 
@@ -434,7 +458,7 @@ def embed_bits(src: torch.Tensor, nw: int, wires, n: int) -> torch.Tensor:
     ld = words_per_row(n)
     out = torch.empty(src.shape[0], ld, dtype=torch.int64, device=src.device)
     check(_lib.load().iqp_embed_bits(_ptr(src), src.shape[0], src.shape[1], _ptr(w), nw, _ptr(out), ld, n,
-                                     ctypes.c_void_p(_stream(src.device))), "iqp_embed_bits")
+                                     _stream(src.device)), "iqp_embed_bits")
     return out
 
 
@@ -457,7 +481,7 @@ def uniform_bits(seed: int, stream: int, rows: int, n: int, device="cuda", out=N
     ld = words_per_row(n)
     out = _bits_out(out, rows, ld, device)
     check(_lib.load().iqp_uniform_bits(seed & (2 ** 64 - 1), stream & (2 ** 64 - 1), rows, n, _ptr(out), ld,
-                                       ctypes.c_void_p(_stream(device))), "iqp_uniform_bits")
+                                       _stream(device)), "iqp_uniform_bits")
     return out
 
 
@@ -467,7 +491,7 @@ def bernoulli_bits(seed: int, stream: int, rows: int, n: int, p: float, device="
     ld = words_per_row(n)
     out = _bits_out(out, rows, ld, device)
     check(_lib.load().iqp_bernoulli_bits(seed & (2 ** 64 - 1), stream & (2 ** 64 - 1), rows, n, float(p),
-                                         _ptr(out), ld, ctypes.c_void_p(_stream(device))), "iqp_bernoulli_bits")
+                                         _ptr(out), ld, _stream(device)), "iqp_bernoulli_bits")
     return out
 
 
@@ -477,10 +501,11 @@ def bitflip_expval_raw(n, theta, G, A):
     th = _theta32(theta)
     m, l = G.shape[0], A.shape[0]
     lib = _lib.load()
-    ws = _WS.get(lib.iqp_workspace_bytes(OP_BITFLIP, n, m, l, 1, 0, FP32), G.device)
+    st = _stream(G.device)
+    ws = _WS.get(_ws_bytes(OP_BITFLIP, n, m, l, 1, 0, FP32), G.device, st)
     ev = torch.empty(l, dtype=torch.float64, device=G.device)
     check(lib.iqp_bitflip_expval(n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(th), _ptr(ev), _ptr(ws),
-                                 ws.numel(), ctypes.c_void_p(_stream(G.device))), "iqp_bitflip_expval")
+                                 ws.numel(), st), "iqp_bitflip_expval")
     return ev
 
 
@@ -489,12 +514,13 @@ def bitflip_grad(n, theta, G, A, w) -> torch.Tensor:
     _bits(G, "G"), _bits(A, "A")
     th = _theta32(theta)
     m, l = G.shape[0], A.shape[0]
-    wd = w.detach().to(device=G.device, dtype=torch.float64).contiguous()
+    wd = _f64(w, G.device)
     lib = _lib.load()
-    ws = _WS.get(lib.iqp_workspace_bytes(OP_BITFLIP, n, m, l, 1, 0, FP32), G.device)
+    st = _stream(G.device)
+    ws = _WS.get(_ws_bytes(OP_BITFLIP, n, m, l, 1, 0, FP32), G.device, st)
     grad = torch.empty(m, dtype=torch.float64, device=G.device)
     check(lib.iqp_bitflip_grad(n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(th), _ptr(wd), _ptr(grad),
-                               _ptr(ws), ws.numel(), ctypes.c_void_p(_stream(G.device))), "iqp_bitflip_grad")
+                               _ptr(ws), ws.numel(), st), "iqp_bitflip_grad")
     return grad
 
 
@@ -522,7 +548,7 @@ def read_status(device=None) -> int:
     """Device-side status recorded in the current stream's workspace (clears it)."""
     device = _resolve("cuda" if device is None else device)
     ws = _WS.get(256, device)
-    return int(_lib.load().iqp_read_status(_ptr(ws), ws.numel(), ctypes.c_void_p(_stream(device))))
+    return int(_lib.load().iqp_read_status(_ptr(ws), ws.numel(), _stream(device)))
 
 
 def launch_count() -> int:
