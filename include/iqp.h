@@ -229,6 +229,23 @@ iqp_status iqp_expval_grad_from_phi(int64_t n, const uint64_t *G, int64_t m, int
                                     iqp_precision prec, const float *phi, int64_t ldphi, double *grad,
                                     void *ws, size_t ws_bytes, void *stream);
 
+/* The same pair for IQP_FP32, where its tensor-core form runs: iqp_planes_used
+ * is 1 for the sizes whose statistics (and gradient) it takes; for the others,
+ * and with workspaces too small for it, the two calls are IQP_ERR_UNSUPPORTED. */
+int iqp_planes_used(int64_t n, int64_t m, int64_t l, int64_t s);
+iqp_status iqp_planes_keep_phi(int64_t n, const uint64_t *G, int64_t m, int64_t ldg,
+                               const uint64_t *A, int64_t l, int64_t lda,
+                               const uint64_t *Z, int64_t s, int64_t ldz,
+                               const float *theta, double *expval, double *std_err,
+                               float *phi, int64_t ldphi,
+                               void *ws, size_t ws_bytes, void *stream);
+iqp_status iqp_planes_grad_from_phi(int64_t n, const uint64_t *G, int64_t m, int64_t ldg,
+                                    const uint64_t *A, int64_t l, int64_t lda,
+                                    const uint64_t *Z, int64_t s, int64_t ldz,
+                                    const float *theta, const double *alpha, const double *beta,
+                                    const float *phi, int64_t ldphi, double *grad,
+                                    void *ws, size_t ws_bytes, void *stream);
+
 /* Estimates and gradient in one call, for a loss whose gradient coefficients
  * alpha, beta (as in iqp_expval_grad) are known before the estimates, e.g.
  * L = sum_a w_a <Z_a> with alpha_a = -w_a / s, beta = NULL. Outputs as

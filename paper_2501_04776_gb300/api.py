@@ -256,12 +256,48 @@ def expval_grad_from_phi(n, theta, G, A, Z, phi, alpha, beta=None, precision="sp
     return grad
 
 
+def _planes_keep_phi(n, theta, G, A, Z):
+    """expval_keep_phi_raw of the FP32 precision's tensor-core form (sizes of iqp_planes_used)."""
+    for t, nm in ((G, "G"), (A, "A"), (Z, "Z")):
+        _bits(t, nm)
+    th = _theta32(theta)
+    m, l, s = G.shape[0], A.shape[0], Z.shape[0]
+    st = _stream(G.device)
+    ws = _WS.get(_ws_bytes(OP_EXPVAL, n, m, l, s, 0, FP32), G.device, st)
+    ev = torch.empty(l, dtype=torch.float64, device=G.device)
+    se = torch.empty(l, dtype=torch.float64, device=G.device)
+    phi = torch.empty((l, phi_ld(s)), dtype=torch.float32, device=G.device)
+    check(_lib.load().iqp_planes_keep_phi(n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(Z), s, Z.shape[1],
+                                          _ptr(th), _ptr(ev), _ptr(se), _ptr(phi), phi.shape[1], _ptr(ws), ws.numel(),
+                                          st), "iqp_planes_keep_phi")
+    return ev, se, phi
+
+
+def _planes_grad_from_phi(n, theta, G, A, Z, phi, alpha) -> torch.Tensor:
+    for t, nm in ((G, "G"), (A, "A"), (Z, "Z")):
+        _bits(t, nm)
+    th = _theta32(theta)
+    m, l, s = G.shape[0], A.shape[0], Z.shape[0]
+    al = _f64(alpha, G.device)
+    st = _stream(G.device)
+    ws = _WS.get(_ws_bytes(OP_EXPVAL_GRAD, n, m, l, s, 0, FP32), G.device, st)
+    grad = torch.empty(m, dtype=torch.float64, device=G.device)
+    check(_lib.load().iqp_planes_grad_from_phi(n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(Z), s,
+                                               Z.shape[1], _ptr(th), _ptr(al), None, _ptr(phi), phi.shape[1],
+                                               _ptr(grad), _ptr(ws), ws.numel(), st), "iqp_planes_grad_from_phi")
+    return grad
+
+
 class _ExpvalFn(torch.autograd.Function):
     @staticmethod
     def forward(ctx, theta, G, A, Z, n, precision, keep_phi):
         phi = None
-        if keep_phi and ctx.needs_input_grad[0] and precision_code(precision) in KEEP_PHI:
+        keep = keep_phi and ctx.needs_input_grad[0]
+        code = precision_code(precision)
+        if keep and code in KEEP_PHI:
             ev, se, phi = expval_keep_phi_raw(n, theta, G, A, Z, precision)
+        elif keep and code == FP32 and _lib.load().iqp_planes_used(n, G.shape[0], A.shape[0], Z.shape[0]):
+            ev, se, phi = _planes_keep_phi(n, theta, G, A, Z)
         else:
             ev, se = expval_raw(n, theta, G, A, Z, precision)
         ctx.save_for_backward(theta, G, A, Z, phi)
@@ -276,7 +312,9 @@ class _ExpvalFn(torch.autograd.Function):
             return (None,) * 7
         s = Z.shape[0]
         alpha = g_ev.to(torch.float64) / -s
-        if phi is not None:
+        if phi is not None and precision_code(ctx.precision) == FP32:
+            grad = _planes_grad_from_phi(ctx.n, theta, G, A, Z, phi, alpha)
+        elif phi is not None:
             grad = expval_grad_from_phi(ctx.n, theta, G, A, Z, phi, alpha, None, ctx.precision)
         else:
             grad = expval_grad(ctx.n, theta, G, A, Z, alpha, None, ctx.precision)
@@ -286,7 +324,7 @@ class _ExpvalFn(torch.autograd.Function):
 def expval(theta, G, A, Z, n: int, precision="split_bf16", keep_phi=True):
     """Monte-Carlo <Z_a> estimates and standard errors (float64), differentiable
     in theta (std_err is not). With keep_phi (split BF16, row-sparse and
-    low-order forms) the forward keeps Phi (4 l s bytes, held until the
+    low-order forms, FP32 on the tensor cores) the forward keeps Phi (4 l s bytes, held until the
     backward) so the backward forms W from it instead of recomputing Phi;
     keep_phi=False holds only the inputs and recomputes."""
     return _ExpvalFn.apply(theta, G, A, Z, n, precision, keep_phi)

@@ -41,6 +41,7 @@ cudaError_t launch_mmd_combine(const int64_t *T, const double *S1, const double 
                                cudaStream_t st);
 cudaError_t launch_phase_tc(int mode, const Plan &p, void *ws, const double *alpha, const double *beta,
                             cudaStream_t st, iqp_status *why);
+cudaError_t launch_x3_w(const Plan &p, void *ws, const double *alpha, const double *beta, cudaStream_t st);
 cudaError_t launch_w_from_phi(const Plan &p, void *ws, const double *alpha, const double *beta, cudaStream_t st);
 cudaError_t launch_grad_tc(const Plan &p, void *ws, cudaStream_t st, iqp_status *why);
 int64_t grad_tc_rows(const Plan &p);
@@ -551,8 +552,9 @@ iqp_status backward(const Plan &p, void *ws, const double *alpha, const double *
         if (launch_grad_tc(p, ws, st, &why) != cudaSuccess) return why != IQP_OK ? why : IQP_ERR_CUDA;
     } else if (p.x3) {
         iqp_status why = IQP_OK;
-        if (launch_phase_x3(1, p, ws, alpha, beta, st, &why) != cudaSuccess ||
-            launch_grad_x3(p, ws, st, &why) != cudaSuccess)
+        const cudaError_t e = p.phi_in ? launch_x3_w(p, ws, alpha, beta, st)
+                                       : launch_phase_x3(1, p, ws, alpha, beta, st, &why);
+        if (e != cudaSuccess || launch_grad_x3(p, ws, st, &why) != cudaSuccess)
             return why != IQP_OK ? why : IQP_ERR_CUDA;
         IQP_TRY(launch_grad_reduce(gpart, 2 * cdiv(p.l, kATile), p.m, grad, st));
         return IQP_OK;
@@ -593,8 +595,8 @@ iqp_status mmd_core(int op, int64_t n, const uint64_t *G, int64_t m, int64_t ldg
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if ((rc = prepare(p, ws, G, ldg, A, lda, Z, ldz, theta, st)) != IQP_OK) return rc;
     double *S1 = at<double>(ws, p.off_s12), *S2 = S1 + l;
-    if (g && (p.prec == IQP_LOWORDER_FP32 || p.off_phi != 0)) {  // Phi kept for the gradient pass
-        p.phi = at<float>(ws, p.prec == IQP_LOWORDER_FP32 ? p.off_w : p.off_phi);
+    if (g && (p.prec == IQP_LOWORDER_FP32 || p.x3 || p.off_phi != 0)) {  // Phi kept for the gradient pass
+        p.phi = at<float>(ws, p.off_phi != 0 ? p.off_phi : p.off_w);
         p.ldphi = p.ldw;
         p.phi_out = p.phi_in = true;
     }
@@ -743,20 +745,21 @@ iqp_status iqp_expval_grad(int64_t n, const uint64_t *G, int64_t m, int64_t ldg,
 
 // Arguments of a caller-owned kept Phi: l x ldphi FP32, ldphi a multiple of
 // 64 and >= s, 16-byte aligned; precisions with a Phi-keeping statistics pass.
-static iqp_status check_phi(const float *phi, int64_t ldphi, int64_t s, iqp_precision prec) {
+static iqp_status check_phi(const float *phi, int64_t ldphi, int64_t s, iqp_precision prec, bool planes) {
     if (phi == nullptr || ldphi < s || ldphi % 64 != 0) return IQP_ERR_ARG;
     if (!aligned(phi, 16)) return IQP_ERR_ALIGN;
+    if (planes) return prec == IQP_FP32 ? IQP_OK : IQP_ERR_UNSUPPORTED;
     if (prec != IQP_SPLIT_BF16 && prec != IQP_SPARSE_FP32 && prec != IQP_LOWORDER_FP32) return IQP_ERR_UNSUPPORTED;
     return IQP_OK;
 }
 
-iqp_status iqp_expval_keep_phi(int64_t n, const uint64_t *G, int64_t m, int64_t ldg, const uint64_t *A, int64_t l,
+static iqp_status keep_phi(bool planes, int64_t n, const uint64_t *G, int64_t m, int64_t ldg, const uint64_t *A, int64_t l,
                                int64_t lda, const uint64_t *Z, int64_t s, int64_t ldz, const float *theta,
                                iqp_precision prec, double *expval, double *std_err, float *phi, int64_t ldphi,
                                void *ws, size_t ws_bytes, void *stream) {
     iqp_status rc = check_common(n, G, m, ldg, A, l, lda, Z, s, ldz, theta, prec);
     if (rc != IQP_OK) return rc;
-    if ((rc = check_phi(phi, ldphi, s, prec)) != IQP_OK) return rc;
+    if ((rc = check_phi(phi, ldphi, s, prec, planes)) != IQP_OK) return rc;
     if ((expval && !aligned(expval, 8)) || (std_err && !aligned(std_err, 8))) return IQP_ERR_ALIGN;
     Plan p = make_plan(IQP_OP_EXPVAL, n, m, l, s, 0, prec);
     p.G = G;
@@ -764,6 +767,7 @@ iqp_status iqp_expval_keep_phi(int64_t n, const uint64_t *G, int64_t m, int64_t 
     p.A = A;
     p.lda = lda;
     if ((rc = check_ws(p, ws, ws_bytes)) != IQP_OK) return rc;
+    if (planes && !p.x3) return IQP_ERR_UNSUPPORTED;
     p.phi = phi;
     p.ldphi = ldphi;
     p.phi_out = true;
@@ -772,14 +776,14 @@ iqp_status iqp_expval_keep_phi(int64_t n, const uint64_t *G, int64_t m, int64_t 
     return forward_stats(p, ws, expval, std_err, nullptr, nullptr, st);
 }
 
-iqp_status iqp_expval_grad_from_phi(int64_t n, const uint64_t *G, int64_t m, int64_t ldg, const uint64_t *A,
+static iqp_status grad_from_phi(bool planes, int64_t n, const uint64_t *G, int64_t m, int64_t ldg, const uint64_t *A,
                                     int64_t l, int64_t lda, const uint64_t *Z, int64_t s, int64_t ldz,
                                     const float *theta, const double *alpha, const double *beta, iqp_precision prec,
                                     const float *phi, int64_t ldphi, double *grad, void *ws, size_t ws_bytes,
                                     void *stream) {
     iqp_status rc = check_common(n, G, m, ldg, A, l, lda, Z, s, ldz, theta, prec);
     if (rc != IQP_OK) return rc;
-    if ((rc = check_phi(phi, ldphi, s, prec)) != IQP_OK) return rc;
+    if ((rc = check_phi(phi, ldphi, s, prec, planes)) != IQP_OK) return rc;
     if (alpha == nullptr || grad == nullptr) return IQP_ERR_ARG;
     if (!aligned(alpha, 8) || !aligned(grad, 8) || (beta && !aligned(beta, 8))) return IQP_ERR_ALIGN;
     Plan p = make_plan(IQP_OP_EXPVAL_GRAD, n, m, l, s, 0, prec);
@@ -788,12 +792,45 @@ iqp_status iqp_expval_grad_from_phi(int64_t n, const uint64_t *G, int64_t m, int
     p.A = A;
     p.lda = lda;
     if ((rc = check_ws(p, ws, ws_bytes)) != IQP_OK) return rc;
+    if (planes && !p.x3) return IQP_ERR_UNSUPPORTED;
     p.phi = const_cast<float *>(phi);  // read only: phi_in
     p.ldphi = ldphi;
     p.phi_in = true;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if ((rc = prepare(p, ws, G, ldg, A, lda, Z, ldz, theta, st)) != IQP_OK) return rc;
     return backward(p, ws, alpha, beta, grad, st);
+}
+
+iqp_status iqp_expval_keep_phi(int64_t n, const uint64_t *G, int64_t m, int64_t ldg, const uint64_t *A, int64_t l,
+    int64_t lda, const uint64_t *Z, int64_t s, int64_t ldz, const float *theta, iqp_precision prec, double *expval,
+    double *std_err, float *phi, int64_t ldphi, void *ws, size_t ws_bytes, void *stream) {
+    return keep_phi(false, n, G, m, ldg, A, l, lda, Z, s, ldz, theta, prec, expval, std_err, phi, ldphi, ws, ws_bytes, stream);
+}
+
+iqp_status iqp_expval_grad_from_phi(int64_t n, const uint64_t *G, int64_t m, int64_t ldg, const uint64_t *A, int64_t l,
+    int64_t lda, const uint64_t *Z, int64_t s, int64_t ldz, const float *theta, const double *alpha,
+    const double *beta, iqp_precision prec, const float *phi, int64_t ldphi, double *grad, void *ws, size_t ws_bytes,
+    void *stream) {
+    return grad_from_phi(false, n, G, m, ldg, A, l, lda, Z, s, ldz, theta, alpha, beta, prec, phi, ldphi, grad, ws, ws_bytes,
+                         stream);
+}
+
+int iqp_planes_used(int64_t n, int64_t m, int64_t l, int64_t s) {
+    if (n < 1 || m < 1 || l < 1 || s < 1) return 0;
+    return make_plan(IQP_OP_EXPVAL, n, m, l, s, 0, IQP_FP32).x3 ? 1 : 0;
+}
+
+iqp_status iqp_planes_keep_phi(int64_t n, const uint64_t *G, int64_t m, int64_t ldg, const uint64_t *A, int64_t l,
+    int64_t lda, const uint64_t *Z, int64_t s, int64_t ldz, const float *theta, double *expval, double *std_err,
+    float *phi, int64_t ldphi, void *ws, size_t ws_bytes, void *stream) {
+    return keep_phi(true, n, G, m, ldg, A, l, lda, Z, s, ldz, theta, IQP_FP32, expval, std_err, phi, ldphi, ws, ws_bytes, stream);
+}
+
+iqp_status iqp_planes_grad_from_phi(int64_t n, const uint64_t *G, int64_t m, int64_t ldg, const uint64_t *A, int64_t l,
+    int64_t lda, const uint64_t *Z, int64_t s, int64_t ldz, const float *theta, const double *alpha,
+    const double *beta, const float *phi, int64_t ldphi, double *grad, void *ws, size_t ws_bytes, void *stream) {
+    return grad_from_phi(true, n, G, m, ldg, A, l, lda, Z, s, ldz, theta, alpha, beta, IQP_FP32, phi, ldphi, grad, ws, ws_bytes,
+                         stream);
 }
 
 iqp_status iqp_expval_value_and_grad(int64_t n, const uint64_t *G, int64_t m, int64_t ldg, const uint64_t *A,

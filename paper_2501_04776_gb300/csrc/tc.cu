@@ -504,8 +504,8 @@ __global__ void __launch_bounds__(256) k_w_from_phi(const float *__restrict__ ph
 // SIMT kernels' sequential FP32 sums (one- and two-body circuit, n = 300, 1000
 // observables, 10^4 samples: gradient 2.4e-7 relative against 3.2e-6).
 // Three products per contraction, bound like the split form by producing the
-// masked planes: that circuit's autograd step takes 4.4 ms, against 59.5 ms on
-// the FP32 FMA pipe (0.54 of its peak).
+// masked planes: that circuit's autograd step takes 2.9 ms (4.2 with Phi contracted
+// a second time for W), against 59.5 ms on the FP32 FMA pipe (0.54 of its peak).
 struct X3Grid {
     float step, inv;  // 2^E and 2^-E
 };
@@ -580,6 +580,38 @@ __global__ void __launch_bounds__(256) k_x3_theta(const float *__restrict__ thet
     }
     if (wmax != nullptr)
         for (int64_t a = blockIdx.x * (int64_t)256 + threadIdx.x; a < l; a += (int64_t)gridDim.x * 256) wmax[a] = 0u;
+}
+
+// W = sin Phi (alpha + beta cos Phi) (FP32) and its row maxima from a kept Phi, as
+// the phase's own epilogue forms them (MODE 1): 2048 samples of a row per block.
+// W may be Phi itself (ldphi = ldw): each thread replaces what it read. 10^7
+// samples take 20 us, the second contraction they replace 1390 (45150 gates).
+__global__ void __launch_bounds__(256) k_x3_w(const float *phi, int64_t ldphi, float *W, int64_t ldw, int64_t l, int64_t s,
+                                              const double *__restrict__ alpha, const double *__restrict__ beta,
+                                              uint32_t *__restrict__ wmax) {
+    const int64_t per_row = cdiv(s, 2048), total = l * per_row;
+    for (int64_t t = blockIdx.x; t < total; t += gridDim.x) {
+        const int64_t a = t / per_row, i0 = (t - a * per_row) * 2048;
+        const float al = (float)alpha[a], be = beta ? (float)beta[a] : 0.f;
+        float mx = 0.f;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int64_t i = i0 + 1024 * k + 4 * threadIdx.x;  // rows are padded to whole fours
+            if (i >= s || !IQP_IN(a * ldw + i + 3, l * ldw, 64) || !IQP_IN(a * ldphi + i + 3, l * ldphi, 65)) continue;
+            const float4 p = *reinterpret_cast<const float4 *>(phi + a * ldphi + i);
+            float w[4] = {p.x, p.y, p.z, p.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                float sn, cn;
+                sincosf(w[e], &sn, &cn);
+                w[e] = i + e < s ? sn * (al + be * cn) : 0.f;
+                if (fabsf(w[e]) <= 3.4e38f) mx = fmaxf(mx, fabsf(w[e]));
+            }
+            *reinterpret_cast<float4 *>(W + a * ldw + i) = make_float4(w[0], w[1], w[2], w[3]);
+        }
+        const uint32_t mb = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(mx));
+        if ((threadIdx.x & 31) == 0 && mb != 0u) atomicMax(wmax + a, mb);
+    }
 }
 
 // The planes of W (l x ldw BF16 each) from W as FP32 and its row maxima, eight
@@ -2429,7 +2461,21 @@ cudaError_t launch_phase_x3(int mode, const Plan &p, void *ws, const double *alp
     a.limit_ns = default_spin_limit_ns();
     a.serp = phase_serp() ? 1 : 0;
     a.gsum = at<float4>(ws, p.off_xsum);
+    if (mode == 0 && p.phi_out) {  // Phi for the gradient pass
+        a.out = p.phi;
+        a.ldo = p.ldphi;
+    }
     return launch_single_tiles(mode, 2, true, ma, mb, a, a.tiles_m * a.tiles_n, at<float>(ws, p.off_skp), kMaxSplitCtas, st);
+}
+
+// Phase pass of the FP32 form's gradient where Phi was kept.
+cudaError_t launch_x3_w(const Plan &p, void *ws, const double *alpha, const double *beta, cudaStream_t st) {
+    int64_t blocks = p.l * cdiv(p.s, (int64_t)2048);
+    if (blocks > 65536) blocks = 65536;
+    LaunchScope ls(IQP_KERNEL_RECOMPUTE_FP32, st);
+    k_x3_w<<<(unsigned)blocks, 256, 0, st>>>(p.phi, p.ldphi, at<float>(ws, p.off_w), p.ldw, p.l, p.s, alpha, beta,
+                                             at<uint32_t>(ws, p.off_xrow));
+    return cudaGetLastError();
 }
 
 cudaError_t launch_x3_theta(const Plan &p, void *ws, const float *theta, cudaStream_t st) {
