@@ -811,7 +811,7 @@ __global__ void __launch_bounds__(kBlk) k_lo_phase(const uint64_t *__restrict__ 
 // eight table loads per lane, and the lanes' sums of 32 pairs are combined by
 // one reduce-scatter.
 // The loads of X from L2 bound the phase where the observables are wide (n =
-// 5000, 4096 observables of 50 qubits, 16384 samples): 927 us, against 1868 with
+// 5000, 4096 observables of 50 qubits, 16384 samples): 810 us, against 1868 with
 // W in the one-CTA form (18 instructions per qubit and four samples); K 356
 // against 1278.
 // MODE 0: statistics partials, and Phi into phi when it is not null; 1: W; 2:
@@ -894,58 +894,55 @@ __global__ void __launch_bounds__(32 * kLoWarps) k_lo_obs(
                         make_float4(acc[4 * k], acc[4 * k + 1], acc[4 * k + 2], acc[4 * k + 3]);
         }
     }
-    const int64_t left = s - i0;  // sample k of the lane is valid when 128 (k / 4) + k % 4 < left
     const float al = MODE != 0 ? (float)alpha[a] : 0.f;
     const float be = (MODE != 0 && beta) ? (float)beta[a] : 0.f;
-    if (MODE == 0 || MODE == 2) {
-        float cv[32], S[4];
+    // The range's four blocks of 256 samples, in a loop that takes the first eight
+    // phases and moves the others down: 32 copies of the cosine's code missed the
+    // instruction cache for half of the kernel's time (2000 observables x 5000
+    // samples: 51 -> 42 us).
+    int64_t i = i0;
+#pragma unroll 1
+    for (int b = 0; b < 4; ++b, i += 256) {
+        const int64_t left = s - i;  // phase k of the eight is valid when 128 (k / 4) + k % 4 < left
+        float cv[8], S = 0.f;
 #pragma unroll
-        for (int b = 0; b < 4; ++b) S[b] = 0.f;
-#pragma unroll
-        for (int k = 0; k < 32; ++k) {
+        for (int k = 0; k < 8; ++k) {
             const bool valid = 128 * (k / 4) + k % 4 < left;
-            if (MODE == 2) {
+            if (MODE == 0) {
+                cv[k] = valid ? cosf(acc[k]) : 0.f;
+            } else {
                 float sn, cn;
                 sincosf(acc[k], &sn, &cn);
                 cv[k] = valid ? cn : 0.f;
                 acc[k] = valid ? sn * (al + be * cn) : 0.f;  // W
-            } else {
-                cv[k] = valid ? cosf(acc[k]) : 0.f;
             }
-            S[k / 8] += cv[k];
+            S += cv[k];
         }
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {  // the 256-sample blocks of the range
+        if (MODE != 1) {
             const int64_t pb = blk * 4 + b;
 #pragma unroll
-            for (int off = 16; off >= 1; off >>= 1) S[b] += __shfl_xor_sync(kFull, S[b], off);
+            for (int off = 16; off >= 1; off >>= 1) S += __shfl_xor_sync(kFull, S, off);
             const int64_t nbv = s - pb * kBlk < kBlk ? s - pb * kBlk : kBlk;
-            const float mean = nbv > 0 ? S[b] / (float)nbv : 0.f;
+            const float mean = nbv > 0 ? S / (float)nbv : 0.f;
             float M2 = 0.f;
 #pragma unroll
-            for (int k = 8 * b; k < 8 * b + 8; ++k) {
+            for (int k = 0; k < 8; ++k) {
                 const float dv = cv[k] - mean;
                 M2 += 128 * (k / 4) + k % 4 < left ? dv * dv : 0.f;
             }
 #pragma unroll
             for (int off = 16; off >= 1; off >>= 1) M2 += __shfl_xor_sync(kFull, M2, off);
-            if (lane == 0 && pb < nparts) part[a * nparts + pb] = make_double2((double)S[b], (double)M2);
+            if (lane == 0 && pb < nparts) part[a * nparts + pb] = make_double2((double)S, (double)M2);
         }
-    }
-    if (MODE != 0) {
-        if (MODE != 2) {
+        if (MODE != 0) {
 #pragma unroll
-            for (int k = 0; k < 32; ++k) {
-                float sn, cn;
-                sincosf(acc[k], &sn, &cn);
-                acc[k] = 128 * (k / 4) + k % 4 < left ? sn * (al + be * cn) : 0.f;
-            }
+            for (int k = 0; k < 8; k += 4)
+                if (i + 32 * k < lds)
+                    *reinterpret_cast<float4 *>(W + a * lds + i + 32 * k) =
+                        make_float4(acc[k], acc[k + 1], acc[k + 2], acc[k + 3]);
         }
 #pragma unroll
-        for (int k = 0; k < 8; ++k)
-            if (i0 + 128 * k < lds)
-                *reinterpret_cast<float4 *>(W + a * lds + i0 + 128 * k) =
-                    make_float4(acc[4 * k], acc[4 * k + 1], acc[4 * k + 2], acc[4 * k + 3]);
+        for (int k = 0; k < 24; ++k) acc[k] = acc[k + 8];
     }
 }
 
