@@ -643,54 +643,6 @@ __global__ void __launch_bounds__(256) k_x3_wsplit(const float *__restrict__ W, 
 }
 
 // ------------------------------------------------------------------ kernel
-// W hi/lo (BF16 pairs) of 32 consecutive samples i0.. of observable row.
-__device__ __forceinline__ void store_w32(const TcArgs &args, int64_t row, int64_t i0, const uint32_t (&ph)[16],
-                                          const uint32_t (&pl)[16]) {
-    if (!IQP_IN(row * args.ldw + i0, args.l * args.ldw, 43) ||
-        !IQP_IN(row * args.ldw + (i0 + 32 <= args.s ? i0 + 31 : args.s - 1), args.l * args.ldw, 44))
-        return;
-    __nv_bfloat16 *dh = args.whi + row * args.ldw + i0;
-    __nv_bfloat16 *dl = args.wlo + row * args.ldw + i0;
-    if (i0 + 32 <= args.s) {
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            reinterpret_cast<uint4 *>(dh)[v] = make_uint4(ph[4 * v], ph[4 * v + 1], ph[4 * v + 2], ph[4 * v + 3]);
-            reinterpret_cast<uint4 *>(dl)[v] = make_uint4(pl[4 * v], pl[4 * v + 1], pl[4 * v + 2], pl[4 * v + 3]);
-        }
-    } else {
-        uint16_t *sh = reinterpret_cast<uint16_t *>(dh);
-        uint16_t *sl = reinterpret_cast<uint16_t *>(dl);
-        for (int e = 0; e < 32 && i0 + e < args.s; ++e) {
-            sh[e] = (uint16_t)(ph[e / 2] >> ((e & 1) * 16));
-            sl[e] = (uint16_t)(pl[e / 2] >> ((e & 1) * 16));
-        }
-    }
-}
-
-// X3: 32 consecutive W values (FP32) of observable row from sample i0 on into
-// args.wf; returns the largest finite |W| among the samples below s.
-__device__ __forceinline__ float store_wf32(const TcArgs &args, int64_t row, int64_t i0, const uint32_t (&r)[32]) {
-    float mx = 0.f;
-    if (!IQP_IN(row * args.ldw + i0, args.l * args.ldw, 43) ||
-        !IQP_IN(row * args.ldw + (i0 + 32 <= args.s ? i0 + 31 : args.s - 1), args.l * args.ldw, 44))
-        return mx;
-    float *d = args.wf + row * args.ldw + i0;
-#pragma unroll
-    for (int e = 0; e < 32; ++e) {
-        const float v = fabsf(__uint_as_float(r[e]));
-        if (i0 + e < args.s && v <= 3.4e38f) mx = fmaxf(mx, v);
-    }
-    if (i0 + 32 <= args.s) {
-#pragma unroll
-        for (int e = 0; e < 32; e += 4)
-            *reinterpret_cast<float4 *>(d + e) = make_float4(__uint_as_float(r[e]), __uint_as_float(r[e + 1]),
-                                                             __uint_as_float(r[e + 2]), __uint_as_float(r[e + 3]));
-    } else {
-        for (int e = 0; e < 32 && i0 + e < args.s; ++e) d[e] = __uint_as_float(r[e]);
-    }
-    return mx;
-}
-
 // W of eight consecutive samples i.. of observable row: BF16 hi/lo rows, or (X3)
 // FP32, returning the largest finite |W| among those below s.
 __device__ __forceinline__ void store_w8(const TcArgs &args, int64_t row, int64_t i, const float (&w)[8]) {
@@ -737,7 +689,7 @@ __device__ __forceinline__ float store_wf8(const TcArgs &args, int64_t row, int6
 // once for the sum and again for the deviations from the whole group's mean,
 // half of its instructions, with no product under way meanwhile where a CTA pair
 // has one tile (all of k_tc, cold: 255 gates, 8 x 2000: 37.6 -> 18.5 us; 5050
-// gates, 1000 x 1003: 71.6 -> 50.3 us).
+// gates, 784 x 1003: 71.6 -> 50.3 us).
 __device__ __forceinline__ void merge_cos32(const uint32_t (&r)[32], int c, int nvalid, float &S, float &M2) {
     const int n = nvalid - 32 * c < 32 ? nvalid - 32 * c : 32;
     if (n <= 0) return;
@@ -757,6 +709,19 @@ __device__ __forceinline__ void merge_cos32(const uint32_t (&r)[32], int c, int 
     }
     S = s;
     M2 = m2;
+}
+
+// r rotated by eight entries: the epilogues take the cosines of eight columns per
+// turn of a loop, so that its code is one copy of eight, not 32, which the
+// instruction cache holds (k_tc, 255 gates, 8 x 2000: 18.5 -> 14.7 us).
+__device__ __forceinline__ void rotate8(uint32_t (&r)[32]) {
+    uint32_t t[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) t[e] = r[e];
+#pragma unroll
+    for (int e = 0; e < 24; ++e) r[e] = r[e + 8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) r[24 + e] = t[e];
 }
 
 // Values of 32 consecutive columns col0.. of `row`, stored into out
@@ -1376,8 +1341,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                         // instead of a second contraction).
                         if (args.out != nullptr && c * 32 < nvalid && row < args.l)
                             store_out32(args, args.out, row, c0 + c * 32, r);
+#pragma unroll 1
+                        for (int v = 0; v < 4; ++v) {
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(cosf(__uint_as_float(r[e])));
+                            for (int e = 0; e < 8; ++e) r[e] = __float_as_uint(cosf(__uint_as_float(r[e])));
+                            rotate8(r);
+                        }
                         merge_cos32(r, c, (int)nvalid, S, M2);
                     }
                     if (row < args.l && nvalid > 0 && IQP_IN(row * args.nparts + c0 / kGroupCols, args.l * args.nparts, 50))
@@ -1402,16 +1371,17 @@ __global__ void __launch_bounds__(kThreads, 1)
                                         IQP_IN(row * args.ldw + (i0 + 32 <= args.s ? i0 + 31 : args.s - 1),
                                                args.l * args.ldw, 44);
                         // eight columns of W at a time, stored as they are formed
-#pragma unroll
+#pragma unroll 1
                         for (int v = 0; v < 4; ++v) {
                             float w[8];
 #pragma unroll
                             for (int e = 0; e < 8; ++e) {
                                 float sn, cn;
-                                sincosf(__uint_as_float(r[8 * v + e]), &sn, &cn);
-                                r[8 * v + e] = __float_as_uint(cn);
+                                sincosf(__uint_as_float(r[e]), &sn, &cn);
+                                r[e] = __float_as_uint(cn);
                                 w[e] = sn * (al + be * cn);
                             }
+                            rotate8(r);
                             const int64_t i = i0 + 8 * v;
                             if (!in || i >= args.s) continue;
                             if (X3)
@@ -1451,27 +1421,25 @@ __global__ void __launch_bounds__(kThreads, 1)
                     for (int c = 0; c < kGroupLoads; ++c) {
                         ldsum(c, r);
                         const int64_t i0 = c0 + c * 32;
-                        uint32_t ph[16], pl[16];
+                        const bool in = rv && i0 < args.s && IQP_IN(row * args.ldw + i0, args.l * args.ldw, 43) &&
+                                        IQP_IN(row * args.ldw + (i0 + 32 <= args.s ? i0 + 31 : args.s - 1),
+                                               args.l * args.ldw, 44);
+#pragma unroll 1
+                        for (int v = 0; v < 4; ++v) {
+                            float w[8];
 #pragma unroll
-                        for (int e = 0; e < 32; e += 2) {
-                            float s0, k0, s1, k1;
-                            sincosf(__uint_as_float(r[e]), &s0, &k0);
-                            sincosf(__uint_as_float(r[e + 1]), &s1, &k1);
-                            const float w0 = s0 * (al + be * k0), w1 = s1 * (al + be * k1);
-                            if (X3) {  // W stays FP32
-                                r[e] = __float_as_uint(w0);
-                                r[e + 1] = __float_as_uint(w1);
-                                continue;
+                            for (int e = 0; e < 8; ++e) {
+                                float sn, cn;
+                                sincosf(__uint_as_float(r[e]), &sn, &cn);
+                                w[e] = sn * (al + be * cn);
                             }
-                            const float h0 = __bfloat162float(__float2bfloat16_rn(w0));
-                            const float h1 = __bfloat162float(__float2bfloat16_rn(w1));
-                            ph[e / 2] = pack_bf16x2(h0, h1);
-                            pl[e / 2] = pack_bf16x2(w0 - h0, w1 - h1);
-                        }
-                        if (X3) {
-                            if (rv && i0 < args.s) wmax = fmaxf(wmax, store_wf32(args, row, i0, r));
-                        } else if (rv && i0 < args.s) {
-                            store_w32(args, row, i0, ph, pl);
+                            rotate8(r);
+                            const int64_t i = i0 + 8 * v;
+                            if (!in || i >= args.s) continue;
+                            if (X3)
+                                wmax = fmaxf(wmax, store_wf8(args, row, i, w));
+                            else
+                                store_w8(args, row, i, w);
                         }
                     }
                     if (X3 && wmax > 0.f && IQP_IN(row, args.l, 60)) atomicMax(args.wmax + row, __float_as_uint(wmax));
