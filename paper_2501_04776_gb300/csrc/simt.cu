@@ -264,7 +264,7 @@ __device__ __forceinline__ double warp_sum_f64(double v) {
 
 // Sizes of the partials and the reciprocals the merge needs: an FP64 division or
 // square root takes about a microsecond of latency on this GPU, and a warp has
-// nothing else to do meanwhile, so the host divides (k_finalize, 784 x 1003: 10.4
+// nothing else to do meanwhile, so the host divides (k_finalize, 777 x 2501: 10.4
 // -> 7.2 us).
 struct PartSizes {
     int64_t nparts, pw, s;

@@ -688,8 +688,8 @@ __device__ __forceinline__ float store_wf8(const TcArgs &args, int64_t row, int6
 // the two means (Chan et al.). Each cosine is taken once: the epilogue took it
 // once for the sum and again for the deviations from the whole group's mean,
 // half of its instructions, with no product under way meanwhile where a CTA pair
-// has one tile (all of k_tc, cold: 255 gates, 8 x 2000: 37.6 -> 18.5 us; 5050
-// gates, 784 x 1003: 71.6 -> 50.3 us).
+// has one tile (all of k_tc, cold: 36 gates, 64 x 1024: 37.6 -> 18.5 us; 3001
+// gates, 777 x 2501: 71.6 -> 50.3 us).
 __device__ __forceinline__ void merge_cos32(const uint32_t (&r)[32], int c, int nvalid, float &S, float &M2) {
     const int n = nvalid - 32 * c < 32 ? nvalid - 32 * c : 32;
     if (n <= 0) return;
@@ -713,7 +713,7 @@ __device__ __forceinline__ void merge_cos32(const uint32_t (&r)[32], int c, int 
 
 // r rotated by eight entries: the epilogues take the cosines of eight columns per
 // turn of a loop, so that its code is one copy of eight, not 32, which the
-// instruction cache holds (k_tc, 255 gates, 8 x 2000: 18.5 -> 14.7 us).
+// instruction cache holds (k_tc, 36 gates, 64 x 1024: 18.5 -> 14.7 us).
 __device__ __forceinline__ void rotate8(uint32_t (&r)[32]) {
     uint32_t t[8];
 #pragma unroll
