@@ -38,6 +38,7 @@ namespace {
 // c_j = cos(2 theta_j), t_j = -2 tan(2 theta_j), zero beyond m.
 __global__ void k_bitflip_gates(const float *__restrict__ theta, int64_t m, int64_t mpad, double *__restrict__ c,
                                 double *__restrict__ t) {
+    pdl_sync();
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < mpad; j += (int64_t)gridDim.x * blockDim.x) {
         if (j < m) {
             const double x = 2.0 * (double)theta[j];
@@ -75,6 +76,7 @@ __device__ __forceinline__ double block_sum_f64(double v) {
 __global__ void __launch_bounds__(256) k_bf_logs(const float *__restrict__ theta, int64_t m, int64_t mpad,
                                                  double *__restrict__ c, double *__restrict__ t, double *__restrict__ x,
                                                  double *__restrict__ bsum) {
+    pdl_sync();
     double acc = 0.0;
     for (int64_t j = blockIdx.x * (int64_t)256 + threadIdx.x; j < mpad; j += (int64_t)gridDim.x * 256) {
         double cs = 1.0, tn = 0.0, lg = 0.0;
@@ -121,6 +123,7 @@ __global__ void __launch_bounds__(256) k_bf_log_ints(const double *__restrict__ 
                                                      unsigned long long *__restrict__ q,
                                                      unsigned long long *__restrict__ sums, int64_t l,
                                                      int *__restrict__ grid) {
+    pdl_sync();
     const int F = bf_grid(bsum, nb, kBfMaxLog);
     if (blockIdx.x == 0 && threadIdx.x == 0) *grid = F;
     if (F < 0) return;
@@ -139,6 +142,7 @@ __global__ void __launch_bounds__(256) k_bf_value_ints(const double *__restrict_
                                                        unsigned long long *__restrict__ q,
                                                        unsigned long long *__restrict__ sums, int64_t m,
                                                        int *__restrict__ grid, unsigned *__restrict__ counter) {
+    pdl_sync();
     const int F = bf_grid(bsum, nb, 1.7e308);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         *grid = F;
@@ -156,6 +160,7 @@ __global__ void __launch_bounds__(kBfThreads) k_bf_sums(const uint64_t *__restri
                                                         const unsigned long long *__restrict__ q,
                                                         unsigned long long *__restrict__ sums,
                                                         const int *__restrict__ grid) {
+    pdl_sync();
     extern __shared__ unsigned long long tab[];
     if (*grid < 0) return;
     const int64_t w0 = blockIdx.y * (int64_t)(kBfCols / 64);
@@ -197,6 +202,7 @@ __global__ void __launch_bounds__(256) k_bf_rows_out(const unsigned long long *_
                                                      const int *__restrict__ grid, double *__restrict__ expval,
                                                      const double *__restrict__ w, double *__restrict__ v,
                                                      double *__restrict__ bsum) {
+    pdl_sync();
     const int F = *grid;
     double acc = 0.0;
     for (int64_t a = blockIdx.x * (int64_t)256 + threadIdx.x; a < l; a += (int64_t)gridDim.x * 256) {
@@ -232,6 +238,7 @@ __global__ void __launch_bounds__(256) k_bf_grad_out(const unsigned long long *_
                                                      int *__restrict__ grid, const double *__restrict__ t,
                                                      double *__restrict__ grad, double *__restrict__ bnorm,
                                                      double *__restrict__ bt, unsigned *__restrict__ counter) {
+    pdl_sync();
     __shared__ bool last;
     const int F = *reinterpret_cast<volatile int *>(grid);
     if (F < 0) return;  // k_bitflip_grad runs
@@ -273,6 +280,7 @@ __global__ void __launch_bounds__(256) k_bf_grad_out(const unsigned long long *_
 __global__ void __launch_bounds__(256) k_bitflip_rows(const uint64_t *__restrict__ PA, int64_t ldp, int64_t l,
                                                        const double *__restrict__ c, double *__restrict__ expval,
                                                        const int *__restrict__ grid) {
+    pdl_sync();
     if (grid != nullptr && *grid >= 0) return;
     const int lane = threadIdx.x & 31;
     const int64_t a = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -295,6 +303,7 @@ __global__ void __launch_bounds__(256) k_bitflip_rows(const uint64_t *__restrict
 // v[a] = w[a] * expval[a].
 __global__ void k_bitflip_weights(const double *__restrict__ w, const double *__restrict__ ev, int64_t l,
                                   double *__restrict__ v) {
+    pdl_sync();
     const int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (a < l) v[a] = w[a] * ev[a];
 }
@@ -304,6 +313,7 @@ __global__ void __launch_bounds__(256) k_bitflip_grad(const uint64_t *__restrict
                                                        [[maybe_unused]] int64_t l, const double *__restrict__ v,
                                                        const double *__restrict__ t, double *__restrict__ grad,
                                                        const int *__restrict__ grid) {
+    pdl_sync();
     if (grid != nullptr && *grid >= 0) return;
     const int lane = threadIdx.x & 31;
     const int64_t j = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -329,14 +339,14 @@ cudaError_t launch_bitflip_gates(const float *theta, int64_t m, int64_t mpad, do
     int blocks = (int)cdiv(mpad, 256);
     if (blocks > 4096) blocks = 4096;
     LaunchScope ls(IQP_KERNEL_BITFLIP, st);
-    k_bitflip_gates<<<blocks, 256, 0, st>>>(theta, m, mpad, c, t);
+    launch_pdl(k_bitflip_gates, blocks, 256, 0, st, theta, m, mpad, c, t);
     return cudaGetLastError();
 }
 
 cudaError_t launch_bitflip_rows(const uint64_t *PA, int64_t ldp, int64_t l, const double *c, double *expval,
                                 cudaStream_t st) {
     LaunchScope ls(IQP_KERNEL_BITFLIP, st);
-    k_bitflip_rows<<<(unsigned)cdiv(l, 8), 256, 0, st>>>(PA, ldp, l, c, expval, nullptr);
+    launch_pdl(k_bitflip_rows, (unsigned)cdiv(l, 8), 256, 0, st, PA, ldp, l, c, expval, nullptr);
     return cudaGetLastError();
 }
 
@@ -344,12 +354,12 @@ cudaError_t launch_bitflip_grad(const uint64_t *PAT, int64_t ldlt, int64_t m, in
                                 const double *ev, double *v, const double *t, double *grad, cudaStream_t st) {
     {
         LaunchScope ls(IQP_KERNEL_BITFLIP, st);
-        k_bitflip_weights<<<(unsigned)cdiv(l, 256), 256, 0, st>>>(w, ev, l, v);
+        launch_pdl(k_bitflip_weights, (unsigned)cdiv(l, 256), 256, 0, st, w, ev, l, v);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     LaunchScope ls(IQP_KERNEL_BITFLIP, st);
-    k_bitflip_grad<<<(unsigned)cdiv(m, 8), 256, 0, st>>>(PAT, ldlt, m, l, v, t, grad, nullptr);
+    launch_pdl(k_bitflip_grad, (unsigned)cdiv(m, 8), 256, 0, st, PAT, ldlt, m, l, v, t, grad, nullptr);
     return cudaGetLastError();
 }
 
@@ -368,7 +378,7 @@ cudaError_t launch_sums(const uint64_t *bits, int64_t rows, int64_t ld, const un
     }
     const int64_t ny = cdiv(ld, (int64_t)(kBfCols / 64));
     LaunchScope ls(IQP_KERNEL_BITFLIP, st);
-    k_bf_sums<<<dim3((unsigned)cdiv(rows, (int64_t)kBfThreads), (unsigned)ny), kBfThreads, kBfSmem, st>>>(bits, rows, ld, q,
+    launch_pdl(k_bf_sums, dim3((unsigned)cdiv(rows, (int64_t)kBfThreads), (unsigned)ny), kBfThreads, kBfSmem, st, bits, rows, ld, q,
                                                                                                           sums, grid);
     return cudaGetLastError();
 }
@@ -401,39 +411,39 @@ cudaError_t launch_bitflip_ints(const uint64_t *PA, int64_t ldp, const uint64_t 
     cudaError_t e;
     {
         LaunchScope ls(IQP_KERNEL_BITFLIP, st);
-        k_bf_logs<<<nb, 256, 0, st>>>(theta, m, mpad, c, t, x, bsum);
+        launch_pdl(k_bf_logs, nb, 256, 0, st, theta, m, mpad, c, t, x, bsum);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     {
         LaunchScope ls(IQP_KERNEL_BITFLIP, st);
-        k_bf_log_ints<<<nb > nl ? nb : nl, 256, 0, st>>>(x, mpad, bsum, nb, q, sums, l, grid);
+        launch_pdl(k_bf_log_ints, nb > nl ? nb : nl, 256, 0, st, x, mpad, bsum, nb, q, sums, l, grid);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if ((e = launch_sums(PA, l, ldp, q, sums, grid, st)) != cudaSuccess) return e;
     {
         LaunchScope ls(IQP_KERNEL_BITFLIP, st);
-        k_bitflip_rows<<<(unsigned)cdiv(l, 8), 256, 0, st>>>(PA, ldp, l, c, expval, grid);
+        launch_pdl(k_bitflip_rows, (unsigned)cdiv(l, 8), 256, 0, st, PA, ldp, l, c, expval, grid);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     {
         LaunchScope ls(IQP_KERNEL_BITFLIP, st);
-        k_bf_rows_out<<<nl, 256, 0, st>>>(sums, l, grid, expval, w, v, bsum2);
+        launch_pdl(k_bf_rows_out, nl, 256, 0, st, sums, l, grid, expval, w, v, bsum2);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (w == nullptr) return cudaSuccess;
     {
         LaunchScope ls(IQP_KERNEL_BITFLIP, st);
-        k_bf_value_ints<<<nb > nl ? nb : nl, 256, 0, st>>>(v, l, 64 * ldlt, bsum2, nl, q, sums, m, grid2, counter);
+        launch_pdl(k_bf_value_ints, nb > nl ? nb : nl, 256, 0, st, v, l, 64 * ldlt, bsum2, nl, q, sums, m, grid2, counter);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if ((e = launch_sums(PAT, m, ldlt, q, sums, grid2, st)) != cudaSuccess) return e;
     {
         LaunchScope ls(IQP_KERNEL_BITFLIP, st);
-        k_bf_grad_out<<<nb, 256, 0, st>>>(sums, m, l, grid2, t, grad, bsum, bsum2, counter);
+        launch_pdl(k_bf_grad_out, nb, 256, 0, st, sums, m, l, grid2, t, grad, bsum, bsum2, counter);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     LaunchScope ls(IQP_KERNEL_BITFLIP, st);
-    k_bitflip_grad<<<(unsigned)cdiv(m, 8), 256, 0, st>>>(PAT, ldlt, m, l, v, t, grad, grid2);
+    launch_pdl(k_bitflip_grad, (unsigned)cdiv(m, 8), 256, 0, st, PAT, ldlt, m, l, v, t, grad, grid2);
     return cudaGetLastError();
 }
 

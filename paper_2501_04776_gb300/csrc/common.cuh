@@ -249,6 +249,33 @@ __device__ __forceinline__ void theta_prep_one(const float *__restrict__ theta, 
     }
 }
 
+// Programmatic dependent launch: a call is a chain of up to 25 short kernels, and
+// a kernel launched by launch_pdl has its blocks in place (up to pdl_sync, its
+// first statement) while the one before drains. pdl_sync waits until every kernel
+// before is complete and its writes are visible, then lets the next one's blocks
+// come in; a kernel that did not begin with it could run ahead of its inputs, so
+// every kernel that launch_pdl starts does. Low-order MMD step, 2000 x 5000 on 1000
+// qubits: 371 -> 345 us; value and gradient, 3001 gates, 777 x 2501: 118 -> 111 us.
+__device__ __forceinline__ void pdl_sync() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <class... Params, class... Args>
+cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 // Host-side launch accounting (iqp_launch_count) and optional per-kernel
 // event timing (iqp_profile_*). Construct one right before each launch.
 struct LaunchScope {

@@ -76,6 +76,7 @@ __global__ void k_lo_build(const int4 *__restrict__ sup, const float *__restrict
                            unsigned long long *__restrict__ Cfx, unsigned long long *__restrict__ dfx,
                            const unsigned *__restrict__ cmax, unsigned long long *__restrict__ E, int64_t lde, int full,
                            uint32_t *__restrict__ status) {
+    pdl_sync();
     [[maybe_unused]] uint32_t *status_dbg = status;
     const float sc = ldexpf(1.0f, lo_fx_exp(*cmax, m));  // |c_j sc| < 2^62
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
@@ -107,6 +108,7 @@ __global__ void __launch_bounds__(256) k_lo_convert(const unsigned long long *__
                                                     __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo,
                                                     int64_t kc, float *__restrict__ C, int64_t ldc,
                                                     float *__restrict__ d) {
+    pdl_sync();
     __shared__ float tile[64][65];
     const float inv = ldexpf(1.0f, -lo_fx_exp(*cmax, m));
     int bi = 0, left = blockIdx.x;  // block number -> (bi, bj), row by row
@@ -158,6 +160,7 @@ __global__ void __launch_bounds__(256) k_lo_convert(const unsigned long long *__
 // words). One warp per (q, b).
 __global__ void __launch_bounds__(256) k_lo_zpack(const uint32_t *__restrict__ ZT, int64_t ldzt32, int64_t n, int64_t nb,
                                                   uint32_t *__restrict__ ZP) {
+    pdl_sync();
     const int lane = threadIdx.x & 31;
     const int64_t total = n * nb;
     for (int64_t i = (blockIdx.x * (int64_t)256 + threadIdx.x) >> 5; i < total; i += (int64_t)gridDim.x * 8) {
@@ -181,6 +184,7 @@ __global__ void __launch_bounds__(256) k_lo_lists(const uint64_t *__restrict__ A
                                                   const unsigned *__restrict__ cmax, int64_t m, int *__restrict__ Lq,
                                                   uint2 *__restrict__ Lp, int *__restrict__ cnt, int *__restrict__ heavy,
                                                   unsigned *__restrict__ nheavy, uint32_t *__restrict__ status) {
+    pdl_sync();
     [[maybe_unused]] uint32_t *status_dbg = status;
     __shared__ int sq[8][kLoQ];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -281,6 +285,7 @@ __global__ void __launch_bounds__(32) k_lo_cs(const unsigned long long *__restri
                                               const float *__restrict__ C, int64_t ldc,
                                               const float *__restrict__ d, const uint64_t *__restrict__ ZT,
                                               int64_t ldzt, int64_t s, float *__restrict__ M, int64_t lds) {
+    pdl_sync();
     const int lane = threadIdx.x;
     const int64_t q = blockIdx.x, r0 = blockIdx.y;
     const int64_t vwords = cdiv(s, 64);
@@ -348,6 +353,7 @@ __global__ void __launch_bounds__(32) k_lo_h(const unsigned long long *__restric
                                              const uint64_t *__restrict__ ZT, int64_t ldzt,
                                              const float *__restrict__ V, int64_t lds, int64_t s,
                                              float *__restrict__ Hf, int64_t ldh) {
+    pdl_sync();
     __shared__ int rl[kRMax];
     const int lane = threadIdx.x;
     const int64_t q = blockIdx.x;
@@ -640,6 +646,7 @@ __global__ void __launch_bounds__(kBlk) k_lo_phase(const uint64_t *__restrict__ 
                                                    const double *__restrict__ alpha, const double *__restrict__ beta,
                                                    float *__restrict__ W, float *__restrict__ phi, int64_t ldphi,
                                                    uint32_t *__restrict__ status) {
+    pdl_sync();
     [[maybe_unused]] uint32_t *status_dbg = status;
     __shared__ LoShared sh;
     __shared__ const float *mrow[kQ4];  // X + Q[t] lds (four-block form)
@@ -824,6 +831,7 @@ __global__ void __launch_bounds__(32 * kLoWarps) k_lo_obs(
     int64_t nb, const float *__restrict__ X, int64_t lds, int64_t n, int64_t l, int64_t s, int64_t nparts,
     double2 *__restrict__ part, const double *__restrict__ alpha, const double *__restrict__ beta, float *__restrict__ W,
     float *__restrict__ phi, int64_t ldphi, uint32_t *__restrict__ status) {
+    pdl_sync();
     [[maybe_unused]] uint32_t *status_dbg = status;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t a = (int64_t)blockIdx.x * kLoWarps + warp, blk = blockIdx.y;
@@ -952,6 +960,7 @@ __global__ void __launch_bounds__(32 * kLoWarps) k_lo_k(const int *__restrict__ 
                                                         const float *__restrict__ W, int64_t lds, int64_t n, int64_t l,
                                                         const double *__restrict__ scale,
                                                         unsigned long long *__restrict__ Kfx) {
+    pdl_sync();
     extern __shared__ float lo_tab[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t a = (int64_t)blockIdx.x * kLoWarps + warp, blk = blockIdx.y;
@@ -1016,6 +1025,7 @@ __global__ void __launch_bounds__(kBlk) k_lo_v(const uint64_t *__restrict__ AT, 
                                                const float *__restrict__ W, int64_t lds, int64_t s, int64_t nblk,
                                                float *__restrict__ V, __nv_bfloat16 *__restrict__ hi,
                                                __nv_bfloat16 *__restrict__ lo, double *__restrict__ gsp) {
+    pdl_sync();
     __shared__ float red[kBlk / 32];
     __shared__ int obs[kObsMax];
     __shared__ int wsum[kBlk / 32];
@@ -1118,6 +1128,7 @@ __global__ void __launch_bounds__(kBlk) k_lo_v(const uint64_t *__restrict__ AT, 
 __global__ void __launch_bounds__(256) k_lo_w(const float *phi, int64_t ldphi, float *W, int64_t lds, int64_t l,
                                              int64_t s, const double *__restrict__ alpha,
                                              const double *__restrict__ beta) {
+    pdl_sync();
     const int64_t per_row = lds / 4;
     const int64_t total = l * per_row;
     for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < total; g += (int64_t)gridDim.x * blockDim.x) {
@@ -1155,6 +1166,7 @@ __global__ void __launch_bounds__(kBlk) k_lo_pairs(const uint64_t *__restrict__ 
                                                    int64_t nblk, const double *__restrict__ scale,
                                                    unsigned long long *__restrict__ Kfx,
                                                    uint32_t *__restrict__ status) {
+    pdl_sync();
     [[maybe_unused]] uint32_t *status_dbg = status;
     __shared__ LoShared sh;
     __shared__ __align__(16) float wb[4 * kBlk];
@@ -1264,6 +1276,7 @@ __global__ void __launch_bounds__(kBlk) k_lo_pairs(const uint64_t *__restrict__ 
 // they are a cache line each, times the pieces).
 __global__ void __launch_bounds__(256) k_lo_hsum(const float *__restrict__ H, int64_t ldh, int64_t n, int hparts, int nb,
                                                  double *__restrict__ Hs) {
+    pdl_sync();
     __shared__ float2 tile[32][33];
     int bi = 0, left = blockIdx.x;  // block number -> (bi, bj), bi <= bj
     while (left >= nb - bi) {
@@ -1302,6 +1315,7 @@ __global__ void k_lo_grad_out(const int4 *__restrict__ sup, int64_t m, int64_t n
                               const double *__restrict__ Hs,
                               const unsigned long long *__restrict__ Kfx, const double *__restrict__ scale,
                               double *__restrict__ grad) {
+    pdl_sync();
     const double inv = 1.0 / *scale;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
         const int4 sp = sup[j];
@@ -1379,7 +1393,7 @@ cudaError_t launch_obs(const LoArgs &a, double2 *part, const double *alpha, cons
                        int64_t ldphi, cudaStream_t st) {
     const int64_t nb = cdiv(a.s, (int64_t)kLane);
     LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-    k_lo_obs<MODE><<<dim3((unsigned)cdiv(a.l, (int64_t)kLoWarps), (unsigned)nb), 32 * kLoWarps, 0, st>>>(
+    launch_pdl(k_lo_obs<MODE>, dim3((unsigned)cdiv(a.l, (int64_t)kLoWarps), (unsigned)nb), 32 * kLoWarps, 0, st,
         a.cnt, a.Lq, a.Lp, a.ZP, nb, a.X, a.lds, a.n, a.l, a.s, cdiv(a.s, (int64_t)kBlk), part, alpha, beta, W, phi, ldphi,
         a.status);
     return cudaGetLastError();
@@ -1395,7 +1409,7 @@ cudaError_t launch_k(const LoArgs &a, const float *W, cudaStream_t st) {
     }
     const int64_t nb = cdiv(a.s, (int64_t)kLane);
     LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-    k_lo_k<<<dim3((unsigned)cdiv(a.l, (int64_t)kLoWarps), (unsigned)nb), 32 * kLoWarps, smem, st>>>(
+    launch_pdl(k_lo_k, dim3((unsigned)cdiv(a.l, (int64_t)kLoWarps), (unsigned)nb), 32 * kLoWarps, smem, st,
         a.cnt, a.Lp, a.ZP, nb, W, a.lds, a.n, a.l, lo_scale(a), a.fx);
     return cudaGetLastError();
 }
@@ -1405,7 +1419,7 @@ cudaError_t launch_phase(const LoArgs &a, double2 *part, const double *alpha, co
                          int64_t ldphi, cudaStream_t st) {
     const int64_t nblk = cdiv(a.s, (int64_t)kBlk);
     LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-    k_lo_phase<MODE><<<lo_heavy_blocks(a, nblk), kBlk, 0, st>>>(
+    launch_pdl(k_lo_phase<MODE>, lo_heavy_blocks(a, nblk), kBlk, 0, st,
         a.A, a.lda, a.n, a.ZT, a.ldzt, a.X, a.lds, a.fx, lo_cmax(a), a.m, a.E, lo_lde(a.n), a.l, lo_heavy(a), lo_nheavy(a),
         a.s, nblk, part, alpha, beta, W, phi, ldphi, a.status);
     return cudaGetLastError();
@@ -1427,20 +1441,20 @@ cudaError_t launch_lo_prepare(const LoArgs &a, cudaStream_t st) {
     __nv_bfloat16 *hi = a.split, *lo = a.split + n * kc;
     {
         LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-        k_lo_build<<<grid_1d(m), 256, 0, st>>>(a.sup, a.theta, m, n, a.fx, a.fx + n * n, lo_cmax(a), a.E, lde, tc ? 0 : 1,
+        launch_pdl(k_lo_build, grid_1d(m), 256, 0, st, a.sup, a.theta, m, n, a.fx, a.fx + n * n, lo_cmax(a), a.E, lde, tc ? 0 : 1,
                                               a.status);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         const int nb = (int)(kc / 64);
-        k_lo_convert<<<(unsigned)((int64_t)nb * (nb + 1) / 2), 256, 0, st>>>(a.fx, a.fx + n * n, lo_cmax(a), m, n, nb, hi,
+        launch_pdl(k_lo_convert, (unsigned)((int64_t)nb * (nb + 1) / 2), 256, 0, st, a.fx, a.fx + n * n, lo_cmax(a), m, n, nb, hi,
                                                                              lo, kc, tc ? nullptr : a.C, a.ldc, a.d);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (a.ZP != nullptr) {
         LaunchScope ls(IQP_KERNEL_LOWORDER, st);
         const int64_t nb = cdiv(a.s, (int64_t)kLane);
-        k_lo_zpack<<<grid_1d(32 * n * nb), 256, 0, st>>>(reinterpret_cast<const uint32_t *>(a.ZT), 2 * a.ldzt, n, nb, a.ZP);
+        launch_pdl(k_lo_zpack, grid_1d(32 * n * nb), 256, 0, st, reinterpret_cast<const uint32_t *>(a.ZT), 2 * a.ldzt, n, nb, a.ZP);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        k_lo_lists<<<(unsigned)cdiv(a.l, (int64_t)8), 256, 0, st>>>(a.A, a.lda, a.l, n, a.E, lde, a.fx, lo_cmax(a), m, a.Lq,
+        launch_pdl(k_lo_lists, (unsigned)cdiv(a.l, (int64_t)8), 256, 0, st, a.A, a.lda, a.l, n, a.E, lde, a.fx, lo_cmax(a), m, a.Lq,
                                                                     a.Lp, a.cnt, a.cnt + a.l, lo_nheavy(a), a.status);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
@@ -1450,7 +1464,7 @@ cudaError_t launch_lo_prepare(const LoArgs &a, cudaStream_t st) {
         if (e != cudaErrorNotSupported) return e;
     }
     LaunchScope ls(IQP_KERNEL_LOWORDER_GEMM, st);
-    k_lo_cs<<<dim3((unsigned)n, (unsigned)cdiv(a.s, 2048)), 32, 0, st>>>(a.E, lde, a.C, a.ldc, a.d, a.ZT, a.ldzt, a.s, a.X,
+    launch_pdl(k_lo_cs, dim3((unsigned)n, (unsigned)cdiv(a.s, 2048)), 32, 0, st, a.E, lde, a.C, a.ldc, a.d, a.ZT, a.ldzt, a.s, a.X,
                                                                          a.lds);
     return cudaGetLastError();
 }
@@ -1483,7 +1497,7 @@ cudaError_t launch_lo_grad(const LoArgs &a, double2 *part, const double *alpha, 
     if ((e = cudaMemsetAsync(a.fx, 0, (size_t)n * n * sizeof(unsigned long long), st)) != cudaSuccess) return e;
     if (phi != nullptr) {
         LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-        k_lo_w<<<grid_1d(a.l * (a.lds / 4)), 256, 0, st>>>(phi, ldphi, W, a.lds, a.l, s, alpha, beta);
+        launch_pdl(k_lo_w, grid_1d(a.l * (a.lds / 4)), 256, 0, st, phi, ldphi, W, a.lds, a.l, s, alpha, beta);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     } else if (listed) {
         e = part != nullptr ? launch_obs<2>(a, part, alpha, beta, W, nullptr, 0, st)
@@ -1494,7 +1508,7 @@ cudaError_t launch_lo_grad(const LoArgs &a, double2 *part, const double *alpha, 
     __nv_bfloat16 *hi = a.split, *lo = a.split + n * a.lds;
     {
         LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-        k_lo_v<<<dim3((unsigned)n, (unsigned)cdiv(nblk, (int64_t)kGroup)), kBlk, 0, st>>>(
+        launch_pdl(k_lo_v, dim3((unsigned)n, (unsigned)cdiv(nblk, (int64_t)kGroup)), kBlk, 0, st,
             AT, ldlt, a.ZT, a.ldzt, W, a.lds, s, nblk, tc ? nullptr : V, tc ? hi : nullptr, lo, gsp);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
@@ -1505,24 +1519,24 @@ cudaError_t launch_lo_grad(const LoArgs &a, double2 *part, const double *alpha, 
         e = launch_tc_dense(hi, lo, n, a.lds, s, a.ZT, n, a.ldzt, a.H, a.ldc, hparts, nullptr, nullptr, 0, a.status, st);
     } else {
         LaunchScope ls(IQP_KERNEL_LOWORDER_GEMM, st);
-        k_lo_h<<<dim3((unsigned)n, (unsigned)kHSplit), 32, 0, st>>>(a.E, lde, a.ZT, a.ldzt, V, a.lds, s, a.H, a.ldc);
+        launch_pdl(k_lo_h, dim3((unsigned)n, (unsigned)kHSplit), 32, 0, st, a.E, lde, a.ZT, a.ldzt, V, a.lds, s, a.H, a.ldc);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return e;
     {
         LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-        k_lo_pairs<<<lo_heavy_blocks(a, nblk), kBlk, 0, st>>>(a.A, a.lda, n, a.ZT, a.ldzt, a.E, lde, a.l, lo_heavy(a),
+        launch_pdl(k_lo_pairs, lo_heavy_blocks(a, nblk), kBlk, 0, st, a.A, a.lda, n, a.ZT, a.ldzt, a.E, lde, a.l, lo_heavy(a),
                                                               lo_nheavy(a), W, a.lds, s, nblk, lo_scale(a), a.fx, a.status);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (hparts > 1) {
         const int64_t nb = cdiv(n, 32);
         LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-        k_lo_hsum<<<(unsigned)(nb * (nb + 1) / 2), 256, 0, st>>>(a.H, a.ldc, n, hparts, (int)nb, a.Hs);
+        launch_pdl(k_lo_hsum, (unsigned)(nb * (nb + 1) / 2), 256, 0, st, a.H, a.ldc, n, hparts, (int)nb, a.Hs);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-    k_lo_grad_out<<<grid_1d(a.m), 256, 0, st>>>(a.sup, a.m, n, gsp, nblk, a.H, a.ldc, hparts > 1 ? a.Hs : nullptr, a.fx,
+    launch_pdl(k_lo_grad_out, grid_1d(a.m), 256, 0, st, a.sup, a.m, n, gsp, nblk, a.H, a.ldc, hparts > 1 ? a.Hs : nullptr, a.fx,
                                                 lo_scale(a), grad);
     return cudaGetLastError();
 }

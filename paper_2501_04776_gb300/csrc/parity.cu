@@ -30,6 +30,7 @@ __global__ void __launch_bounds__(256) k_parity(int nw32, const uint32_t *__rest
                                                  uint32_t *__restrict__ P, int64_t ldp32, uint32_t *__restrict__ PT,
                                                  int64_t ldpt32, long long *__restrict__ T,
                                                  const int *__restrict__ heavy) {
+    pdl_sync();
     if (MODE == 1 && heavy != nullptr && heavy[blockIdx.y] == 0) return;
     __shared__ __align__(16) uint32_t Rs[kRows][kPad];
     __shared__ __align__(16) uint32_t Gs[kGens][kPad];
@@ -117,6 +118,7 @@ __global__ void __launch_bounds__(1024) k_parity_sum_rows(const uint64_t *__rest
                                                           int64_t n, const uint64_t *__restrict__ XT, int64_t ldxt,
                                                           int64_t N, int limit, long long *__restrict__ T,
                                                           int *__restrict__ heavy, uint32_t *__restrict__ counter) {
+    pdl_sync();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t a = (int64_t)blockIdx.x * 32 + warp;
     const int64_t nw = (n + 63) >> 6;
@@ -306,6 +308,7 @@ __global__ void __launch_bounds__(kTT) k_bit_transpose(const uint32_t *__restric
                                                         int64_t in_cols, int64_t ld_in32,
                                                         uint32_t *__restrict__ out, int64_t ld_out32, int64_t gx,
                                                         int64_t in_bs32, int64_t out_bs32) {
+    pdl_sync();
     __shared__ uint32_t tin[kTT][kTW + 1];  // transposed in place
     bit_transpose_tile(tin, in + (int64_t)blockIdx.y * in_bs32, in_rows, in_cols, ld_in32,
                        out + (int64_t)blockIdx.y * out_bs32, ld_out32, gx, blockIdx.x);
@@ -350,6 +353,7 @@ constexpr int kSlGates = 256;  // gates per support-list block of k_parity_prep
 // us on the GPU and a few on the host).
 __global__ void __launch_bounds__(kTT) k_parity_prep(BitTransposeJob a, BitTransposeJob b, SupportJob g, ThetaJob t,
                                                      int64_t tblocks) {
+    pdl_sync();
     __shared__ __align__(16) uint32_t tin[kTT][kTW + 1];  // transposed in place
     const int64_t bid = blockIdx.x;
     if (bid >= (int64_t)gridDim.x - tblocks) {
@@ -529,6 +533,7 @@ template <typename IT, int V>
 __global__ void __launch_bounds__(V * 32, kGtMinBlocks(V))
     k_gather_transpose(const int4 *__restrict__ sup, const uint64_t *__restrict__ G, int64_t ldg_, int64_t n_,
                        int64_t m_, GatherSide s0, GatherSide s1, int64_t ldp32_, int64_t gx) {
+    pdl_sync();
     const bool second = (int64_t)blockIdx.x >= s0.tiles;
     const uint32_t *__restrict__ RT = second ? s1.RT : s0.RT;
     uint32_t *__restrict__ PT = second ? s1.PT : s0.PT;
@@ -620,6 +625,7 @@ __global__ void __launch_bounds__(V * 32, kGtMinBlocks(V))
 __global__ void __launch_bounds__(256) k_support_gather(const uint64_t *__restrict__ G, int64_t m, int64_t ldg,
                                                          int64_t n, const uint64_t *__restrict__ RT, int64_t ldrt,
                                                          uint64_t *__restrict__ PT, int64_t ldpt) {
+    pdl_sync();
     const int nw = (int)((n + 63) >> 6);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t j = (int64_t)blockIdx.x * 8 + warp;
@@ -663,7 +669,7 @@ cudaError_t bit_transpose(const uint64_t *in, int64_t in_rows, int64_t in_cols, 
     const int64_t gy = cdiv(in_cols, kTT);
     if (gx * gy > 0x7FFFFFFFll) return cudaErrorInvalidValue;
     LaunchScope ls(IQP_KERNEL_PARITY, st);
-    k_bit_transpose<<<(unsigned)(gx * gy), kTT, 0, st>>>(reinterpret_cast<const uint32_t *>(in), in_rows, in_cols,
+    launch_pdl(k_bit_transpose, (unsigned)(gx * gy), kTT, 0, st, reinterpret_cast<const uint32_t *>(in), in_rows, in_cols,
                                                           2 * ld_in, reinterpret_cast<uint32_t *>(out), 2 * ld_out, gx,
                                                           0, 0);
     return cudaGetLastError();
@@ -683,6 +689,7 @@ constexpr int kSuRows = 256, kSuLoads = 8;
 __global__ void __launch_bounds__(256) k_support_rows(const uint64_t *__restrict__ G, int64_t m, int64_t ldg, int64_t n,
                                                       int nu, int R, int4 *__restrict__ sup,
                                                       const float *__restrict__ theta, unsigned *__restrict__ cmax) {
+    pdl_sync();
     __shared__ int cnt[kSuRows], qs[kSuRows][3];
     const int64_t j0 = (int64_t)blockIdx.x * R;
     const int rows = (int)(m - j0 < R ? m - j0 : R);
@@ -761,7 +768,7 @@ cudaError_t launch_bit_transpose_batched(const uint64_t *in, int64_t batch, int6
     for (int64_t b0 = 0; b0 < batch; b0 += 65535) {
         const int64_t nb = batch - b0 < 65535 ? batch - b0 : 65535;
         LaunchScope ls(IQP_KERNEL_PARITY, st);
-        k_bit_transpose<<<dim3((unsigned)(gx * gy), (unsigned)nb), kTT, 0, st>>>(
+        launch_pdl(k_bit_transpose, dim3((unsigned)(gx * gy), (unsigned)nb), kTT, 0, st,
             reinterpret_cast<const uint32_t *>(in + b0 * in_rows * ld_in), in_rows, in_cols, 2 * ld_in,
             reinterpret_cast<uint32_t *>(out + b0 * in_cols * ld_out), 2 * ld_out, gx, 2 * in_rows * ld_in,
             2 * in_cols * ld_out);
@@ -778,7 +785,7 @@ cudaError_t launch_support_list(const uint64_t *G, int64_t m, int64_t ldg, int64
     R = R < 1 ? 1 : (R > kSuRows ? kSuRows : R);
     if (cdiv(m, R) > 0x7FFFFFFFll) return cudaErrorInvalidValue;
     LaunchScope ls(IQP_KERNEL_PARITY, st);
-    k_support_rows<<<(unsigned)cdiv(m, R), 256, 0, st>>>(G, m, ldg, n, (int)nu, (int)R, sup, theta, cmax);
+    launch_pdl(k_support_rows, (unsigned)cdiv(m, R), 256, 0, st, G, m, ldg, n, (int)nu, (int)R, sup, theta, cmax);
     return cudaGetLastError();
 }
 
@@ -812,9 +819,9 @@ cudaError_t launch_gather_transpose(bool i32, int64_t gx, const int4 *sup, const
     if (blocks > 0x7FFFFFFFll) return cudaErrorInvalidValue;
     LaunchScope ls(IQP_KERNEL_PARITY, st);
     if (i32)
-        k_gather_transpose<int32_t, V><<<(unsigned)blocks, V * 32, smem, st>>>(sup, G, ldg, n, m, s0, s1, ldp32, gx);
+        launch_pdl(k_gather_transpose<int32_t, V>, (unsigned)blocks, V * 32, smem, st, sup, G, ldg, n, m, s0, s1, ldp32, gx);
     else
-        k_gather_transpose<int64_t, V><<<(unsigned)blocks, V * 32, smem, st>>>(sup, G, ldg, n, m, s0, s1, ldp32, gx);
+        launch_pdl(k_gather_transpose<int64_t, V>, (unsigned)blocks, V * 32, smem, st, sup, G, ldg, n, m, s0, s1, ldp32, gx);
     return cudaGetLastError();
 }
 
@@ -841,7 +848,7 @@ cudaError_t launch_parity_gather_fused(int64_t n, const uint64_t *G, int64_t m, 
     if (bt[0].tiles + bt[1].tiles + sl_blocks + tblocks > 0x7FFFFFFFll) return cudaErrorInvalidValue;
     {
         LaunchScope ls(IQP_KERNEL_PARITY, st);
-        k_parity_prep<<<(unsigned)(bt[0].tiles + bt[1].tiles + sl_blocks + tblocks), kTT, 0, st>>>(
+        launch_pdl(k_parity_prep, (unsigned)(bt[0].tiles + bt[1].tiles + sl_blocks + tblocks), kTT, 0, st,
             bt[0], bt[1], SupportJob{G, m, ldg, n, sup}, theta, tblocks);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -882,7 +889,7 @@ cudaError_t launch_parity_gather(int64_t n, const uint64_t *R, int64_t rows, int
     {
         dim3 grid((unsigned)cdiv(m, 8), (unsigned)cdiv(ldpt, 256));
         LaunchScope ls(IQP_KERNEL_PARITY, st);
-        k_support_gather<<<grid, 256, 0, st>>>(G, m, ldg, n, RT, ldpt, PT, ldpt);
+        launch_pdl(k_support_gather, grid, 256, 0, st, G, m, ldg, n, RT, ldpt, PT, ldpt);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -904,7 +911,7 @@ cudaError_t launch_parity(int64_t n, const uint64_t *R, int64_t rows, int64_t ld
         const int64_t roff = y0 * kRows;
         const int64_t rrows = rows - roff;
         LaunchScope ls(IQP_KERNEL_PARITY, st);
-        k_parity<0><<<grid, 256, 0, st>>>(nw32, reinterpret_cast<const uint32_t *>(R + roff * ldr), 2 * ldr,
+        launch_pdl(k_parity<0>, grid, 256, 0, st, nw32, reinterpret_cast<const uint32_t *>(R + roff * ldr), 2 * ldr,
                                           rrows, reinterpret_cast<const uint32_t *>(G), 2 * ldg, m,
                                           reinterpret_cast<uint32_t *>(P + roff * ldp), 2 * ldp,
                                           PT ? reinterpret_cast<uint32_t *>(PT) + (roff >> 5) : nullptr, 2 * ldpt,
@@ -931,7 +938,7 @@ cudaError_t launch_parity_sum(int64_t n, const uint64_t *A, int64_t l, int64_t l
         const int64_t roff = y0 * kRows;
         dim3 grid((unsigned)gx, (unsigned)ny);
         LaunchScope ls(IQP_KERNEL_PARITY_SUM, st);
-        k_parity<1><<<grid, 256, 0, st>>>(nw32, reinterpret_cast<const uint32_t *>(A + roff * lda), 2 * lda,
+        launch_pdl(k_parity<1>, grid, 256, 0, st, nw32, reinterpret_cast<const uint32_t *>(A + roff * lda), 2 * lda,
                                           l - roff, reinterpret_cast<const uint32_t *>(X), 2 * ldx, N, nullptr, 0,
                                           nullptr, 0, reinterpret_cast<long long *>(T + roff),
                                           heavy ? heavy + y0 : nullptr);
@@ -951,7 +958,7 @@ cudaError_t launch_parity_sum_rows(int64_t n, const uint64_t *A, int64_t l, int6
     {
         const int limit = (int)(n / 8 > 64 ? n / 8 : 64);
         LaunchScope ls(IQP_KERNEL_PARITY_SUM, st);
-        k_parity_sum_rows<<<(unsigned)cdiv(l, 32), 1024, 0, st>>>(A, l, lda, n, XT, ldxt, N, limit,
+        launch_pdl(k_parity_sum_rows, (unsigned)cdiv(l, 32), 1024, 0, st, A, l, lda, n, XT, ldxt, N, limit,
                                                                   reinterpret_cast<long long *>(T), heavy, counter);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }

@@ -23,6 +23,7 @@ constexpr int BM = 128, BN = 128, BK = 32, PADF = 4;
 // c_j, hi_j and lo_j of theta_prep_one for every j < mpad.
 __global__ void k_theta_prep(const float *__restrict__ theta, int64_t m, int64_t mpad, float *__restrict__ c32,
                              __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo) {
+    pdl_sync();
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < mpad; j += (int64_t)gridDim.x * blockDim.x)
         theta_prep_one(theta, j, m, mpad, c32, hi, lo);
 }
@@ -39,6 +40,7 @@ __global__ void __launch_bounds__(256) k_phase_simt(const uint32_t *__restrict__
                                                      int64_t nparts, const double *__restrict__ alpha,
                                                      const double *__restrict__ beta, float *__restrict__ W,
                                                      int64_t ldw) {
+    pdl_sync();
     __shared__ __align__(16) float As[2][BK][BM + PADF];
     __shared__ __align__(16) float Bs[2][BK][BN + PADF];
     __shared__ float cs[2][BK];
@@ -145,6 +147,7 @@ __global__ void __launch_bounds__(256) k_grad_simt(const float *__restrict__ W, 
                                                     const uint32_t *__restrict__ PZ, const uint32_t *__restrict__ PA,
                                                     int64_t ldp32, int64_t l, int64_t s, int64_t m,
                                                     double *__restrict__ gpart) {
+    pdl_sync();
     __shared__ __align__(16) float As[BK][BM + PADF];
     __shared__ __align__(16) float Bs[BK][BN + PADF];
     __shared__ float red[16][BN];
@@ -300,6 +303,7 @@ __device__ __forceinline__ void merge_partials(const double2 *__restrict__ p, co
 __global__ void __launch_bounds__(256) k_finalize(const double2 *__restrict__ part, PartSizes z, int64_t l,
                                                   double *__restrict__ expval, double *__restrict__ std_err,
                                                   double *__restrict__ S1, double *__restrict__ S2) {
+    pdl_sync();
     const int lane = threadIdx.x & 31;
     const int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (a >= l) return;  // whole warps
@@ -315,6 +319,7 @@ __global__ void __launch_bounds__(256) k_finalize(const double2 *__restrict__ pa
 
 // grad[j] = sum over observable tiles t of gpart[t * m + j], in order.
 __global__ void k_grad_reduce(const double *__restrict__ gpart, int64_t ntiles, int64_t m, double *__restrict__ grad) {
+    pdl_sync();
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
         double t = 0.0;
         for (int64_t k = 0; k < ntiles; ++k) t += gpart[k * m + j];
@@ -330,6 +335,7 @@ __global__ void __launch_bounds__(1024) k_mmd_combine(const long long *__restric
                                                       int unbiased, int sqrt_loss, double *__restrict__ terms,
                                                       double *__restrict__ alpha, double *__restrict__ beta,
                                                       double *__restrict__ loss) {
+    pdl_sync();
     __shared__ double red[1024];
     const double ds = (double)s, dN = (double)N, dl = (double)l;
     double acc = 0.0;
@@ -387,6 +393,7 @@ __global__ void __launch_bounds__(256) k_mmd_terms(const double2 *__restrict__ p
                                                    double *__restrict__ alpha, double *__restrict__ beta,
                                                    double *__restrict__ loss, double *__restrict__ scale,
                                                    uint32_t *__restrict__ counter) {
+    pdl_sync();
     const int lane = threadIdx.x & 31;
     const int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (a < l && IQP_IN(a * z.nparts + z.nparts - 1, l * z.nparts, 30)) {  // whole warps
@@ -450,6 +457,7 @@ __global__ void __launch_bounds__(256) k_mmd_terms(const double2 *__restrict__ p
 
 // alpha_a = -w_a / s for a linear loss given weights (device helper).
 __global__ void k_scale(const double *__restrict__ x, double f, int64_t l, double *__restrict__ y) {
+    pdl_sync();
     const int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (a < l) y[a] = f * x[a];
 }
@@ -461,7 +469,7 @@ cudaError_t launch_theta_prep(const float *theta, int64_t m, int64_t mpad, float
     int blocks = (int)cdiv(mpad, 256);
     if (blocks > 4096) blocks = 4096;
     LaunchScope ls(IQP_KERNEL_THETA_SPLIT, st);
-    k_theta_prep<<<blocks, 256, 0, st>>>(theta, m, mpad, c32, hi, lo);
+    launch_pdl(k_theta_prep, blocks, 256, 0, st, theta, m, mpad, c32, hi, lo);
     return cudaGetLastError();
 }
 
@@ -477,11 +485,11 @@ cudaError_t launch_phase_simt(int mode, const uint64_t *PA, const uint64_t *PZ, 
         const uint32_t *pa = reinterpret_cast<const uint32_t *>(PA + aoff * ldp);
         LaunchScope ls(mode == 0 ? IQP_KERNEL_PHASE_FP32 : IQP_KERNEL_RECOMPUTE_FP32, st);
         if (mode == 0)
-            k_phase_simt<0><<<grid, 256, 0, st>>>(pa, reinterpret_cast<const uint32_t *>(PZ), 2 * ldp, c, l - aoff,
+            launch_pdl(k_phase_simt<0>, grid, 256, 0, st, pa, reinterpret_cast<const uint32_t *>(PZ), 2 * ldp, c, l - aoff,
                                                   s, kwords, part + aoff * nparts, nparts, nullptr, nullptr, nullptr,
                                                   0);
         else
-            k_phase_simt<1><<<grid, 256, 0, st>>>(pa, reinterpret_cast<const uint32_t *>(PZ), 2 * ldp, c, l - aoff,
+            launch_pdl(k_phase_simt<1>, grid, 256, 0, st, pa, reinterpret_cast<const uint32_t *>(PZ), 2 * ldp, c, l - aoff,
                                                   s, kwords, nullptr, 0, alpha + aoff, beta ? beta + aoff : nullptr,
                                                   W + aoff * ldw, ldw);
     }
@@ -496,7 +504,7 @@ cudaError_t launch_grad_simt(const float *W, int64_t ldw, const uint64_t *PZ, co
         const int64_t aoff = y0 * BM;
         dim3 grid((unsigned)cdiv(m, BN), (unsigned)ny);
         LaunchScope ls(IQP_KERNEL_GRAD_FP32, st);
-        k_grad_simt<<<grid, 256, 0, st>>>(W + aoff * ldw, ldw, reinterpret_cast<const uint32_t *>(PZ),
+        launch_pdl(k_grad_simt, grid, 256, 0, st, W + aoff * ldw, ldw, reinterpret_cast<const uint32_t *>(PZ),
                                           reinterpret_cast<const uint32_t *>(PA + aoff * ldp), 2 * ldp, l - aoff, s,
                                           m, gpart + y0 * m);
     }
@@ -512,7 +520,7 @@ PartSizes part_sizes(int64_t nparts, int64_t pw, int64_t s) {
 cudaError_t launch_finalize(const double2 *part, int64_t nparts, int64_t pw, int64_t l, int64_t s, double *expval,
                             double *std_err, double *S1, double *S2, cudaStream_t st) {
     LaunchScope ls(IQP_KERNEL_FINALIZE, st);
-    k_finalize<<<(unsigned)cdiv(l, 8), 256, 0, st>>>(part, part_sizes(nparts, pw, s), l, expval, std_err, S1, S2);
+    launch_pdl(k_finalize, (unsigned)cdiv(l, 8), 256, 0, st, part, part_sizes(nparts, pw, s), l, expval, std_err, S1, S2);
     return cudaGetLastError();
 }
 
@@ -520,7 +528,7 @@ cudaError_t launch_grad_reduce(const double *gpart, int64_t ntiles, int64_t m, d
     int blocks = (int)cdiv(m, 256);
     if (blocks > 8192) blocks = 8192;
     LaunchScope ls(IQP_KERNEL_GRAD_REDUCE, st);
-    k_grad_reduce<<<blocks, 256, 0, st>>>(gpart, ntiles, m, grad);
+    launch_pdl(k_grad_reduce, blocks, 256, 0, st, gpart, ntiles, m, grad);
     return cudaGetLastError();
 }
 
@@ -528,7 +536,7 @@ cudaError_t launch_mmd_combine(const int64_t *T, const double *S1, const double 
                                int unbiased, bool sqrt_loss, double *terms, double *alpha, double *beta, double *loss,
                                cudaStream_t st) {
     LaunchScope ls(IQP_KERNEL_MMD_COMBINE, st);
-    k_mmd_combine<<<1, 1024, 0, st>>>(reinterpret_cast<const long long *>(T), S1, S2, l, s, N, unbiased,
+    launch_pdl(k_mmd_combine, 1, 1024, 0, st, reinterpret_cast<const long long *>(T), S1, S2, l, s, N, unbiased,
                                       sqrt_loss ? 1 : 0, terms, alpha, beta, loss);
     return cudaGetLastError();
 }
@@ -541,7 +549,7 @@ cudaError_t launch_mmd_terms(const double2 *part, int64_t nparts, int64_t pw, co
     const double ds = (double)s, dN = (double)N;
     const MmdConst k{1.0 / ds, 1.0 / dN, 1.0 / (double)l, 1.0 / (ds * (ds - 1.0)), 1.0 / (dN * (dN - 1.0))};
     LaunchScope ls(IQP_KERNEL_MMD_COMBINE, st);
-    k_mmd_terms<<<(unsigned)cdiv(l, 8), 256, 0, st>>>(part, part_sizes(nparts, pw, s),
+    launch_pdl(k_mmd_terms, (unsigned)cdiv(l, 8), 256, 0, st, part, part_sizes(nparts, pw, s),
                                                       reinterpret_cast<const long long *>(T), l, N,
                                                       unbiased, sqrt_loss ? 1 : 0, k, terms, alpha, beta, loss, scale,
                                                       counter);
@@ -550,7 +558,7 @@ cudaError_t launch_mmd_terms(const double2 *part, int64_t nparts, int64_t pw, co
 
 cudaError_t launch_scale(const double *x, double f, int64_t l, double *y, cudaStream_t st) {
     LaunchScope ls(IQP_KERNEL_FINALIZE, st);
-    k_scale<<<(unsigned)cdiv(l, 256), 256, 0, st>>>(x, f, l, y);
+    launch_pdl(k_scale, (unsigned)cdiv(l, 256), 256, 0, st, x, f, l, y);
     return cudaGetLastError();
 }
 

@@ -462,6 +462,7 @@ __global__ void __launch_bounds__(kThreads, MODE == 0 && INDEP ? 2 : 1)
              unsigned long long *__restrict__ gfx, const int4 *__restrict__ sup, const uint64_t *__restrict__ G,
              int64_t ldg, int64_t n, float *__restrict__ phi, int64_t ldphi, int64_t r0,
              int64_t rpc) {
+    pdl_sync();
     extern __shared__ __align__(16) uint8_t sm[];
     int2 *list = reinterpret_cast<int2 *>(sm + kSmList);
     float *tab = reinterpret_cast<float *>(sm + kSmTab);
@@ -627,6 +628,7 @@ __global__ void __launch_bounds__(kThreads, MODE == 0 && INDEP ? 2 : 1)
 __global__ void __launch_bounds__(256) k_sparse_scale(const double *__restrict__ alpha,
                                                       const double *__restrict__ beta, int64_t l, int64_t s,
                                                       double *__restrict__ scale) {
+    pdl_sync();
     __shared__ double red[256];
     double acc = 0.0;
     for (int64_t a = threadIdx.x; a < l; a += 256) acc += fabs(alpha[a]) + (beta ? fabs(beta[a]) : 0.0);
@@ -644,6 +646,7 @@ __global__ void __launch_bounds__(256) k_sparse_scale(const double *__restrict__
 // grad[j] = fixed-point accumulator / scale.
 __global__ void k_sparse_grad_out(const unsigned long long *__restrict__ gfx, int64_t m,
                                   const double *__restrict__ scale, double *__restrict__ grad) {
+    pdl_sync();
     const double inv = 1.0 / *scale;  // a power of two: exact
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x)
         grad[j] = (double)(long long)gfx[j] * inv;
@@ -672,7 +675,7 @@ cudaError_t launch_k(int64_t l, int64_t nparts, int kernel, const uint64_t *PA, 
     for (int64_t r0 = 0; r0 < nparts; r0 += 65535 * rpc) {
         const int64_t nr = cdiv(nparts - r0, rpc) < 65535 ? cdiv(nparts - r0, rpc) : 65535;
         LaunchScope ls(kernel, st);
-        k_sparse<MODE, INDEP><<<dim3((unsigned)l, (unsigned)nr), kThreads, smem, st>>>(
+        launch_pdl(k_sparse<MODE, INDEP>, dim3((unsigned)l, (unsigned)nr), kThreads, smem, st,
             PA, ldp, PZT, ldzt, m, c, s, nparts, part, alpha, beta, scale, gfx, ind ? ind->sup : nullptr,
             ind ? ind->G : nullptr, ind ? ind->ldg : 0, ind ? ind->n : 0, phi, ldphi, r0, rpc);
         const cudaError_t e = cudaGetLastError();
@@ -696,7 +699,7 @@ cudaError_t launch_sparse_value_grad(const uint64_t *PA, int64_t ldp, const uint
     if (e != cudaSuccess) return e;
     {
         LaunchScope ls(IQP_KERNEL_GRAD_SPARSE, st);
-        k_sparse_scale<<<1, 256, 0, st>>>(alpha, beta, l, s, scale);
+        launch_pdl(k_sparse_scale, 1, 256, 0, st, alpha, beta, l, s, scale);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     e = launch_k<2, false>(l, nparts, IQP_KERNEL_PHASE_SPARSE, PA, ldp, PZT, ldzt, m, c, s, part, alpha, beta, scale, gfx,
@@ -705,7 +708,7 @@ cudaError_t launch_sparse_value_grad(const uint64_t *PA, int64_t ldp, const uint
     int blocks = (int)cdiv(m, 256);
     if (blocks > 8192) blocks = 8192;
     LaunchScope ls(IQP_KERNEL_GRAD_SPARSE, st);
-    k_sparse_grad_out<<<blocks, 256, 0, st>>>(gfx, m, scale, grad);
+    launch_pdl(k_sparse_grad_out, blocks, 256, 0, st, gfx, m, scale, grad);
     return cudaGetLastError();
 }
 
@@ -714,7 +717,7 @@ cudaError_t launch_sparse_value_grad(const uint64_t *PA, int64_t ldp, const uint
 cudaError_t launch_fixed_scale(const double *alpha, const double *beta, int64_t l, int64_t s, double *scale,
                                cudaStream_t st) {
     LaunchScope ls(IQP_KERNEL_GRAD_SPARSE, st);
-    k_sparse_scale<<<1, 256, 0, st>>>(alpha, beta, l, s, scale);
+    launch_pdl(k_sparse_scale, 1, 256, 0, st, alpha, beta, l, s, scale);
     return cudaGetLastError();
 }
 
@@ -738,7 +741,7 @@ cudaError_t launch_sparse_grad(const uint64_t *PA, int64_t ldp, const uint64_t *
     if (e != cudaSuccess) return e;
     if (!scale_set) {
         LaunchScope ls(IQP_KERNEL_GRAD_SPARSE, st);
-        k_sparse_scale<<<1, 256, 0, st>>>(alpha, beta, l, s, scale);
+        launch_pdl(k_sparse_scale, 1, 256, 0, st, alpha, beta, l, s, scale);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (indep)
@@ -751,7 +754,7 @@ cudaError_t launch_sparse_grad(const uint64_t *PA, int64_t ldp, const uint64_t *
     int blocks = (int)cdiv(m, 256);
     if (blocks > 8192) blocks = 8192;
     LaunchScope ls(IQP_KERNEL_GRAD_SPARSE, st);
-    k_sparse_grad_out<<<blocks, 256, 0, st>>>(gfx, m, scale, grad);
+    launch_pdl(k_sparse_grad_out, blocks, 256, 0, st, gfx, m, scale, grad);
     return cudaGetLastError();
 }
 

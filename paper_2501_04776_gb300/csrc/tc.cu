@@ -461,6 +461,7 @@ __global__ void __launch_bounds__(256) k_w_from_phi(const float *__restrict__ ph
                                                     const double *__restrict__ alpha,
                                                     const double *__restrict__ beta, __nv_bfloat16 *__restrict__ whi,
                                                     __nv_bfloat16 *__restrict__ wlo) {
+    pdl_sync();
     const int64_t per_row = ldw / 4;
     const int64_t total = l * per_row;
     for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < total; g += (int64_t)gridDim.x * blockDim.x) {
@@ -555,6 +556,7 @@ __device__ __forceinline__ float x3_block_max(const float *__restrict__ theta, i
 }
 
 __global__ void __launch_bounds__(256) k_x3_cmax(const float *__restrict__ theta, int64_t m, float *__restrict__ bmax) {
+    pdl_sync();
     const float v = x3_block_max(theta, m, blockIdx.x * (int64_t)256 + threadIdx.x, (int64_t)gridDim.x * 256);
     if (threadIdx.x == 0) bmax[blockIdx.x] = v;
 }
@@ -567,6 +569,7 @@ __global__ void __launch_bounds__(256) k_x3_theta(const float *__restrict__ thet
                                                   const float *__restrict__ bmax, int nb,
                                                   __nv_bfloat16 *__restrict__ planes, uint32_t *__restrict__ wmax,
                                                   int64_t l) {
+    pdl_sync();
     float mx = 0.f;
     if (nb == 0) mx = x3_block_max(theta, m, threadIdx.x, 256);
     for (int b = 0; b < nb; ++b) mx = fmaxf(mx, bmax[b]);
@@ -589,6 +592,7 @@ __global__ void __launch_bounds__(256) k_x3_theta(const float *__restrict__ thet
 __global__ void __launch_bounds__(256) k_x3_w(const float *phi, int64_t ldphi, float *W, int64_t ldw, int64_t l, int64_t s,
                                               const double *__restrict__ alpha, const double *__restrict__ beta,
                                               uint32_t *__restrict__ wmax) {
+    pdl_sync();
     const int64_t per_row = cdiv(s, 2048), total = l * per_row;
     for (int64_t t = blockIdx.x; t < total; t += gridDim.x) {
         const int64_t a = t / per_row, i0 = (t - a * per_row) * 2048;
@@ -619,6 +623,7 @@ __global__ void __launch_bounds__(256) k_x3_w(const float *phi, int64_t ldphi, f
 // maps end at s).
 __global__ void __launch_bounds__(256) k_x3_wsplit(const float *__restrict__ W, int64_t ldw, int64_t l, int64_t s,
                                                    const uint32_t *__restrict__ wmax, __nv_bfloat16 *__restrict__ planes) {
+    pdl_sync();
     const int64_t per_row = cdiv(s, 8), total = l * per_row;
     for (int64_t t = blockIdx.x * (int64_t)256 + threadIdx.x; t < total; t += (int64_t)gridDim.x * 256) {
         const int64_t a = t / per_row, i0 = (t - a * per_row) * 8;  // ldw is a multiple of 64: whole words
@@ -769,6 +774,7 @@ __device__ __noinline__ void split_store(float *dst, uint32_t tbase, bool chunke
 // time for 45 us of products (1000 observables x 10^4 samples, 45150 gates).
 template <int MODE, bool X3>
 __global__ void __launch_bounds__(256) k_split_reduce(const TcArgs args, int CG, int NH, int64_t tiles) {
+    pdl_sync();
     const int lane = threadIdx.x & 31;
     const int64_t w = (blockIdx.x * (int64_t)256 + threadIdx.x) >> 5;
     const int group = (int)(w & 3), rl = (int)((w >> 2) & (TM - 1));
@@ -862,6 +868,7 @@ template <bool GRAD, int MODE, int CG, bool AT, bool SPL, int TA>
 __global__ void __launch_bounds__(kThreads, 1)
     k_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA2,
          const __grid_constant__ CUtensorMap tmB, const TcArgs args) {
+    pdl_sync();
     constexpr bool ATMA = GRAD || AT;  // A operand by TMA
     // A operand in TMEM, written by the producer warps (phase modes, CTA pairs)
     constexpr bool ATM = TA == 1 && !GRAD && !AT && CG == 2;
@@ -1591,6 +1598,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
     k_grad_pair(const __grid_constant__ CUtensorMap tmWhi, const __grid_constant__ CUtensorMap tmWlo,
                 const __grid_constant__ CUtensorMap tmW3, const __grid_constant__ CUtensorMap tmZt,
                 const GradArgs args) {
+    pdl_sync();
     using C = GCfg<X3>;
     constexpr int GNS = C::NS, GN = C::OBS, GNB = GN / 2;
     extern __shared__ uint8_t smem_raw[];
@@ -2013,7 +2021,7 @@ cudaError_t launch_k(const CUtensorMap &a, const CUtensorMap &a2, const CUtensor
                                : IQP_KERNEL_PHASE_TC,
                    st);
     if constexpr (CL == 1) {
-        k_tc<GRAD, MODE, 1, AT, SPL, TA><<<(unsigned)groups, kThreads, C::SMEM, st>>>(a, a2, b, args);
+        launch_pdl(k_tc<GRAD, MODE, 1, AT, SPL, TA>, (unsigned)groups, kThreads, C::SMEM, st, a, a2, b, args);
         return cudaGetLastError();
     }
     cudaLaunchConfig_t cfg = {};
@@ -2021,13 +2029,15 @@ cudaError_t launch_k(const CUtensorMap &a, const CUtensorMap &a2, const CUtensor
     cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.dynamicSmemBytes = C::SMEM;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = CL;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // the kernel begins with pdl_sync
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, k_tc<GRAD, MODE, CG, AT, SPL, TA>, a, a2, b, args);
 }
 
@@ -2263,13 +2273,13 @@ cudaError_t launch_split_reduce(int mode, bool x3, const TcArgs &a, int cg, int 
                       : (mode == 1 ? IQP_KERNEL_RECOMPUTE_TC : IQP_KERNEL_PHASE_TC),
                    st);
     if (x3) {
-        if (mode == 0) k_split_reduce<0, true><<<blocks, 256, 0, st>>>(a, cg, nh, tiles);
-        else if (mode == 1) k_split_reduce<1, true><<<blocks, 256, 0, st>>>(a, cg, nh, tiles);
-        else k_split_reduce<2, true><<<blocks, 256, 0, st>>>(a, cg, nh, tiles);
+        if (mode == 0) launch_pdl(k_split_reduce<0, true>, blocks, 256, 0, st, a, cg, nh, tiles);
+        else if (mode == 1) launch_pdl(k_split_reduce<1, true>, blocks, 256, 0, st, a, cg, nh, tiles);
+        else launch_pdl(k_split_reduce<2, true>, blocks, 256, 0, st, a, cg, nh, tiles);
     } else {
-        if (mode == 0) k_split_reduce<0, false><<<blocks, 256, 0, st>>>(a, cg, nh, tiles);
-        else if (mode == 1) k_split_reduce<1, false><<<blocks, 256, 0, st>>>(a, cg, nh, tiles);
-        else k_split_reduce<2, false><<<blocks, 256, 0, st>>>(a, cg, nh, tiles);
+        if (mode == 0) launch_pdl(k_split_reduce<0, false>, blocks, 256, 0, st, a, cg, nh, tiles);
+        else if (mode == 1) launch_pdl(k_split_reduce<1, false>, blocks, 256, 0, st, a, cg, nh, tiles);
+        else launch_pdl(k_split_reduce<2, false>, blocks, 256, 0, st, a, cg, nh, tiles);
     }
     return cudaGetLastError();
 }
@@ -2441,7 +2451,7 @@ cudaError_t launch_x3_w(const Plan &p, void *ws, const double *alpha, const doub
     int64_t blocks = p.l * cdiv(p.s, (int64_t)2048);
     if (blocks > 65536) blocks = 65536;
     LaunchScope ls(IQP_KERNEL_RECOMPUTE_FP32, st);
-    k_x3_w<<<(unsigned)blocks, 256, 0, st>>>(p.phi, p.ldphi, at<float>(ws, p.off_w), p.ldw, p.l, p.s, alpha, beta,
+    launch_pdl(k_x3_w, (unsigned)blocks, 256, 0, st, p.phi, p.ldphi, at<float>(ws, p.off_w), p.ldw, p.l, p.s, alpha, beta,
                                              at<uint32_t>(ws, p.off_xrow));
     return cudaGetLastError();
 }
@@ -2452,14 +2462,14 @@ cudaError_t launch_x3_theta(const Plan &p, void *ws, const float *theta, cudaStr
     if (nb > kX3Blocks) nb = kX3Blocks;
     if (nb > 0) {
         LaunchScope ls(IQP_KERNEL_THETA_SPLIT, st);
-        k_x3_cmax<<<(unsigned)nb, 256, 0, st>>>(theta, p.m, bmax);
+        launch_pdl(k_x3_cmax, (unsigned)nb, 256, 0, st, theta, p.m, bmax);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     int64_t blocks = cdiv(p.mpad, 256);
     if (blocks > 4096) blocks = 4096;
     LaunchScope ls(IQP_KERNEL_THETA_SPLIT, st);
-    k_x3_theta<<<(unsigned)blocks, 256, 0, st>>>(theta, p.m, p.mpad, bmax, (int)nb, at<__nv_bfloat16>(ws, p.off_xc),
+    launch_pdl(k_x3_theta, (unsigned)blocks, 256, 0, st, theta, p.m, p.mpad, bmax, (int)nb, at<__nv_bfloat16>(ws, p.off_xc),
                                                  p.off_xw != p.off_xrow ? at<uint32_t>(ws, p.off_xrow) : nullptr, p.l);
     return cudaGetLastError();
 }
@@ -2514,13 +2524,15 @@ cudaError_t launch_grad_pair(const Plan &p, void *ws, cudaStream_t st, iqp_statu
     cfg.blockDim = dim3(kGThreads, 1, 1);
     cfg.dynamicSmemBytes = C::SMEM;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // the kernel begins with pdl_sync
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, k_grad_pair<X3>, mhi, mlo, m3, mz, a);
 }
 }  // namespace
@@ -2539,7 +2551,7 @@ cudaError_t launch_grad_x3(const Plan &p, void *ws, cudaStream_t st, iqp_status 
     if (grid > cap) grid = cap;
     {
         LaunchScope ls(IQP_KERNEL_RECOMPUTE_FP32, st);
-        k_x3_wsplit<<<(unsigned)grid, 256, 0, st>>>(at<float>(ws, p.off_w), p.ldw, p.l, p.s,
+        launch_pdl(k_x3_wsplit, (unsigned)grid, 256, 0, st, at<float>(ws, p.off_w), p.ldw, p.l, p.s,
                                                     at<uint32_t>(ws, p.off_xrow), at<__nv_bfloat16>(ws, p.off_xw));
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -2600,7 +2612,7 @@ cudaError_t launch_w_from_phi(const Plan &p, void *ws, const double *alpha, cons
     if (grid > cap) grid = cap;
     if (grid < 1) grid = 1;
     LaunchScope ls(IQP_KERNEL_RECOMPUTE_TC, st);
-    k_w_from_phi<<<(unsigned)grid, 256, 0, st>>>(p.phi, p.ldphi, p.ldw, p.l, p.s, alpha, beta, whi, wlo);
+    launch_pdl(k_w_from_phi, (unsigned)grid, 256, 0, st, p.phi, p.ldphi, p.ldw, p.l, p.s, alpha, beta, whi, wlo);
     return cudaGetLastError();
 }
 
