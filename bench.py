@@ -386,7 +386,7 @@ def parity_roofline(kt, peaks, n, m, l, s, steps, calls=2, loworder=False):
     ms = kt["parity"]["total_ms"] / max(1, steps)
     hbm = peaks.get("hbm_gbs") or 6800.0
     gbs = nbytes / (ms * 1e-3) / 1e9
-    names = "k_support_list + k_bit_transpose" if loworder else "k_parity_prep + k_gather_transpose"
+    names = "k_support_rows + k_bit_transpose" if loworder else "k_parity_prep + k_gather_transpose"
     return {"bound": "hbm", "kernels": names, "bytes_per_step": nbytes,
             "ms_per_step": round(ms, 4), "achieved": round(gbs, 1), "peak": hbm, "unit": "GB/s",
             "frac": round(gbs / hbm, 4), "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)"}
@@ -460,30 +460,26 @@ def other_rows(args, lib, dev, st, timed, peaks, clocks, G, A, theta, w, n, m, l
     ms, _ = timed(None, args.steps, args.warmup, profile=True, fn=bitflip)
     kt = _kernel_times(lib)
     ldp, ldlt = -(-m // 256) * 4, -(-l // 256) * 4
-    # The product / gradient-sum kernels read P_A (l x ldp words) or P_A^T
-    # (m x ldlt words) once, a small fraction of HBM time; their work is one
-    # FP64 multiply (product over a row's set bits, run by both calls) or add
-    # (gradient sum over a column's set bits) per set bit: 3 nnz(P_A) FP64
-    # operations per call pair, against the FP64 pipe's sustained rate of one
-    # operation per SM per clock (the rate ncu's pipe_fp64 percentages imply
-    # for these DMULs).
+    # The sums of the logarithms (both calls, over P_A) and of the values
+    # (over P_A^T) read one 8-byte entry of a table in shared memory per four
+    # bits, whatever bits are set: 3 l m / 4 of them per call pair, against the
+    # shared memories' 128 bytes per clock. The bits themselves are a small
+    # fraction of HBM time.
     nbytes = 8.0 * (l * ldp + m * ldlt)
-    nnz = nnz_parities(api, n, A, G)
-    fp64_ops = 3.0 * nnz
+    lds_bytes = 2.0 * 64 * (2.0 * l * ldp + m * ldlt)
     bf_ms = kt.get("bitflip", {}).get("total_ms", 0.0) / max(1, args.steps)
     mhz = (clocks or {}).get("sm_max_mhz") or 2070.0
-    fp64_peak = 152 * 1 * mhz * 1e6 / 1e12  # TFLOP/s, one DMUL / DADD per SM per clock
-    ach = fp64_ops / (bf_ms * 1e-3) / 1e12 if bf_ms else None
+    lds_peak = 152 * 128 * mhz * 1e6 / 1e9
+    ach = lds_bytes / (bf_ms * 1e-3) / 1e9 if bf_ms else None
     out["bitflip_fwd_grad"] = {
         "workload": f"bitflip circuit, n={n} m={m} l={l} (the headline's G, A, theta), FP64",
         "ms_per_call_pair": round(statistics.mean(ms), 3), "kernels": kt,
-        "roofline": {"bound": "alu", "kernel": "bitflip (FP64 product and gradient sums)",
-                     "achieved": round(ach, 4) if ach else None, "peak": round(fp64_peak, 4), "unit": "TFLOP/s",
-                     "frac": round(ach / fp64_peak, 4) if ach else None, "fp64_ops_per_call_pair": fp64_ops,
-                     "nnz_PA": nnz, "bytes_per_call_pair": nbytes,
+        "roofline": {"bound": "smem", "kernel": "bitflip (64-bit integer sums from four-bit tables)",
+                     "achieved": round(ach, 1) if ach else None, "peak": round(lds_peak, 1), "unit": "GB/s",
+                     "frac": round(ach / lds_peak, 4) if ach else None, "table_bytes_per_call_pair": lds_bytes,
+                     "bytes_per_call_pair": nbytes,
                      "hbm_frac": round(nbytes / (bf_ms * 1e-3) / 1e9 / hbm, 4) if bf_ms else None,
-                     "peak_source": "FP64 pipe: 152 SMs x 1 operation per clock x max SM clock (from ncu's "
-                                    "sm__inst_executed_pipe_fp64 percentage of peak for k_bitflip_rows)"}}
+                     "peak_source": "shared memory: 152 SMs x 128 bytes x max SM clock"}}
     del ws
 
     # MMD^2 loss and gradient, one training step's call (unbiased form), in
@@ -559,21 +555,38 @@ def alu_peak(clocks, per_lane_per_clock=1):
     return 152 * 128 * per_lane_per_clock * mhz * 1e6 / 1e12
 
 
+def fp32_roofline(lib, kt, n, m, l, s, steps, clocks, peaks):
+    """The FP32 form's slowest contraction, 2 l s m useful flops per step in one or more launches: on the
+    tensor cores (iqp_planes_used) three BF16 products, 6 l s m executed flops; else on the FP32 FMA pipe."""
+    dom = max(("phase_fp32", "recompute_fp32", "grad_fp32"), key=lambda k: kt.get(k, {}).get("total_ms", 0.0))
+    useful = 2.0 * l * s * m
+    sec = kt[dom]["total_ms"] / max(1, steps) * 1e-3
+    if lib.iqp_planes_used(n, m, l, s):
+        peak = peaks.get("bf16_tflops_sustained") or 1700.0
+        ach = 3.0 * useful / sec / 1e12
+        return {"bound": "tensor", "kernel": dom + " (three BF16 planes)", "achieved": round(ach, 1), "peak": peak,
+                "unit": "TFLOP/s", "frac": round(ach / peak, 4), "traffic": None, "flops_per_step": 3.0 * useful,
+                "useful_flops_per_step": useful,
+                "peak_source": "MEASURED_PEAKS.json bf16_tflops_sustained (of measured)"
+                if "bf16_tflops_sustained" in peaks else "fallback 1.7 PFLOP/s sustained (of fallback)"}
+    peak = alu_peak(clocks, 2)
+    ach = useful / sec / 1e12
+    return {"bound": "alu", "kernel": dom, "achieved": round(ach, 2), "peak": round(peak, 1), "unit": "TFLOP/s",
+            "frac": round(ach / peak, 4), "traffic": None, "flops_per_step": useful,
+            "peak_source": "FP32 FMA: 152 SMs x 128 lanes x 2 x max SM clock"}
+
+
 def row_roofline(prec, kt, p, steps, peaks, clocks, api, dev_A, dev_G, step_ms, contractions, fused):
     """Roofline of a row's dominant kernel, by form: split BF16 on the tensor pipe (useful 2 l s m per
-    contraction), FP32 on the FMA pipe (2 l s m per launch), row-sparse on FP32 adds (nnz(P_A) s per pass,
+    contraction), FP32 on it with three products (or on the FMA pipe), row-sparse on FP32 adds (nnz(P_A) s per pass,
     twice in the fused one-pass kernel), low-order on its pair contractions."""
     l, s, m = p.A.shape[0], p.Z.shape[0], p.G.shape[0]
     if prec == "split_bf16":
         dom = max(("phase_tc", "recompute_tc", "grad_tc"), key=lambda k: kt.get(k, {}).get("total_ms", 0.0))
         return split_bf16_roofline(kt, dom, l, s, m, steps, peaks, step_ms, contractions)
     if prec == "fp32":
-        dom = max(("phase_fp32", "recompute_fp32", "grad_fp32"), key=lambda k: kt.get(k, {}).get("total_ms", 0.0))
-        ach = 2.0 * l * s * m / (kt[dom]["avg_ms"] * 1e-3) / 1e12
-        peak = alu_peak(clocks, 2)
-        return {"bound": "alu", "kernel": dom, "achieved": round(ach, 2), "peak": round(peak, 1), "unit": "TFLOP/s",
-                "frac": round(ach / peak, 4), "flops_per_launch": 2.0 * l * s * m,
-                "peak_source": "FP32 FMA: 152 SMs x 128 lanes x 2 x max SM clock"}
+        from paper_2501_04776_gb300 import _lib
+        return fp32_roofline(_lib.load(), kt, p.n, m, l, s, steps, clocks, peaks)
     if prec == "sparse_fp32":
         nnz = nnz_parities(api, p.n, dev_A, dev_G)
         adds = (2 if fused else 1) * nnz * s
@@ -651,16 +664,25 @@ def workload_rows(args, lib, dev, st, timed, peaks, clocks):
                 nb = max(lib.iqp_workspace_bytes(_lib.OP_EXPVAL, n, m, l, s, 0, code),
                          lib.iqp_workspace_bytes(_lib.OP_EXPVAL_GRAD, n, m, l, s, 0, code))
                 ws = torch.zeros(nb, dtype=torch.uint8, device=dev)
-                keep = code in api.KEEP_PHI and not fused
+                planes = code == _lib.FP32 and lib.iqp_planes_used(n, m, l, s) == 1
+                keep = (code in api.KEEP_PHI or planes) and not fused
                 phi = torch.empty((l, api.phi_ld(s)) if keep else (1, 64), dtype=torch.float32, device=dev)
                 args_bits = (n, P(G.data_ptr()), m, G.shape[1], P(A.data_ptr()), l, A.shape[1], P(Z.data_ptr()), s,
                              Z.shape[1], P(th.data_ptr()))
 
-                def call(args_bits=args_bits, code=code, ws=ws, phi=phi, keep=keep):
+                def call(args_bits=args_bits, code=code, ws=ws, phi=phi, keep=keep, planes=planes):
                     if fused:
                         _lib.check(lib.iqp_expval_value_and_grad(*args_bits, P(al.data_ptr()), None, code,
                                                                  P(ev.data_ptr()), P(se.data_ptr()), P(g.data_ptr()),
                                                                  P(ws.data_ptr()), ws.numel(), st), "value_and_grad")
+                    elif keep and planes:
+                        _lib.check(lib.iqp_planes_keep_phi(*args_bits, P(ev.data_ptr()), P(se.data_ptr()),
+                                                           P(phi.data_ptr()), phi.shape[1], P(ws.data_ptr()),
+                                                           ws.numel(), st), "planes_keep_phi")
+                        _lib.check(lib.iqp_planes_grad_from_phi(*args_bits, P(al.data_ptr()), None,
+                                                                P(phi.data_ptr()), phi.shape[1], P(g.data_ptr()),
+                                                                P(ws.data_ptr()), ws.numel(), st),
+                                   "planes_grad_from_phi")
                     elif keep:
                         _lib.check(lib.iqp_expval_keep_phi(*args_bits, code, P(ev.data_ptr()), P(se.data_ptr()),
                                                            P(phi.data_ptr()), phi.shape[1], P(ws.data_ptr()),
@@ -771,8 +793,9 @@ def main():
     ev = torch.empty(l, dtype=torch.float64, device=dev)
     se = torch.empty(l, dtype=torch.float64, device=dev)
     grad = torch.empty(m, dtype=torch.float64, device=dev)
-    nbytes = max(lib.iqp_workspace_bytes(_lib.OP_EXPVAL, n, m, l, s, 0, prec),
-                 lib.iqp_workspace_bytes(_lib.OP_EXPVAL_GRAD, n, m, l, s, 0, prec))
+    # also for the FP32 form timed beside it: short of its planes' regions it would run its SIMT kernels
+    nbytes = max(lib.iqp_workspace_bytes(op, n, m, l, s, 0, pr) for op in (_lib.OP_EXPVAL, _lib.OP_EXPVAL_GRAD)
+                 for pr in (prec, _lib.FP32 if args.fp32_steps else prec))
     ws = torch.zeros(nbytes, dtype=torch.uint8, device=dev)
     flush = torch.empty(L2_FLUSH_BYTES, dtype=torch.uint8, device=dev)
     stream = torch.cuda.current_stream(dev)
@@ -893,13 +916,7 @@ def main():
                 "nnz_PA": nnz, "density_PA": round(nnz / (l * m), 5),
                 "peak_source": "FP32 add: 152 SMs x 128 lanes x max SM clock"}
     else:
-        dom = max(("phase_fp32", "recompute_fp32", "grad_fp32"), key=lambda k: kt.get(k, {}).get("total_ms", 0.0))
-        flops = 2.0 * l * s * m
-        achieved = flops / (kt[dom]["avg_ms"] * 1e-3) / 1e12
-        peak = 152 * 128 * 2 * (clocks or {}).get("sm_mhz", 1425.0) * 1e6 / 1e12
-        roof = {"bound": "alu", "kernel": dom, "achieved": round(achieved, 2), "peak": round(peak, 1),
-                "unit": "TFLOP/s", "frac": round(achieved / peak, 4), "traffic": None,
-                "flops_per_launch": flops, "peak_source": "FP32 FMA: 152 SMs x 128 lanes x 2 x median SM clock"}
+        roof = fp32_roofline(lib, kt, n, m, l, s, args.steps, clocks, peaks)
 
     # The other step form on the same workload (same timing rules).
     other_fn = (lambda: two_call_step(prec)) if args.step == "fused" else (lambda: fused_step(prec))

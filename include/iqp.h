@@ -53,14 +53,17 @@ typedef enum {
 } iqp_status;
 
 /* Arithmetic of the phase contraction Phi = (2 theta . P_A) S_Z^T.
- * IQP_FP32: FP32 FMA on the SIMT cores (the plain form).
+ * IQP_FP32: FP32 accuracy. From 2^23 terms (l s m) on the tensor cores: 2 theta
+ * and W as three BF16 planes each, the first summed exactly (error against
+ * FP64 no larger than FP32 FMAs'); below, FP32 FMA on the SIMT cores.
  * IQP_SPLIT_BF16: tcgen05 tensor cores; 2 theta is split into hi + lo BF16
  * parts (hi = RN_bf16(2 theta), lo = RN_bf16(2 theta - hi)), the +-1 and 0/1
  * operands are exact in BF16, and both products accumulate in FP32 in TMEM.
  * IQP_SPARSE_FP32: row-sparse FP32 form on the SIMT cores: for each
  * observable only the gates with [g_j.a odd] are visited, so the work is
- * nnz(P_A) * s instead of l * m * s; the choice when P_A is sparse (density
- * below a few percent, e.g. low-weight observables drawn with small p_sigma).
+ * nnz(P_A) * s (a fraction of an instruction per term: five gates' signs at a
+ * time) instead of l * m * s; the choice when P_A is sparse (density below a
+ * few percent, e.g. low-weight observables drawn with small p_sigma).
  * Same tolerances as IQP_FP32; its gradient is bitwise reproducible.
  * IQP_LOWORDER_FP32: for generators of weight <= 2 only (one- and two-body
  * gates, e.g. local_gates of Sec. 3.1.1). With s_q(i) = (-1)^{z_iq} the
@@ -212,7 +215,7 @@ iqp_status iqp_expval_grad(int64_t n, const uint64_t *G, int64_t m, int64_t ldg,
  * with the same n, G, A, Z, theta and prec (not re-checked). The gradient
  * call only reads phi.
  * prec: IQP_SPLIT_BF16, IQP_SPARSE_FP32 or IQP_LOWORDER_FP32
- * (IQP_ERR_UNSUPPORTED for IQP_FP32). Errors: phi NULL, ldphi < s or not a
+ * (IQP_ERR_UNSUPPORTED for IQP_FP32, which has the pair below). Errors: phi NULL, ldphi < s or not a
  * multiple of 64 -> IQP_ERR_ARG; phi not 16-byte aligned -> IQP_ERR_ALIGN.
  * ws: iqp_workspace_bytes(IQP_OP_EXPVAL, ...) for the first,
  * iqp_workspace_bytes(IQP_OP_EXPVAL_GRAD, ...) for the second. */
@@ -251,8 +254,8 @@ iqp_status iqp_planes_grad_from_phi(int64_t n, const uint64_t *G, int64_t m, int
  * L = sum_a w_a <Z_a> with alpha_a = -w_a / s, beta = NULL. Outputs as
  * iqp_expval plus grad[m]. The parities are formed once. In IQP_SPLIT_BF16
  * and IQP_SPARSE_FP32 a single pass over Phi yields the statistics and W (no
- * recompute); IQP_LOWORDER_FP32 keeps Phi from its statistics pass for W;
- * IQP_FP32 recomputes it. ws: iqp_workspace_bytes(IQP_OP_EXPVAL_GRAD, ...). */
+ * recompute), so does IQP_FP32 on the tensor cores; IQP_LOWORDER_FP32 keeps
+ * Phi from its statistics pass for W; the SIMT kernels recompute it. ws: iqp_workspace_bytes(IQP_OP_EXPVAL_GRAD, ...). */
 iqp_status iqp_expval_value_and_grad(int64_t n, const uint64_t *G, int64_t m, int64_t ldg,
                                      const uint64_t *A, int64_t l, int64_t lda,
                                      const uint64_t *Z, int64_t s, int64_t ldz, const float *theta,
@@ -287,10 +290,10 @@ iqp_status iqp_mmd_loss(int64_t n, const uint64_t *G, int64_t m, int64_t ldg,
 
 /* Loss as iqp_mmd_loss and its gradient grad[m] in theta, by the chain rule
  * through S1 and S2 (alpha, beta of iqp_expval_grad formed on the device).
- * With IQP_SPLIT_BF16, IQP_SPARSE_FP32 and IQP_LOWORDER_FP32 (shared
- * batches) the call runs one phase contraction: the statistics pass keeps Phi
- * (l x s FP32, in the workspace) and W is formed from it once alpha, beta are
- * known; IQP_FP32 and independent batches recompute Phi for W.
+ * With shared batches the call runs one phase contraction: the statistics
+ * pass keeps Phi (l x s FP32, in the workspace) and W is formed from it once
+ * alpha, beta are known; independent batches and IQP_FP32's SIMT kernels
+ * recompute Phi for W.
  * ws: iqp_workspace_bytes(IQP_OP_MMD_LOSS_GRAD, ...). */
 iqp_status iqp_mmd_loss_grad(int64_t n, const uint64_t *G, int64_t m, int64_t ldg,
                              const uint64_t *A, int64_t l, int64_t lda,
