@@ -55,7 +55,9 @@ typedef enum {
 /* Arithmetic of the phase contraction Phi = (2 theta . P_A) S_Z^T.
  * IQP_FP32: FP32 accuracy. From 2^23 terms (l s m) on the tensor cores: 2 theta
  * and W as three BF16 planes each, the first summed exactly (error against
- * FP64 no larger than FP32 FMAs'); below, FP32 FMA on the SIMT cores.
+ * FP64 no larger than FP32 FMAs', also where a few parameters dominate; where
+ * gates 2^11 times below the mean of thousands of others are an observable's only
+ * ones, its phase is off by up to 2e-6); below, FP32 FMA on the SIMT cores.
  * IQP_SPLIT_BF16: tcgen05 tensor cores; 2 theta is split into hi + lo BF16
  * parts (hi = RN_bf16(2 theta), lo = RN_bf16(2 theta - hi)), the +-1 and 0/1
  * operands are exact in BF16, and both products accumulate in FP32 in TMEM.

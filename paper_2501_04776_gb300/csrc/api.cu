@@ -189,13 +189,13 @@ Plan make_plan(int op, int64_t n, int64_t m, int64_t l, int64_t s, int64_t N, in
     if (prec == IQP_FP32 && !bitflip && !indep) {
         p.off_opt = off;
         p.off_xc = take(3 * p.mpad * 2);
-        p.off_xmax = take(128 * 4);
+        p.off_xsums = take(cdiv(m, (int64_t)kX3Gates) * 4);
         p.off_xpart = take(l * cdiv(s, (int64_t)kPartColsTc) * 16);
         p.off_xrow = take(grad ? l * 4 : 0);
         p.off_xw = take(grad ? 3 * l * p.ldw * 2 : 0);
         p.off_skp = take((int64_t)kMaxSplitCtas * kSplitSlotFloats * 4 + (int64_t)kMaxSplitCtas * 4);
         // running sums: only where the gates take more than one accumulation chunk
-        p.off_xsum = take(m > 65536 ? (int64_t)kMaxSplitCtas * kSplitSlotFloats * 4 : 0);
+        p.off_xsum = take(m > kX3Gates ? (int64_t)kMaxSplitCtas * kSplitSlotFloats * 4 : 0);
         // Below 2^23 terms (and, where a gradient follows, at most 1024
         // samples) the SIMT kernels' few tiles take no longer than the tensor
         // form's launches do: at n = 8, m = 36, l = 64, s = 1024 a step is 0.52 ms of

@@ -28,6 +28,9 @@ constexpr int kSplitSlots = 640;
 // Two-sample-tile phase kernels: the running sums of both accumulators, per
 // CTA (at most kMaxSplitCtas CTAs).
 constexpr int64_t kDtSumFloats = 2 * 128 * 256;
+// FP32 form on the tensor cores: gates per accumulation chunk, and the
+// logarithm of the gradient's samples per chunk (tc.cu, x3_planes).
+constexpr int kX3Gates = 8192, kX3SampleBits = 14;
 
 __host__ __device__ inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 __host__ __device__ inline int64_t round_up(int64_t a, int64_t b) { return cdiv(a, b) * b; }
@@ -53,9 +56,9 @@ struct Plan {
     size_t off_gsum; // split BF16: per-CTA running sums of the two-sample-tile phase kernels (0 if none)
     size_t off_skx;  // split BF16: pieces and counters of the two-tile phase's balanced last round (0 if none)
     // FP32 form on the tensor cores (optional region at the end of the FP32 plan; x3 = it is there and in use):
-    // the three planes of 2 theta, block maxima of |2 theta|, (S, M2) partials of 64 samples, row maxima of |W|, the
+    // the three planes of 2 theta, sums of |2 theta| over blocks of kX3Gates, (S, M2) partials of 64 samples, row maxima of |W|, the
     // three planes of W, running sums (off_skp: the split tiles' scratch)
-    size_t off_xc, off_xmax, off_xpart, off_xrow, off_xw, off_xsum;
+    size_t off_xc, off_xsums, off_xpart, off_xrow, off_xw, off_xsum;
     bool x3;
     size_t off_opt;  // where the optional regions begin (0: none)
     // MMD (optional, at the end): the data transposed (n x ldxt words), marks of the heavy observable blocks, the counter

@@ -492,34 +492,45 @@ __global__ void __launch_bounds__(256) k_w_from_phi(const float *__restrict__ ph
 }
 
 // ---- FP32 form: three BF16 planes of an FP32 value
-// A value x is taken apart on the grid of its operand (2 theta as a whole, or
-// one row of W): plane 0 is x rounded to a multiple of 2^E, an integer of at
-// most 256 in magnitude, so exact in BF16; planes 1 and 2 are the BF16 head
-// and tail of the rest (|rest| <= 2^(E-1)). 2^(E+8) is the power of two above
-// the operand's largest magnitude: the three planes keep x to 2^-26 of that
-// maximum or better, and sums of plane 0 against +-1 stay integers below
-// 2^24 of the grid, which the tensor core's FP32 accumulator holds exactly.
-// So the first plane's products need no accumulation chunks (up to 65536
-// terms), and the truncation of the other two, in an accumulator of their own,
-// is 2^-8 smaller than the sum: against FP64 the results are closer than the
-// SIMT kernels' sequential FP32 sums (one- and two-body circuit, n = 300, 1000
-// observables, 10^4 samples: gradient 2.4e-7 relative against 3.2e-6).
+// A value x is taken apart on the grid 2^E of its operand (2 theta as a whole,
+// or one row of W): plane 0 is x rounded to a multiple of 2^E, or, from 256 grid
+// steps on, to BF16's 8 bits, which is a multiple of 2^E too; planes 1 and 2 are
+// the BF16 head and tail of the rest (at most 2^(E-1) or 2^-9 |x|). E is the
+// least for which the |plane 0| of one accumulation chunk add up to at most 2^24
+// grid steps, so that its sums against +-1 are integers that the tensor core's FP32
+// accumulator holds exactly. The other two planes have an accumulator of their
+// own, which truncates like any, at 2^-9 of the sum where plane 0 holds the values
+// and at the sum itself for the values below the grid.
+// Those decide the chunk and the grid. With one chunk of 65536 gates and
+// 2^E = 2^-8 of the largest |2 theta|, one parameter 500 times the others left them
+// all below the grid. With the sum of |2 theta| over a chunk of 8192 gates in
+// place of the maximum, only values below about 2^-11 of its mean are, and the
+// truncation is an eighth. Measured against FP64 (65536 gates, 256 x 19456, one
+// parameter near pi / 2, the others of 0.003): estimates off by 2.2e-5 -> 1.3e-8, gradient
+// 6.2e-5 -> 1.0e-7; every other parameter large: 1.1e-5 -> 1.3e-8, 6.1e-5 -> 5.1e-7;
+// SIMT kernels 3.7e-8 and 3.9e-6. Values below 2^-11 of the mean have up to 1e-5 relative
+// in a model of the arithmetic (16 terms per step, truncated to 24 bits), in a
+// phase of at most 0.2 (2 theta is at most pi here): 2e-6.
 // Three products per contraction, bound like the split form by producing the
-// masked planes: that circuit's autograd step takes 2.9 ms (4.2 with Phi contracted
-// a second time for W), against 59.5 ms on the FP32 FMA pipe (0.54 of its peak).
+// masked planes (one- and two-body circuit, n = 300, 1000 observables, 10^4
+// samples): its autograd step takes 2.95 ms (2.91 with one chunk; error 1.2e-7),
+// against 59.5 ms on the FP32 FMA pipe (0.54 of its peak; 3.3e-6).
 struct X3Grid {
-    float step, inv;  // 2^E and 2^-E
+    float step, inv, big;  // 2^E, 2^-E, 2^(E+8)
 };
-__device__ __forceinline__ X3Grid x3_grid(float mx) {
-    int e = (int)((__float_as_uint(mx) >> 23) & 255u) - 126;  // mx < 2^e
-    e = e < -100 ? -100 : (e > 120 ? 120 : e);
+// |values| that add up to at most 2^bits bound.
+__device__ __forceinline__ X3Grid x3_grid(float bound, int bits) {
+    int e = (int)((__float_as_uint(bound) >> 23) & 255u) - 126 + bits - 24;  // bound 2^bits < 2^(e + 24)
+    e = e < -104 ? -104 : (e > 104 ? 104 : e);
     X3Grid g;
-    g.step = __uint_as_float((uint32_t)(e - 8 + 127) << 23);
-    g.inv = __uint_as_float((uint32_t)(8 - e + 127) << 23);
+    g.step = __uint_as_float((uint32_t)(e + 127) << 23);
+    g.inv = __uint_as_float((uint32_t)(127 - e) << 23);
+    g.big = 256.f * g.step;
     return g;
 }
 __device__ __forceinline__ void x3_planes(float x, const X3Grid &g, float (&p)[3]) {
-    p[0] = rintf(x * g.inv) * g.step;  // scaling by powers of two and the difference below are exact
+    // scaling by powers of two and both differences are exact
+    p[0] = fabsf(x) >= g.big ? __bfloat162float(__float2bfloat16_rn(x)) : rintf(x * g.inv) * g.step;
     const float rest = x - p[0];
     p[1] = __bfloat162float(__float2bfloat16_rn(rest));
     p[2] = rest - p[1];
@@ -535,45 +546,55 @@ __device__ __forceinline__ float x3_angle(float theta) {
     return (float)(d - 6.283185307179586476925 * rint(d * 0.15915494309189533577));
 }
 
-constexpr int kX3Blocks = 128;   // blocks of the maximum's own pass, one maximum each
-constexpr int kX3Own = 8192;     // up to this many gates every block of the planes' pass takes the maximum itself
-
-// The largest finite |2 theta_j| over j = first, first + step, ... for this thread, reduced over the block.
-__device__ __forceinline__ float x3_block_max(const float *__restrict__ theta, int64_t m, int64_t first, int64_t step) {
+// Sum of the finite |2 theta_j| over the gates first + threadIdx.x, + 256, ... below end, over the block (fixed order).
+__device__ __forceinline__ float x3_block_sum(const float *__restrict__ theta, int64_t first, int64_t end) {
     __shared__ float red[8];
     float v = 0.f;
-    for (int64_t j = first; j < m; j += step) {
+    for (int64_t j = first + threadIdx.x; j < end; j += 256) {
         const float c = fabsf(x3_angle(theta[j]));
-        if (c <= 4.f) v = fmaxf(v, c);
+        if (c <= 4.f) v += c;
     }
 #pragma unroll
-    for (int w = 16; w >= 1; w >>= 1) v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, w));
+    for (int w = 16; w >= 1; w >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, w);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
     v = red[0];
-    for (int w = 1; w < 8; ++w) v = fmaxf(v, red[w]);
+    for (int w = 1; w < 8; ++w) v += red[w];
     return v;
 }
 
-__global__ void __launch_bounds__(256) k_x3_cmax(const float *__restrict__ theta, int64_t m, float *__restrict__ bmax) {
+// bsum[b] = sum of |2 theta| over the gates of block b (kX3Gates of them).
+__global__ void __launch_bounds__(256) k_x3_csum(const float *__restrict__ theta, int64_t m, float *__restrict__ bsum) {
     pdl_sync();
-    const float v = x3_block_max(theta, m, blockIdx.x * (int64_t)256 + threadIdx.x, (int64_t)gridDim.x * 256);
-    if (threadIdx.x == 0) bmax[blockIdx.x] = v;
+    const int64_t j0 = blockIdx.x * (int64_t)kX3Gates;
+    const float v = x3_block_sum(theta, j0, j0 + kX3Gates < m ? j0 + kX3Gates : m);
+    if (threadIdx.x == 0) bsum[blockIdx.x] = v;
 }
 
 // The planes of 2 theta (mpad BF16 each, zero beyond m), on the grid of the
-// block maxima (nb of them; nb = 0: each block takes the maximum itself, which
-// saves a launch where the gates are few). Row maxima wmax (l words, or
-// none) start at zero for the phase that follows.
+// block sums (nb of them; nb = 0: each block takes the sum itself, which saves
+// a launch where the gates are one chunk). A chunk is kX3Gates consecutive
+// gates that may begin anywhere, so it lies in two blocks at most. Row maxima
+// wmax (l words, or none) start at zero for the phase that follows.
 __global__ void __launch_bounds__(256) k_x3_theta(const float *__restrict__ theta, int64_t m, int64_t mpad,
-                                                  const float *__restrict__ bmax, int nb,
+                                                  const float *__restrict__ bsum, int64_t nb,
                                                   __nv_bfloat16 *__restrict__ planes, uint32_t *__restrict__ wmax,
                                                   int64_t l) {
     pdl_sync();
-    float mx = 0.f;
-    if (nb == 0) mx = x3_block_max(theta, m, threadIdx.x, 256);
-    for (int b = 0; b < nb; ++b) mx = fmaxf(mx, bmax[b]);
-    const X3Grid g = x3_grid(mx);
+    float sum = 0.f;
+    if (nb == 0) {
+        sum = x3_block_sum(theta, 0, m);
+    } else {
+        __shared__ uint32_t most;
+        if (threadIdx.x == 0) most = 0u;
+        __syncthreads();
+        float v = 0.f;
+        for (int64_t b = threadIdx.x; b < nb; b += 256) v = fmaxf(v, bsum[b]);
+        atomicMax(&most, __float_as_uint(v));  // non-negative floats order like their bits
+        __syncthreads();
+        sum = 2.f * __uint_as_float(most);
+    }
+    const X3Grid g = x3_grid(1.01f * sum, 0);  // rounding adds 2^-9 and half a step per gate, 2^-12 of 2^24 steps
     for (int64_t j = blockIdx.x * (int64_t)256 + threadIdx.x; j < mpad; j += (int64_t)gridDim.x * 256) {
         float p[3] = {0.f, 0.f, 0.f};
         if (j < m) x3_planes(x3_angle(theta[j]), g, p);
@@ -628,7 +649,7 @@ __global__ void __launch_bounds__(256) k_x3_wsplit(const float *__restrict__ W, 
     for (int64_t t = blockIdx.x * (int64_t)256 + threadIdx.x; t < total; t += (int64_t)gridDim.x * 256) {
         const int64_t a = t / per_row, i0 = (t - a * per_row) * 8;  // ldw is a multiple of 64: whole words
         if (!IQP_IN(a * ldw + i0 + 7, l * ldw, 62)) continue;
-        const X3Grid g = x3_grid(__uint_as_float(wmax[a]));
+        const X3Grid g = x3_grid(__uint_as_float(wmax[a]), kX3SampleBits);
         const float4 u = *reinterpret_cast<const float4 *>(W + a * ldw + i0);
         const float4 v = *reinterpret_cast<const float4 *>(W + a * ldw + i0 + 4);
         const float x[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
@@ -2169,10 +2190,6 @@ bool fp32_tc() {
     return v == 1;
 }
 
-// Gates (samples in the gradient) per accumulation chunk of the FP32 form:
-// plane 0's integers of at most 256 stay below 2^24 over 65536 terms.
-constexpr int64_t kX3Chunk = 65536;
-
 // Every tile whole (no split parts).
 void whole_tiles(TcArgs &a, int64_t ntiles) {
     a.nunits = a.whole = ntiles;
@@ -2418,7 +2435,7 @@ cudaError_t launch_phase_x3(int mode, const Plan &p, void *ws, const double *alp
     a.s = p.s;
     a.m = p.m;
     a.nks = cdiv(p.m, KS);
-    a.chunk = kX3Chunk / KS;
+    a.chunk = cdiv(a.nks, cdiv(a.nks, (int64_t)(kX3Gates / KS)));  // fewest chunks, balanced
     a.tiles_m = cdiv(p.l, 2 * TM);
     a.tiles_n = cdiv(p.s, TN);
     a.group_m = tile_group();
@@ -2457,19 +2474,18 @@ cudaError_t launch_x3_w(const Plan &p, void *ws, const double *alpha, const doub
 }
 
 cudaError_t launch_x3_theta(const Plan &p, void *ws, const float *theta, cudaStream_t st) {
-    float *bmax = at<float>(ws, p.off_xmax);
-    int64_t nb = p.m <= kX3Own ? 0 : cdiv(p.m, 1024);
-    if (nb > kX3Blocks) nb = kX3Blocks;
+    float *bsum = at<float>(ws, p.off_xsums);
+    const int64_t nb = p.m <= kX3Gates ? 0 : cdiv(p.m, (int64_t)kX3Gates);
     if (nb > 0) {
         LaunchScope ls(IQP_KERNEL_THETA_SPLIT, st);
-        launch_pdl(k_x3_cmax, (unsigned)nb, 256, 0, st, theta, p.m, bmax);
+        launch_pdl(k_x3_csum, (unsigned)nb, 256, 0, st, theta, p.m, bsum);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     int64_t blocks = cdiv(p.mpad, 256);
     if (blocks > 4096) blocks = 4096;
     LaunchScope ls(IQP_KERNEL_THETA_SPLIT, st);
-    launch_pdl(k_x3_theta, (unsigned)blocks, 256, 0, st, theta, p.m, p.mpad, bmax, (int)nb, at<__nv_bfloat16>(ws, p.off_xc),
+    launch_pdl(k_x3_theta, (unsigned)blocks, 256, 0, st, theta, p.m, p.mpad, bsum, nb, at<__nv_bfloat16>(ws, p.off_xc),
                                                  p.off_xw != p.off_xrow ? at<uint32_t>(ws, p.off_xrow) : nullptr, p.l);
     return cudaGetLastError();
 }
@@ -2497,7 +2513,7 @@ cudaError_t launch_grad_pair(const Plan &p, void *ws, cudaStream_t st, iqp_statu
     a.s = p.s;
     a.m = p.m;
     a.nks = cdiv(p.s, GKS);
-    const int64_t cmax = (X3 ? kX3Chunk : grad_chunk_samples()) / GKS;
+    const int64_t cmax = (X3 ? (int64_t)1 << kX3SampleBits : grad_chunk_samples()) / GKS;
     a.chunk = cdiv(a.nks, cdiv(a.nks, cmax));  // fewest chunks, balanced
     a.tiles_g = cdiv(p.m, 2 * TM);
     a.tiles_o = cdiv(p.l, (int64_t)C::OBS);
