@@ -370,12 +370,9 @@ int bf_blocks(int64_t n) {
 }
 cudaError_t launch_sums(const uint64_t *bits, int64_t rows, int64_t ld, const unsigned long long *q,
                         unsigned long long *sums, const int *grid, cudaStream_t st) {
-    static bool attr_set = false;
-    if (!attr_set) {
-        const cudaError_t e = cudaFuncSetAttribute(k_bf_sums, cudaFuncAttributeMaxDynamicSharedMemorySize, kBfSmem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static DeviceOnce once;
+    const cudaError_t e = allow_smem(once, k_bf_sums, kBfSmem);
+    if (e != cudaSuccess) return e;
     const int64_t ny = cdiv(ld, (int64_t)(kBfCols / 64));
     LaunchScope ls(IQP_KERNEL_BITFLIP, st);
     launch_pdl(k_bf_sums, dim3((unsigned)cdiv(rows, (int64_t)kBfThreads), (unsigned)ny), kBfThreads, kBfSmem, st, bits, rows, ld, q,

@@ -8,6 +8,7 @@
 #include <stdint.h>
 #include <stddef.h>
 
+#include "device_once.cuh"
 #include "iqp.h"
 
 namespace iqp {
@@ -262,6 +263,17 @@ __device__ __forceinline__ void theta_prep_one(const float *__restrict__ theta, 
 __device__ __forceinline__ void pdl_sync() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Lets `kernel` take `bytes` of dynamic shared memory on the current device (an
+// attribute of the kernel on one device: `once` is the call site's).
+template <class... Params>
+cudaError_t allow_smem(DeviceOnce &once, void (*kernel)(Params...), int bytes) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    return (cudaError_t)once.run(
+        dev, [&] { return (int)cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
 }
 
 template <class... Params, class... Args>

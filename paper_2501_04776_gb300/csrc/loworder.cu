@@ -1404,12 +1404,9 @@ cudaError_t launch_obs(const LoArgs &a, double2 *part, const double *alpha, cons
 
 cudaError_t launch_k(const LoArgs &a, const float *W, cudaStream_t st) {
     constexpr int smem = kLoWarps * kLoTab * 4;
-    static bool attr_set = false;
-    if (!attr_set) {
-        const cudaError_t e = cudaFuncSetAttribute(k_lo_k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static DeviceOnce once;
+    const cudaError_t e = allow_smem(once, k_lo_k, smem);
+    if (e != cudaSuccess) return e;
     const int64_t nb = cdiv(a.s, (int64_t)kLane);
     LaunchScope ls(IQP_KERNEL_LOWORDER, st);
     launch_pdl(k_lo_k, dim3((unsigned)cdiv(a.l, (int64_t)kLoWarps), (unsigned)nb), 32 * kLoWarps, smem, st,

@@ -805,16 +805,10 @@ cudaError_t launch_gather_transpose(bool i32, int64_t gx, const int4 *sup, const
                                     int64_t m, const GatherSide &s0, const GatherSide &s1, int64_t ldp32,
                                     cudaStream_t st) {
     constexpr int smem = gt_smem_bytes(V);
-    static bool attr_set[2] = {false, false};
-    if (!attr_set[i32]) {
-        const cudaError_t e =
-            i32 ? cudaFuncSetAttribute(k_gather_transpose<int32_t, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       smem)
-                : cudaFuncSetAttribute(k_gather_transpose<int64_t, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       smem);
-        if (e != cudaSuccess) return e;
-        attr_set[i32] = true;
-    }
+    static DeviceOnce once[2];
+    const cudaError_t e = i32 ? allow_smem(once[1], k_gather_transpose<int32_t, V>, smem)
+                              : allow_smem(once[0], k_gather_transpose<int64_t, V>, smem);
+    if (e != cudaSuccess) return e;
     const int64_t blocks = s0.tiles + s1.tiles;
     if (blocks > 0x7FFFFFFFll) return cudaErrorInvalidValue;
     LaunchScope ls(IQP_KERNEL_PARITY, st);

@@ -658,13 +658,9 @@ cudaError_t launch_k(int64_t l, int64_t nparts, int kernel, const uint64_t *PA, 
                      const double *beta, const double *scale, unsigned long long *gfx, const SparseIndep *ind, float *phi,
                      int64_t ldphi, cudaStream_t st) {
     constexpr int smem = smem_bytes(MODE != 0, INDEP);
-    static bool attr_set = false;
-    if (!attr_set) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(k_sparse<MODE, INDEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static DeviceOnce once;
+    cudaError_t e = allow_smem(once, k_sparse<MODE, INDEP>, smem);
+    if (e != cudaSuccess) return e;
     // Observables on grid x (the CTAs running at once share a range's P_Z^T
     // segments in L2), ranges on y: a CTA takes as many of them as leave four
     // CTAs per SM, so that J_a is listed once for them all (5% of the time where
@@ -678,7 +674,7 @@ cudaError_t launch_k(int64_t l, int64_t nparts, int kernel, const uint64_t *PA, 
         launch_pdl(k_sparse<MODE, INDEP>, dim3((unsigned)l, (unsigned)nr), kThreads, smem, st,
             PA, ldp, PZT, ldzt, m, c, s, nparts, part, alpha, beta, scale, gfx, ind ? ind->sup : nullptr,
             ind ? ind->G : nullptr, ind ? ind->ldg : 0, ind ? ind->n : 0, phi, ldphi, r0, rpc);
-        const cudaError_t e = cudaGetLastError();
+        e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

@@ -2025,13 +2025,9 @@ cudaError_t launch_k(const CUtensorMap &a, const CUtensorMap &a2, const CUtensor
     constexpr bool kPhasePair = !GRAD && !AT && CG == 2;
     using C = Cfg<CG, GRAD || AT, TA == 1 && kPhasePair, TA == 3 && kPhasePair, TA == 4 && kPhasePair>;
     constexpr int CL = CG;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_tc<GRAD, MODE, CG, AT, SPL, TA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)C::SMEM);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static DeviceOnce once;
+    const cudaError_t e0 = allow_smem(once, k_tc<GRAD, MODE, CG, AT, SPL, TA>, (int)C::SMEM);
+    if (e0 != cudaSuccess) return e0;
     int sms = num_sms();
     if (sms < CL) sms = CL;
     const int64_t groups = args.nunits < sms / CL ? args.nunits : sms / CL;
@@ -2523,13 +2519,9 @@ cudaError_t launch_grad_pair(const Plan &p, void *ws, cudaStream_t st, iqp_statu
     a.gpart = at<double>(ws, p.off_gpart);
     a.status = at<uint32_t>(ws, p.off_status);
     a.limit_ns = default_spin_limit_ns();
-    static bool attr_set = false;
-    if (!attr_set) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(k_grad_pair<X3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static DeviceOnce once;
+    const cudaError_t e0 = allow_smem(once, k_grad_pair<X3>, (int)C::SMEM);
+    if (e0 != cudaSuccess) return e0;
     int sms = num_sms();
     if (sms < 2) sms = 2;
     const int64_t ntiles = a.tiles_g * a.tiles_o;
