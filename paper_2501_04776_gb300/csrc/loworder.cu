@@ -1439,16 +1439,19 @@ cudaError_t launch_lo_prepare(const LoArgs &a, cudaStream_t st) {
     if ((e = launch_support_list(a.G, m, a.ldg, n, a.sup, st, a.theta, lo_cmax(a))) != cudaSuccess) return e;
     if ((e = launch_bit_transpose_batched(a.Z, 1, a.s, n, a.ldz, a.ZT, a.ldzt, st)) != cudaSuccess) return e;
     __nv_bfloat16 *hi = a.split, *lo = a.split + n * kc;
-    {
+    // dense: the contractions' operand; else C itself and both halves of E, for k_lo_cs and k_lo_h
+    auto build = [&](bool dense) {
         LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-        launch_pdl(k_lo_build, grid_1d(m), 256, 0, st, a.sup, a.theta, m, n, a.fx, a.fx + n * n, lo_cmax(a), a.E, lde, tc ? 0 : 1,
-                                              a.status);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        launch_pdl(k_lo_build, grid_1d(m), 256, 0, st, a.sup, a.theta, m, n, a.fx, a.fx + n * n, lo_cmax(a), a.E, lde,
+                   dense ? 0 : 1, a.status);
+        const cudaError_t rc = cudaGetLastError();
+        if (rc != cudaSuccess) return rc;
         const int nb = (int)(kc / 64);
         launch_pdl(k_lo_convert, (unsigned)((int64_t)nb * (nb + 1) / 2), 256, 0, st, a.fx, a.fx + n * n, lo_cmax(a), m, n, nb, hi,
-                                                                             lo, kc, tc ? nullptr : a.C, a.ldc, a.d);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
+                   lo, kc, dense ? nullptr : a.C, a.ldc, a.d);
+        return cudaGetLastError();
+    };
+    if ((e = build(tc)) != cudaSuccess) return e;
     if (a.ZP != nullptr) {
         LaunchScope ls(IQP_KERNEL_LOWORDER, st);
         const int64_t nb = cdiv(a.s, (int64_t)kLane);
@@ -1462,6 +1465,9 @@ cudaError_t launch_lo_prepare(const LoArgs &a, cudaStream_t st) {
     if (tc) {
         e = launch_tc_dense(hi, lo, n, kc, n, a.Z, a.s, a.ldz, a.X, a.lds, 1, a.d, a.ZT, a.ldzt, a.status, st);
         if (e != cudaErrorNotSupported) return e;
+        // No tensor map for Z (rows 2^40 bytes apart): the sums once more, for the kernel that adds them up.
+        if ((e = cudaMemsetAsync(a.fx, 0, (size_t)(n * n + n) * 8, st)) != cudaSuccess) return e;
+        if ((e = build(false)) != cudaSuccess) return e;
     }
     LaunchScope ls(IQP_KERNEL_LOWORDER_GEMM, st);
     launch_pdl(k_lo_cs, dim3((unsigned)n, (unsigned)cdiv(a.s, 2048)), 32, 0, st, a.E, lde, a.C, a.ldc, a.d, a.ZT, a.ldzt, a.s, a.X,
