@@ -106,7 +106,7 @@ struct LoArgs {
     uint2 *Lp;                 // l x kLoP: their pairs with a generator (q | r << 16, bits of -2 C_qr)
     int *cnt;                  // l: qubits | pairs << 16, or -1 for an observable too heavy for the lists; then those
     float *H;                  // hparts x n x ldc
-    double *Hs;                // n x ldc: the pieces' symmetric sum (hparts > 1)
+    double *Hs;                // n x ldc: the pieces' symmetric sum (hparts > 1), or H without the tensor cores
     int hparts;
     uint32_t *status;
 };

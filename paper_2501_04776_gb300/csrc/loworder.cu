@@ -344,7 +344,8 @@ __global__ void __launch_bounds__(32) k_lo_cs(const unsigned long long *__restri
 // H[q][r] = sum_i s_q(i) V[q][i] s_r(i) for r in E_q. Warp (q, k) takes
 // every kHSplit-th set bit of E_q starting at the k-th (listed in shared
 // memory, kRMax at a time) and walks the sample ranges in order, so each
-// H[q][r] is accumulated by one warp alone (fixed order).
+// H[q][r] is accumulated by one warp alone (fixed order, FP32 per range, FP64
+// across ranges).
 constexpr int kHSplit = 8;
 constexpr int kRMax = 1024;
 constexpr int kHPre = 4;
@@ -352,7 +353,7 @@ constexpr int kHPre = 4;
 __global__ void __launch_bounds__(32) k_lo_h(const unsigned long long *__restrict__ E, int64_t lde,
                                              const uint64_t *__restrict__ ZT, int64_t ldzt,
                                              const float *__restrict__ V, int64_t lds, int64_t s,
-                                             float *__restrict__ Hf, int64_t ldh) {
+                                             double *__restrict__ Hd, int64_t ldh) {
     pdl_sync();
     __shared__ int rl[kRMax];
     const int lane = threadIdx.x;
@@ -360,7 +361,7 @@ __global__ void __launch_bounds__(32) k_lo_h(const unsigned long long *__restric
     const int split = blockIdx.y;
     const int64_t vwords = cdiv(s, 64);
     const int64_t nranges = cdiv(vwords, 32);
-    float *hrow = Hf + q * ldh;
+    double *hrow = Hd + q * ldh;
     const unsigned long long *erow = E + q * lde;
     int seen = 0;        // set bits of E_q visited so far
     int64_t w0 = 0;      // next E word to scan
@@ -433,7 +434,7 @@ __global__ void __launch_bounds__(32) k_lo_h(const unsigned long long *__restric
                 float dsum = ((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]));
 #pragma unroll
                 for (int off = 16; off >= 1; off >>= 1) dsum += __shfl_xor_sync(kFull, dsum, off);
-                if (lane == 0) hrow[r] = r0 == 0 ? dsum : hrow[r] + dsum;
+                if (lane == 0) hrow[r] = r0 == 0 ? (double)dsum : hrow[r] + (double)dsum;
                 }
             }
         }
@@ -1309,10 +1310,11 @@ __global__ void __launch_bounds__(256) k_lo_hsum(const float *__restrict__ H, in
     }
 }
 
-// grad_j from the parts above (see the header).
+// grad_j from the parts above (see the header). H: one piece in FP32 (H), the
+// pieces' symmetric sum (Hs), or FP64 sums (Hd).
 __global__ void k_lo_grad_out(const int4 *__restrict__ sup, int64_t m, int64_t n, const double *__restrict__ gsp,
                               int64_t nblk, const float *__restrict__ H, int64_t ldh,
-                              const double *__restrict__ Hs,
+                              const double *__restrict__ Hs, const double *__restrict__ Hd,
                               const unsigned long long *__restrict__ Kfx, const double *__restrict__ scale,
                               double *__restrict__ grad) {
     pdl_sync();
@@ -1330,7 +1332,9 @@ __global__ void k_lo_grad_out(const int4 *__restrict__ sup, int64_t m, int64_t n
             g = 2.0 * t;
         } else if (sp.w == 2) {
             const int64_t q = sp.x, r = sp.y;
-            const double h = Hs != nullptr ? Hs[q * ldh + r] : (double)H[q * ldh + r] + (double)H[r * ldh + q];
+            const double h = Hs != nullptr   ? Hs[q * ldh + r]
+                             : Hd != nullptr ? Hd[q * ldh + r] + Hd[r * ldh + q]
+                                             : (double)H[q * ldh + r] + (double)H[r * ldh + q];
             g = fma((double)(long long)Kfx[q * n + r], inv, h + h);  // 2 h - 4 k, rounded once
         }
         grad[j] = g;
@@ -1525,7 +1529,7 @@ cudaError_t launch_lo_grad(const LoArgs &a, double2 *part, const double *alpha, 
         e = launch_tc_dense(hi, lo, n, a.lds, s, a.ZT, n, a.ldzt, a.H, a.ldc, hparts, nullptr, nullptr, 0, a.status, st);
     } else {
         LaunchScope ls(IQP_KERNEL_LOWORDER_GEMM, st);
-        launch_pdl(k_lo_h, dim3((unsigned)n, (unsigned)kHSplit), 32, 0, st, a.E, lde, a.ZT, a.ldzt, V, a.lds, s, a.H, a.ldc);
+        launch_pdl(k_lo_h, dim3((unsigned)n, (unsigned)kHSplit), 32, 0, st, a.E, lde, a.ZT, a.ldzt, V, a.lds, s, a.Hs, a.ldc);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return e;
@@ -1542,8 +1546,8 @@ cudaError_t launch_lo_grad(const LoArgs &a, double2 *part, const double *alpha, 
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-    launch_pdl(k_lo_grad_out, grid_1d(a.m), 256, 0, st, a.sup, a.m, n, gsp, nblk, a.H, a.ldc, hparts > 1 ? a.Hs : nullptr, a.fx,
-                                                lo_scale(a), grad);
+    launch_pdl(k_lo_grad_out, grid_1d(a.m), 256, 0, st, a.sup, a.m, n, gsp, nblk, a.H, a.ldc, hparts > 1 ? a.Hs : nullptr,
+               tc ? nullptr : a.Hs, a.fx, lo_scale(a), grad);
     return cudaGetLastError();
 }
 
