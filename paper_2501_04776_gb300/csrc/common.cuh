@@ -32,6 +32,14 @@ constexpr int64_t kDtSumFloats = 2 * 128 * 256;
 // FP32 form on the tensor cores: gates per accumulation chunk, and the
 // logarithm of the gradient's samples per chunk (tc.cu, x3_planes).
 constexpr int kX3Gates = 8192, kX3SampleBits = 14;
+// Observables whose W is held as three planes at a time: all of them up to 2 GiB
+// (3.5e8 samples of W), else whole tiles of 128, so that the FP32 form's scratch stays near the 4 bytes
+// per sample that W itself takes.
+constexpr int64_t kX3PlaneBytes = (int64_t)1 << 31;
+__host__ __device__ inline int64_t x3_rows(int64_t l, int64_t ldw) {
+    const int64_t r = kX3PlaneBytes / (6 * ldw) / kATile * kATile, most = r < kATile ? kATile : r;
+    return l < most ? l : most;
+}
 
 __host__ __device__ inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 __host__ __device__ inline int64_t round_up(int64_t a, int64_t b) { return cdiv(a, b) * b; }

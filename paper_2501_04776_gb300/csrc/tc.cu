@@ -2487,17 +2487,18 @@ cudaError_t launch_x3_theta(const Plan &p, void *ws, const float *theta, cudaStr
 }
 
 namespace {
+// Observables o0 .. o0 + l (X3: the planes hold these alone; else all).
 template <bool X3>
-cudaError_t launch_grad_pair(const Plan &p, void *ws, cudaStream_t st, iqp_status *why) {
+cudaError_t launch_grad_pair(const Plan &p, void *ws, int64_t o0, int64_t l, cudaStream_t st, iqp_status *why) {
     using C = GCfg<X3>;
     CUtensorMap mhi, mlo, m3, mz;
     const __nv_bfloat16 *whi = at<__nv_bfloat16>(ws, X3 ? p.off_xw : p.off_w);
-    const __nv_bfloat16 *wlo = whi + p.l * p.ldw;
-    if (!make_map(&mhi, whi, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, p.s, p.l, p.ldw * 2, KS, GNB,
+    const __nv_bfloat16 *wlo = whi + l * p.ldw;
+    if (!make_map(&mhi, whi, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, p.s, l, p.ldw * 2, KS, GNB,
                   CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map(&mlo, wlo, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, p.s, p.l, p.ldw * 2, KS, GNB,
+        !make_map(&mlo, wlo, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, p.s, l, p.ldw * 2, KS, GNB,
                   CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map(&m3, X3 ? wlo + p.l * p.ldw : wlo, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, p.s, p.l, p.ldw * 2, KS, 64,
+        !make_map(&m3, X3 ? wlo + l * p.ldw : wlo, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, p.s, l, p.ldw * 2, KS, 64,
                   CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map(&mz, at<uint64_t>(ws, p.off_pzt), CU_TENSOR_MAP_DATA_TYPE_UINT64, p.ldzt, p.m, p.ldzt * 8, 4, TM,
                   CU_TENSOR_MAP_SWIZZLE_NONE)) {
@@ -2505,18 +2506,18 @@ cudaError_t launch_grad_pair(const Plan &p, void *ws, cudaStream_t st, iqp_statu
         return cudaErrorNotSupported;
     }
     GradArgs a;
-    a.l = p.l;
+    a.l = l;
     a.s = p.s;
     a.m = p.m;
     a.nks = cdiv(p.s, GKS);
     const int64_t cmax = (X3 ? (int64_t)1 << kX3SampleBits : grad_chunk_samples()) / GKS;
     a.chunk = cdiv(a.nks, cdiv(a.nks, cmax));  // fewest chunks, balanced
     a.tiles_g = cdiv(p.m, 2 * TM);
-    a.tiles_o = cdiv(p.l, (int64_t)C::OBS);
+    a.tiles_o = cdiv(l, (int64_t)C::OBS);
     a.group_o = grad_group() * (GN / C::OBS);
-    a.pat32 = at<uint32_t>(ws, p.off_pat);
+    a.pat32 = at<uint32_t>(ws, p.off_pat) + o0 / 32;  // whole tiles of 128 observables end inside a row
     a.ldlt32 = 2 * p.ldlt;
-    a.gpart = at<double>(ws, p.off_gpart);
+    a.gpart = at<double>(ws, p.off_gpart) + 2 * (o0 / C::OBS) * p.m;
     a.status = at<uint32_t>(ws, p.off_status);
     a.limit_ns = default_spin_limit_ns();
     static DeviceOnce once;
@@ -2551,24 +2552,30 @@ cudaError_t launch_grad_pair(const Plan &p, void *ws, cudaStream_t st, iqp_statu
 int64_t grad_tc_rows(const Plan &p) { return cta_group() == 2 && grad_pair() ? 2 * cdiv(p.l, GN) : cdiv(p.l, TM); }
 
 // The FP32 form's gradient contraction (p.x3): W taken apart into its planes,
-// then k_grad_pair<true>; 2 ceil(l / 128) rows of partials.
+// then k_grad_pair<true>, for as many observables at a time as the planes hold; 2
+// ceil(l / 128) rows of partials.
 cudaError_t launch_grad_x3(const Plan &p, void *ws, cudaStream_t st, iqp_status *why) {
-    const int64_t total = p.l * cdiv(p.s, (int64_t)8);
-    int64_t grid = cdiv(total, 256);
-    const int64_t cap = (int64_t)num_sms() * 8;
-    if (grid > cap) grid = cap;
-    {
-        LaunchScope ls(IQP_KERNEL_RECOMPUTE_FP32, st);
-        launch_pdl(k_x3_wsplit, (unsigned)grid, 256, 0, st, at<float>(ws, p.off_w), p.ldw, p.l, p.s,
-                                                    at<uint32_t>(ws, p.off_xrow), at<__nv_bfloat16>(ws, p.off_xw));
-        const cudaError_t e = cudaGetLastError();
+    const int64_t rows = x3_rows(p.l, p.ldw);
+    for (int64_t o0 = 0; o0 < p.l; o0 += rows) {
+        const int64_t l = p.l - o0 < rows ? p.l - o0 : rows;
+        int64_t grid = cdiv(l * cdiv(p.s, (int64_t)8), 256);
+        const int64_t cap = (int64_t)num_sms() * 8;
+        if (grid > cap) grid = cap;
+        {
+            LaunchScope ls(IQP_KERNEL_RECOMPUTE_FP32, st);
+            launch_pdl(k_x3_wsplit, (unsigned)grid, 256, 0, st, at<float>(ws, p.off_w) + o0 * p.ldw, p.ldw, l, p.s,
+                       at<uint32_t>(ws, p.off_xrow) + o0, at<__nv_bfloat16>(ws, p.off_xw));
+            const cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
+        }
+        const cudaError_t e = launch_grad_pair<true>(p, ws, o0, l, st, why);
         if (e != cudaSuccess) return e;
     }
-    return launch_grad_pair<true>(p, ws, st, why);
+    return cudaSuccess;
 }
 
 cudaError_t launch_grad_tc(const Plan &p, void *ws, cudaStream_t st, iqp_status *why) {
-    if (cta_group() == 2 && grad_pair()) return launch_grad_pair<false>(p, ws, st, why);
+    if (cta_group() == 2 && grad_pair()) return launch_grad_pair<false>(p, ws, 0, p.l, st, why);
     const int cg = 1;
     CUtensorMap mhi, mlo, mb;
     const __nv_bfloat16 *whi = at<__nv_bfloat16>(ws, p.off_w);
