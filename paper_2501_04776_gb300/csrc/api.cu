@@ -150,7 +150,9 @@ Plan make_plan(int op, int64_t n, int64_t m, int64_t l, int64_t s, int64_t N, in
     p.off_pat = take(lo ? 0 : m * p.ldlt * 8);
     p.off_rt = take(n * (p.ldzt + p.ldlt) * 8);  // R^T of A, then of Z (one fused parity launch for both)
     p.off_c = take(bitflip ? p.mpad * 16 : p.mpad * 4);  // bitflip: cos(2 theta), -2 tan(2 theta) in FP64
-    p.off_part = take(bitflip ? l * 16 : l * p.nparts * 16);  // bitflip: expval, w * expval
+    // bitflip: expval, w * expval; row-sparse: half as many of twice the samples, where a workspace has no room for all
+    // at the end (check_ws)
+    p.off_part = p.off_part2 = take(bitflip ? l * 16 : l * (p.prec == IQP_SPARSE_FP32 ? cdiv(p.nparts, 2) : p.nparts) * 16);
     p.off_w = take(grad && !sparse ? l * p.ldw * 4 : 0);
     p.off_lo_c = take(lo ? (n + 1) * p.ldc * 4 + n * cdiv(n, 64) * 8 : 0);  // C, d, pair-existence bits E
     p.off_lo_m = take(lo ? n * p.ldw * 4 : 0);
@@ -226,6 +228,11 @@ Plan make_plan(int op, int64_t n, int64_t m, int64_t l, int64_t s, int64_t N, in
     if (bitflip && bitflip_ints(m, l)) {
         p.off_opt = off;
         p.off_bf = take(8 * bitflip_int_words(m, l));
+    }
+    // Row-sparse: partials of one range each.
+    if (sparse && p.nparts > 1) {
+        p.off_opt = off;
+        p.off_part = take(l * p.nparts * 16);
     }
     // MMD: scratch of the data parities by row gather (a workspace that ends
     // before its end folds them densely).
@@ -367,6 +374,11 @@ iqp_status check_ws(Plan &p, void *ws, size_t ws_bytes) {
         p.x3 = false;  // FP32: the SIMT kernels
         p.off_xt = 0;  // data parities folded densely
         p.off_bf = 0;
+        if (p.off_part != p.off_part2 && ws_bytes < p.off_part + (size_t)round_up(p.l * p.nparts * 16, 256)) {
+            p.off_part = p.off_part2;
+            p.nparts = cdiv(p.nparts, 2);
+            p.pw *= 2;
+        }
         p.off_lo_zp = p.off_lo_hp = 0;  // low-order: no lists, H in one piece
         // The optional regions at the end, in order: each is used only where
         // the workspace reaches its end.

@@ -77,6 +77,7 @@ struct Plan {
     // low-order lists (optional): lane-ordered sample bits, the observables' qubits, pairs and counts
     size_t off_lo_zp, off_lo_q, off_lo_p, off_lo_cnt, off_lo_hp;
     size_t off_bf;   // bitflip (optional): scratch of the integer sums
+    size_t off_part2;  // row-sparse: room for half as many partials (off_part: optional, all of them)
     bool scale_set;  // the gradient's fixed-point scale is in place already (set with the MMD terms)
     size_t off_phi;  // MMD gradient (split BF16, row-sparse): room for Phi, l x ldw fp32 (0 if none)
     // Kept Phi (l x ldphi fp32, ldphi a multiple of 64 >= s; the layout is the

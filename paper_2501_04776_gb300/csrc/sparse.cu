@@ -35,7 +35,8 @@
 // backward: 1.43 -> 0.51 ms.
 //
 // Statistics: (sum cos, sum (cos - mean)^2) partials of 1024 samples (FP32
-// within a warp, FP64 across warps), merged by the shared finaliser.
+// within a warp, FP64 across warps), merged by the shared finaliser; where the
+// workspace has room for half as many, a CTA takes pairs of ranges and merges their two.
 // Gradient sums: the per-range dot products are added into a 64-bit fixed-point
 // accumulator per gate with integer atomics. Integer addition is associative,
 // so the result does not depend on the order of the atomics: the gradient is
@@ -454,6 +455,7 @@ __device__ __forceinline__ double block_sum(float v, float *red) {
 // each, observable a at PZT + a n ldzt) and the parities are formed on the fly.
 // phi: element e = 32-sample position k, lane q of a range's nl valid lanes at
 // range start + k nl + q.
+// nparts: ranges of 1024 samples; pair: partials of 2048 (rpc and r0 are even).
 template <int MODE, bool INDEP>
 __global__ void __launch_bounds__(kThreads, MODE == 0 && INDEP ? 2 : 1)
     k_sparse(const uint64_t *__restrict__ PA, int64_t ldp, const uint64_t *__restrict__ PZT, int64_t ldzt,
@@ -461,7 +463,7 @@ __global__ void __launch_bounds__(kThreads, MODE == 0 && INDEP ? 2 : 1)
              const double *__restrict__ alpha, const double *__restrict__ beta, const double *__restrict__ scale,
              unsigned long long *__restrict__ gfx, const int4 *__restrict__ sup, const uint64_t *__restrict__ G,
              int64_t ldg, int64_t n, float *__restrict__ phi, int64_t ldphi, int64_t r0,
-             int64_t rpc) {
+             int64_t rpc, int pair) {
     pdl_sync();
     extern __shared__ __align__(16) uint8_t sm[];
     int2 *list = reinterpret_cast<int2 *>(sm + kSmList);
@@ -569,7 +571,22 @@ __global__ void __launch_bounds__(kThreads, MODE == 0 && INDEP ? 2 : 1)
             m2 += valid[h] ? d * d : 0.f;
         }
         const double M2 = block_sum(m2, redf);
-        if (tid == 0 && IQP_IN(a * nparts + r, l * nparts, 75)) part[a * nparts + r] = make_double2(S, M2);
+        if (tid == 0 && !pair) {
+            if (IQP_IN(a * nparts + r, l * nparts, 75)) part[a * nparts + r] = make_double2(S, M2);
+        } else if (tid == 0) {
+            double *held = reinterpret_cast<double *>(red + 32);  // the even range's
+            if ((r & 1) != 0) {  // Chan et al.: the even range has all its samples
+                const double nk = (double)(left < kRange ? left : kRange), d = S / nk - held[0] / kRange;
+                held[1] += M2 + d * d * (kRange * nk / (kRange + nk));
+                held[0] += S;
+            } else {
+                held[0] = S;
+                held[1] = M2;
+            }
+            const int64_t np = (nparts + 1) / 2;
+            if (((r & 1) != 0 || r + 1 == nparts) && IQP_IN(a * np + r / 2, l * np, 75))
+                part[a * np + r / 2] = make_double2(held[0], held[1]);
+        }
     }
     if (MODE != 0) {
         const float al = (float)alpha[a];
@@ -652,8 +669,9 @@ __global__ void k_sparse_grad_out(const unsigned long long *__restrict__ gfx, in
         grad[j] = (double)(long long)gfx[j] * inv;
 }
 
+// npart: partials per observable, one per range or per two.
 template <int MODE, bool INDEP>
-cudaError_t launch_k(int64_t l, int64_t nparts, int kernel, const uint64_t *PA, int64_t ldp, const uint64_t *PZT,
+cudaError_t launch_k(int64_t l, int64_t npart, int kernel, const uint64_t *PA, int64_t ldp, const uint64_t *PZT,
                      int64_t ldzt, int64_t m, const float *c, int64_t s, double2 *part, const double *alpha,
                      const double *beta, const double *scale, unsigned long long *gfx, const SparseIndep *ind, float *phi,
                      int64_t ldphi, cudaStream_t st) {
@@ -665,15 +683,18 @@ cudaError_t launch_k(int64_t l, int64_t nparts, int kernel, const uint64_t *PA, 
     // segments in L2), ranges on y: a CTA takes as many of them as leave four
     // CTAs per SM, so that J_a is listed once for them all (5% of the time where
     // P_A's density is 0.008), at most 65535 blocks per launch.
+    const int64_t nparts = cdiv(s, (int64_t)kRange);
+    const bool pair = part != nullptr && npart < nparts;
     int64_t rpc = l * nparts / (4 * (int64_t)num_sms() + 1);
     rpc = rpc < 1 ? 1 : (rpc > nparts ? nparts : rpc);
     rpc = cdiv(nparts, cdiv(nparts, rpc));  // equal shares
+    if (pair) rpc = round_up(rpc, 2);
     for (int64_t r0 = 0; r0 < nparts; r0 += 65535 * rpc) {
         const int64_t nr = cdiv(nparts - r0, rpc) < 65535 ? cdiv(nparts - r0, rpc) : 65535;
         LaunchScope ls(kernel, st);
         launch_pdl(k_sparse<MODE, INDEP>, dim3((unsigned)l, (unsigned)nr), kThreads, smem, st,
             PA, ldp, PZT, ldzt, m, c, s, nparts, part, alpha, beta, scale, gfx, ind ? ind->sup : nullptr,
-            ind ? ind->G : nullptr, ind ? ind->ldg : 0, ind ? ind->n : 0, phi, ldphi, r0, rpc);
+            ind ? ind->G : nullptr, ind ? ind->ldg : 0, ind ? ind->n : 0, phi, ldphi, r0, rpc, pair ? 1 : 0);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
