@@ -111,6 +111,17 @@ typedef enum {
 size_t iqp_workspace_bytes(iqp_op op, int64_t n, int64_t m, int64_t l, int64_t s, int64_t N,
                            iqp_precision prec);
 
+/* Bytes of the smallest workspace that `op` runs with: iqp_workspace_bytes less
+ * its optional end. Beside IQP_SPLIT_BF16's parts that is, where a form has them:
+ * IQP_FP32's planes (without: FP32 FMA on the SIMT cores), IQP_SPARSE_FP32's
+ * partials of 1024 samples (without: of 2048), IQP_LOWORDER_FP32's lists and
+ * the pieces of its pair contraction (without: one CTA per observable, one
+ * piece), the bitflip model's integers (without: FP64 products and sums), the
+ * transposed data of the MMD losses (without: every data row folded).
+ * 0 for invalid sizes. Host only. */
+size_t iqp_workspace_min_bytes(iqp_op op, int64_t n, int64_t m, int64_t l, int64_t s, int64_t N,
+                               iqp_precision prec);
+
 /* GF(2) products of Sec. 2.2 (A.G^T and Z.G^T mod 2):
  *   P[r][j] = (R_r . g_j) mod 2,  r < rows, j < m,
  * written bit-packed: row r of P is ldp words, bit j of the row is parity

@@ -27,6 +27,7 @@ _i64, _p, _int, _sz, _dbl = ctypes.c_int64, ctypes.c_void_p, ctypes.c_int, ctype
 _MAT = [_p, _i64, _i64]
 SIGNATURES = {
     "iqp_workspace_bytes": (_sz, [_int, _i64, _i64, _i64, _i64, _i64, _int]),
+    "iqp_workspace_min_bytes": (_sz, [_int, _i64, _i64, _i64, _i64, _i64, _int]),
     "iqp_parity": (_int, [_i64] + _MAT + _MAT + [_p, _i64, _p]),
     "iqp_parity_gather": (_int, [_i64] + _MAT + _MAT + [_p, _i64, _p, _i64, _p, _p]),
     "iqp_parity_sum": (_int, [_i64] + _MAT + _MAT + [_p, _p]),

@@ -71,6 +71,7 @@ class _Workspace:
 
     def __init__(self):
         self._bufs = {}
+        self.refused = {}  # the least size that the device had no room for
 
     def get(self, nbytes: int, device, stream: int | None = None) -> torch.Tensor:
         if not isinstance(device, torch.device) or device.index is None:
@@ -88,6 +89,21 @@ _WS = _Workspace()
 
 def _ws_bytes(op: int, n: int, m: int, l: int, s: int, N: int, prec: int) -> int:
     return int(_lib.load().iqp_workspace_bytes(op, n, m, l, s, N, prec))
+
+
+def _scratch(op: int, n: int, m: int, l: int, s: int, N: int, prec: int, device, stream: int) -> torch.Tensor:
+    """Workspace of an operation: of its full size, or, where the device has no
+    room for that, of the smallest it runs with (the optional regions, which
+    are there for speed, are left out). A size that was refused is not asked for
+    again, since every refusal empties the allocator's cache."""
+    full = _ws_bytes(op, n, m, l, s, N, prec)
+    key = (device.index, stream)
+    if full < _WS.refused.get(key, full + 1):
+        try:
+            return _WS.get(full, device, stream)
+        except torch.OutOfMemoryError:
+            _WS.refused[key] = full
+    return _WS.get(int(_lib.load().iqp_workspace_min_bytes(op, n, m, l, s, N, prec)), device, stream)
 
 
 def workspace_bytes(op: int, n: int, m: int, l: int, s: int, N: int = 0, precision="split_bf16") -> int:
@@ -150,7 +166,7 @@ def expval_raw(n, theta, G, A, Z, precision="split_bf16"):
     prec = precision_code(precision)
     lib = _lib.load()
     st = _stream(G.device)
-    ws = _WS.get(_ws_bytes(OP_EXPVAL, n, m, l, s, 0, prec), G.device, st)
+    ws = _scratch(OP_EXPVAL, n, m, l, s, 0, prec, G.device, st)
     ev = torch.empty(l, dtype=torch.float64, device=G.device)
     se = torch.empty(l, dtype=torch.float64, device=G.device)
     check(lib.iqp_expval(n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(Z), s, Z.shape[1], _ptr(th), prec,
@@ -169,7 +185,7 @@ def expval_grad(n, theta, G, A, Z, alpha, beta=None, precision="split_bf16") -> 
     be = _f64(beta, G.device)
     lib = _lib.load()
     st = _stream(G.device)
-    ws = _WS.get(_ws_bytes(OP_EXPVAL_GRAD, n, m, l, s, 0, prec), G.device, st)
+    ws = _scratch(OP_EXPVAL_GRAD, n, m, l, s, 0, prec, G.device, st)
     grad = torch.empty(m, dtype=torch.float64, device=G.device)
     check(lib.iqp_expval_grad(n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(Z), s, Z.shape[1], _ptr(th),
                               _ptr(al), _ptr(be), prec, _ptr(grad), _ptr(ws), ws.numel(),
@@ -191,7 +207,7 @@ def expval_value_and_grad(n, theta, G, A, Z, alpha, beta=None, precision="split_
     be = _f64(beta, G.device)
     lib = _lib.load()
     st = _stream(G.device)
-    ws = _WS.get(_ws_bytes(OP_EXPVAL_GRAD, n, m, l, s, 0, prec), G.device, st)
+    ws = _scratch(OP_EXPVAL_GRAD, n, m, l, s, 0, prec, G.device, st)
     ev = torch.empty(l, dtype=torch.float64, device=G.device)
     se = torch.empty(l, dtype=torch.float64, device=G.device)
     grad = torch.empty(m, dtype=torch.float64, device=G.device)
@@ -221,7 +237,7 @@ def expval_keep_phi_raw(n, theta, G, A, Z, precision="split_bf16", ld=None):
     prec = precision_code(precision)
     lib = _lib.load()
     st = _stream(G.device)
-    ws = _WS.get(_ws_bytes(OP_EXPVAL, n, m, l, s, 0, prec), G.device, st)
+    ws = _scratch(OP_EXPVAL, n, m, l, s, 0, prec, G.device, st)
     ev = torch.empty(l, dtype=torch.float64, device=G.device)
     se = torch.empty(l, dtype=torch.float64, device=G.device)
     ld = phi_ld(s) if ld is None else int(ld)
@@ -247,13 +263,18 @@ def expval_grad_from_phi(n, theta, G, A, Z, phi, alpha, beta=None, precision="sp
     be = _f64(beta, G.device)
     lib = _lib.load()
     st = _stream(G.device)
-    ws = _WS.get(_ws_bytes(OP_EXPVAL_GRAD, n, m, l, s, 0, prec), G.device, st)
+    ws = _scratch(OP_EXPVAL_GRAD, n, m, l, s, 0, prec, G.device, st)
     grad = torch.empty(m, dtype=torch.float64, device=G.device)
     check(lib.iqp_expval_grad_from_phi(n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(Z), s, Z.shape[1],
                                        _ptr(th), _ptr(al), _ptr(be), prec, _ptr(phi), phi.shape[1], _ptr(grad),
                                        _ptr(ws), ws.numel(), st),
           "iqp_expval_grad_from_phi")
     return grad
+
+
+# FP32 keeps Phi from the forward up to this size: the recompute that it saves is a third of a step,
+# and FP32 held no more than its inputs before.
+FP32_PHI_BYTES = 2 ** 33
 
 
 def _planes_keep_phi(n, theta, G, A, Z):
@@ -296,8 +317,12 @@ class _ExpvalFn(torch.autograd.Function):
         code = precision_code(precision)
         if keep and code in KEEP_PHI:
             ev, se, phi = expval_keep_phi_raw(n, theta, G, A, Z, precision)
-        elif keep and code == FP32 and _lib.load().iqp_planes_used(n, G.shape[0], A.shape[0], Z.shape[0]):
-            ev, se, phi = _planes_keep_phi(n, theta, G, A, Z)
+        elif (keep and code == FP32 and 4 * A.shape[0] * phi_ld(Z.shape[0]) <= FP32_PHI_BYTES
+              and _lib.load().iqp_planes_used(n, G.shape[0], A.shape[0], Z.shape[0])):
+            try:
+                ev, se, phi = _planes_keep_phi(n, theta, G, A, Z)
+            except torch.OutOfMemoryError:
+                ev, se = expval_raw(n, theta, G, A, Z, precision)
         else:
             ev, se = expval_raw(n, theta, G, A, Z, precision)
         ctx.save_for_backward(theta, G, A, Z, phi)
@@ -313,7 +338,10 @@ class _ExpvalFn(torch.autograd.Function):
         s = Z.shape[0]
         alpha = g_ev.to(torch.float64) / -s
         if phi is not None and precision_code(ctx.precision) == FP32:
-            grad = _planes_grad_from_phi(ctx.n, theta, G, A, Z, phi, alpha)
+            try:
+                grad = _planes_grad_from_phi(ctx.n, theta, G, A, Z, phi, alpha)
+            except torch.OutOfMemoryError:
+                grad = expval_grad(ctx.n, theta, G, A, Z, alpha, None, ctx.precision)
         elif phi is not None:
             grad = expval_grad_from_phi(ctx.n, theta, G, A, Z, phi, alpha, None, ctx.precision)
         else:
@@ -324,7 +352,7 @@ class _ExpvalFn(torch.autograd.Function):
 def expval(theta, G, A, Z, n: int, precision="split_bf16", keep_phi=True):
     """Monte-Carlo <Z_a> estimates and standard errors (float64), differentiable
     in theta (std_err is not). With keep_phi (split BF16, row-sparse and
-    low-order forms, FP32 on the tensor cores) the forward keeps Phi (4 l s bytes, held until the
+    low-order forms, FP32 on the tensor cores up to 8 GiB) the forward keeps Phi (4 l s bytes, held until the
     backward) so the backward forms W from it instead of recomputing Phi;
     keep_phi=False holds only the inputs and recomputes."""
     return _ExpvalFn.apply(theta, G, A, Z, n, precision, keep_phi)
@@ -349,7 +377,7 @@ def mmd_loss_raw(n, theta, G, A, Z, X, precision="split_bf16", unbiased=True, wi
         op = OP_MMD_LOSS_GRAD if with_grad else OP_MMD_LOSS
     flags = (MMD_UNBIASED if unbiased else 0) | (MMD_SQRT if sqrt_loss else 0) | (MMD_INDEP if indep else 0)
     st = _stream(G.device)
-    ws = _WS.get(_ws_bytes(op, n, m, l, s, N, prec), G.device, st)
+    ws = _scratch(op, n, m, l, s, N, prec, G.device, st)
     loss = torch.empty(1, dtype=torch.float64, device=G.device)
     args = (n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(Z), s, Z.shape[1], _ptr(X), N, X.shape[1],
             _ptr(th), prec, flags)
@@ -399,7 +427,7 @@ def expval_indep_raw(n, theta, G, A, Z):
     s = Z.shape[0] // l
     lib = _lib.load()
     st = _stream(G.device)
-    ws = _WS.get(_ws_bytes(OP_EXPVAL_INDEP, n, m, l, s, 0, SPARSE_FP32), G.device, st)
+    ws = _scratch(OP_EXPVAL_INDEP, n, m, l, s, 0, SPARSE_FP32, G.device, st)
     ev = torch.empty(l, dtype=torch.float64, device=G.device)
     se = torch.empty(l, dtype=torch.float64, device=G.device)
     check(lib.iqp_expval_indep(n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(Z), s, Z.shape[1], _ptr(th),
@@ -419,7 +447,7 @@ def expval_indep_grad(n, theta, G, A, Z, alpha, beta=None) -> torch.Tensor:
     be = _f64(beta, G.device)
     lib = _lib.load()
     st = _stream(G.device)
-    ws = _WS.get(_ws_bytes(OP_EXPVAL_INDEP_GRAD, n, m, l, s, 0, SPARSE_FP32), G.device, st)
+    ws = _scratch(OP_EXPVAL_INDEP_GRAD, n, m, l, s, 0, SPARSE_FP32, G.device, st)
     grad = torch.empty(m, dtype=torch.float64, device=G.device)
     check(lib.iqp_expval_indep_grad(n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(Z), s, Z.shape[1],
                                     _ptr(th), _ptr(al), _ptr(be), _ptr(grad), _ptr(ws), ws.numel(),
@@ -540,7 +568,7 @@ def bitflip_expval_raw(n, theta, G, A):
     m, l = G.shape[0], A.shape[0]
     lib = _lib.load()
     st = _stream(G.device)
-    ws = _WS.get(_ws_bytes(OP_BITFLIP, n, m, l, 1, 0, FP32), G.device, st)
+    ws = _scratch(OP_BITFLIP, n, m, l, 1, 0, FP32, G.device, st)
     ev = torch.empty(l, dtype=torch.float64, device=G.device)
     check(lib.iqp_bitflip_expval(n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(th), _ptr(ev), _ptr(ws),
                                  ws.numel(), st), "iqp_bitflip_expval")
@@ -555,7 +583,7 @@ def bitflip_grad(n, theta, G, A, w) -> torch.Tensor:
     wd = _f64(w, G.device)
     lib = _lib.load()
     st = _stream(G.device)
-    ws = _WS.get(_ws_bytes(OP_BITFLIP, n, m, l, 1, 0, FP32), G.device, st)
+    ws = _scratch(OP_BITFLIP, n, m, l, 1, 0, FP32, G.device, st)
     grad = torch.empty(m, dtype=torch.float64, device=G.device)
     check(lib.iqp_bitflip_grad(n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(th), _ptr(wd), _ptr(grad),
                                _ptr(ws), ws.numel(), st), "iqp_bitflip_grad")

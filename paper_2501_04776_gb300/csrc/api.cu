@@ -252,9 +252,8 @@ Plan make_plan(int op, int64_t n, int64_t m, int64_t l, int64_t s, int64_t N, in
 // its end left out).
 size_t plan_min_bytes(const Plan &p) { return p.off_opt != 0 ? p.off_opt : p.total; }
 
-// The smallest workspace `op` runs with (iqp_workspace_bytes less the
-// optional split-tile scratch at its end); 0 for invalid arguments (the
-// checks of iqp_workspace_bytes).
+// The smallest workspace `op` runs with (iqp_workspace_bytes less its optional
+// regions); 0 for invalid arguments (the checks of iqp_workspace_bytes).
 size_t workspace_min_bytes(int op, int64_t n, int64_t m, int64_t l, int64_t s, int64_t N, int prec) {
     if (n < 1 || m < 1 || l < 1 || s < 1) return 0;
     if (op < IQP_OP_EXPVAL || op > IQP_OP_MMD_LOSS_GRAD_INDEP) return 0;
@@ -668,6 +667,10 @@ uint64_t default_spin_limit_ns() { return spin_limit_ns(); }
 using namespace iqp;
 
 extern "C" {
+
+size_t iqp_workspace_min_bytes(iqp_op op, int64_t n, int64_t m, int64_t l, int64_t s, int64_t N, iqp_precision prec) {
+    return workspace_min_bytes(op, n, m, l, s, N, prec);
+}
 
 size_t iqp_workspace_bytes(iqp_op op, int64_t n, int64_t m, int64_t l, int64_t s, int64_t N, iqp_precision prec) {
     if (n < 1 || m < 1 || l < 1 || s < 1) return 0;
