@@ -760,6 +760,17 @@ def workload_rows(args, lib, dev, st, timed, peaks, clocks):
 
 # ---------------------------------------------------------------- GPU arm
 
+def short_rows(rows):
+    """The rows' workloads and times, for the one line on stdout: whoever reads it may keep only its last
+    16 KB, and the rows' kernels and rooflines (on stderr) are more than that by themselves."""
+    def short(row):
+        out = {k: v for k, v in row.items() if k == "workload" or k.startswith("ms")}
+        if "forms" in row:
+            out["forms"] = {k: short(f) for k, f in row["forms"].items()}
+        return out
+    return {k: short(r) for k, r in rows.items()}
+
+
 def main():
     args = parse()
     world = int(os.environ.get("WORLD_SIZE", "1"))
@@ -995,6 +1006,9 @@ def main():
         torch.cuda.synchronize()
         line["cpu_baseline"] = cpu_baseline(p, args, ev.cpu().numpy(), se.cpu().numpy(), gpu_grad_fn)
     if rank == 0:
+        if "rows" in line:
+            print(json.dumps({"rows": line["rows"]}), file=sys.stderr, flush=True)
+            line["rows"] = short_rows(line["rows"])
         print(json.dumps(line), flush=True)
     if world > 1:
         dist.barrier()
