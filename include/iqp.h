@@ -53,7 +53,8 @@ typedef enum {
 } iqp_status;
 
 /* Arithmetic of the phase contraction Phi = (2 theta . P_A) S_Z^T.
- * IQP_FP32: FP32 accuracy. From 2^23 terms (l s m) on the tensor cores: 2 theta
+ * IQP_FP32: FP32 accuracy. From 2^23 terms (l s m), and for gradients of more
+ * than 1024 samples, on the tensor cores (where the workspace has room): 2 theta
  * and W as three BF16 planes each, the first summed exactly (error against
  * FP64 no larger than FP32 FMAs', also where a few parameters dominate; where
  * gates 2^11 times below the mean of thousands of others are an observable's only
@@ -101,12 +102,12 @@ typedef enum {
  * except for the MMD ops). Returns 0 for invalid sizes. Host only.
  * With IQP_SPLIT_BF16 its end is optional, in three parts, each used only
  * when `ws_bytes` reaches its end:
- *  - 20.5 MB (160 x 128 KiB plus 640 bytes): a last round of phase tiles that
+ *  - 20.5 MB (160 x 128 KiB, and 640 bytes that are not used): a last round of phase tiles that
  *    would leave SMs idle is split along the gates across them (else every
  *    phase tile runs whole);
  *  - 40 MiB (160 x 256 KiB): the running sums of the phase kernels that take
  *    two sample tiles per tile (else one sample tile per tile);
- *  - 80 MiB (640 x 128 KiB plus 640 bytes): the last round of those kernels
+ *  - 80 MiB (640 x 128 KiB, and 640 bytes that are not used): the last round of those kernels
  *    is split evenly across the SMs (else it runs as single tiles). */
 size_t iqp_workspace_bytes(iqp_op op, int64_t n, int64_t m, int64_t l, int64_t s, int64_t N,
                            iqp_precision prec);
@@ -265,10 +266,9 @@ iqp_status iqp_planes_grad_from_phi(int64_t n, const uint64_t *G, int64_t m, int
 /* Estimates and gradient in one call, for a loss whose gradient coefficients
  * alpha, beta (as in iqp_expval_grad) are known before the estimates, e.g.
  * L = sum_a w_a <Z_a> with alpha_a = -w_a / s, beta = NULL. Outputs as
- * iqp_expval plus grad[m]. The parities are formed once. In IQP_SPLIT_BF16
- * and IQP_SPARSE_FP32 a single pass over Phi yields the statistics and W (no
- * recompute), so does IQP_FP32 on the tensor cores; IQP_LOWORDER_FP32 keeps
- * Phi from its statistics pass for W; the SIMT kernels recompute it. ws: iqp_workspace_bytes(IQP_OP_EXPVAL_GRAD, ...). */
+ * iqp_expval plus grad[m]. The parities are formed once, and a single pass over
+ * Phi yields the statistics and W (no recompute) except in IQP_FP32's SIMT
+ * kernels. ws: iqp_workspace_bytes(IQP_OP_EXPVAL_GRAD, ...). */
 iqp_status iqp_expval_value_and_grad(int64_t n, const uint64_t *G, int64_t m, int64_t ldg,
                                      const uint64_t *A, int64_t l, int64_t lda,
                                      const uint64_t *Z, int64_t s, int64_t ldz, const float *theta,
@@ -319,14 +319,18 @@ iqp_status iqp_mmd_loss_grad(int64_t n, const uint64_t *G, int64_t m, int64_t ld
  * coherently, flips the bits of g_j with probability sin^2(theta_j). Its
  * expectation values are exact products (eq. expval_bitflip), no sampling:
  *   expval[a] = prod_{j : g_j.a odd} cos(2 theta_j).
- * FP64. ws: iqp_workspace_bytes(IQP_OP_BITFLIP, n, m, l, 1, 0, prec). */
+ * FP64 accuracy; from 2^25 parities (l m) on as sums of logarithms in 64-bit
+ * integers where these add up to at most 512 over all gates, within one FP64 rounding per factor.
+ * ws: iqp_workspace_bytes(IQP_OP_BITFLIP, n, m, l, 1, 0, prec). */
 iqp_status iqp_bitflip_expval(int64_t n, const uint64_t *G, int64_t m, int64_t ldg,
                               const uint64_t *A, int64_t l, int64_t lda, const float *theta,
                               double *expval, void *ws, size_t ws_bytes, void *stream);
 
 /* Gradient of L = sum_a w[a] expval[a] for the bitflip circuit:
  *   grad[j] = -2 tan(2 theta_j) sum_{a : g_j.a odd} w[a] expval[a].
- * w: float64[l] on the device (e.g. dL/d expval). grad: float64[m]. FP64.
+ * w: float64[l] on the device (e.g. dL/d expval). grad: float64[m]. FP64
+ * accuracy for every gate: from 2^25 parities on in integers where their rounding
+ * stays below 2^-53 of the gate's sum, else in FP64.
  * Same workspace as iqp_bitflip_expval. */
 iqp_status iqp_bitflip_grad(int64_t n, const uint64_t *G, int64_t m, int64_t ldg,
                             const uint64_t *A, int64_t l, int64_t lda, const float *theta,

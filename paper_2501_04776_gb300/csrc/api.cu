@@ -198,11 +198,15 @@ Plan make_plan(int op, int64_t n, int64_t m, int64_t l, int64_t s, int64_t N, in
         p.off_skp = take((int64_t)kMaxSplitCtas * kSplitSlotFloats * 4 + (int64_t)kMaxSplitCtas * 4);
         // running sums: only where the gates take more than one accumulation chunk
         p.off_xsum = take(m > kX3Gates ? (int64_t)kMaxSplitCtas * kSplitSlotFloats * 4 : 0);
-        // Below 2^23 terms (and, where a gradient follows, at most 1024
-        // samples) the SIMT kernels' few tiles take no longer than the tensor
-        // form's launches do: at n = 8, m = 36, l = 64, s = 1024 a step is 0.52 ms of
-        // host time either way, 25 us more of it with the tensor maps. Past that
-        // the SIMT gradient's serial loop (4.6 us per 32 samples) decides.
+        // Below 2^23 terms the SIMT kernels' estimates take as long as the
+        // tensor form's (36 gates, 64 x 4096, 2^23.2 terms: 35 and 30 us; 640 x
+        // 512: 35 and 30), and up to 1024 samples a gradient step through autograd is
+        // host time either way (64 x 1024: 0.45 ms, 25 us more of it with the
+        // tensor maps). Past 1024 samples the SIMT gradient's serial loop (4 us per
+        // 32 samples, whatever l and m) decides: one call's gradient, 64 x 1025
+        // samples 157 us (planes 43), 1 x 1025 136 (41), 64 x 2048 280 (49); 700
+        // gates, 4 x 1025: 226 (50). The estimates of such a step stay below
+        // 2^23 terms on the SIMT kernels; both forms hold the FP32 tolerance.
         p.x3 = x3_available() && ((double)l * (double)s * (double)m >= 8388608.0 || (grad && s > 1024));
     }
     if (prec == IQP_SPLIT_BF16 && !bitflip && !indep) {
@@ -357,11 +361,11 @@ iqp_status check_common(int64_t n, const uint64_t *G, int64_t m, int64_t ldg, co
     if (prec != IQP_FP32 && prec != IQP_SPLIT_BF16 && prec != IQP_SPARSE_FP32 && prec != IQP_LOWORDER_FP32)
         return IQP_ERR_ARG;
     if (prec == IQP_SPLIT_BF16 && !iqp_tensor_path_available()) return IQP_ERR_UNSUPPORTED;
-    // low-order form: observables on grid x, 256-sample blocks on y; its n x n
-    // pair matrices (C, H, K: 20 n^2 bytes) bound n
+    // low-order form: samples in 256-sample blocks, at most 65535 of them; its
+    // n x n pair matrices (C, H, K: 20 n^2 bytes) bound n
     if (prec == IQP_LOWORDER_FP32 && (l > INT32_MAX || n > 65536 || cdiv(s, (int64_t)256) > 65535))
         return IQP_ERR_ARG;
-    // sparse grid: observables on x (< 2^31), 2048-sample blocks on y (< 65536)
+    // row-sparse form: observables on grid x (< 2^31), at most 65535 x 2048 samples
     if (prec == IQP_SPARSE_FP32 && (l > INT32_MAX || cdiv(s, (int64_t)2048) > 65535)) return IQP_ERR_ARG;
     return IQP_OK;
 }
@@ -480,15 +484,9 @@ iqp_status prepare(const Plan &p, void *ws, const uint64_t *G, int64_t ldg, cons
         return IQP_OK;
     }
     // The sparse form reads only P_Z^T (bits over samples).
-    IQP_TRY(launch_parity_gather(p.n, Z, p.s, ldz, G, p.m, ldg,
-                                 p.prec == IQP_SPARSE_FP32 ? nullptr : at<uint64_t>(ws, p.off_pz), p.ldp,
-                                 at<uint64_t>(ws, p.off_pzt), p.ldzt, rt, st, sup));
-    if (p.prec == IQP_SPLIT_BF16) {
-        __nv_bfloat16 *hi = at<__nv_bfloat16>(ws, p.off_c);
-        IQP_TRY(launch_theta_prep(theta, p.m, p.mpad, nullptr, hi, hi + p.mpad, st));
-    } else {
-        IQP_TRY(launch_theta_prep(theta, p.m, p.mpad, at<float>(ws, p.off_c), nullptr, nullptr, st));
-    }
+    IQP_TRY(launch_parity_gather(p.n, Z, p.s, ldz, G, p.m, ldg, nullptr, p.ldp, at<uint64_t>(ws, p.off_pzt), p.ldzt, rt, st,
+                                 sup));
+    IQP_TRY(launch_theta_prep(theta, p.m, p.mpad, at<float>(ws, p.off_c), nullptr, nullptr, st));
     return IQP_OK;
 }
 

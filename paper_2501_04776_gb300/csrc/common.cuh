@@ -20,11 +20,12 @@ constexpr int kPartColsTc = 64;     // samples per (S, M2) partial, tensor-core 
 constexpr int kATile = 128;      // observables per gradient partial row (single-CTA gradient kernel)
 constexpr int kGradObs = 256;    // observables per tile of the CTA-pair gradient kernel (two partial rows each)
 // Split phase tiles: one 128 x 256 FP32 partial accumulator per (part, CTA),
-// for at most kMaxSplitCtas CTAs, then one int counter per (tile, CTA).
+// for at most kMaxSplitCtas CTAs (then kMaxSplitCtas ints that no kernel uses: the sizes are part of the
+// documented layout).
 constexpr int64_t kSplitSlotFloats = 128 * 256;
 constexpr int kMaxSplitCtas = 160;
 // Balanced split of the two-sample-tile phase's last round: kSplitSlots slots
-// (one per piece, CTA and accumulator), then kMaxSplitCtas counters.
+// (one per piece, CTA and accumulator), then kMaxSplitCtas unused ints.
 constexpr int kSplitSlots = 640;
 // Two-sample-tile phase kernels: the running sums of both accumulators, per
 // CTA (at most kMaxSplitCtas CTAs).
@@ -59,11 +60,11 @@ struct Plan {
     int64_t natile; // room for gradient partial rows: 2 ceil(l / 128)
     size_t off_status, off_pa, off_pz, off_pzt, off_pat, off_rt, off_c, off_part, off_w, off_gpart;
     size_t off_ab, off_s12, off_T, off_terms, off_zt, off_sup, total;
-    // low-order form: C (+ d), M = C S, V, H, single-gate partials; ldc floats per row of C and H
+    // low-order form: C (+ d), X = s (d + C S), V, H, single-gate partials; ldc elements per row of C and H
     size_t off_lo_c, off_lo_m, off_lo_v, off_lo_h, off_lo_gs, off_lo_a;
-    size_t off_skp;  // split BF16: partial accumulators and counters of split phase tiles (0 if none)
+    size_t off_skp;  // split BF16, FP32 planes: partial accumulators of split phase tiles (0 if none)
     size_t off_gsum; // split BF16: per-CTA running sums of the two-sample-tile phase kernels (0 if none)
-    size_t off_skx;  // split BF16: pieces and counters of the two-tile phase's balanced last round (0 if none)
+    size_t off_skx;  // split BF16: pieces of the two-tile phase's balanced last round (0 if none)
     // FP32 form on the tensor cores (optional region at the end of the FP32 plan; x3 = it is there and in use):
     // the three planes of 2 theta, sums of |2 theta| over blocks of kX3Gates, (S, M2) partials of 64 samples, row maxima of |W|, the
     // three planes of W, running sums (off_skp: the split tiles' scratch)

@@ -455,13 +455,6 @@ __global__ void __launch_bounds__(256) k_mmd_terms(const double2 *__restrict__ p
     }
 }
 
-// alpha_a = -w_a / s for a linear loss given weights (device helper).
-__global__ void k_scale(const double *__restrict__ x, double f, int64_t l, double *__restrict__ y) {
-    pdl_sync();
-    const int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (a < l) y[a] = f * x[a];
-}
-
 }  // namespace
 
 cudaError_t launch_theta_prep(const float *theta, int64_t m, int64_t mpad, float *c32, __nv_bfloat16 *hi,
@@ -553,12 +546,6 @@ cudaError_t launch_mmd_terms(const double2 *part, int64_t nparts, int64_t pw, co
                                                       reinterpret_cast<const long long *>(T), l, N,
                                                       unbiased, sqrt_loss ? 1 : 0, k, terms, alpha, beta, loss, scale,
                                                       counter);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_scale(const double *x, double f, int64_t l, double *y, cudaStream_t st) {
-    LaunchScope ls(IQP_KERNEL_FINALIZE, st);
-    launch_pdl(k_scale, (unsigned)cdiv(l, 256), 256, 0, st, x, f, l, y);
     return cudaGetLastError();
 }
 

@@ -349,21 +349,6 @@ __device__ __forceinline__ void expand_a3(const uint8_t *bitsA, const uint8_t *c
     }
 }
 
-// Sum over the 32 lanes of v[lane][k]: afterwards lane L returns the sum of column L.
-__device__ __forceinline__ float reduce_scatter32(float (&v)[32], int lane) {
-#pragma unroll
-    for (int w = 16; w >= 1; w >>= 1) {
-        const bool upper = (lane & w) != 0;
-#pragma unroll
-        for (int k = 0; k < w; ++k) {
-            const float send = upper ? v[k] : v[k + w];
-            const float keep = upper ? v[k + w] : v[k];
-            v[k] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, w);
-        }
-    }
-    return v[0];
-}
-
 // Bounded wait polled by every lane (each needs the acquire), with the outcome
 // made warp-uniform so that a give-up never splits a warp.
 __device__ __forceinline__ bool wait_warp(uint64_t *b, uint32_t parity, volatile int *abort_flag, uint32_t *status,
@@ -1486,7 +1471,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         float v[32];
 #pragma unroll
                         for (int e = 0; e < 32; ++e) v[e] = ((mask >> e) & 1u) ? 2.f * __uint_as_float(r[e]) : 0.f;
-                        red[quarter * 256 + group * kGroupCols + c * 32 + lane] = reduce_scatter32(v, lane);
+                        red[quarter * 256 + group * kGroupCols + c * 32 + lane] = reduce_scatter(v, lane);
                     }
                     // All producer warps' column sums are in `red`; combine the four
                     // lane quarters in fixed order. (The next tile's writes to
