@@ -506,7 +506,7 @@ struct X3Grid {
 // |values| that add up to at most 2^bits bound.
 __device__ __forceinline__ X3Grid x3_grid(float bound, int bits) {
     int e = (int)((__float_as_uint(bound) >> 23) & 255u) - 126 + bits - 24;  // bound 2^bits < 2^(e + 24)
-    e = e < -104 ? -104 : (e > 104 ? 104 : e);
+    e = e < -120 ? -120 : (e > 104 ? 104 : e);
     X3Grid g;
     g.step = __uint_as_float((uint32_t)(e + 127) << 23);
     g.inv = __uint_as_float((uint32_t)(127 - e) << 23);
