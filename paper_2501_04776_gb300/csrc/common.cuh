@@ -109,7 +109,7 @@ struct LoArgs {
     float *C, *d;              // C (n x ldc; only where the contractions run as sums), d (n)
     int64_t ldc;
     unsigned long long *E;     // pair-existence bits
-    unsigned long long *fx;    // n x n fixed-point sums (C, then the gradient's K), n more (d, then the scale), cmax, counter
+    unsigned long long *fx;    // n x n fixed-point sums (C, then the gradient's K), n more (d, then the scale), cmax, counters
     __nv_bfloat16 *split;      // split-BF16 operand of the contractions
     uint32_t *ZP;              // n x 32 ceil(s / 1024): the sample bits in lane order (null: no lists, the one-CTA form)
     int *Lq;                   // l x kLoQ: the observables' qubits

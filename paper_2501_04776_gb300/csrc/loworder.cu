@@ -622,6 +622,16 @@ __device__ void lo_load_bits4(LoShared &sh, int nq, int64_t n, const uint64_t *_
     __syncthreads();
 }
 
+// The CTA's next work item of the heavy observables' kernels (the first is its block's; the items differ in size, so
+// the rest are handed out as CTAs come free). Its barriers also part one item's use of shared memory from the next's.
+__device__ __forceinline__ int64_t next_item(unsigned long long *__restrict__ counter) {
+    __shared__ unsigned long long item;
+    __syncthreads();
+    if (threadIdx.x == 0) item = atomicAdd(counter, 1ull);
+    __syncthreads();
+    return (int64_t)(gridDim.x + item);
+}
+
 // The observables too heavy for the lists (or all of them, without lists):
 // work item (h, g) is observable heavy[h] (h itself without `heavy`).
 // MODE 0: (sum cos, sum (cos - mean)^2) per (observable, 256 samples) into
@@ -635,14 +645,16 @@ __device__ void lo_load_bits4(LoShared &sh, int nq, int64_t n, const uint64_t *_
 // so every support qubit costs one 16-byte load of M and every pair one
 // word pair of sample bits for four samples; larger supports take one block
 // per pass, one sample per thread.
+constexpr int kPhaseCtas = 5, kPairCtas = 3;  // CTAs per SM of the heavy observables' kernels (45 KB of shared memory each)
 template <int MODE>
-__global__ void __launch_bounds__(kBlk) k_lo_phase(const uint64_t *__restrict__ A, int64_t lda, int64_t n,
+__global__ void __launch_bounds__(kBlk, kPhaseCtas) k_lo_phase(const uint64_t *__restrict__ A, int64_t lda, int64_t n,
                                                    const uint64_t *__restrict__ ZT, int64_t ldzt,
                                                    const float *__restrict__ X, int64_t lds,
                                                    const unsigned long long *__restrict__ Cfx,
                                                    const unsigned *__restrict__ cmax, int64_t m,
                                                    const unsigned long long *__restrict__ E, int64_t lde, int64_t l,
                                                    const int *__restrict__ heavy, const unsigned *__restrict__ nheavy,
+                                                   unsigned long long *__restrict__ counter,
                                                    int64_t s, int64_t nparts, double2 *__restrict__ part,
                                                    const double *__restrict__ alpha, const double *__restrict__ beta,
                                                    float *__restrict__ W, float *__restrict__ phi, int64_t ldphi,
@@ -654,8 +666,7 @@ __global__ void __launch_bounds__(kBlk) k_lo_phase(const uint64_t *__restrict__ 
     const int64_t ngroups = cdiv(nparts, (int64_t)kPGroup);
     const int64_t nobs = heavy ? (int64_t)*nheavy : l;
     const float inv = ldexpf(1.0f, -lo_fx_exp(*cmax, m));
-    for (int64_t it = blockIdx.x; it < nobs * ngroups; it += gridDim.x) {
-    __syncthreads();  // the previous item's readers of sh are done
+    for (int64_t it = blockIdx.x; it < nobs * ngroups; it = next_item(counter)) {
     const int64_t h = it % nobs, a = heavy ? heavy[h] : h;
     const int nq = support_of_row(A + a * lda, n, sh.Q, sh.scan, status);
     const int tid = threadIdx.x, w = tid >> 5, bit = tid & 31;
@@ -1159,10 +1170,11 @@ __global__ void __launch_bounds__(256) k_lo_w(const float *phi, int64_t ldphi, f
 // are staged per pair of barriers (one block at a time otherwise).
 // Work item (a, g) takes blocks kPGroup g ...; heavy observables as in k_lo_phase.
 constexpr int kPairPass = 128;
-__global__ void __launch_bounds__(kBlk) k_lo_pairs(const uint64_t *__restrict__ A, int64_t lda, int64_t n,
+__global__ void __launch_bounds__(kBlk, kPairCtas) k_lo_pairs(const uint64_t *__restrict__ A, int64_t lda, int64_t n,
                                                    const uint64_t *__restrict__ ZT, int64_t ldzt,
                                                    const unsigned long long *__restrict__ E, int64_t lde, int64_t l,
                                                    const int *__restrict__ heavy, const unsigned *__restrict__ nheavy,
+                                                   unsigned long long *__restrict__ counter,
                                                    const float *__restrict__ W, int64_t lds, int64_t s,
                                                    int64_t nblk, const double *__restrict__ scale,
                                                    unsigned long long *__restrict__ Kfx,
@@ -1174,8 +1186,7 @@ __global__ void __launch_bounds__(kBlk) k_lo_pairs(const uint64_t *__restrict__ 
     constexpr int kPerWarp = kPairPass / (kBlk / 32);
     const int64_t ngroups = cdiv(nblk, (int64_t)kPGroup);
     const int64_t nobs = heavy ? (int64_t)*nheavy : l;
-    for (int64_t it = blockIdx.x; it < nobs * ngroups; it += gridDim.x) {
-    __syncthreads();  // the previous item's readers of sh are done
+    for (int64_t it = blockIdx.x; it < nobs * ngroups; it = next_item(counter)) {
     const int64_t h = it % nobs, a = heavy ? heavy[h] : h;
     const int nq = support_of_row(A + a * lda, n, sh.Q, sh.scan, status);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1384,13 +1395,17 @@ namespace {
 unsigned *lo_cmax(const LoArgs &a) { return reinterpret_cast<unsigned *>(a.fx + a.n * a.n + a.n); }
 unsigned *lo_nheavy(const LoArgs &a) { return lo_cmax(a) + 1; }
 double *lo_scale(const LoArgs &a) { return reinterpret_cast<double *>(a.fx + a.n * a.n); }
+unsigned long long *lo_items(const LoArgs &a) { return a.fx + a.n * a.n + a.n + 1; }  // of the phase, of the pairs
 const int *lo_heavy(const LoArgs &a) { return a.ZP != nullptr ? a.cnt + a.l : nullptr; }
 
-// Blocks of the heavy observables' kernels: two per SM take what there is
-// (usually nothing); without lists one per work item.
-unsigned lo_heavy_blocks(const LoArgs &a, int64_t nblk) {
+// Blocks of the heavy observables' kernels: as many as the SMs hold take what
+// there is (usually nothing); without lists one per work item. They are not
+// launched as dependents: where there are fewer items than the SMs hold, the blocks would come
+// in while the contraction before them ends and crowd the SMs that it leaves first (300 observables of
+// 300 qubits x 3000: 21 ms, 37 as dependents).
+unsigned lo_heavy_blocks(const LoArgs &a, int64_t nblk, int per_sm) {
     int64_t b = a.l * cdiv(nblk, (int64_t)kPGroup);
-    if (a.ZP != nullptr && b > 2 * num_sms()) b = 2 * num_sms();
+    if (a.ZP != nullptr && b > per_sm * num_sms()) b = per_sm * num_sms();
     if (b > 0x7FFFFFFF) b = 0x7FFFFFFF;
     return (unsigned)(b < 1 ? 1 : b);
 }
@@ -1423,9 +1438,9 @@ cudaError_t launch_phase(const LoArgs &a, double2 *part, const double *alpha, co
                          int64_t ldphi, cudaStream_t st) {
     const int64_t nblk = cdiv(a.s, (int64_t)kBlk);
     LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-    launch_pdl(k_lo_phase<MODE>, lo_heavy_blocks(a, nblk), kBlk, 0, st,
+    k_lo_phase<MODE><<<lo_heavy_blocks(a, nblk, kPhaseCtas), kBlk, 0, st>>>(
         a.A, a.lda, a.n, a.ZT, a.ldzt, a.X, a.lds, a.fx, lo_cmax(a), a.m, a.E, lo_lde(a.n), a.l, lo_heavy(a), lo_nheavy(a),
-        a.s, nblk, part, alpha, beta, W, phi, ldphi, a.status);
+        lo_items(a), a.s, nblk, part, alpha, beta, W, phi, ldphi, a.status);
     return cudaGetLastError();
 }
 
@@ -1437,9 +1452,9 @@ cudaError_t launch_lo_prepare(const LoArgs &a, cudaStream_t st) {
     const bool tc = lo_tensor() && a.split != nullptr && a.ldz >= 4 && a.ldz % 2 == 0 &&
                     (reinterpret_cast<uintptr_t>(a.Z) & 15) == 0;
     cudaError_t e;
-    // fx: Cfx (n x n), dfx (n), then the largest |c_j| (float bits) and the count of heavy observables.
+    // fx: Cfx (n x n), dfx (n), then the largest |c_j| (float bits), the count of heavy observables and the items handed out.
     if ((e = cudaMemsetAsync(a.E, 0, (size_t)n * lde * 8, st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(a.fx, 0, (size_t)(n * n + n) * 8 + 16, st)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(a.fx, 0, (size_t)(n * n + n) * 8 + 24, st)) != cudaSuccess) return e;
     if ((e = launch_support_list(a.G, m, a.ldg, n, a.sup, st, a.theta, lo_cmax(a))) != cudaSuccess) return e;
     if ((e = launch_bit_transpose_batched(a.Z, 1, a.s, n, a.ldz, a.ZT, a.ldzt, st)) != cudaSuccess) return e;
     __nv_bfloat16 *hi = a.split, *lo = a.split + n * kc;
@@ -1535,8 +1550,9 @@ cudaError_t launch_lo_grad(const LoArgs &a, double2 *part, const double *alpha, 
     if (e != cudaSuccess) return e;
     {
         LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-        launch_pdl(k_lo_pairs, lo_heavy_blocks(a, nblk), kBlk, 0, st, a.A, a.lda, n, a.ZT, a.ldzt, a.E, lde, a.l, lo_heavy(a),
-                                                              lo_nheavy(a), W, a.lds, s, nblk, lo_scale(a), a.fx, a.status);
+        k_lo_pairs<<<lo_heavy_blocks(a, nblk, kPairCtas), kBlk, 0, st>>>(a.A, a.lda, n, a.ZT, a.ldzt, a.E, lde, a.l,
+                                                                         lo_heavy(a), lo_nheavy(a), lo_items(a) + 1, W, a.lds, s, nblk,
+                                                                         lo_scale(a), a.fx, a.status);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (hparts > 1) {

@@ -62,3 +62,28 @@ def test_limits_match_oracle(build, edges, s):
         assert np.max(np.abs(e.cpu().numpy() - want)) <= 1e-5 and np.max(np.abs(d.cpu().numpy() - want_se)) <= 1e-5
     for x in (g, kept, one[2]):
         assert np.linalg.norm(x.cpu().numpy() - want_g) <= 1e-4 * np.linalg.norm(want_g)
+
+
+def test_more_heavy_observables_than_blocks():
+    """1000 observables of 130 to 140 qubits and 5000 samples: 2000 work items for at most five blocks per SM."""
+    import torch
+    from paper_2501_04776_gb300 import api
+    n, l, s = 140, 1000, 5000
+    rng = I.Rng(9)
+    G = I.random_k_body(rng, 300, n, [1, 2], 1)
+    bits = np.ones((l, n), dtype=np.uint8)
+    for a in range(l):
+        bits[a, np.argsort(rng.uniform(n, 100 + a))[:a % 11]] = 0
+    A, Z = I.pack_bits(bits), I.uniform_bits(rng, s, n, 3)
+    th = (0.5 * rng.normal(300, 2) / np.sqrt(300)).astype(np.float32)
+    al, be = rng.normal(l, 7) / s, rng.normal(l, 8) / s
+    Gd, Ad, Zd = (api.to_device_bits(x) for x in (G, A, Z))
+    thd, ald, bed = (torch.from_numpy(x).cuda() for x in (th, al, be))
+    ev, se = api.expval_raw(n, thd, Gd, Ad, Zd, "loworder_fp32")
+    g = api.expval_grad(n, thd, Gd, Ad, Zd, ald, bed, "loworder_fp32")
+    assert api.read_status() == 0
+    t64 = th.astype(np.float64)
+    want, want_se, _, _ = oracle.expval(n, G, A, Z, t64)
+    want_g = oracle.expval_grad(n, G, A, Z, t64, al, be)
+    assert np.max(np.abs(ev.cpu().numpy() - want)) <= 1e-5 and np.max(np.abs(se.cpu().numpy() - want_se)) <= 1e-5
+    assert np.linalg.norm(g.cpu().numpy() - want_g) <= 1e-4 * np.linalg.norm(want_g)
