@@ -268,7 +268,8 @@ __device__ __forceinline__ void theta_prep_one(const float *__restrict__ theta, 
 // first statement) while the one before drains. pdl_sync waits until every kernel
 // before is complete and its writes are visible, then lets the next one's blocks
 // come in; a kernel that did not begin with it could run ahead of its inputs, so
-// every kernel that launch_pdl starts does. Low-order MMD step, 2000 x 5000 on 1000
+// every kernel that launch_pdl starts does (one of the low-order form waits at its
+// end: see AfterHeavy). Low-order MMD step, 2000 x 5000 on 1000
 // qubits: 371 -> 345 us; value and gradient, 3001 gates, 777 x 2501: 118 -> 111 us.
 __device__ __forceinline__ void pdl_sync() {
     asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -175,13 +175,17 @@ __global__ void __launch_bounds__(256) k_lo_zpack(const uint32_t *__restrict__ Z
 }
 
 // Every observable's qubits (in increasing order) and, with C, the pairs among
-// them that carry a generator, one warp per observable. One of more than kLoQ
-// qubits or kLoP pairs is left to the heavy observables' kernels: cnt = -1, and
-// its number in `heavy` (counted in *nheavy).
+// them that carry a generator, one warp per observable. One of more than qmax
+// (at most kLoQ) qubits or kLoP pairs is left to the heavy observables' kernels: cnt = -1, and
+// its number in `heavy` (counted in *nheavy). qmax: the listed kernels take a row of X per
+// step and warp, the block kernels several at a time, so where the warps are few (at most four per SM) they take the
+// observables from 65 qubits on (30 observables of 120 qubits x
+// 100: 158 us before the lists, 188 listed, 129).
+constexpr int kListed = 8;  // pairs per lane and round
 __global__ void __launch_bounds__(256) k_lo_lists(const uint64_t *__restrict__ A, int64_t lda, int64_t l, int64_t n,
                                                   const unsigned long long *__restrict__ E, int64_t lde,
                                                   const unsigned long long *__restrict__ Cfx,
-                                                  const unsigned *__restrict__ cmax, int64_t m, int *__restrict__ Lq,
+                                                  const unsigned *__restrict__ cmax, int64_t m, int qmax, int *__restrict__ Lq,
                                                   uint2 *__restrict__ Lp, int *__restrict__ cnt, int *__restrict__ heavy,
                                                   unsigned *__restrict__ nheavy, uint32_t *__restrict__ status) {
     pdl_sync();
@@ -213,37 +217,46 @@ __global__ void __launch_bounds__(256) k_lo_lists(const uint64_t *__restrict__ A
     }
     __syncwarp();
     int np = 0;
-    if (nq <= kLoQ) {
+    if (nq <= qmax) {
         for (int t = lane; t < nq; t += 32) Lq[a * kLoQ + t] = sq[warp][t];
-        // candidates t nq + u in order, 128 per round: the round's E words are all loaded before the first is used
-        for (int c0 = 0; c0 < nq * nq; c0 += 128) {
-            int qq[4], rr[4];
-            bool ok[4];
-            unsigned long long ew[4];
+        // the pairs t < u in order, 256 per round: the round's E words are all loaded before the first is used (with all
+        // nq^2 candidates, 128 per round, 30 observables of 100 qubits waited 78 rounds, 60 us, on their four SMs)
+        const int all = nq * (nq - 1) / 2;
+        for (int c0 = 0; c0 < all; c0 += 32 * kListed) {
+            int qr[kListed];
+            bool ok[kListed];
+            unsigned long long ew[kListed];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int e = c0 + 32 * k + lane, t = e / nq, u = e - t * nq;
-                ok[k] = e < nq * nq && u > t;
-                qq[k] = ok[k] ? sq[warp][t] : 0;
-                rr[k] = ok[k] ? sq[warp][u] : 0;
-                ok[k] = ok[k] && LO_OK(qq[k] >= 0 && qq[k] < rr[k] && rr[k] < n, 10);
-                ew[k] = ok[k] ? E[(int64_t)qq[k] * lde + (rr[k] >> 6)] : 0ull;
+            for (int k = 0; k < kListed; ++k) {
+                const int e = c0 + 32 * k + lane;
+                ok[k] = e < all;
+                // row t holds pairs t (2 nq - t - 1) / 2 ..: the root's rounding is put right by the two steps below
+                const float h = (float)(2 * nq - 1);
+                int t = ok[k] ? (int)(0.5f * (h - sqrtf(h * h - 8.f * (float)e))) : 0;
+                t -= t * (2 * nq - t - 1) / 2 > e ? 1 : 0;
+                t += (t + 1) * (2 * nq - t - 2) / 2 <= e ? 1 : 0;
+                const int u = ok[k] ? t + 1 + e - t * (2 * nq - t - 1) / 2 : 0;
+                const int q = ok[k] ? sq[warp][t] : 0, r = ok[k] ? sq[warp][u] : 0;
+                ok[k] = ok[k] && LO_OK(q >= 0 && q < r && r < n, 10);
+                qr[k] = q | (r << 16);
+                ew[k] = ok[k] ? E[(int64_t)q * lde + (r >> 6)] : 0ull;
             }
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const bool has = ok[k] && ((ew[k] >> (rr[k] & 63)) & 1ull) != 0ull;
+            for (int k = 0; k < kListed; ++k) {
+                const int q = qr[k] & 0xFFFF, r = (int)((unsigned)qr[k] >> 16);
+                const bool has = ok[k] && ((ew[k] >> (r & 63)) & 1ull) != 0ull;
                 const uint32_t bal = __ballot_sync(kFull, has);
                 const int pos = np + __popc(bal & ((1u << lane) - 1u));
                 if (has && pos < kLoP) {
-                    const float cv = __ll2float_rn((long long)Cfx[(int64_t)qq[k] * n + rr[k]]) * inv;
-                    Lp[a * kLoP + pos] = make_uint2((uint32_t)qq[k] | ((uint32_t)rr[k] << 16), __float_as_uint(-2.0f * cv));
+                    const float cv = __ll2float_rn((long long)Cfx[(int64_t)q * n + r]) * inv;
+                    Lp[a * kLoP + pos] = make_uint2((uint32_t)qr[k], __float_as_uint(-2.0f * cv));
                 }
                 np += __popc(bal);
             }
         }
     }
     if (lane != 0) return;
-    const bool listed = nq <= kLoQ && np <= kLoP;
+    const bool listed = nq <= qmax && np <= kLoP;
     cnt[a] = listed ? nq | (np << 16) : -1;
     if (!listed) {
         const unsigned h = atomicAdd(nheavy, 1u);
@@ -836,6 +849,15 @@ __global__ void __launch_bounds__(kBlk, kPhaseCtas) k_lo_phase(const uint64_t *_
 // MODE 0: statistics partials, and Phi into phi when it is not null; 1: W; 2:
 // partials and W.
 constexpr int kLoWarps = 4;
+
+// The listed observables' phase follows the heavy observables', which waits for all that came before, and shares no output with
+// it: where it is launched as its dependent (obs_beside) it runs beside it and waits for it at its end, on every path, so that
+// what follows it follows both. A few heavy observables take as long as one of them alone: 2000 observables of about 100 of
+// 1000 qubits x 3000, three of more than 128: 412 -> 320 us.
+struct AfterHeavy {
+    __device__ AfterHeavy() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+    __device__ ~AfterHeavy() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+};
 constexpr int kLoTab = 8 * 16 * 32;  // floats of a warp's tables
 template <int MODE>
 __global__ void __launch_bounds__(32 * kLoWarps) k_lo_obs(
@@ -843,7 +865,7 @@ __global__ void __launch_bounds__(32 * kLoWarps) k_lo_obs(
     int64_t nb, const float *__restrict__ X, int64_t lds, int64_t n, int64_t l, int64_t s, int64_t nparts,
     double2 *__restrict__ part, const double *__restrict__ alpha, const double *__restrict__ beta, float *__restrict__ W,
     float *__restrict__ phi, int64_t ldphi, uint32_t *__restrict__ status) {
-    pdl_sync();
+    const AfterHeavy after;
     [[maybe_unused]] uint32_t *status_dbg = status;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t a = (int64_t)blockIdx.x * kLoWarps + warp, blk = blockIdx.y;
@@ -1410,14 +1432,23 @@ unsigned lo_heavy_blocks(const LoArgs &a, int64_t nblk, int per_sm) {
     return (unsigned)(b < 1 ? 1 : b);
 }
 
+// Whether the listed observables' phase runs beside the heavy ones' (AfterHeavy): up to 16384 warps of it (7 per
+// scheduler). Past that a few heavy observables' time counts for less than the L1 that their kernel's shared memory
+// takes from the first blocks on every SM (4096 x 16384 on 5000 qubits: 4.47 ms in order, 4.56 beside).
+bool obs_beside(const LoArgs &a) { return a.l * cdiv(a.s, (int64_t)kLane) <= 16384; }
+
 template <int MODE>
 cudaError_t launch_obs(const LoArgs &a, double2 *part, const double *alpha, const double *beta, float *W, float *phi,
                        int64_t ldphi, cudaStream_t st) {
     const int64_t nb = cdiv(a.s, (int64_t)kLane);
+    const dim3 grid((unsigned)cdiv(a.l, (int64_t)kLoWarps), (unsigned)nb);
     LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-    launch_pdl(k_lo_obs<MODE>, dim3((unsigned)cdiv(a.l, (int64_t)kLoWarps), (unsigned)nb), 32 * kLoWarps, 0, st,
-        a.cnt, a.Lq, a.Lp, a.ZP, nb, a.X, a.lds, a.n, a.l, a.s, cdiv(a.s, (int64_t)kBlk), part, alpha, beta, W, phi, ldphi,
-        a.status);
+    if (obs_beside(a))
+        launch_pdl(k_lo_obs<MODE>, grid, 32 * kLoWarps, 0, st, a.cnt, a.Lq, a.Lp, a.ZP, nb, a.X, a.lds, a.n, a.l, a.s,
+                   cdiv(a.s, (int64_t)kBlk), part, alpha, beta, W, phi, ldphi, a.status);
+    else
+        k_lo_obs<MODE><<<grid, 32 * kLoWarps, 0, st>>>(a.cnt, a.Lq, a.Lp, a.ZP, nb, a.X, a.lds, a.n, a.l, a.s,
+                                                       cdiv(a.s, (int64_t)kBlk), part, alpha, beta, W, phi, ldphi, a.status);
     return cudaGetLastError();
 }
 
@@ -1476,7 +1507,8 @@ cudaError_t launch_lo_prepare(const LoArgs &a, cudaStream_t st) {
         const int64_t nb = cdiv(a.s, (int64_t)kLane);
         launch_pdl(k_lo_zpack, grid_1d(32 * n * nb), 256, 0, st, reinterpret_cast<const uint32_t *>(a.ZT), 2 * a.ldzt, n, nb, a.ZP);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        launch_pdl(k_lo_lists, (unsigned)cdiv(a.l, (int64_t)8), 256, 0, st, a.A, a.lda, a.l, n, a.E, lde, a.fx, lo_cmax(a), m, a.Lq,
+        launch_pdl(k_lo_lists, (unsigned)cdiv(a.l, (int64_t)8), 256, 0, st, a.A, a.lda, a.l, n, a.E, lde, a.fx, lo_cmax(a), m,
+                   a.l * nb <= 4 * (int64_t)num_sms() ? kLoQ / 2 : kLoQ, a.Lq,
                                                                     a.Lp, a.cnt, a.cnt + a.l, lo_nheavy(a), a.status);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
@@ -1512,22 +1544,24 @@ cudaError_t launch_lo_grad(const LoArgs &a, double2 *part, const double *alpha, 
     const bool listed = a.ZP != nullptr, tc = lo_tensor() && a.split != nullptr;
     cudaError_t e = launch_bit_transpose_batched(a.A, 1, a.l, n, a.lda, AT, ldlt, st);
     if (e != cudaSuccess) return e;
-    // The heavy observables' phase reads C's sums, which K then takes the place of.
+    if (!scale_set && (e = launch_fixed_scale(alpha, beta, a.l, s, lo_scale(a), st)) != cudaSuccess) return e;
+    // K's sums take the place of C's, which the heavy observables' phase reads.
+    const bool beside = phi == nullptr && obs_beside(a);
+    auto clear = [&] { return cudaMemsetAsync(a.fx, 0, (size_t)n * n * sizeof(unsigned long long), st); };
     if (phi == nullptr) {
         e = part != nullptr ? launch_phase<2>(a, part, alpha, beta, W, nullptr, 0, st)
                             : launch_phase<1>(a, nullptr, alpha, beta, W, nullptr, 0, st);
+        if (e == cudaSuccess && !beside) e = clear();
+        if (e == cudaSuccess && listed)
+            e = part != nullptr ? launch_obs<2>(a, part, alpha, beta, W, nullptr, 0, st)
+                                : launch_obs<1>(a, nullptr, alpha, beta, W, nullptr, 0, st);
+        if (e == cudaSuccess && beside) e = clear();
         if (e != cudaSuccess) return e;
-    }
-    if (!scale_set && (e = launch_fixed_scale(alpha, beta, a.l, s, lo_scale(a), st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(a.fx, 0, (size_t)n * n * sizeof(unsigned long long), st)) != cudaSuccess) return e;
-    if (phi != nullptr) {
+    } else {
+        if ((e = clear()) != cudaSuccess) return e;
         LaunchScope ls(IQP_KERNEL_LOWORDER, st);
         launch_pdl(k_lo_w, grid_1d(a.l * (a.lds / 4)), 256, 0, st, phi, ldphi, W, a.lds, a.l, s, alpha, beta);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    } else if (listed) {
-        e = part != nullptr ? launch_obs<2>(a, part, alpha, beta, W, nullptr, 0, st)
-                            : launch_obs<1>(a, nullptr, alpha, beta, W, nullptr, 0, st);
-        if (e != cudaSuccess) return e;
     }
     if (listed && (e = launch_k(a, W, st)) != cudaSuccess) return e;
     __nv_bfloat16 *hi = a.split, *lo = a.split + n * a.lds;
@@ -1550,9 +1584,9 @@ cudaError_t launch_lo_grad(const LoArgs &a, double2 *part, const double *alpha, 
     if (e != cudaSuccess) return e;
     {
         LaunchScope ls(IQP_KERNEL_LOWORDER, st);
-        k_lo_pairs<<<lo_heavy_blocks(a, nblk, kPairCtas), kBlk, 0, st>>>(a.A, a.lda, n, a.ZT, a.ldzt, a.E, lde, a.l,
-                                                                         lo_heavy(a), lo_nheavy(a), lo_items(a) + 1, W, a.lds, s, nblk,
-                                                                         lo_scale(a), a.fx, a.status);
+        k_lo_pairs<<<lo_heavy_blocks(a, nblk, kPairCtas), kBlk, 0, st>>>(
+            a.A, a.lda, n, a.ZT, a.ldzt, a.E, lde, a.l, lo_heavy(a), lo_nheavy(a), lo_items(a) + 1, W, a.lds, s, nblk,
+            lo_scale(a), a.fx, a.status);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (hparts > 1) {

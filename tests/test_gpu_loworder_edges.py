@@ -1,6 +1,7 @@
-"""Low-order form at the limits of its observable lists, 128 qubits and 256 pairs,
-against the FP64 oracle: observables one below, at and one above each, alone over
-the limit and beside listed ones, with sample counts that end inside a lane's four.
+"""Low-order form at the limits of its observable lists, 128 qubits (64 where
+the observables and samples are few) and 256 pairs, against the FP64 oracle:
+observables one below, at and one above each, alone over the limit and beside
+listed ones, with sample counts that end inside a lane's four.
 Tolerances are the form's own (1e-5 on estimates, 1e-4 relative on gradients)."""
 import numpy as np
 import pytest
@@ -30,9 +31,9 @@ def by_pairs():
     return gates, [np.arange(23 + j) for j in (2, 3, 4, 0, 3, 4)] + [np.arange(200, 240)]
 
 
-@pytest.mark.parametrize("s", [1021, 2050])
+@pytest.mark.parametrize("repeat,s", [(1, 1021), (1, 2050), (100, 1021)])
 @pytest.mark.parametrize("build,edges", [(by_qubits, [127, 128, 129]), (by_pairs, [255, 256, 257])], ids=["qubits", "pairs"])
-def test_limits_match_oracle(build, edges, s):
+def test_limits_match_oracle(build, edges, repeat, s):
     import torch
     from paper_2501_04776_gb300 import api
     gates, rows = build()
@@ -41,6 +42,7 @@ def test_limits_match_oracle(build, edges, s):
     sizes = [len(r) for r in rows]
     assert set(edges) <= set(sizes if build is by_qubits else inside)  # the edges are there ...
     assert max(inside if build is by_qubits else sizes) <= 100          # ... and the other limit is far
+    rows = rows * repeat
     bits = np.zeros((len(rows), N), dtype=np.uint8)
     for k, r in enumerate(rows):
         bits[k, r] = 1
