@@ -195,7 +195,7 @@ Plan make_plan(int op, int64_t n, int64_t m, int64_t l, int64_t s, int64_t N, in
         p.off_xpart = take(l * cdiv(s, (int64_t)kPartColsTc) * 16);
         p.off_xrow = take(grad ? l * 4 : 0);
         p.off_xw = take(grad ? 3 * x3_rows(l, p.ldw) * p.ldw * 2 : 0);
-        p.off_skp = take((int64_t)kMaxSplitCtas * kSplitSlotFloats * 4 + (int64_t)kMaxSplitCtas * 4);
+        p.off_skp = take((int64_t)kX3Slots * kSplitSlotFloats * 4);
         // running sums: only where the gates take more than one accumulation chunk
         p.off_xsum = take(m > kX3Gates ? (int64_t)kMaxSplitCtas * kSplitSlotFloats * 4 : 0);
         // Below 2^23 terms the SIMT kernels' estimates take as long as the

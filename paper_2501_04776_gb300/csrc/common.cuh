@@ -33,6 +33,7 @@ constexpr int64_t kDtSumFloats = 2 * 128 * 256;
 // FP32 form on the tensor cores: gates per accumulation chunk, and the
 // logarithm of the gradient's samples per chunk (tc.cu, x3_planes).
 constexpr int kX3Gates = 8192, kX3SampleBits = 14;
+constexpr int kX3Slots = 2 * kMaxSplitCtas;  // slots of its split tiles: 76 ranges over up to 75 tiles of CTA pairs
 // Observables whose W is held as three planes at a time: all of them up to 2 GiB
 // (3.5e8 samples of W), else whole tiles of 128, so that the FP32 form's scratch stays near the 4 bytes
 // per sample that W itself takes.

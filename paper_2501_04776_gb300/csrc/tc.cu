@@ -209,9 +209,13 @@ struct TcArgs {
     // bits stages of the tiles from `whole` on, laid end to end, are cut into
     // skP equal contiguous ranges, one per CTA group; unit u is piece u / skP
     // of range u % skP (the part of the range inside one tile; empty when the
-    // range has fewer pieces). The pieces of tile whole + t take the slots
-    // t * skKP + j, j = 0, 1, ... in range order.
-    int64_t skW, skP, skKP;
+    // range has fewer pieces). Range g's piece of tile whole + t takes slot g + t:
+    // one after the other in a tile, and from one piece to the next the range
+    // or the tile goes up, so that they fit skP + tiles - 1 slots. (With as many
+    // slots per tile as the most that one tile takes, 56 double tiles over 76
+    // ranges had no room and ran as 56 ranges: n = 5000, 10^6 gates, 4096 x 16384,
+    // phase 123 -> 131 ms.)
+    int64_t skW, skP;
     int64_t skcap;  // floats of split-part scratch at skp
 };
 
@@ -271,9 +275,7 @@ __device__ __forceinline__ void unit_of(int64_t u, const TcArgs &a, int nks, int
     ks0 = (KB / KS) * (int)(start - tt * nkb);
     const int64_t e = (KB / KS) * (end - tt * nkb);
     ks1 = e < nks ? (int)e : nks;
-    // the range holding the tile's first bits stage: the largest g0 with g0 W / P <= tt nkb
-    const int64_t g0 = ((tt * nkb + 1) * a.skP - 1) / a.skW;
-    v = tt * a.skKP + (g - g0);
+    v = g + tt;
 }
 
 // Split tile tt (from `whole` on): the number of its parts and the slot of the first.
@@ -282,7 +284,7 @@ __device__ __forceinline__ void part_info(int64_t tt, const TcArgs &a, int nks, 
     const int64_t g0 = ((tt * nkb + 1) * a.skP - 1) / a.skW;
     const int64_t g1 = ((tt + 1) * nkb * a.skP - 1) / a.skW;
     np = g1 - g0 + 1;
-    base = tt * a.skKP;
+    base = g0 + tt;
 }
 
 __device__ __forceinline__ uint8_t *aligned_smem(uint8_t *raw) {
@@ -2244,25 +2246,18 @@ bool balance(TcArgs &a, int64_t first, int64_t left, int64_t P, int cg, int nh, 
     const int64_t nkb = cdiv(a.nks, KB / KS), W = left * nkb;
     const double stage = nh == 2 ? kStageDtUs : kStageUs, cost = nh == 2 ? kSplitDtUs : kSplitUs;
     if (!split_tail() || skp == nullptr || left <= 0 || nkb < 2) return false;
-    if (!always && 2 * left > P && (double)(nkb * (P - left)) * stage <= cost * (double)P) return false;
     if (P > W) P = W;  // at least one bits stage per range
-    for (; P >= left && P >= 1; --P) {
-        int64_t KP = 1;
-        for (int64_t t = 0; t < left; ++t) {
-            const int64_t g0 = ((t * nkb + 1) * P - 1) / W, g1 = ((t + 1) * nkb * P - 1) / W;
-            if (g1 - g0 + 1 > KP) KP = g1 - g0 + 1;
-        }
-        if (left * KP * cg * nh > slots) continue;
-        a.whole = first;
-        a.nunits = P * (cdiv(W / P + 1, nkb) + 2);
-        a.skW = W;
-        a.skP = P;
-        a.skKP = KP;
-        a.skp = skp;
-        a.skcap = slots * kSplitSlotFloats;
-        return true;
-    }
-    return false;
+    const int64_t fit = slots / (cg * nh) - left + 1;  // P ranges over `left` tiles are at most P + left - 1 pieces
+    if (P > fit) P = fit;
+    if (P <= left) return false;
+    if (!always && 2 * left > P && (double)(nkb * (P - left)) * stage <= cost * (double)P) return false;
+    a.whole = first;
+    a.nunits = P * (cdiv(W / P + 1, nkb) + 2);
+    a.skW = W;
+    a.skP = P;
+    a.skp = skp;
+    a.skcap = slots * kSplitSlotFloats;
+    return true;
 }
 
 cudaError_t launch_split_reduce(int mode, bool x3, const TcArgs &a, int cg, int nh, int64_t tiles, cudaStream_t st) {
@@ -2441,7 +2436,7 @@ cudaError_t launch_phase_x3(int mode, const Plan &p, void *ws, const double *alp
         a.out = p.phi;
         a.ldo = p.ldphi;
     }
-    return launch_single_tiles(mode, 2, true, ma, mb, a, a.tiles_m * a.tiles_n, at<float>(ws, p.off_skp), kMaxSplitCtas, st);
+    return launch_single_tiles(mode, 2, true, ma, mb, a, a.tiles_m * a.tiles_n, at<float>(ws, p.off_skp), kX3Slots, st);
 }
 
 // Phase pass of the FP32 form's gradient where Phi was kept.
