@@ -460,13 +460,13 @@ def other_rows(args, lib, dev, st, timed, peaks, clocks, G, A, theta, w, n, m, l
     ms, _ = timed(None, args.steps, args.warmup, profile=True, fn=bitflip)
     kt = _kernel_times(lib)
     ldp, ldlt = -(-m // 256) * 4, -(-l // 256) * 4
-    # The sums of the logarithms (both calls, over P_A) and of the values
-    # (over P_A^T) read one 8-byte entry of a table in shared memory per four
-    # bits, whatever bits are set: 3 l m / 4 of them per call pair, against the
-    # shared memories' 128 bytes per clock. The bits themselves are a small
+    # The sums of the logarithms (both calls, over P_A) read one 8-byte entry of
+    # a table in shared memory per four bits, whatever bits are set, those of the
+    # values (over P_A^T) one of 8 and one of 4 bytes: 3 l m / 4 reads per call
+    # pair, against the shared memories' 128 bytes per clock. The bits themselves are a small
     # fraction of HBM time.
     nbytes = 8.0 * (l * ldp + m * ldlt)
-    lds_bytes = 2.0 * 64 * (2.0 * l * ldp + m * ldlt)
+    lds_bytes = 16.0 * (2.0 * 8 * l * ldp + 12 * m * ldlt)
     bf_ms = kt.get("bitflip", {}).get("total_ms", 0.0) / max(1, args.steps)
     mhz = (clocks or {}).get("sm_max_mhz") or 2070.0
     lds_peak = 152 * 128 * mhz * 1e6 / 1e9
