@@ -91,11 +91,13 @@ def _ws_bytes(op: int, n: int, m: int, l: int, s: int, N: int, prec: int) -> int
     return int(_lib.load().iqp_workspace_bytes(op, n, m, l, s, N, prec))
 
 
-def _scratch(op: int, n: int, m: int, l: int, s: int, N: int, prec: int, device, stream: int) -> torch.Tensor:
+def _scratch(op: int, n: int, m: int, l: int, s: int, N: int, prec: int, device, stream: int,
+             full_only: bool = False) -> torch.Tensor:
     """Workspace of an operation: of its full size, or, where the device has no
     room for that, of the smallest it runs with (the optional regions, which
-    are there for speed, are left out). A size that was refused is not asked for
-    again, since every refusal empties the allocator's cache."""
+    are there for speed, are left out); full_only: OutOfMemoryError then. A size
+    that was refused is not asked for again, since every refusal empties the
+    allocator's cache."""
     full = _ws_bytes(op, n, m, l, s, N, prec)
     key = (device.index, stream)
     if full < _WS.refused.get(key, full + 1):
@@ -103,6 +105,8 @@ def _scratch(op: int, n: int, m: int, l: int, s: int, N: int, prec: int, device,
             return _WS.get(full, device, stream)
         except torch.OutOfMemoryError:
             _WS.refused[key] = full
+    if full_only:
+        raise torch.OutOfMemoryError(f"no room for a workspace of {full} bytes")
     return _WS.get(int(_lib.load().iqp_workspace_min_bytes(op, n, m, l, s, N, prec)), device, stream)
 
 
@@ -284,7 +288,7 @@ def _planes_keep_phi(n, theta, G, A, Z):
     th = _theta32(theta)
     m, l, s = G.shape[0], A.shape[0], Z.shape[0]
     st = _stream(G.device)
-    ws = _WS.get(_ws_bytes(OP_EXPVAL, n, m, l, s, 0, FP32), G.device, st)
+    ws = _scratch(OP_EXPVAL, n, m, l, s, 0, FP32, G.device, st, full_only=True)
     ev = torch.empty(l, dtype=torch.float64, device=G.device)
     se = torch.empty(l, dtype=torch.float64, device=G.device)
     phi = torch.empty((l, phi_ld(s)), dtype=torch.float32, device=G.device)
@@ -301,7 +305,7 @@ def _planes_grad_from_phi(n, theta, G, A, Z, phi, alpha) -> torch.Tensor:
     m, l, s = G.shape[0], A.shape[0], Z.shape[0]
     al = _f64(alpha, G.device)
     st = _stream(G.device)
-    ws = _WS.get(_ws_bytes(OP_EXPVAL_GRAD, n, m, l, s, 0, FP32), G.device, st)
+    ws = _scratch(OP_EXPVAL_GRAD, n, m, l, s, 0, FP32, G.device, st, full_only=True)
     grad = torch.empty(m, dtype=torch.float64, device=G.device)
     check(_lib.load().iqp_planes_grad_from_phi(n, _ptr(G), m, G.shape[1], _ptr(A), l, A.shape[1], _ptr(Z), s,
                                                Z.shape[1], _ptr(th), _ptr(al), None, _ptr(phi), phi.shape[1],

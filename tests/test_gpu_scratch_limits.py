@@ -107,4 +107,5 @@ def test_a_refused_size_is_not_asked_for_again(tight):
     refused = tight((_lib.OP_EXPVAL, n, G.shape[0], A.shape[0], Z.shape[0], 0, _lib.FP32))
     for _ in range(3):
         api.expval_raw(n, th, G, A, Z, "fp32")
+        ev, _ = api.expval(th.clone().requires_grad_(True), G, A, Z, n, "fp32")  # would keep Phi, with the planes
     assert len(refused) == 1
